@@ -378,6 +378,7 @@ struct PCGState {
     double inv_gamma, inv_gamma_prev, inv_alpha, inv_alpha_prev;   // FP64 divisions are slow here
     double tot0[10];   // first pass's set-up sums [0, 10) (fixed during a solve; MG refinement reuses them)
     int it, it_total, conv;
+    int met;           // refinement: the FP64 residual has met the tolerance
 };
 
 // Scalar part of one CG update, thread 0 only: beta and alpha from gamma and
@@ -496,6 +497,7 @@ __global__ void __launch_bounds__(tile_threads<D, SH>(), 512 / tile_threads<D, S
         S.inv_gamma = S.inv_gamma_prev = S.inv_alpha = S.inv_alpha_prev = 1.0;
         it = 0;
         it_total = 0;
+        S.met = 0;
         if (A.warm)
             for (int v = 0; v < NV; v++) (refine ? E64 : XE)[v] = A.sc->E[v];
     }
@@ -608,19 +610,25 @@ __global__ void __launch_bounds__(tile_threads<D, SH>(), 512 / tile_threads<D, S
                 bnorm = sqrt(bbt);
                 rho_final = rho;
                 int ctl = CTL_RUN;
+                // refinement goes on to half the tolerance: its passes end
+                // anywhere below their targets, and a residual just under the
+                // tolerance would leave an error several times the usual one
+                const double res = sqrt(rho), tol = A.rtol * bnorm;
+                if (refine && res <= tol) S.met = 1;
                 if (bnorm == 0.0) ctl = CTL_ZERO;
-                else if (sqrt(rho) <= A.rtol * bnorm) ctl = CTL_DONE;
+                else if (res <= (refine ? 0.5 * tol : tol)) ctl = CTL_DONE;
                 // refinement that no longer halves the FP64 residual has
-                // reached what the FP32 passes can resolve: stop (not converged)
-                else if (refine && outer > 0 && sqrt(rho) > 0.5 * S.prev_res) ctl = CTL_STOP;
-                S.prev_res = sqrt(rho);
+                // reached what the FP32 passes can resolve: stop (not
+                // converged unless the tolerance is met)
+                else if (refine && outer > 0 && res > 0.5 * S.prev_res) ctl = S.met ? CTL_DONE : CTL_STOP;
+                S.prev_res = res;
                 // target of this pass: the requested tolerance, or in refinement
                 // mode what an FP32 iteration can deliver on this correction
                 // (eta); when the final tolerance is within a factor 100 of that,
                 // the pass aims for it directly, which saves a pass that would
                 // otherwise start just above the tolerance
                 if (refine) {
-                    const double fin = 0.5 * A.rtol * bnorm, pass = A.eta * sqrt(rho);
+                    const double fin = 0.25 * tol, pass = A.eta * res;
                     target = fin >= 0.01 * pass ? fin : pass;
                 } else {
                     target = A.rtol * bnorm;
@@ -958,7 +966,7 @@ __global__ void __launch_bounds__(tile_threads<D, SH>(), 512 / tile_threads<D, S
         Acc<T> dummy[1];
         double dres[1];
         if (!reduce_barrier<Acc<T>, 1>(dummy, A.partials, A.result, A.bar_count, A.bar_gen, err, dres, bid, nbk)) return;
-        if (stop == CTL_STOP) { if (lead) conv = false; break; }
+        if (stop == CTL_STOP) { if (lead) conv = S.met != 0; break; }
     }
     if (refine) {
         for (long long n = t0; n < N; n += st)
