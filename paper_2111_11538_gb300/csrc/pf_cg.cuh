@@ -37,6 +37,7 @@ template <> struct Tile<3, 0> { static constexpr int X = 16, Y = 4, Z = 4; };
 template <> struct Tile<3, 1> { static constexpr int X = 32, Y = 4, Z = 2; };
 constexpr int PCG_SHAPES = 2;
 
+constexpr int MG_MAX_LEVELS = 12;
 template <typename T> struct MGHier;
 
 template <typename T, int D>
@@ -63,6 +64,8 @@ struct PCGArgs {
     const MGHier<T> *mg;           // multigrid hierarchy (2D, k_pcg<..., MG = true> only)
     double *b64[3];                // MG refinement mode: the FP64 right-hand side, kept from the
                                    // first pass for the later ones
+    int zc1[MG_MAX_LEVELS], zc2[MG_MAX_LEVELS];   // 2D MG: rows per work item of a level's one- and
+                                                  // two-product sweeps (pf_march2.cuh)
 };
 
 // Grid barrier that also reduces K per-block values in a fixed order: the
@@ -421,6 +424,7 @@ enum { CTL_RUN = 0, CTL_DONE = 1, CTL_ZERO = 2, CTL_STOP = 3 };
 
 }  // namespace pfdev
 
+#include "pf_march2.cuh"
 #include "pf_mg.cuh"
 #include "pf_mg3.cuh"
 
@@ -432,6 +436,10 @@ namespace pfdev {
 // FP64, solves for a correction with the FP32 iteration (A.x holds the
 // correction), adds it in FP64, and stops when the FP64 residual meets rtol;
 // the FP32 displacement A.u is written from x64 at the end.
+// the hierarchy's place in shared memory, none without multigrid
+template <typename T, bool MG> struct MGStore { MGHier<T> h; };
+template <typename T> struct MGStore<T, false> {};
+
 template <int D, int S>
 constexpr int tile_threads() { return Tile<D, S>::X * Tile<D, S>::Y * Tile<D, S>::Z; }
 
@@ -455,17 +463,16 @@ __global__ void __launch_bounds__(tile_threads<D, SH>(), 512 / tile_threads<D, S
     constexpr int CX = TX + 1, CY = TY + 1, CZ = D == 3 ? TZ + 1 : 1;
     constexpr int HN = HX * HY * HZ, HC = CX * CY * CZ;
     constexpr int MAX_OUTER = 24;
-    // the node and cell tiles of the plain sweep (the 3D multigrid variant
-    // keeps its tiles in the dynamic shared memory)
-    constexpr bool Z3 = MG && D == 3;
-    __shared__ T su[Z3 ? 1 : D * HN];
-    __shared__ T sl[Z3 ? 1 : HC], sm[Z3 ? 1 : HC];
+    // the node and cell tiles of the plain sweep (the multigrid variants
+    // keep theirs in the dynamic shared memory)
+    __shared__ T su[MG ? 1 : D * HN];
+    __shared__ T sl[MG ? 1 : HC], sm[MG ? 1 : HC];
     // per-cell stress and hourglass forces: 2D 5 values per cell; 3D FP32 on
     // the 16x4x4 tile 20 (five float4); other 3D variants use the
     // element-matrix path and need none
     constexpr bool CELL3 = D == 3 && sizeof(T) == 4 && SH == 0;
-    __shared__ __align__(16) T scell2[D == 2 ? 5 * HC : 1];
-    extern __shared__ __align__(16) unsigned char pcg_dyn[];   // CELL3: 20 * HC floats; MG: block-run levels
+    __shared__ __align__(16) T scell2[D == 2 && !MG ? 5 * HC : 1];
+    // pcg_dyn, CELL3: 20 * HC floats; MG: block-run levels, sweeps
     T *scell = CELL3 ? reinterpret_cast<T *>(pcg_dyn) : scell2;
     __shared__ T s_ta, s_tb, s_ue[6], s_xe[6];
     __shared__ int s_ctl;
@@ -502,14 +509,22 @@ __global__ void __launch_bounds__(tile_threads<D, SH>(), 512 / tile_threads<D, S
             for (int v = 0; v < NV; v++) (refine ? E64 : XE)[v] = A.sc->E[v];
     }
 
-    // MG: the hierarchy descriptor (read only during the launch) stays in
-    // global memory; the coarse levels' moduli are rebuilt for this solve
-    // the block-run levels' arrays: dynamic shared memory (pcg_dyn_smem)
+    // MG: a copy of the hierarchy descriptor in shared memory (its pointers
+    // are read all over a V-cycle); the coarse levels' moduli are rebuilt for
+    // this solve; the block-run levels' arrays: dynamic shared memory
+    // (pcg_dyn_smem)
+    __shared__ MGStore<T, MG> sH;
     T *sblk = reinterpret_cast<T *>(pcg_dyn);
-    if constexpr (MG && D == 2) {
-        if (!mg_setup<T>(*A.mg, A.bar_count, A.bar_gen, err, bid, nbk)) return;
-    } else if constexpr (MG) {
-        if (!mg_setup3<T>(*A.mg, A.bar_count, A.bar_gen, err, bid, nbk)) return;
+    if constexpr (MG) {
+        const int *src = reinterpret_cast<const int *>(A.mg);
+        int *dst = reinterpret_cast<int *>(&sH.h);
+        for (int i = threadIdx.x; i < (int)(sizeof(MGHier<T>) / sizeof(int)); i += blockDim.x) dst[i] = src[i];
+        __syncthreads();
+        if constexpr (D == 2) {
+            if (!mg_setup<T>(sH.h, A.bar_count, A.bar_gen, err, bid, nbk)) return;
+        } else {
+            if (!mg_setup3<T>(sH.h, A.bar_count, A.bar_gen, err, bid, nbk)) return;
+        }
     }
 
     for (int outer = 0; outer < (refine ? MAX_OUTER : 1); outer++) {
@@ -661,9 +676,9 @@ __global__ void __launch_bounds__(tile_threads<D, SH>(), 512 / tile_threads<D, S
         if constexpr (MG) {
             int rc;
             if constexpr (D == 2)
-                rc = mg_pass<T, TX, TY>(A, *A.mg, S, su, sl, sm, scell, sblk, s_ta, s_tb, s_ue, s_ctl, bid, nbk, err);
+                rc = mg_pass<T, TX, TY>(A, sH.h, S, sblk, s_ta, s_tb, s_ue, s_ctl, bid, nbk, err);
             else
-                rc = mg_pass3<T>(A, *A.mg, S, reinterpret_cast<T *>(pcg_dyn), s_ta, s_tb, s_ue, s_ctl, bid, nbk, err);
+                rc = mg_pass3<T>(A, sH.h, S, reinterpret_cast<T *>(pcg_dyn), s_ta, s_tb, s_ue, s_ctl, bid, nbk, err);
             if (rc < 0) return;
             if (lead) conv = rc == CTL_DONE;
         } else {
@@ -991,19 +1006,16 @@ __global__ void __launch_bounds__(tile_threads<D, SH>(), 512 / tile_threads<D, S
 // tables (constant memory is per unit).  Dynamic shared memory: the 3D FP32
 // cell buffer of the 16x4x4 tile; with MG, the arrays of the block-run
 // levels (the bound for any hierarchy, so one attribute serves all), which
-// the FP64 set-up sweep uses as scratch before them, and the fused
-// two-step smoothing sweep's scratch.
+// the FP64 set-up sweep uses as scratch before them, and the operation
+// record of the marching sweeps.
 template <typename T, int D>
 size_t pcg_dyn_smem(int shape, bool mg)
 {
     if (D == 2 && mg) {
         // the block-run levels' arrays (or, before them in each pass, the
-        // set-up sweep's FP64 scratch), then the fused two-step sweep's scratch
-        if (shape == 1)
-            return mg_pair_offset<T, Tile<2, 1>::X, Tile<2, 1>::Y>() +
-                   sizeof(T) * (size_t)sweep2_words<Tile<2, 1>::X, Tile<2, 1>::Y>();
-        return mg_pair_offset<T, Tile<2, 0>::X, Tile<2, 0>::Y>() +
-               sizeof(T) * (size_t)sweep2_words<Tile<2, 0>::X, Tile<2, 0>::Y>();
+        // set-up sweep's FP64 scratch), then the sweeps' operation record
+        return shape == 1 ? mg_march_offset<T, Tile<2, 1>::X, Tile<2, 1>::Y>() + M2_OP_BYTES
+                          : mg_march_offset<T, Tile<2, 0>::X, Tile<2, 0>::Y>() + M2_OP_BYTES;
     }
     if (D == 3 && mg) {
         // the 3D V-cycle's sweeps (mg_sweep3z in T), or the set-up sweep's

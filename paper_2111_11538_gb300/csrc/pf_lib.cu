@@ -297,12 +297,19 @@ struct pf_handle {
     template <typename X>
     int alloc(X **ptr, size_t bytes_)
     {
+        return alloc_comps(ptr, 1, bytes_);
+    }
+    // ptr[0 .. n): n components of bytes_ each, one after the other
+    template <typename X>
+    int alloc_comps(X **ptr, int n, size_t each)
+    {
+        const size_t bytes_ = (size_t)n * each;
         void *v = nullptr;
         cudaError_t e = cudaMalloc(&v, bytes_ ? bytes_ : 16);
         if (e != cudaSuccess) return fail(PF_ENOMEM, "cudaMalloc(%zu): %s", bytes_, cudaGetErrorString(e));
         allocs.push_back(v);
         bytes += (long long)bytes_;
-        *ptr = (X *)v;
+        for (int k = 0; k < n; k++) ptr[k] = (X *)((unsigned char *)v + (size_t)k * each);
         return PF_OK;
     }
 };
@@ -471,15 +478,14 @@ int build_mg(pf_handle *h)
             PF_TRY(h->alloc(&V.lam, b));
             PF_TRY(h->alloc(&V.mu, b));
             PF_TRY(h->alloc(&V.dinv, b));
-            for (int c = 0; c < D; c++) PF_TRY(h->alloc(&V.f[c], b));
+            PF_TRY(h->alloc_comps(V.f, D, b));
         }
-        for (int c = 0; c < D; c++) {
-            PF_TRY(h->alloc(&V.xpost[c], b));
-            if (blk) continue;
-            PF_TRY(h->alloc(&V.xpre[c], b));
+        PF_TRY(h->alloc_comps(V.xpost, D, b));
+        if (!blk) {
+            PF_TRY(h->alloc_comps(V.xpre, D, b));
             for (int q = 0; q < 2; q++) {
-                PF_TRY(h->alloc(&V.r[q][c], b));
-                PF_TRY(h->alloc(&V.d[q][c], b));
+                PF_TRY(h->alloc_comps(V.r[q], D, b));
+                PF_TRY(h->alloc_comps(V.d[q], D, b));
             }
         }
         nx /= 2;
@@ -691,10 +697,20 @@ int build_plan(pf_handle *h)
         int g0 = 0;
         for (int i = 0; i < n; i++) {
             long long nb = 1 + (long long)((double)(cap - n) * work[i] / wtot);
-            if (nb > tiles[i]) nb = tiles[i] > 0 ? tiles[i] : 1;
+            // the marching sweeps of the 2D V-cycle share out single rows:
+            // a block for every 64 nodes in FP64 (its SM's FP64 pipe is what
+            // they wait for), for every 256 in FP32
+            const long long most = D == 2 && I[i]->mg ? (I[i]->P.N + (sizeof(T) == 8 ? 63 : 255)) / (sizeof(T) == 8 ? 64 : 256)
+                                                      : tiles[i];
+            if (nb > most) nb = most > 0 ? most : 1;
             pj[i] = pcg_args<T, D>(I[i]);
             pj[i].block0 = g0;
             pj[i].nblocks = (int)nb;
+            if (D == 2 && I[i]->mg)
+                for (int k = 0, nx = I[i]->P.nx, ny = I[i]->P.ny; k < mg_levels(I[i]->P.nx, I[i]->P.ny); k++, nx /= 2, ny /= 2) {
+                    pj[i].zc1[k] = m2_chunk(nx, ny, (int)nb, h->cg_block / 32, 30, 2, sizeof(T) == 8);
+                    pj[i].zc2[k] = m2_chunk(nx, ny, (int)nb, h->cg_block / 32, 28, 4, sizeof(T) == 8);
+                }
             g0 += (int)nb;
         }
         h->pcg_grid = g0;
@@ -1075,11 +1091,12 @@ int alloc_fields(pf_handle *h)
     if (h->cfg.mechanics) {
         PF_TRY(h->alloc(&h->lam, b)); PF_TRY(h->alloc(&h->mu, b));
         for (int v = 0; v < NV; v++) PF_TRY(h->alloc(&h->sig[v], b));
-        for (int d = 0; d < D; d++) {
-            PF_TRY(h->alloc(&h->p[d], b));
-            for (int k = 0; k < 2; k++) {
-                PF_TRY(h->alloc(&h->r[k][d], b)); PF_TRY(h->alloc(&h->w[k][d], b)); PF_TRY(h->alloc(&h->s[k][d], b));
-            }
+        // (the solver's sweeps address a vector's components by their distance)
+        PF_TRY(h->alloc_comps(h->p, D, b));
+        for (int k = 0; k < 2; k++) {
+            PF_TRY(h->alloc_comps(h->r[k], D, b));
+            PF_TRY(h->alloc_comps(h->w[k], D, b));
+            PF_TRY(h->alloc_comps(h->s[k], D, b));
         }
         PF_TRY(h->alloc(&h->result, sizeof(double) * 32));
         PF_TRY(h->alloc(&h->diag, b));

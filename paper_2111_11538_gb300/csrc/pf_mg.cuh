@@ -11,20 +11,18 @@
 // serves as a CG preconditioner.  The mean-strain dofs keep their Jacobi
 // scaling (block-diagonal preconditioner).
 //
-// Levels with more than a few tiles: every Chebyshev step is one sweep of
-// the tiled Q1 operator (the cell decomposition of cell_force2) and one grid
-// barrier.  Operands that are pointwise in stored vectors are formed while
-// the tile halo is staged (the Chebyshev direction from r and the previous
-// direction, the restricted residual, the prolonged correction, the CG
-// update), and the last step of a smoothing, which needs no operator
-// product, is applied in the epilogue of the step before it, so no sweep is
-// spent on either.  The coarse levels are run by the job's first block in
-// its shared memory (whole levels, one pass per phase, block barriers).
+// Levels beyond the block-run ones: a smoothing is one warp-marching sweep of
+// the Q1 operator (pf_march2.cuh) and one grid barrier.  Operands that are
+// pointwise in stored vectors are formed as the sweep reaches their row (the
+// restricted residual, the prolonged correction, the CG update), two steps
+// run in one sweep, and the last step of a smoothing, which needs no operator
+// product, is applied in the epilogue of the step before it.  The coarse
+// levels are run by the job's first block in its shared memory (whole levels,
+// one pass per phase, block barriers).
 #pragma once
 
 namespace pfdev {
 
-constexpr int MG_MAX_LEVELS = 12;
 constexpr int MG_MAX_STEPS = 16;
 
 template <typename T>
@@ -72,87 +70,6 @@ __device__ __forceinline__ bool grid_sync(unsigned int *count, unsigned int *gen
 
 __device__ __forceinline__ int mg_wrap(int a, int n, bool small) { return small ? wrapm(a, n) : wrap(a, n); }
 
-// One sweep of the level's Q1 operator over node tiles TX x TY: val(gx, gy, v)
-// gives the operand at any node (called for the tile and its halo), and
-// epi(n, v, q, se) receives, at each own node n, the operand v, q = A v and
-// (WITH_E) the own cell's average stress without the mean strain, the mean
-// strain ue being added to every cell's stress for q.
-template <typename T, int TX, int TY, bool WITH_E, class Val, class Epi>
-__device__ __forceinline__ void mg_sweep(int nx, int ny, const T *lam, const T *mu, int bid, int nbk, T *su, T *sl,
-                                         T *sm, T *scell, const T *ue, Val &&val, Epi &&epi)
-{
-    constexpr int HX = TX + 2, HY = TY + 2, CX = TX + 1, CY = TY + 1, HN = HX * HY, HC = CX * CY, NT = TX * TY;
-    const int ntx = (nx + TX - 1) / TX, nty = (ny + TY - 1) / TY, ntiles = ntx * nty;
-    const bool small = nx < HX || ny < HY;
-    const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
-    for (int tile = bid; tile < ntiles; tile += nbk) {
-        const int x0 = (tile % ntx) * TX, y0 = (tile / ntx) * TY;
-        for (int h = threadIdx.x; h < HN; h += NT) {
-            T v[2];
-            val(mg_wrap(x0 - 1 + h % HX, nx, small), mg_wrap(y0 - 1 + h / HX, ny, small), v);
-            su[h] = v[0];
-            su[HN + h] = v[1];
-        }
-        for (int h = threadIdx.x; h < HC; h += NT) {
-            const int g = mg_wrap(x0 - 1 + h % CX, nx, small) + nx * mg_wrap(y0 - 1 + h / CX, ny, small);
-            sl[h] = __ldcg(lam + g);
-            sm[h] = __ldcg(mu + g);
-        }
-        __syncthreads();
-        for (int h = threadIdx.x; h < HC; h += NT) {
-            const int cx = h % CX, cy = h / CX;
-            T uc[4][2];
-#pragma unroll
-            for (int b = 0; b < 4; b++) {
-                const int hn = (cx + (b & 1)) + HX * (cy + (b >> 1));
-                uc[b][0] = su[hn];
-                uc[b][1] = su[HN + hn];
-            }
-            const T l = sl[h], m = sm[h];
-            T s3[3], fh[2];
-            cell_force2<T>(l, m, uc, s3, fh);
-            if constexpr (WITH_E) {
-                T sx[3];
-                voigt_stress<T, 2>(l, m, ue, sx);
-#pragma unroll
-                for (int v = 0; v < 3; v++) s3[v] += sx[v];
-            }
-            scell[h] = s3[0];
-            scell[HC + h] = s3[1];
-            scell[2 * HC + h] = s3[2];
-            scell[3 * HC + h] = fh[0];
-            scell[4 * HC + h] = fh[1];
-        }
-        __syncthreads();
-        const int gx = x0 + tx, gy = y0 + ty;
-        if (gx < nx && gy < ny) {
-            const int lx = tx + 1, ly = ty + 1, hn = lx + HX * ly;
-            const T un[2] = {su[hn], su[HN + hn]};
-            T q[2] = {T(0), T(0)}, se[3] = {T(0), T(0), T(0)};
-#pragma unroll
-            for (int a = 0; a < 4; a++) {
-                const int cl = (lx - (a & 1)) + CX * (ly - (a >> 1));
-                const T s3[3] = {scell[cl], scell[HC + cl], scell[2 * HC + cl]};
-                const T fh[2] = {scell[3 * HC + cl], scell[4 * HC + cl]};
-                T f[2];
-                node_force2<T>(a, s3, fh, f);
-                q[0] += f[0];
-                q[1] += f[1];
-            }
-            if constexpr (WITH_E) {
-                const int c0 = lx + CX * ly;
-                T sx[3];
-                voigt_stress<T, 2>(sl[c0], sm[c0], ue, sx);
-                se[0] = scell[c0] - sx[0];
-                se[1] = scell[HC + c0] - sx[1];
-                se[2] = scell[2 * HC + c0] - sx[2];
-            }
-            epi(gx + nx * gy, un, q, se);
-        }
-        __syncthreads();
-    }
-}
-
 // Shared memory of the block-run levels [Lg, L), in words of T: per level 11
 // arrays of its node count (x, r, d, f by component, then the inverse
 // diagonal and the cell moduli), then the scratch of the largest level: the
@@ -178,7 +95,7 @@ __host__ __device__ inline long long mg_block_words(const MGHier<T> &H)
     return nmax ? w + MG_BLK_SCRATCH * nmax : 0;
 }
 
-__host__ __device__ inline long long mg_block_words_cap(long long nb)
+__host__ __device__ constexpr long long mg_block_words_cap(long long nb)
 {
     return MG_BLK_ARRAYS * (nb * 4 / 3 + 1) + MG_BLK_SCRATCH * nb;
 }
@@ -268,132 +185,6 @@ __device__ __forceinline__ void blk_sweep(const BLevel<T> &B, T *scr, int nmax, 
         epi(i, v, q);
     }
     __syncthreads();
-}
-
-// Shared memory (words of T) of mg_sweep2 for a TX x TY tile: two operands
-// on the width-2 halo, the intermediate residual and second operand on the
-// width-1 halo, and five values per cell of the width-2 halo.
-template <int TX, int TY>
-__host__ __device__ constexpr int sweep2_words()
-{
-    return 4 * (TX + 4) * (TY + 4) + 4 * (TX + 2) * (TY + 2) + 5 * (TX + 3) * (TY + 3);
-}
-
-// Two consecutive operator products on each tile with no grid barrier
-// between them (the ring of halo nodes both need is recomputed by the
-// neighbouring tiles): val(gx, gy, v0, a0) gives the first operand v0 and an
-// auxiliary a0 on the width-2 halo; mid(g, v0, a0, q0, r1, v1) forms, on the
-// width-1 halo, from v0, a0 and q0 = A v0, an intermediate r1 and the second
-// operand v1; epi(n, v0, a0, r1, v1, q1, se) gets q1 = A v1 at every own
-// node.  E2: the second product adds the mean strain ue to every cell's
-// stress and se is the own cell's stress of v1 without it (else zero).
-// Scratch: sweep2_words<TX, TY>() words of shared memory at scr.
-template <typename T, int TX, int TY, bool E2, class Val, class Mid, class Epi>
-__device__ __forceinline__ void mg_sweep2(int nx, int ny, const T *lam, const T *mu, int bid, int nbk, T *scr,
-                                          const T *ue, Val &&val, Mid &&mid, Epi &&epi)
-{
-    constexpr int AX = TX + 4, AY = TY + 4, AN = AX * AY;     // width-2 halo nodes
-    constexpr int BX = TX + 2, BY = TY + 2, BN = BX * BY;     // width-1 halo nodes
-    constexpr int CX = TX + 3, CY = TY + 3, CN = CX * CY;     // cells of the width-2 halo
-    constexpr int DX = TX + 1, DN = (TX + 1) * (TY + 1);      // cells of the width-1 halo
-    constexpr int NT = TX * TY;
-    T *v0 = scr, *a0 = scr + 2 * AN, *r1 = scr + 4 * AN, *v1 = r1 + 2 * BN, *cf = v1 + 2 * BN;
-    const int ntx = (nx + TX - 1) / TX, nty = (ny + TY - 1) / TY, ntiles = ntx * nty;
-    const bool small = nx < AX || ny < AY;
-    const int tx = threadIdx.x % TX, ty = threadIdx.x / TX;
-    auto cells = [&](const T *u, int ux, int un, int ncx, int ncell, int ox, int oy, bool withE) {
-        // cells with lower-left node (cx, cy) of the operand grid u (row
-        // length ux, un nodes per component), global origin (ox, oy)
-        for (int h = threadIdx.x; h < ncell; h += NT) {
-            const int cx = h % ncx, cy = h / ncx;
-            const int g = mg_wrap(ox + cx, nx, small) + nx * mg_wrap(oy + cy, ny, small);
-            T uc[4][2];
-#pragma unroll
-            for (int b = 0; b < 4; b++) {
-                const int hn = (cx + (b & 1)) + ux * (cy + (b >> 1));
-                uc[b][0] = u[hn];
-                uc[b][1] = u[un + hn];
-            }
-            T s3[3], fh[2];
-            const T l = __ldcg(lam + g), m = __ldcg(mu + g);
-            cell_force2<T>(l, m, uc, s3, fh);
-            if (E2 && withE) {
-                T sx[3];
-                voigt_stress<T, 2>(l, m, ue, sx);
-#pragma unroll
-                for (int v = 0; v < 3; v++) s3[v] += sx[v];
-            }
-            cf[h] = s3[0];
-            cf[CN + h] = s3[1];
-            cf[2 * CN + h] = s3[2];
-            cf[3 * CN + h] = fh[0];
-            cf[4 * CN + h] = fh[1];
-        }
-    };
-    auto force = [&](int lx, int ly, int ncx, T (&q)[2]) {
-        // q at the node whose lower-left cell is (lx, ly) in cell coordinates
-        q[0] = T(0);
-        q[1] = T(0);
-#pragma unroll
-        for (int a = 0; a < 4; a++) {
-            const int cl = (lx - (a & 1)) + ncx * (ly - (a >> 1));
-            const T s3[3] = {cf[cl], cf[CN + cl], cf[2 * CN + cl]};
-            const T fh[2] = {cf[3 * CN + cl], cf[4 * CN + cl]};
-            T f[2];
-            node_force2<T>(a, s3, fh, f);
-            q[0] += f[0];
-            q[1] += f[1];
-        }
-    };
-    for (int tile = bid; tile < ntiles; tile += nbk) {
-        const int x0 = (tile % ntx) * TX, y0 = (tile / ntx) * TY;
-        for (int h = threadIdx.x; h < AN; h += NT) {
-            T v[2], a[2];
-            val(mg_wrap(x0 - 2 + h % AX, nx, small), mg_wrap(y0 - 2 + h / AX, ny, small), v, a);
-            v0[h] = v[0];
-            v0[AN + h] = v[1];
-            a0[h] = a[0];
-            a0[AN + h] = a[1];
-        }
-        __syncthreads();
-        cells(v0, AX, AN, CX, CN, x0 - 2, y0 - 2, false);
-        __syncthreads();
-        for (int h = threadIdx.x; h < BN; h += NT) {
-            const int mx = h % BX, my = h / BX, ah = (mx + 1) + AX * (my + 1);
-            T q[2];
-            force(mx + 1, my + 1, CX, q);
-            const T vv[2] = {v0[ah], v0[AN + ah]}, aa[2] = {a0[ah], a0[AN + ah]};
-            T rr[2], ww[2];
-            mid(mg_wrap(x0 - 1 + mx, nx, small) + nx * mg_wrap(y0 - 1 + my, ny, small), vv, aa, q, rr, ww);
-            r1[h] = rr[0];
-            r1[BN + h] = rr[1];
-            v1[h] = ww[0];
-            v1[BN + h] = ww[1];
-        }
-        __syncthreads();
-        cells(v1, BX, BN, DX, DN, x0 - 1, y0 - 1, true);
-        __syncthreads();
-        const int gx = x0 + tx, gy = y0 + ty;
-        if (gx < nx && gy < ny) {
-            const int ah = (tx + 2) + AX * (ty + 2), bh = (tx + 1) + BX * (ty + 1);
-            T q[2];
-            force(tx + 1, ty + 1, DX, q);
-            const T vv[2] = {v0[ah], v0[AN + ah]}, aa[2] = {a0[ah], a0[AN + ah]};
-            const T rr[2] = {r1[bh], r1[BN + bh]}, ww[2] = {v1[bh], v1[BN + bh]};
-            const int n = gx + nx * gy;
-            T se[3] = {T(0), T(0), T(0)};
-            if constexpr (E2) {
-                const int c0 = (tx + 1) + DX * (ty + 1);
-                T sx[3];
-                voigt_stress<T, 2>(__ldcg(lam + n), __ldcg(mu + n), ue, sx);
-                se[0] = cf[c0] - sx[0];
-                se[1] = cf[CN + c0] - sx[1];
-                se[2] = cf[2 * CN + c0] - sx[2];
-            }
-            epi(n, vv, aa, rr, ww, q, se);
-        }
-        __syncthreads();
-    }
 }
 
 // Coarse level C from fine level F (both in global memory): cell moduli =
@@ -577,11 +368,11 @@ __device__ __forceinline__ void node_force2_df(int a, const DF (&s)[3], const DF
 template <int TX, int TY>
 __host__ __device__ constexpr int setup_tiled_doubles() { return 2 * (TX + 2) * (TY + 2) + 5 * (TX + 1) * (TY + 1); }
 
-// Byte offset of mg_sweep2's scratch in the dynamic shared memory: after
-// the block-run levels' arrays and the set-up sweep's scratch (which share
-// the start), rounded to 16 bytes.  The total is pcg_dyn_smem.
+// Byte offset of the sweeps' operation record in the dynamic shared
+// memory: after the block-run levels' arrays and the set-up sweep's scratch
+// (which share the start), rounded to 16 bytes.  The total is pcg_dyn_smem.
 template <typename T, int TX, int TY>
-__host__ __device__ constexpr size_t mg_pair_offset()
+__host__ __device__ constexpr size_t mg_march_offset()
 {
     const size_t blk = sizeof(T) * (size_t)mg_block_words_cap(mg_block_nodes<T>());
     const size_t stp = sizeof(double) * (size_t)setup_tiled_doubles<TX, TY>();
@@ -765,53 +556,57 @@ __device__ void setup_tiled(const PCGArgs<T, 2> &A, bool use_x, bool refine, boo
 //   w_i.u_i and the mean-strain row in one sweep and one reduction.
 // Returns CTL_DONE or CTL_STOP, or -1 when a barrier timed out.
 template <typename T, int TX, int TY>
-__device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, T *su, T *sl, T *sm, T *scell,
-                       T *sblk, T &s_ta, T &s_tb, T *s_ue, int &s_ctl, int bid, int nbk, int *err)
+__device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, T *sblk, T &s_ta, T &s_tb, T *s_ue,
+                       int &s_ctl, int bid, int nbk, int *err)
 {
-    constexpr int NV = 3;
+    constexpr int NV = 3, NT = TX * TY;
     const bool lead = threadIdx.x == 0;
     const int L = H.L, Lgw = H.Lg < H.L ? H.Lg : H.L, cs = H.csteps;
     const MGLevel<T> &L0 = H.lv[0];
     unsigned int *bc = A.bar_count, *bg = A.bar_gen;
+    // the sweeps' place in the dynamic shared memory; the operation's record
+    // there is filled by the lead thread (every sweep follows a barrier of the
+    // whole block) and read by all
+    constexpr size_t OFF = mg_march_offset<T, TX, TY>();
+    unsigned char *s_op = pcg_dyn + OFF;
 
     // ---- grid levels --------------------------------------------------
-    // Chebyshev step j on level k: d_j on the halo from buffer par, then
-    // X += d_j, r_{j+1} = r_j - A d_j into buffer 1 - par.  last: apply
+    // Chebyshev step j >= 1 of the pre-smoothing on level k: d_j from buffer
+    // par, x += d_j, r_{j+1} = r_j - A d_j into buffer 1 - par.  last: apply
     // step j + 1 too (pointwise) and leave the final correction in xpost.
-    auto cheb = [&](int k, int j, int par, bool post, bool last) {
+    auto cheb = [&](int k, int j, int par, bool last) {
         const MGLevel<T> &V = H.lv[k];
-        T *const *X = post ? V.xpost : V.xpre;
-        const T c1 = H.c1[j], c2 = H.c2[j], n1 = H.c1[j + 1], n2 = H.c2[j + 1];
-        mg_sweep<T, TX, TY, false>(
-            V.nx, V.ny, V.lam, V.mu, bid, nbk, su, sl, sm, scell, nullptr,
-            [&](int gx, int gy, T (&v)[2]) {
-                const int g = gx + V.nx * gy;
-                const T di = c2 * __ldcg(V.dinv + g);
-#pragma unroll
-                for (int c = 0; c < 2; c++) {
-                    T a = di * __ldcg(V.r[par][c] + g);
-                    if (j > 0) a += c1 * __ldcg(V.d[par][c] + g);
-                    v[c] = a;
-                }
-            },
-            [&](int n, const T (&v)[2], const T (&q)[2], const T (&)[3]) {
-                const T di = last ? n2 * __ldcg(V.dinv + n) : T(0);
-#pragma unroll
-                for (int c = 0; c < 2; c++) {
-                    const T x = __ldcg(X[c] + n) + v[c];
-                    const T rn = __ldcg(V.r[par][c] + n) - q[c];
-                    if (last) {
-                        V.xpost[c][n] = x + (n1 * v[c] + di * rn);
-                    } else {
-                        X[c][n] = x;
-                        V.r[1 - par][c][n] = rn;
-                        V.d[1 - par][c][n] = v[c];
-                    }
-                }
-            });
+        OpCheb2<T> &op = *reinterpret_cast<OpCheb2<T> *>(s_op);
+        static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
+        if (lead) {
+            op.lam = V.lam; op.mu = V.mu; op.dinv = V.dinv; op.n = V.nx * V.ny;
+            op.r = V.r[par][0]; op.d = V.d[par][0]; op.xi = V.xpre[0];
+            op.xo = last ? V.xpost[0] : V.xpre[0];
+            op.rn = V.r[1 - par][0]; op.dn = V.d[1 - par][0];
+            op.c1 = H.c1[j]; op.c2 = H.c2[j]; op.n1 = H.c1[j + 1]; op.n2 = H.c2[j + 1];
+            op.last = last;
+        }
+        __syncthreads();
+        m2_sweep<T, NT, OFF, OpCheb2<T>>(V.nx, V.ny, A.zc1[k], bid, nbk);
+    };
+    auto restrict_of = [&](int k) {
+        const MGLevel<T> &F = H.lv[k - 1];
+        const int pf = H.deg[k - 1] & 1;
+        Restrict2<T> R;
+        R.r = F.r[pf][0];
+        R.fnx = F.nx; R.fny = F.ny;
+        return R;
+    };
+    auto prolong_of = [&](int k) {
+        const MGLevel<T> &C = H.lv[k + 1];
+        Prolong2<T> P;
+        P.x = C.xpost[0];
+        P.cnx = C.nx; P.cny = C.ny;
+        return P;
     };
     // restriction (transpose of bilinear prolongation) of grid level k-1's
-    // residual after its pre-smoothing, at node (gx, gy) of level k
+    // residual after its pre-smoothing, at node (gx, gy) of level k (the top
+    // block-run level's right-hand side)
     auto restrict_g = [&](int k, int gx, int gy, T (&f)[2]) {
         const MGLevel<T> &F = H.lv[k - 1];
         const int pf = H.deg[k - 1] & 1;
@@ -830,175 +625,52 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
             }
         }
     };
-    // first pre-smoothing sweep of a grid level k >= 1: f = R r_{k-1}, x = d_0
-    auto pre_first = [&](int k) {
+    // post-smoothing of a grid level k >= 1 (two steps, one sweep)
+    auto post = [&](int k) {
         const MGLevel<T> &V = H.lv[k];
-        const T c2 = H.c2[0];
-        mg_sweep<T, TX, TY, false>(
-            V.nx, V.ny, V.lam, V.mu, bid, nbk, su, sl, sm, scell, nullptr,
-            [&](int gx, int gy, T (&v)[2]) {
-                T f[2];
-                restrict_g(k, gx, gy, f);
-                const T di = c2 * __ldcg(V.dinv + gx + V.nx * gy);
-                v[0] = di * f[0];
-                v[1] = di * f[1];
-            },
-            [&](int n, const T (&v)[2], const T (&q)[2], const T (&)[3]) {
-                T f[2];
-                restrict_g(k, n % V.nx, n / V.nx, f);
-#pragma unroll
-                for (int c = 0; c < 2; c++) {
-                    V.f[c][n] = f[c];
-                    V.xpre[c][n] = v[c];
-                    V.r[1][c][n] = f[c] - q[c];
-                    V.d[1][c][n] = v[c];
-                }
-            });
-    };
-    // first post-smoothing sweep of grid level k: x = x_pre + P e_{k+1}
-    // (e: level k+1's final correction), r = f - A x; last (one-step
-    // smoothing): apply that step, x + c2[0] D^-1 r, as the final correction
-    auto post_first = [&](int k, int par, int cur, bool last) {
-        const MGLevel<T> &V = H.lv[k];
-        const MGLevel<T> &C = H.lv[k + 1];
-        mg_sweep<T, TX, TY, false>(
-            V.nx, V.ny, V.lam, V.mu, bid, nbk, su, sl, sm, scell, nullptr,
-            [&](int gx, int gy, T (&v)[2]) {
-                const int g = gx + V.nx * gy;
-                const int ox = gx & 1, oy = gy & 1, ix = gx >> 1, iy = gy >> 1;
-                const T w = (ox && oy) ? T(0.25) : ((ox || oy) ? T(0.5) : T(1));
-                const int ix1 = ox ? (ix + 1 == C.nx ? 0 : ix + 1) : ix, iy1 = oy ? (iy + 1 == C.ny ? 0 : iy + 1) : iy;
-                const int c00 = ix + C.nx * iy, c10 = ix1 + C.nx * iy, c01 = ix + C.nx * iy1, c11 = ix1 + C.nx * iy1;
-#pragma unroll
-                for (int c = 0; c < 2; c++) {
-                    T e = __ldcg(C.xpost[c] + c00);
-                    if (ox) e += __ldcg(C.xpost[c] + c10);
-                    if (oy) e += __ldcg(C.xpost[c] + c01);
-                    if (ox && oy) e += __ldcg(C.xpost[c] + c11);
-                    v[c] = __ldcg(V.xpre[c] + g) + w * e;
-                }
-            },
-            [&](int n, const T (&v)[2], const T (&q)[2], const T (&)[3]) {
-                const T di = last ? H.c2[0] * __ldcg(V.dinv + n) : T(0);
-#pragma unroll
-                for (int c = 0; c < 2; c++) {
-                    const T f = k == 0 ? __ldcg(A.r[cur][c] + n) : __ldcg(V.f[c] + n);
-                    if (last) {
-                        V.xpost[c][n] = v[c] + di * (f - q[c]);
-                    } else {
-                        V.xpost[c][n] = v[c];
-                        V.r[1 - par][c][n] = f - q[c];
-                    }
-                }
-            });
-    };
-    // Two-step smoothing of a grid level k >= 1 in one fused sweep (degree 2,
-    // not the coarsest): pre-smoothing from f = R r_{k-1} (x = d_0 + d_1,
-    // r_2 and d_1 into buffer 0, which the restriction to level k+1 reads),
-    // and post-smoothing from x_pre + P e_{k+1} with the final correction
-    // into xpost.
-    T *s2 = reinterpret_cast<T *>(reinterpret_cast<unsigned char *>(sblk) + mg_pair_offset<T, TX, TY>());
-    auto pre2 = [&](int k) {
-        const MGLevel<T> &V = H.lv[k];
-        const T c20 = H.c2[0], c11 = H.c1[1], c21 = H.c2[1];
-        mg_sweep2<T, TX, TY, false>(
-            V.nx, V.ny, V.lam, V.mu, bid, nbk, s2, nullptr,
-            [&](int gx, int gy, T (&v)[2], T (&a)[2]) {
-                restrict_g(k, gx, gy, a);
-                const T di = c20 * __ldcg(V.dinv + gx + V.nx * gy);
-                v[0] = di * a[0];
-                v[1] = di * a[1];
-            },
-            [&](int g, const T (&v)[2], const T (&a)[2], const T (&q)[2], T (&r)[2], T (&w)[2]) {
-                const T di = c21 * __ldcg(V.dinv + g);
-#pragma unroll
-                for (int c = 0; c < 2; c++) {
-                    r[c] = a[c] - q[c];
-                    w[c] = c11 * v[c] + di * r[c];
-                }
-            },
-            [&](int n, const T (&v)[2], const T (&a)[2], const T (&r)[2], const T (&w)[2], const T (&q)[2],
-                const T (&)[3]) {
-#pragma unroll
-                for (int c = 0; c < 2; c++) {
-                    V.f[c][n] = a[c];
-                    V.xpre[c][n] = v[c] + w[c];
-                    V.r[0][c][n] = r[c] - q[c];
-                    V.d[0][c][n] = w[c];
-                }
-            });
-    };
-    auto post2 = [&](int k) {
-        const MGLevel<T> &V = H.lv[k];
-        const MGLevel<T> &C = H.lv[k + 1];
-        const T c20 = H.c2[0], c11 = H.c1[1], c21 = H.c2[1];
-        mg_sweep2<T, TX, TY, false>(
-            V.nx, V.ny, V.lam, V.mu, bid, nbk, s2, nullptr,
-            [&](int gx, int gy, T (&v)[2], T (&a)[2]) {
-                const int g = gx + V.nx * gy;
-                const int ox = gx & 1, oy = gy & 1, ix = gx >> 1, iy = gy >> 1;
-                const T wgt = (ox && oy) ? T(0.25) : ((ox || oy) ? T(0.5) : T(1));
-                const int ix1 = ox ? (ix + 1 == C.nx ? 0 : ix + 1) : ix, iy1 = oy ? (iy + 1 == C.ny ? 0 : iy + 1) : iy;
-                const int c00 = ix + C.nx * iy, c10 = ix1 + C.nx * iy, c01 = ix + C.nx * iy1, c11i = ix1 + C.nx * iy1;
-#pragma unroll
-                for (int c = 0; c < 2; c++) {
-                    T e = __ldcg(C.xpost[c] + c00);
-                    if (ox) e += __ldcg(C.xpost[c] + c10);
-                    if (oy) e += __ldcg(C.xpost[c] + c01);
-                    if (ox && oy) e += __ldcg(C.xpost[c] + c11i);
-                    v[c] = __ldcg(V.xpre[c] + g) + wgt * e;
-                    a[c] = __ldcg(V.f[c] + g);
-                }
-            },
-            [&](int g, const T (&v)[2], const T (&a)[2], const T (&q)[2], T (&r)[2], T (&w)[2]) {
-                const T di = c20 * __ldcg(V.dinv + g);
-#pragma unroll
-                for (int c = 0; c < 2; c++) {
-                    r[c] = a[c] - q[c];
-                    w[c] = di * r[c];
-                }
-            },
-            [&](int n, const T (&v)[2], const T (&)[2], const T (&r)[2], const T (&w)[2], const T (&q)[2],
-                const T (&)[3]) {
-                const T di = c21 * __ldcg(V.dinv + n);
-#pragma unroll
-                for (int c = 0; c < 2; c++) V.xpost[c][n] = v[c] + w[c] + (c11 * w[c] + di * (r[c] - q[c]));
-            });
-    };
-    // the fused form serves grid levels with two-step smoothing
-    auto fused = [&](int k) { return k >= 1 && k < L - 1 && H.deg[k] == 2; };
-
-    // post-smoothing of grid level k
-    auto post = [&](int k, int cur) {
-        if (fused(k)) {
-            post2(k);
-            return grid_sync(bc, bg, err, nbk);
+        OpPostPair2<T> &op = *reinterpret_cast<OpPostPair2<T> *>(s_op);
+        static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
+        if (lead) {
+            op.lam = V.lam; op.mu = V.mu; op.dinv = V.dinv; op.n = V.nx * V.ny;
+            op.f = V.f[0]; op.xpre = V.xpre[0]; op.xpost = V.xpost[0];
+            op.P = prolong_of(k);
+            op.c20 = H.c2[0]; op.c11 = H.c1[1]; op.c21 = H.c2[1];
         }
-        const int dk = H.deg[k];
-        int par = dk & 1;
-        post_first(k, par, cur, dk == 1);
-        if (!grid_sync(bc, bg, err, nbk)) return false;
-        par ^= 1;
-        for (int j = 0; j + 1 < dk; j++) {
-            cheb(k, j, par, true, j + 2 == dk);
-            if (!grid_sync(bc, bg, err, nbk)) return false;
-            par ^= 1;
-        }
-        return true;
+        __syncthreads();
+        m2_sweep2<T, NT, OFF, OpPostPair2<T>>(V.nx, V.ny, A.zc2[k], bid, nbk);
+        return grid_sync(bc, bg, err, nbk);
     };
-    // pre-smoothing (or the coarsest solve, csteps >= 3) of grid level k >= 1
+    // pre-smoothing of grid level k >= 1 (two steps, one sweep), or the
+    // coarsest solve (csteps >= 3) if the coarsest level is a grid level
     auto pre = [&](int k) {
-        if (fused(k)) {
-            pre2(k);
+        const MGLevel<T> &V = H.lv[k];
+        if (k < L - 1) {
+            OpPrePair2<T> &op = *reinterpret_cast<OpPrePair2<T> *>(s_op);
+            static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
+            if (lead) {
+                op.lam = V.lam; op.mu = V.mu; op.dinv = V.dinv; op.n = V.nx * V.ny;
+                op.f = V.f[0]; op.xpre = V.xpre[0]; op.r2 = V.r[0][0];
+                op.Rs = restrict_of(k);
+                op.c20 = H.c2[0]; op.c11 = H.c1[1]; op.c21 = H.c2[1];
+            }
+            __syncthreads();
+            m2_sweep2<T, NT, OFF, OpPrePair2<T>>(V.nx, V.ny, A.zc2[k], bid, nbk);
             return grid_sync(bc, bg, err, nbk);
         }
-        pre_first(k);
+        OpPre2<T> &op = *reinterpret_cast<OpPre2<T> *>(s_op);
+        static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
+        if (lead) {
+            op.lam = V.lam; op.mu = V.mu; op.dinv = V.dinv; op.n = V.nx * V.ny;
+            op.f = V.f[0]; op.xpre = V.xpre[0]; op.r1 = V.r[1][0]; op.d1 = V.d[1][0];
+            op.Rs = restrict_of(k);
+            op.c2 = H.c2[0];
+        }
+        __syncthreads();
+        m2_sweep<T, NT, OFF, OpPre2<T>>(V.nx, V.ny, A.zc1[k], bid, nbk);
         if (!grid_sync(bc, bg, err, nbk)) return false;
         int par = 1;
-        const bool co = k == L - 1;
-        const int nk = co ? cs - 1 : H.deg[k];
-        for (int j = 1; j < nk; j++) {
-            cheb(k, j, par, false, co && j + 1 == nk);
+        for (int j = 1; j < cs - 1; j++) {
+            cheb(k, j, par, j + 2 == cs);
             if (!grid_sync(bc, bg, err, nbk)) return false;
             par ^= 1;
         }
@@ -1129,43 +801,21 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
 
         // ---- finest level, first pre-smoothing sweep; from the second
         // iteration on its own nodes also take the CG update
-        //   p = u + beta p, s = w + beta s, x += alpha p, r -= alpha s
-        // (u: the previous V-cycle's result, in L0.xpost) and the halo uses
-        // the updated r formed on the fly
         Acc<T> racc[1];
         {
-            const T c2 = H.c2[0];
-            mg_sweep<T, TX, TY, false>(
-                L0.nx, L0.ny, L0.lam, L0.mu, bid, nbk, su, sl, sm, scell, nullptr,
-                [&](int gx, int gy, T (&v)[2]) {
-                    const int g = gx + L0.nx * gy;
-                    const T di = c2 * __ldcg(L0.dinv + g);
-#pragma unroll
-                    for (int c = 0; c < 2; c++) {
-                        T rv = __ldcg(A.r[cur][c] + g);
-                        if (!first) rv -= ta * (__ldcg(A.w[cur][c] + g) + tb * __ldcg(A.s[cur][c] + g));
-                        v[c] = di * rv;
-                    }
-                },
-                [&](int n, const T (&v)[2], const T (&q)[2], const T (&)[3]) {
-#pragma unroll
-                    for (int c = 0; c < 2; c++) {
-                        T f = __ldcg(A.r[cur][c] + n);
-                        if (!first) {
-                            const T si = __ldcg(A.w[cur][c] + n) + tb * __ldcg(A.s[cur][c] + n);
-                            const T pi = __ldcg(L0.xpost[c] + n) + tb * A.p[c][n];
-                            A.p[c][n] = pi;
-                            A.x[c][n] = A.x[c][n] + ta * pi;
-                            A.s[nxt][c][n] = si;
-                            f = f - ta * si;
-                            A.r[nxt][c][n] = f;
-                            racc[0].fma_plain(f, f);
-                        }
-                        L0.xpre[c][n] = v[c];
-                        L0.r[1][c][n] = f - q[c];
-                        L0.d[1][c][n] = v[c];
-                    }
-                });
+            OpFirst2<T> &op = *reinterpret_cast<OpFirst2<T> *>(s_op);
+            static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
+            if (lead) {
+                op.lam = L0.lam; op.mu = L0.mu; op.dinv = L0.dinv; op.n = L0.nx * L0.ny;
+                op.r = A.r[cur][0]; op.w = A.w[cur][0]; op.s = A.s[cur][0]; op.u = L0.xpost[0];
+                op.p = A.p[0]; op.x[0] = A.x[0]; op.x[1] = A.x[1]; op.sn = A.s[nxt][0]; op.rn = A.r[nxt][0];
+                op.xpre = L0.xpre[0]; op.r1 = L0.r[1][0]; op.d1 = L0.d[1][0];
+                op.ta = ta; op.tb = tb; op.c2 = H.c2[0];
+                op.upd = !first;
+                op.dir = L == 1;
+            }
+            __syncthreads();
+            racc[0] = m2_sweep<T, NT, OFF, OpFirst2<T>>(L0.nx, L0.ny, A.zc1[0], bid, nbk);
         }
         if (!first) {
             double tr[1];
@@ -1188,12 +838,11 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
             return -1;
         }
 
-        // ---- rest of the V-cycle
-        {
+        // ---- rest of the V-cycle (one-level hierarchies: the coarsest solve)
+        if (L == 1) {
             int par = 1;
-            const int n0 = L == 1 ? cs - 1 : H.deg[0];
-            for (int j = 1; j < n0; j++) {
-                cheb(0, j, par, false, L == 1 && j + 1 == n0);
+            for (int j = 1; j < cs - 1; j++) {
+                cheb(0, j, par, j + 2 == cs);
                 if (!grid_sync(bc, bg, err, nbk)) return -1;
                 par ^= 1;
             }
@@ -1213,75 +862,39 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
             }
             if (!grid_sync(bc, bg, err, nbk)) return -1;
         }
-        // the finest level's one-step post-smoothing fuses with the next sweep
-        const bool fuse0 = L > 1 && H.deg[0] == 1;
-        for (int k = (Lgw < L - 1 ? Lgw : L - 1) - 1; k >= (fuse0 ? 1 : 0); k--)
-            if (!post(k, cur)) return -1;
+        for (int k = (Lgw < L - 1 ? Lgw : L - 1) - 1; k >= 1; k--)
+            if (!post(k)) return -1;
 
-        // ---- u = V-cycle result, w = A u (+ mean strain), gamma, delta, mean-strain row
+        // ---- u = V-cycle result (the finest level's one-step post-smoothing,
+        // fused), w = A u (+ mean strain), gamma, delta, mean-strain row
         Acc<T> acc[2 + NV];
-        if (fuse0) {
-            // x = x_pre + P e_1, r = f - A x (f: the CG residual), u = x + c2[0] D^-1 r
-            // on the width-1 ring, then w = A u on the tile
-            const MGLevel<T> &C = H.lv[1];
-            const T c20 = H.c2[0];
-            mg_sweep2<T, TX, TY, true>(
-                L0.nx, L0.ny, L0.lam, L0.mu, bid, nbk,
-                reinterpret_cast<T *>(reinterpret_cast<unsigned char *>(sblk) + mg_pair_offset<T, TX, TY>()), s_ue,
-                [&](int gx, int gy, T (&v)[2], T (&a)[2]) {
-                    const int g = gx + L0.nx * gy;
-                    const int ox = gx & 1, oy = gy & 1, ix = gx >> 1, iy = gy >> 1;
-                    const T wgt = (ox && oy) ? T(0.25) : ((ox || oy) ? T(0.5) : T(1));
-                    const int ix1 = ox ? (ix + 1 == C.nx ? 0 : ix + 1) : ix, iy1 = oy ? (iy + 1 == C.ny ? 0 : iy + 1) : iy;
-                    const int c00 = ix + C.nx * iy, c10 = ix1 + C.nx * iy, c01 = ix + C.nx * iy1, c11 = ix1 + C.nx * iy1;
-#pragma unroll
-                    for (int c = 0; c < 2; c++) {
-                        T e = __ldcg(C.xpost[c] + c00);
-                        if (ox) e += __ldcg(C.xpost[c] + c10);
-                        if (oy) e += __ldcg(C.xpost[c] + c01);
-                        if (ox && oy) e += __ldcg(C.xpost[c] + c11);
-                        v[c] = __ldcg(L0.xpre[c] + g) + wgt * e;
-                        a[c] = __ldcg(A.r[cur][c] + g);
-                    }
-                },
-                [&](int g, const T (&v)[2], const T (&a)[2], const T (&q)[2], T (&r)[2], T (&w)[2]) {
-                    const T di = c20 * __ldcg(L0.dinv + g);
-#pragma unroll
-                    for (int c = 0; c < 2; c++) {
-                        r[c] = a[c] - q[c];
-                        w[c] = v[c] + di * r[c];
-                    }
-                },
-                [&](int n, const T (&)[2], const T (&a)[2], const T (&)[2], const T (&u)[2], const T (&q)[2],
-                    const T (&se)[3]) {
-#pragma unroll
-                    for (int c = 0; c < 2; c++) {
-                        L0.xpost[c][n] = u[c];
-                        A.w[cur][c][n] = q[c];
-                        acc[0].fma_plain(a[c], u[c]);
-                        acc[1].fma_plain(q[c], u[c]);
-                    }
-#pragma unroll
-                    for (int vv = 0; vv < NV; vv++) acc[2 + vv].add_plain(se[vv]);
-                });
+        auto take = [&](const Sums2<T> &sums) {
+            acc[0] = sums.ru;
+            acc[1] = sums.wu;
+            for (int v = 0; v < 3; v++) acc[2 + v].s = T(2) * sums.se[v].s;     // twice half of each cell's stress
+        };
+        if (L > 1) {
+            OpFine2<T> &op = *reinterpret_cast<OpFine2<T> *>(s_op);
+            static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
+            if (lead) {
+                op.lam = L0.lam; op.mu = L0.mu; op.dinv = L0.dinv; op.n = L0.nx * L0.ny;
+                op.r = A.r[cur][0]; op.xpre = L0.xpre[0]; op.u = L0.xpost[0]; op.w = A.w[cur][0];
+                for (int v = 0; v < 3; v++) op.ue[v] = s_ue[v];
+                op.P = prolong_of(0);
+                op.c20 = H.c2[0];
+            }
+            __syncthreads();
+            take(m2_sweep2<T, NT, OFF, OpFine2<T>>(L0.nx, L0.ny, A.zc2[0], bid, nbk));
         } else {
-            mg_sweep<T, TX, TY, true>(
-                L0.nx, L0.ny, L0.lam, L0.mu, bid, nbk, su, sl, sm, scell, s_ue,
-                [&](int gx, int gy, T (&v)[2]) {
-                    const int g = gx + L0.nx * gy;
-                    v[0] = __ldcg(L0.xpost[0] + g);
-                    v[1] = __ldcg(L0.xpost[1] + g);
-                },
-                [&](int n, const T (&v)[2], const T (&q)[2], const T (&se)[3]) {
-#pragma unroll
-                    for (int c = 0; c < 2; c++) {
-                        A.w[cur][c][n] = q[c];
-                        acc[0].fma_plain(__ldcg(A.r[cur][c] + n), v[c]);
-                        acc[1].fma_plain(q[c], v[c]);
-                    }
-#pragma unroll
-                    for (int vv = 0; vv < NV; vv++) acc[2 + vv].add_plain(se[vv]);
-                });
+            OpApply2<T> &op = *reinterpret_cast<OpApply2<T> *>(s_op);
+            static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
+            if (lead) {
+                op.lam = L0.lam; op.mu = L0.mu; op.n = L0.nx * L0.ny;
+                op.u = L0.xpost[0]; op.r = A.r[cur][0]; op.w = A.w[cur][0];
+                for (int v = 0; v < 3; v++) op.ue[v] = s_ue[v];
+            }
+            __syncthreads();
+            take(m2_sweep<T, NT, OFF, OpApply2<T>>(L0.nx, L0.ny, A.zc1[0], bid, nbk));
         }
         double tt[2 + NV];
         if (!reduce_barrier<Acc<T>, 2 + NV>(acc, A.partials, A.result, A.bar_count, A.bar_gen, err, tt, bid, nbk)) return -1;
