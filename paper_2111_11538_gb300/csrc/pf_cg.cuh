@@ -68,57 +68,114 @@ struct PCGArgs {
                                                   // two-product sweeps (pf_march2.cuh)
 };
 
-// Grid barrier that also reduces K per-block values in a fixed order: the
-// last block to arrive sums the partials (warp 0, lane-strided over blocks,
-// then a butterfly) and publishes them before releasing the others.  After
-// the call thread 0 holds the totals in out[].  Waits are bounded
-// (SPIN_LIMIT polls, then PF_ETIMEOUT in *err and false is returned).
+// Grid barrier that also reduces K per-thread values: the warps of a block
+// reduce them, one warp per value combines the warps' and writes the block's
+// partial, and after the barrier every block sums all partials in the same
+// fixed order, again one warp per value.  (The last block to arrive used to
+// sum them before it released the others, one warp for all values: a second
+// trip through L2 for every other block and K reductions in a row.)  After
+// the call every thread may read the totals in out[], which stay until the
+// block's next call.  FP32 values are reduced as error-free (hi, lo) pairs.
+// `region` picks one of PCG_REGIONS sets of partials: a set may be written
+// again only after another barrier has passed since it was read.  Waits are
+// bounded (SPIN_LIMIT polls, then PF_ETIMEOUT in *err and false is returned).
+constexpr int PCG_REGIONS = 3;
+
 template <typename AccT, int K>
-__device__ bool reduce_barrier(AccT (&acc)[K], double *partials, double *result, unsigned int *count,
-                               unsigned int *gen, int *err, double (&out)[K], int bid, int nbk)
+__device__ __forceinline__ bool reduce_barrier(AccT (&acc)[K], double *partials, int region, unsigned int *count,
+                                            unsigned int *gen, int *err, double *out, int bid, int nbk)
 {
     constexpr bool pairs = std::is_same<AccT, Acc<float>>::value;
-    __shared__ int s_last, s_ok;
-    __shared__ unsigned int s_gen;
-    if constexpr (pairs) block_reduce_pairs<K>(acc, reinterpret_cast<float2 *>(partials + (size_t)bid * PSTRIDE));
-    else block_reduce_store<K>(acc, partials + (size_t)bid * PSTRIDE);
+    __shared__ float sh[pairs ? K : 1][32], sl[pairs ? K : 1][32];
+    __shared__ double sd[pairs ? 1 : K][32];
+    __shared__ int s_ok;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+    double *const part = partials + (size_t)region * nbk * PSTRIDE;
+#pragma unroll
+    for (int k = 0; k < K; k++) {
+        if constexpr (pairs) {
+            float h = acc[k].s, l = acc[k].c;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const float h2 = __shfl_xor_sync(0xffffffffu, h, o), l2 = __shfl_xor_sync(0xffffffffu, l, o);
+                pair_add(h, l, h2, l2);
+            }
+            if (lane == 0) { sh[k][wid] = h; sl[k][wid] = l; }
+        } else {
+            const double v = warp_sum(acc[k].value());
+            if (lane == 0) sd[k][wid] = v;
+        }
+    }
+    __syncthreads();
+    for (int k = wid; k < K; k += nw) {
+        if constexpr (pairs) {
+            float h = lane < nw ? sh[k][lane] : 0.f, l = lane < nw ? sl[k][lane] : 0.f;
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const float h2 = __shfl_xor_sync(0xffffffffu, h, o), l2 = __shfl_xor_sync(0xffffffffu, l, o);
+                pair_add(h, l, h2, l2);
+            }
+            if (lane == 0) reinterpret_cast<float2 *>(part + (size_t)bid * PSTRIDE)[k] = make_float2(h, l);
+        } else {
+            const double v = warp_sum(lane < nw ? sd[k][lane] : 0.0);
+            if (lane == 0) part[(size_t)bid * PSTRIDE + k] = v;
+        }
+    }
+    __syncthreads();
     if (threadIdx.x == 0) {
         s_ok = 1;
-        s_gen = ld_relaxed_gpu(gen);
+        const unsigned int g = ld_relaxed_gpu(gen);
         const unsigned int arrived = atom_add_acq_rel_gpu(count, 1u);
-        s_last = (arrived == (unsigned int)nbk - 1) ? 1 : 0;
-    }
-    __syncthreads();
-    if (s_last && pairs) {
-        last_block_pairs<K>(partials, nbk, result);
-        if (threadIdx.x == 0) {
+        if (arrived == (unsigned int)nbk - 1) {
             *count = 0u;
             red_add_release_gpu(gen, 1u);
+        } else if (!wait_generation(gen, g, err, SPIN_LIMIT)) {
+            s_ok = 0;
         }
-    } else if (s_last) {
-        if (threadIdx.x < 32) {
-            const int lane = threadIdx.x;
-#pragma unroll
-            for (int k = 0; k < K; k++) {
-                double sacc = 0.0;
-                for (int b = lane; b < nbk; b += 32) sacc += __ldcg(partials + (size_t)b * PSTRIDE + k);
-                sacc = warp_sum(sacc);
-                if (lane == 0) result[k] = sacc;
-            }
-            if (lane == 0) {
-                *count = 0u;
-                red_add_release_gpu(gen, 1u);
-            }
-        }
-    } else if (threadIdx.x == 0) {
-        if (!wait_generation(gen, s_gen, err, SPIN_LIMIT)) s_ok = 0;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
+    for (int k = wid; k < K; k += nw) {
+        if constexpr (pairs) {
+            float h = 0.f, l = 0.f;
+            for (int b = lane; b < nbk; b += 32) {
+                const float2 v = __ldcg(reinterpret_cast<const float2 *>(part + (size_t)b * PSTRIDE) + k);
+                pair_add(h, l, v.x, v.y);
+            }
 #pragma unroll
-        for (int k = 0; k < K; k++) out[k] = __ldcg(result + k);
+            for (int o = 16; o > 0; o >>= 1) {
+                const float h2 = __shfl_xor_sync(0xffffffffu, h, o), l2 = __shfl_xor_sync(0xffffffffu, l, o);
+                pair_add(h, l, h2, l2);
+            }
+            if (lane == 0) out[k] = (double)h + (double)l;
+        } else {
+            double v = 0.0;
+            for (int b = lane; b < nbk; b += 32) v += __ldcg(part + (size_t)b * PSTRIDE + k);
+            v = warp_sum(v);
+            if (lane == 0) out[k] = v;
+        }
     }
+    __syncthreads();
     return s_ok != 0;
+}
+
+// Plain grid barrier (no reduction).  Waits are bounded like reduce_barrier.
+__device__ __forceinline__ bool grid_sync(unsigned int *count, unsigned int *gen, int *err, int nbk)
+{
+    __shared__ int s_gok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s_gok = 1;
+        const unsigned int g = ld_relaxed_gpu(gen);
+        const unsigned int arrived = atom_add_acq_rel_gpu(count, 1u);
+        if (arrived == (unsigned int)nbk - 1) {
+            *count = 0u;
+            red_add_release_gpu(gen, 1u);
+        } else if (!wait_generation(gen, g, err, SPIN_LIMIT)) {
+            s_gok = 0;
+        }
+    }
+    __syncthreads();
+    return s_gok != 0;
 }
 
 // q = sum over the 2^d cells around a node of (lam K_lam + mu K_mu) u_e, plus
@@ -380,6 +437,7 @@ struct PCGState {
     double gamma, delta, gamma_prev, alpha_prev, alpha, beta;
     double inv_gamma, inv_gamma_prev, inv_alpha, inv_alpha_prev;   // FP64 divisions are slow here
     double tot0[10];   // first pass's set-up sums [0, 10) (fixed during a solve; MG refinement reuses them)
+    double red[16];    // totals of the last reduction
     int it, it_total, conv;
     int met;           // refinement: the FP64 residual has met the tolerance
 };
@@ -588,8 +646,8 @@ __global__ void __launch_bounds__(tile_threads<D, SH>(), 512 / tile_threads<D, S
                     acc[1].addprod(rv[d], rv[d]);
                 }
             }
-            double tot[16];
-            if (!reduce_barrier<Acc<double>, 16>(acc, A.partials, A.result, A.bar_count, A.bar_gen, err, tot, bid, nbk)) return;
+            double *const tot = S.red;
+            if (!reduce_barrier<Acc<double>, 16>(acc, A.partials, 2, A.bar_count, A.bar_gen, err, tot, bid, nbk)) return;
             if (lead) {
                 // a residual-only pass reuses the first pass's sums of b, the
                 // moduli and the eigenstress
@@ -683,7 +741,7 @@ __global__ void __launch_bounds__(tile_threads<D, SH>(), 512 / tile_threads<D, S
             if (lead) conv = rc == CTL_DONE;
         } else {
             bool first = true;
-            int cur = 0;
+            int cur = 0, redpar = 0;
             while (true) {
                 if (lead) {
                     if (!first) cg_scalar_update<NV>(S);
@@ -930,8 +988,9 @@ __global__ void __launch_bounds__(tile_threads<D, SH>(), 512 / tile_threads<D, S
                     }
                     __syncthreads();
                 }
-                double tt[3 + NV];
-                if (!reduce_barrier<Acc<T>, 3 + NV>(acc, A.partials, A.result, A.bar_count, A.bar_gen, err, tt, bid, nbk)) return;
+                double *const tt = S.red;
+                if (!reduce_barrier<Acc<T>, 3 + NV>(acc, A.partials, redpar, A.bar_count, A.bar_gen, err, tt, bid, nbk)) return;
+                redpar ^= 1;
                 const bool was_first = first;
                 if (lead) {
                     double s6[6];
@@ -978,9 +1037,7 @@ __global__ void __launch_bounds__(tile_threads<D, SH>(), 512 / tile_threads<D, S
         }
         __syncthreads();
         const int stop = s_ctl;
-        Acc<T> dummy[1];
-        double dres[1];
-        if (!reduce_barrier<Acc<T>, 1>(dummy, A.partials, A.result, A.bar_count, A.bar_gen, err, dres, bid, nbk)) return;
+        if (!grid_sync(A.bar_count, A.bar_gen, err, nbk)) return;
         if (stop == CTL_STOP) { if (lead) conv = S.met != 0; break; }
     }
     if (refine) {

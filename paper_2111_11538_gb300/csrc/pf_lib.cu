@@ -492,6 +492,10 @@ int build_mg(pf_handle *h)
         ny /= 2;
         if (D == 3) nz /= 2;
     }
+    if (D == 2 && sizeof(T) == 8 && H.Lg < L) {
+        const size_t nun = 2 * (size_t)H.lv[H.Lg].nx * (size_t)H.lv[H.Lg].ny;
+        PF_TRY(h->alloc(&H.dense, sizeof(T) * nun * nun));
+    }
     for (int k = 0; k < L; k++) H.deg[k] = k == 0 ? MG_DEG_FINE : (k < H.Lg ? MG_DEG_GRID : MG_DEG_BLOCK);
     // Chebyshev iteration on [bmin, bmax]: d_0 = D^-1 r_0 / theta,
     // rho_j = 1 / (2 sigma - rho_{j-1}), d_j = rho_j rho_{j-1} d_{j-1} + 2 rho_j / delta D^-1 r_j
@@ -698,9 +702,10 @@ int build_plan(pf_handle *h)
         for (int i = 0; i < n; i++) {
             long long nb = 1 + (long long)((double)(cap - n) * work[i] / wtot);
             // the marching sweeps of the 2D V-cycle share out single rows:
-            // a block for every 64 nodes in FP64 (its SM's FP64 pipe is what
-            // they wait for), for every 256 in FP32
-            const long long most = D == 2 && I[i]->mg ? (I[i]->P.N + (sizeof(T) == 8 ? 63 : 255)) / (sizeof(T) == 8 ? 64 : 256)
+            // a block for every 16 nodes in FP64 (its SM's FP64 pipes are what
+            // they wait for, and blocks without rows prepare the dense map of
+            // the block-run levels), for every 256 in FP32
+            const long long most = D == 2 && I[i]->mg ? (I[i]->P.N + (sizeof(T) == 8 ? 15 : 255)) / (sizeof(T) == 8 ? 16 : 256)
                                                       : tiles[i];
             if (nb > most) nb = most > 0 ? most : 1;
             pj[i] = pcg_args<T, D>(I[i]);

@@ -22,6 +22,21 @@
 
 namespace pfdev {
 
+// A lane and the lanes of its right and left neighbour columns.  A grid of
+// at most 32 columns is one strip of whole periodic rows (per: its last lane's
+// neighbour is lane 0), without halo columns.
+struct Lanes2 {
+    int lane, nxt, prv;
+    bool per;
+    __device__ __forceinline__ Lanes2(int nx)
+    {
+        lane = threadIdx.x & 31;
+        per = nx <= 32;
+        nxt = per ? (lane + 1 >= nx ? 0 : lane + 1) : min(lane + 1, 31);
+        prv = per ? (lane == 0 ? nx - 1 : lane - 1) : max(lane - 1, 0);
+    }
+};
+
 // the row's displacement with its right neighbour: sum and difference
 template <typename T>
 struct Row2 {
@@ -29,11 +44,11 @@ struct Row2 {
 };
 
 template <typename T>
-__device__ __forceinline__ void row2(const T (&v)[2], Row2<T> &R)
+__device__ __forceinline__ void row2(const T (&v)[2], const Lanes2 &Ln, Row2<T> &R)
 {
 #pragma unroll
     for (int c = 0; c < 2; c++) {
-        const T r = __shfl_down_sync(0xffffffffu, v[c], 1);
+        const T r = __shfl_sync(0xffffffffu, v[c], Ln.nxt);
         R.e[c] = v[c] + r;
         R.d[c] = r - v[c];
     }
@@ -86,12 +101,12 @@ struct Node2 {
         O[0] = C.ax0 + C.xy[0];
         O[1] = C.sh + C.xy[1];
     }
-    __device__ __forceinline__ void finish(const Cell2<T> &C, T (&q)[2])   // lower corners of the cell row above
+    __device__ __forceinline__ void finish(const Cell2<T> &C, const Lanes2 &Ln, T (&q)[2])   // lower corners of the cell row above
     {
         const T e[2] = {E[0] - C.sh, E[1] - C.ay1};
         const T o[2] = {O[0] + (C.ax0 - C.xy[0]), O[1] + (C.sh - C.xy[1])};
 #pragma unroll
-        for (int c = 0; c < 2; c++) q[c] = (e[c] - o[c]) + __shfl_up_sync(0xffffffffu, e[c] + o[c], 1);
+        for (int c = 0; c < 2; c++) q[c] = (e[c] - o[c]) + __shfl_sync(0xffffffffu, e[c] + o[c], Ln.prv);
     }
 };
 
@@ -108,7 +123,7 @@ extern __shared__ __align__(16) unsigned char pcg_dyn[];
 // row of a lone warp takes as long as its FP64 instructions, 64 cycles each).
 inline int m2_chunk(int nx, int ny, int nbk, int nwb, int OW, int extra, bool fp64)
 {
-    const long long ns = (nx + OW - 1) / OW;
+    const long long ns = nx <= 32 ? 1 : (nx + OW - 1) / OW;
     int best = ny;
     long long bcost = -1;
     for (int zc = 1; zc <= ny; zc++) {
@@ -123,8 +138,8 @@ inline int m2_chunk(int nx, int ny, int nbk, int nwb, int OW, int extra, bool fp
     return best;
 }
 
-// One product: op.load(g, gx, gy, own, lane, R) loads the words of node g
-// (own: an output row), op.form(R, g, own, lane, v, keep, S) gives the operand
+// One product: op.load(g, gx, gy, own, lanes, R) loads the words of node g
+// (own: an output row), op.form(R, g, own, lanes, gx, v, keep, S) gives the operand
 // v of the node (own: an output node; keep[3] is handed to the epilogue),
 // op.mod(R, l, m) the moduli of the cell at the node and op.epi(g, v, q, keep,
 // S) receives q = A v at every output node.  op.cell(C, S) gets every own cell
@@ -134,27 +149,28 @@ template <typename T, int NT, size_t OFF, class OP>
 __device__ __noinline__ typename OP::Sums m2_sweep(int nx, int ny, int zc, int bid, int nbk)
 {
     const OP op = *reinterpret_cast<const OP *>(pcg_dyn + OFF);
-    const int lane = threadIdx.x & 31, nw = (NT / 32) * nbk;
+    const Lanes2 Ln(nx);
+    const int lane = Ln.lane, nw = (NT / 32) * nbk;
     typename OP::Sums S;
-    const int ns = (nx + 29) / 30, items = ns * ((ny + zc - 1) / zc);
+    const int ns = Ln.per ? 1 : (nx + 29) / 30, items = ns * ((ny + zc - 1) / zc);
     for (int item = (int)(threadIdx.x >> 5) * nbk + bid; item < items; item += nw) {
         const int x0 = (item % ns) * 30, y0 = (item / ns) * zc, y1 = min(y0 + zc, ny);
-        const int gxr = x0 - 1 + lane, gx = wrapm(gxr, nx);
-        const bool ownx = lane >= 1 && lane <= 30 && gxr < nx;
+        const int gxr = Ln.per ? lane : x0 - 1 + lane, gx = wrapm(gxr, nx);
+        const bool ownx = (Ln.per || (lane >= 1 && lane <= 30)) && gxr < nx;
         typename OP::Raw R;
         int gy = wrap(y0 - 1, ny);
-        op.load(gx + nx * gy, gx, gy, false, lane, R);
+        op.load(gx + nx * gy, gx, gy, false, Ln, R);
         Row2<T> lo;
         Node2<T> nd;
         T vl[2] = {T(0), T(0)}, kl[3] = {T(0), T(0), T(0)}, l4 = T(0), m4 = T(0);
         for (int y = y0 - 1; y <= y1; y++) {
             T v[2], k[3], ln, mn;
-            op.form(R, gx + nx * gy, ownx && y >= y0 && y < y1, lane, gx, v, k, S);
+            op.form(R, gx + nx * gy, ownx && y >= y0 && y < y1, Ln, gx, v, k, S);
             op.mod(R, ln, mn);
             gy = gy + 1 == ny ? 0 : gy + 1;
-            if (y < y1) op.load(gx + nx * gy, gx, gy, y + 1 < y1, lane, R);
+            if (y < y1) op.load(gx + nx * gy, gx, gy, y + 1 < y1, Ln, R);
             Row2<T> hi;
-            row2(v, hi);
+            row2(v, Ln, hi);
             if (y >= y0) {
                 Cell2<T> C = cell2(l4, m4, lo, hi);
                 const bool own = ownx && y > y0;             // node row y - 1 and the cells at it
@@ -164,7 +180,7 @@ __device__ __noinline__ typename OP::Sums m2_sweep(int nx, int ny, int zc, int b
                 }
                 if (y > y0) {
                     T q[2];
-                    nd.finish(C, q);
+                    nd.finish(C, Ln, q);
                     if (own) op.epi(gx + nx * (y - 1), vl, q, kl, S);
                 }
                 nd.start(C);
@@ -181,7 +197,7 @@ __device__ __noinline__ typename OP::Sums m2_sweep(int nx, int ny, int zc, int b
     return S;
 }
 
-// Two products, the second one row behind the first: op.form(R, lane, gx, v, a)
+// Two products, the second one row behind the first: op.form(R, lanes, gx, v, a)
 // gives the first operand v and an auxiliary a[3]; op.mid(v, a, q, r, w)
 // the intermediate r and second operand w from q = A v; op.epi(g, v, a, r,
 // w, q, S) gets q = A w at every output node (28 columns per strip).
@@ -189,16 +205,17 @@ template <typename T, int NT, size_t OFF, class OP>
 __device__ __noinline__ typename OP::Sums m2_sweep2(int nx, int ny, int zc, int bid, int nbk)
 {
     const OP op = *reinterpret_cast<const OP *>(pcg_dyn + OFF);
-    const int lane = threadIdx.x & 31, nw = (NT / 32) * nbk;
+    const Lanes2 Ln(nx);
+    const int lane = Ln.lane, nw = (NT / 32) * nbk;
     typename OP::Sums S;
-    const int ns = (nx + 27) / 28, items = ns * ((ny + zc - 1) / zc);
+    const int ns = Ln.per ? 1 : (nx + 27) / 28, items = ns * ((ny + zc - 1) / zc);
     for (int item = (int)(threadIdx.x >> 5) * nbk + bid; item < items; item += nw) {
         const int x0 = (item % ns) * 28, y0 = (item / ns) * zc, y1 = min(y0 + zc, ny);
-        const int gxr = x0 - 2 + lane, gx = wrapm(gxr, nx);
-        const bool ownx = lane >= 2 && lane <= 29 && gxr < nx;
+        const int gxr = Ln.per ? lane : x0 - 2 + lane, gx = wrapm(gxr, nx);
+        const bool ownx = (Ln.per || (lane >= 2 && lane <= 29)) && gxr < nx;
         typename OP::Raw R;
         int gy = wrapm(y0 - 2, ny);
-        op.load(gx + nx * gy, gx, gy, lane, R);
+        op.load(gx + nx * gy, gx, gy, Ln, R);
         Row2<T> lo0, lo1;
         Node2<T> n0, n1;
         // row y - 1 of the first operand, row y - 2 of the second
@@ -206,22 +223,22 @@ __device__ __noinline__ typename OP::Sums m2_sweep2(int nx, int ny, int zc, int 
         T v2[2] = {T(0), T(0)}, a2[3] = {T(0), T(0), T(0)}, r2[2] = {T(0), T(0)}, w2[2] = {T(0), T(0)}, l2 = T(0), m2 = T(0);
         for (int y = y0 - 2; y <= y1 + 1; y++) {
             T v[2], a[3], ln, mn;
-            op.form(R, lane, gx, v, a);
+            op.form(R, Ln, gx, v, a);
             op.mod(R, ln, mn);
             gy = gy + 1 == ny ? 0 : gy + 1;
-            if (y <= y1) op.load(gx + nx * gy, gx, gy, lane, R);
+            if (y <= y1) op.load(gx + nx * gy, gx, gy, Ln, R);
             Row2<T> hi;
-            row2(v, hi);
+            row2(v, Ln, hi);
             T r[2] = {T(0), T(0)}, w[2] = {T(0), T(0)};
             if (y > y0 - 2) {
                 const Cell2<T> C = cell2(l1, m1, lo0, hi);
                 if (y >= y0) {
                     // second operand at row y - 1, its cells at row y - 2
                     T q[2];
-                    n0.finish(C, q);
+                    n0.finish(C, Ln, q);
                     op.mid(v1, a1, q, r, w);
                     Row2<T> h1;
-                    row2(w, h1);
+                    row2(w, Ln, h1);
                     if (y > y0) {
                         Cell2<T> C1 = cell2(l2, m2, lo1, h1);
                         const bool own = ownx && y > y0 + 1;
@@ -231,7 +248,7 @@ __device__ __noinline__ typename OP::Sums m2_sweep2(int nx, int ny, int zc, int 
                         }
                         if (y > y0 + 1) {
                             T q1[2];
-                            n1.finish(C1, q1);
+                            n1.finish(C1, Ln, q1);
                             if (own) op.epi(gx + nx * (y - 2), v2, a2, r2, w2, q1, S);
                         }
                         n1.start(C1);
@@ -272,8 +289,8 @@ __device__ __forceinline__ void ld_pair(const double *p, double (&v)[2])
 // The coarse correction at a fine node (bilinear prolongation of C's xpost;
 // component 1 lies n values after component 0).  Each lane loads the two
 // coarse rows' values at its own gx >> 1; an odd column takes the other half
-// from the lane on its right, the last lane of a strip (an odd column) from
-// loads of its own.
+// from its right neighbour's lane, the last lane of a strip with halo columns
+// (an odd column) from loads of its own.
 template <typename T>
 struct Prolong2 {
     const T *x;
@@ -281,7 +298,7 @@ struct Prolong2 {
     struct Raw {
         T a[4], b[4];
     };
-    __device__ __forceinline__ void load(int gx, int gy, int lane, Raw &R) const
+    __device__ __forceinline__ void load(int gx, int gy, const Lanes2 &Ln, Raw &R) const
     {
         const int ix = gx >> 1, iy = gy >> 1, iy1 = (gy & 1) ? (iy + 1 == cny ? 0 : iy + 1) : iy, n = cnx * cny;
 #pragma unroll
@@ -289,7 +306,7 @@ struct Prolong2 {
             R.a[2 * c] = __ldca(x + c * n + ix + cnx * iy);
             R.a[2 * c + 1] = __ldca(x + c * n + ix + cnx * iy1);
         }
-        if (lane == 31) {
+        if (!Ln.per && Ln.lane == 31) {
             const int ix1 = ix + 1 == cnx ? 0 : ix + 1;
 #pragma unroll
             for (int c = 0; c < 2; c++) {
@@ -298,14 +315,14 @@ struct Prolong2 {
             }
         }
     }
-    __device__ __forceinline__ void add(const Raw &R, int gx, int lane, T (&v)[2]) const
+    __device__ __forceinline__ void add(const Raw &R, int gx, const Lanes2 &Ln, T (&v)[2]) const
     {
 #pragma unroll
         for (int c = 0; c < 2; c++) {
             // rows averaged (the same row twice on an even row)
             const T e = T(0.5) * (R.a[2 * c] + R.a[2 * c + 1]);
-            T r = __shfl_down_sync(0xffffffffu, e, 1);
-            if (lane == 31) r = T(0.5) * (R.b[2 * c] + R.b[2 * c + 1]);
+            T r = __shfl_sync(0xffffffffu, e, Ln.nxt);
+            if (!Ln.per && Ln.lane == 31) r = T(0.5) * (R.b[2 * c] + R.b[2 * c + 1]);
             v[c] += (gx & 1) ? T(0.5) * (e + r) : e;
         }
     }
@@ -314,7 +331,8 @@ struct Prolong2 {
 // The restriction (transpose of the bilinear prolongation) of the finer
 // level's residual r at a coarse node: pairs (2 gx, 2 gx + 1) of the three
 // fine rows around it; the value at 2 gx - 1 is the left lane's second
-// entry, or a load of its own for the first lane.
+// entry, or a load of its own for the first lane of a
+// strip with halo columns.
 template <typename T>
 struct Restrict2 {
     const T *r;
@@ -322,7 +340,7 @@ struct Restrict2 {
     struct Raw {
         T p[6][2], b[6];
     };
-    __device__ __forceinline__ void load(int gx, int gy, int lane, Raw &R) const
+    __device__ __forceinline__ void load(int gx, int gy, const Lanes2 &Ln, Raw &R) const
     {
         const int n = fnx * fny;
 #pragma unroll
@@ -331,19 +349,19 @@ struct Restrict2 {
 #pragma unroll
             for (int c = 0; c < 2; c++) {
                 ld_pair(row + c * n + 2 * gx, R.p[2 * b + c]);
-                if (lane == 0) R.b[2 * b + c] = __ldca(row + c * n + (gx == 0 ? fnx - 1 : 2 * gx - 1));
+                if (!Ln.per && Ln.lane == 0) R.b[2 * b + c] = __ldca(row + c * n + (gx == 0 ? fnx - 1 : 2 * gx - 1));
             }
         }
     }
-    __device__ __forceinline__ void get(const Raw &R, int lane, T (&f)[2]) const
+    __device__ __forceinline__ void get(const Raw &R, const Lanes2 &Ln, T (&f)[2]) const
     {
         f[0] = f[1] = T(0);
 #pragma unroll
         for (int b = 0; b < 3; b++)
 #pragma unroll
             for (int c = 0; c < 2; c++) {
-                T am = __shfl_up_sync(0xffffffffu, R.p[2 * b + c][1], 1);
-                if (lane == 0) am = R.b[2 * b + c];
+                T am = __shfl_sync(0xffffffffu, R.p[2 * b + c][1], Ln.prv);
+                if (!Ln.per && Ln.lane == 0) am = R.b[2 * b + c];
                 const T s = R.p[2 * b + c][0] + T(0.5) * (am + R.p[2 * b + c][1]);
                 f[c] += b == 1 ? s : T(0.5) * s;
             }
@@ -378,7 +396,7 @@ struct OpFirst2 {
     struct Raw {
         T l, m, di, r[2], w[2], s[2], u[2], p[2], x[2];
     };
-    __device__ __forceinline__ void load(int g, int, int, bool own, int, Raw &R) const
+    __device__ __forceinline__ void load(int g, int, int, bool own, const Lanes2 &, Raw &R) const
     {
         R.l = __ldcg(lam + g);
         R.m = __ldcg(mu + g);
@@ -398,7 +416,7 @@ struct OpFirst2 {
         }
     }
     __device__ __forceinline__ void mod(const Raw &R, T &l, T &m) const { l = R.l; m = R.m; }
-    __device__ __forceinline__ void form(const Raw &R, int g, bool own, int, int, T (&v)[2], T (&k)[3], Sums &S) const
+    __device__ __forceinline__ void form(const Raw &R, int g, bool own, const Lanes2 &, int, T (&v)[2], T (&k)[3], Sums &S) const
     {
         const T di = c2 * R.di;
         k[2] = T(0);
@@ -441,12 +459,12 @@ struct OpCheb2 {
     T *xo, *rn, *dn;
     T c1, c2, n1, n2;
     int n;
-    bool last;
+    bool last, dir;            // dir: the step has a previous direction d
     typedef Acc<T> Sums;
     struct Raw {
         T l, m, di, r[2], d[2], x[2];
     };
-    __device__ __forceinline__ void load(int g, int, int, bool own, int, Raw &R) const
+    __device__ __forceinline__ void load(int g, int, int, bool own, const Lanes2 &, Raw &R) const
     {
         R.l = __ldcg(lam + g);
         R.m = __ldcg(mu + g);
@@ -454,12 +472,12 @@ struct OpCheb2 {
 #pragma unroll
         for (int c = 0; c < 2; c++) {
             R.r[c] = __ldcg(r + g + c * n);
-            R.d[c] = __ldcg(d + g + c * n);
+            R.d[c] = dir ? __ldcg(d + g + c * n) : T(0);
             if (own) R.x[c] = __ldcg(xi + g + c * n);
         }
     }
     __device__ __forceinline__ void mod(const Raw &R, T &l, T &m) const { l = R.l; m = R.m; }
-    __device__ __forceinline__ void form(const Raw &R, int g, bool own, int, int, T (&v)[2], T (&k)[3], Sums &) const
+    __device__ __forceinline__ void form(const Raw &R, int g, bool own, const Lanes2 &, int, T (&v)[2], T (&k)[3], Sums &) const
     {
         const T di = c2 * R.di, dl = n2 * R.di;
         k[2] = dl;
@@ -502,18 +520,18 @@ struct OpPre2 {
         T l, m, di;
         typename Restrict2<T>::Raw f;
     };
-    __device__ __forceinline__ void load(int g, int gx, int gy, bool, int lane, Raw &R) const
+    __device__ __forceinline__ void load(int g, int gx, int gy, bool, const Lanes2 &Ln, Raw &R) const
     {
         R.l = __ldcg(lam + g);
         R.m = __ldcg(mu + g);
         R.di = __ldcg(dinv + g);
-        Rs.load(gx, gy, lane, R.f);
+        Rs.load(gx, gy, Ln, R.f);
     }
     __device__ __forceinline__ void mod(const Raw &R, T &l, T &m) const { l = R.l; m = R.m; }
-    __device__ __forceinline__ void form(const Raw &R, int g, bool own, int lane, int, T (&v)[2], T (&k)[3], Sums &) const
+    __device__ __forceinline__ void form(const Raw &R, int g, bool own, const Lanes2 &Ln, int, T (&v)[2], T (&k)[3], Sums &) const
     {
         T ff[2];
-        Rs.get(R.f, lane, ff);
+        Rs.get(R.f, Ln, ff);
         const T di = c2 * R.di;
         k[2] = T(0);
 #pragma unroll
@@ -543,7 +561,7 @@ struct OpApply2 {
     struct Raw {
         T l, m, u[2], r[2];
     };
-    __device__ __forceinline__ void load(int g, int, int, bool own, int, Raw &R) const
+    __device__ __forceinline__ void load(int g, int, int, bool own, const Lanes2 &, Raw &R) const
     {
         R.l = __ldcg(lam + g);
         R.m = __ldcg(mu + g);
@@ -554,7 +572,7 @@ struct OpApply2 {
         }
     }
     __device__ __forceinline__ void mod(const Raw &R, T &l, T &m) const { l = R.l; m = R.m; }
-    __device__ __forceinline__ void form(const Raw &R, int, bool own, int, int, T (&v)[2], T (&k)[3], Sums &S) const
+    __device__ __forceinline__ void form(const Raw &R, int, bool own, const Lanes2 &, int, T (&v)[2], T (&k)[3], Sums &S) const
     {
         k[2] = T(0);
 #pragma unroll
@@ -595,18 +613,18 @@ struct OpPrePair2 {
         T l, m, di;
         typename Restrict2<T>::Raw f;
     };
-    __device__ __forceinline__ void load(int g, int gx, int gy, int lane, Raw &R) const
+    __device__ __forceinline__ void load(int g, int gx, int gy, const Lanes2 &Ln, Raw &R) const
     {
         R.l = __ldcg(lam + g);
         R.m = __ldcg(mu + g);
         R.di = __ldcg(dinv + g);
-        Rs.load(gx, gy, lane, R.f);
+        Rs.load(gx, gy, Ln, R.f);
     }
     __device__ __forceinline__ void mod(const Raw &R, T &l, T &m) const { l = R.l; m = R.m; }
-    __device__ __forceinline__ void form(const Raw &R, int lane, int, T (&v)[2], T (&a)[3]) const
+    __device__ __forceinline__ void form(const Raw &R, const Lanes2 &Ln, int, T (&v)[2], T (&a)[3]) const
     {
         T ff[2];
-        Rs.get(R.f, lane, ff);
+        Rs.get(R.f, Ln, ff);
         const T di = c20 * R.di;
         a[2] = c21 * R.di;
 #pragma unroll
@@ -639,7 +657,7 @@ struct PostRaw2 {
     typename Prolong2<T>::Raw e;
 };
 template <typename T, class OP>
-__device__ __forceinline__ void post_load2(const OP &op, const T *f, int g, int gx, int gy, int lane, PostRaw2<T> &R)
+__device__ __forceinline__ void post_load2(const OP &op, const T *f, int g, int gx, int gy, const Lanes2 &Ln, PostRaw2<T> &R)
 {
     R.l = __ldcg(op.lam + g);
     R.m = __ldcg(op.mu + g);
@@ -649,8 +667,45 @@ __device__ __forceinline__ void post_load2(const OP &op, const T *f, int g, int 
         R.f[c] = __ldcg(f + g + c * op.n);
         R.x[c] = __ldcg(op.xpre + g + c * op.n);
     }
-    op.P.load(gx, gy, lane, R.e);
+    op.P.load(gx, gy, Ln, R.e);
 }
+
+// First post-smoothing step alone (FP64): x = x_pre + P e, r = f - A x; last
+// (one-step smoothing): x + c2 D^-1 r into xpost, else x and r.
+template <typename T>
+struct OpPost2 {
+    static constexpr bool E = false;
+    const T *lam, *mu, *dinv, *f, *xpre;
+    Prolong2<T> P;
+    T *xpost, *r;
+    T c2;
+    int n;
+    bool last;
+    typedef Acc<T> Sums;
+    typedef PostRaw2<T> Raw;
+    __device__ __forceinline__ void load(int g, int gx, int gy, bool, const Lanes2 &Ln, Raw &R) const { post_load2(*this, f, g, gx, gy, Ln, R); }
+    __device__ __forceinline__ void mod(const Raw &R, T &l, T &m) const { l = R.l; m = R.m; }
+    __device__ __forceinline__ void form(const Raw &R, int g, bool own, const Lanes2 &Ln, int gx, T (&v)[2], T (&k)[3], Sums &) const
+    {
+#pragma unroll
+        for (int c = 0; c < 2; c++) v[c] = R.x[c];
+        P.add(R.e, gx, Ln, v);
+        k[2] = c2 * R.di;
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+            k[c] = last ? v[c] + k[2] * R.f[c] : R.f[c];
+            if (own && !last) xpost[g + c * n] = v[c];
+        }
+    }
+    __device__ __forceinline__ void epi(int g, const T (&)[2], const T (&q)[2], const T (&k)[3], Sums &) const
+    {
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+            if (last) xpost[g + c * n] = k[c] - k[2] * q[c];
+            else r[g + c * n] = k[c] - q[c];
+        }
+    }
+};
 
 // Two-step post-smoothing of a coarse level from x = x_pre + P e.
 template <typename T>
@@ -663,14 +718,14 @@ struct OpPostPair2 {
     int n;
     typedef Acc<T> Sums;
     typedef PostRaw2<T> Raw;
-    __device__ __forceinline__ void load(int g, int gx, int gy, int lane, Raw &R) const { post_load2(*this, f, g, gx, gy, lane, R); }
+    __device__ __forceinline__ void load(int g, int gx, int gy, const Lanes2 &Ln, Raw &R) const { post_load2(*this, f, g, gx, gy, Ln, R); }
     __device__ __forceinline__ void mod(const Raw &R, T &l, T &m) const { l = R.l; m = R.m; }
-    __device__ __forceinline__ void form(const Raw &R, int lane, int gx, T (&v)[2], T (&a)[3]) const
+    __device__ __forceinline__ void form(const Raw &R, const Lanes2 &Ln, int gx, T (&v)[2], T (&a)[3]) const
     {
         a[2] = R.di;
 #pragma unroll
         for (int c = 0; c < 2; c++) { a[c] = R.f[c]; v[c] = R.x[c]; }
-        P.add(R.e, gx, lane, v);
+        P.add(R.e, gx, Ln, v);
     }
     __device__ __forceinline__ void mid(const T (&)[2], const T (&a)[3], const T (&q)[2], T (&r)[2], T (&w)[2]) const
     {
@@ -703,14 +758,14 @@ struct OpFine2 {
     int n;
     typedef Sums2<T> Sums;
     typedef PostRaw2<T> Raw;
-    __device__ __forceinline__ void load(int g, int gx, int gy, int lane, Raw &R) const { post_load2(*this, r, g, gx, gy, lane, R); }
+    __device__ __forceinline__ void load(int g, int gx, int gy, const Lanes2 &Ln, Raw &R) const { post_load2(*this, r, g, gx, gy, Ln, R); }
     __device__ __forceinline__ void mod(const Raw &R, T &l, T &m) const { l = R.l; m = R.m; }
-    __device__ __forceinline__ void form(const Raw &R, int lane, int gx, T (&v)[2], T (&a)[3]) const
+    __device__ __forceinline__ void form(const Raw &R, const Lanes2 &Ln, int gx, T (&v)[2], T (&a)[3]) const
     {
         a[2] = c20 * R.di;
 #pragma unroll
         for (int c = 0; c < 2; c++) { a[c] = R.f[c]; v[c] = R.x[c]; }
-        P.add(R.e, gx, lane, v);
+        P.add(R.e, gx, Ln, v);
     }
     __device__ __forceinline__ void mid(const T (&v)[2], const T (&a)[3], const T (&q)[2], T (&r_)[2], T (&w_)[2]) const
     {

@@ -45,28 +45,9 @@ struct MGHier {
     int deg[MG_MAX_LEVELS];        // Chebyshev steps of each pre- and post-smoothing, per level
     int csteps;                    // Chebyshev steps of the coarsest solve (>= 2)
     T c1[MG_MAX_STEPS], c2[MG_MAX_STEPS];   // d_j = c1[j] d_{j-1} + c2[j] D^-1 r_j  (c1[0] = 0)
+    T *dense;                      // 2D FP64: the block-run levels' map, (2 nodes)^2 values
     MGLevel<T> lv[MG_MAX_LEVELS];
 };
-
-// Plain grid barrier (no reduction).  Waits are bounded like reduce_barrier.
-__device__ __forceinline__ bool grid_sync(unsigned int *count, unsigned int *gen, int *err, int nbk)
-{
-    __shared__ int s_gok;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        s_gok = 1;
-        const unsigned int g = ld_relaxed_gpu(gen);
-        const unsigned int arrived = atom_add_acq_rel_gpu(count, 1u);
-        if (arrived == (unsigned int)nbk - 1) {
-            *count = 0u;
-            red_add_release_gpu(gen, 1u);
-        } else if (!wait_generation(gen, g, err, SPIN_LIMIT)) {
-            s_gok = 0;
-        }
-    }
-    __syncthreads();
-    return s_gok != 0;
-}
 
 __device__ __forceinline__ int mg_wrap(int a, int n, bool small) { return small ? wrapm(a, n) : wrap(a, n); }
 
@@ -571,20 +552,22 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
     unsigned char *s_op = pcg_dyn + OFF;
 
     // ---- grid levels --------------------------------------------------
-    // Chebyshev step j >= 1 of the pre-smoothing on level k: d_j from buffer
-    // par, x += d_j, r_{j+1} = r_j - A d_j into buffer 1 - par.  last: apply
-    // step j + 1 too (pointwise) and leave the final correction in xpost.
-    auto cheb = [&](int k, int j, int par, bool last) {
+    // Chebyshev step j on level k: d_j from buffer par, x += d_j, r_{j+1} =
+    // r_j - A d_j into buffer 1 - par (post: of the post-smoothing, whose
+    // iterate is xpost).  last: apply step j + 1 too (pointwise) and leave the
+    // final correction in xpost.
+    auto cheb = [&](int k, int j, int par, bool last, bool post) {
         const MGLevel<T> &V = H.lv[k];
         OpCheb2<T> &op = *reinterpret_cast<OpCheb2<T> *>(s_op);
         static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
         if (lead) {
             op.lam = V.lam; op.mu = V.mu; op.dinv = V.dinv; op.n = V.nx * V.ny;
-            op.r = V.r[par][0]; op.d = V.d[par][0]; op.xi = V.xpre[0];
-            op.xo = last ? V.xpost[0] : V.xpre[0];
+            op.r = V.r[par][0]; op.d = V.d[par][0]; op.xi = post ? V.xpost[0] : V.xpre[0];
+            op.xo = last || post ? V.xpost[0] : V.xpre[0];
             op.rn = V.r[1 - par][0]; op.dn = V.d[1 - par][0];
             op.c1 = H.c1[j]; op.c2 = H.c2[j]; op.n1 = H.c1[j + 1]; op.n2 = H.c2[j + 1];
             op.last = last;
+            op.dir = j > 0;
         }
         __syncthreads();
         m2_sweep<T, NT, OFF, OpCheb2<T>>(V.nx, V.ny, A.zc1[k], bid, nbk);
@@ -625,26 +608,49 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
             }
         }
     };
-    // post-smoothing of a grid level k >= 1 (two steps, one sweep)
-    auto post = [&](int k) {
+    // FP64 sweeps are bound by the FP64 pipes: two one-product sweeps and a
+    // barrier are cheaper there than one two-product sweep, which repeats two
+    // more rows of each chunk (64^2: 18 against 10 us on the 32^2 level)
+    constexpr bool PAIR = sizeof(T) == 4;
+    // post-smoothing of a grid level k (k = 0: one step, FP64 only; else two)
+    auto post = [&](int k, int cur) {
         const MGLevel<T> &V = H.lv[k];
-        OpPostPair2<T> &op = *reinterpret_cast<OpPostPair2<T> *>(s_op);
-        static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
-        if (lead) {
-            op.lam = V.lam; op.mu = V.mu; op.dinv = V.dinv; op.n = V.nx * V.ny;
-            op.f = V.f[0]; op.xpre = V.xpre[0]; op.xpost = V.xpost[0];
-            op.P = prolong_of(k);
-            op.c20 = H.c2[0]; op.c11 = H.c1[1]; op.c21 = H.c2[1];
+        if constexpr (PAIR) {
+            OpPostPair2<T> &op = *reinterpret_cast<OpPostPair2<T> *>(s_op);
+            static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
+            if (lead) {
+                op.lam = V.lam; op.mu = V.mu; op.dinv = V.dinv; op.n = V.nx * V.ny;
+                op.f = V.f[0]; op.xpre = V.xpre[0]; op.xpost = V.xpost[0];
+                op.P = prolong_of(k);
+                op.c20 = H.c2[0]; op.c11 = H.c1[1]; op.c21 = H.c2[1];
+            }
+            __syncthreads();
+            m2_sweep2<T, NT, OFF, OpPostPair2<T>>(V.nx, V.ny, A.zc2[k], bid, nbk);
+            return grid_sync(bc, bg, err, nbk);
+        } else {
+            OpPost2<T> &op = *reinterpret_cast<OpPost2<T> *>(s_op);
+            static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
+            if (lead) {
+                op.lam = V.lam; op.mu = V.mu; op.dinv = V.dinv; op.n = V.nx * V.ny;
+                op.f = k == 0 ? A.r[cur][0] : V.f[0];
+                op.xpre = V.xpre[0]; op.xpost = V.xpost[0]; op.r = V.r[0][0];
+                op.P = prolong_of(k);
+                op.c2 = H.c2[0];
+                op.last = k == 0;
+            }
+            __syncthreads();
+            m2_sweep<T, NT, OFF, OpPost2<T>>(V.nx, V.ny, A.zc1[k], bid, nbk);
+            if (!grid_sync(bc, bg, err, nbk)) return false;
+            if (k == 0) return true;
+            cheb(k, 0, 0, true, true);
+            return grid_sync(bc, bg, err, nbk);
         }
-        __syncthreads();
-        m2_sweep2<T, NT, OFF, OpPostPair2<T>>(V.nx, V.ny, A.zc2[k], bid, nbk);
-        return grid_sync(bc, bg, err, nbk);
     };
-    // pre-smoothing of grid level k >= 1 (two steps, one sweep), or the
-    // coarsest solve (csteps >= 3) if the coarsest level is a grid level
+    // pre-smoothing of grid level k >= 1 (two steps), or the coarsest solve
+    // (csteps >= 3) if the coarsest level is a grid level
     auto pre = [&](int k) {
         const MGLevel<T> &V = H.lv[k];
-        if (k < L - 1) {
+        if (PAIR && k < L - 1) {
             OpPrePair2<T> &op = *reinterpret_cast<OpPrePair2<T> *>(s_op);
             static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
             if (lead) {
@@ -669,15 +675,20 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
         m2_sweep<T, NT, OFF, OpPre2<T>>(V.nx, V.ny, A.zc1[k], bid, nbk);
         if (!grid_sync(bc, bg, err, nbk)) return false;
         int par = 1;
-        for (int j = 1; j < cs - 1; j++) {
-            cheb(k, j, par, j + 2 == cs);
+        const bool co = k == L - 1;
+        const int nk = co ? cs - 1 : H.deg[k];
+        for (int j = 1; j < nk; j++) {
+            cheb(k, j, par, co && j + 1 == nk, false);
             if (!grid_sync(bc, bg, err, nbk)) return false;
             par ^= 1;
         }
         return true;
     };
 
-    // ---- block-run levels (first block, shared memory, in place) ----------
+    // ---- block-run levels (shared memory) ---------------------------------
+    // (the marching sweeps on one block's warps took longer than these phases,
+    // 29 against 23 us per V-cycle at 512^2: a chain of rows per warp is longer
+    // than a phase over all nodes)
     const int nmax = Lgw < L ? H.lv[Lgw].nx * H.lv[Lgw].ny : 0;
     T *scr = bscratch<T>(sblk, H);
     auto bcheb = [&](int k, int j, bool last) {
@@ -706,7 +717,9 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
                 }
             });
     };
-    auto bpre = [&](int k) {
+    // (unit >= 0: from the unit vector of that entry in place of the
+    // restricted residual)
+    auto bpre = [&](int k, int unit) {
         const BLevel<T> B = blevel<T>(sblk, H, k);
         const T c2 = H.c2[0];
         const bool top = k == Lgw;
@@ -715,7 +728,10 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
             [&](int i, T (&v)[2]) {
                 const int ix = i % B.nx, iy = i / B.nx;
                 T f[2];
-                if (top) {
+                if (top && unit >= 0) {
+                    f[0] = i == unit ? T(1) : T(0);
+                    f[1] = i + B.n == unit ? T(1) : T(0);
+                } else if (top) {
                     restrict_g(k, ix, iy, f);
                 } else {
                     const BLevel<T> F = blevel<T>(sblk, H, k - 1);
@@ -784,7 +800,47 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
         for (int j = 0; j + 1 < dk; j++) bcheb(k, j, j + 2 == dk);
     };
 
-    if (bid == 0 && Lgw < L) mg_setup_block<T>(H, sblk);
+    // FP64: the correction of the block-run levels is a fixed symmetric linear
+    // map of their right-hand side.  While the first block runs them, the
+    // other blocks, which would wait, each compute the map's column of one
+    // unit vector; once all columns are there (after a few V-cycles of the
+    // solve), the map is applied as a dense product spread over all warps (at
+    // 64^2, 512 unknowns: 51 -> 4 us per V-cycle)
+    const int nun = Lgw < L ? 2 * H.lv[Lgw].nx * H.lv[Lgw].ny : 0;
+    int ncol = 0;
+    auto bcycle = [&](int unit, T *dst) {
+        for (int k = Lgw; k < L; k++) bpre(k, unit);
+        for (int k = L - 2; k >= Lgw; k--) bpost(k);
+        const BLevel<T> B = blevel<T>(sblk, H, Lgw);
+        for (int i = threadIdx.x; i < 2 * B.n; i += blockDim.x) dst[i] = B.x[0][i];
+        __syncthreads();
+    };
+    auto block64 = [&]() {
+        if (ncol < nun) {
+            if (bid == 0) bcycle(-1, H.lv[Lgw].xpost[0]);
+            else if (ncol + bid - 1 < nun) bcycle(ncol + bid - 1, H.dense + (size_t)(ncol + bid - 1) * nun);
+            ncol += nbk - 1;
+            return;
+        }
+        T *f = bscratch<T>(sblk, H);
+        const int nn = nun / 2, nx = H.lv[Lgw].nx, lane = threadIdx.x & 31;
+        for (int i = threadIdx.x; i < nn; i += blockDim.x) {
+            T v[2];
+            restrict_g(Lgw, i % nx, i / nx, v);
+            f[i] = v[0];
+            f[nn + i] = v[1];
+        }
+        __syncthreads();
+        for (int i = (threadIdx.x >> 5) * nbk + bid; i < nun; i += (NT / 32) * nbk) {
+            const T *row = H.dense + (size_t)i * nun;
+            T y = T(0);
+            for (int j = lane; j < nun; j += 32) y = fma(__ldcg(row + j), f[j], y);
+            y = warp_sum(y);
+            if (lane == 0) H.lv[Lgw].xpost[0][i] = y;
+        }
+    };
+
+    if ((bid == 0 || !PAIR) && Lgw < L) mg_setup_block<T>(H, sblk);
 
     int cur = 0;
     bool first = true;
@@ -818,8 +874,8 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
             racc[0] = m2_sweep<T, NT, OFF, OpFirst2<T>>(L0.nx, L0.ny, A.zc1[0], bid, nbk);
         }
         if (!first) {
-            double tr[1];
-            if (!reduce_barrier<Acc<T>, 1>(racc, A.partials, A.result, A.bar_count, A.bar_gen, err, tr, bid, nbk)) return -1;
+            double *const tr = S.red;
+            if (!reduce_barrier<Acc<T>, 1>(racc, A.partials, 1, A.bar_count, A.bar_gen, err, tr, bid, nbk)) return -1;
             if (lead) {
                 double rnew = tr[0];
                 for (int vv = 0; vv < NV; vv++) rnew += S.RE[vv] * S.RE[vv];
@@ -842,7 +898,7 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
         if (L == 1) {
             int par = 1;
             for (int j = 1; j < cs - 1; j++) {
-                cheb(0, j, par, j + 2 == cs);
+                cheb(0, j, par, j + 2 == cs, false);
                 if (!grid_sync(bc, bg, err, nbk)) return -1;
                 par ^= 1;
             }
@@ -850,30 +906,25 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
         for (int k = 1; k < Lgw; k++)
             if (!pre(k)) return -1;
         if (Lgw < L) {
-            if (bid == 0) {
-                for (int k = Lgw; k < L; k++) bpre(k);
-                for (int k = L - 2; k >= Lgw; k--) bpost(k);
-                // the top block-run level's correction, for the grid level above
-                const BLevel<T> B = blevel<T>(sblk, H, Lgw);
-                for (int i = threadIdx.x; i < B.n; i += blockDim.x) {
-                    H.lv[Lgw].xpost[0][i] = B.x[0][i];
-                    H.lv[Lgw].xpost[1][i] = B.x[1][i];
-                }
+            if constexpr (PAIR) {
+                if (bid == 0) bcycle(-1, H.lv[Lgw].xpost[0]);
+            } else {
+                block64();
             }
             if (!grid_sync(bc, bg, err, nbk)) return -1;
         }
-        for (int k = (Lgw < L - 1 ? Lgw : L - 1) - 1; k >= 1; k--)
-            if (!post(k)) return -1;
+        for (int k = (Lgw < L - 1 ? Lgw : L - 1) - 1; k >= (PAIR ? 1 : 0); k--)
+            if (!post(k, cur)) return -1;
 
-        // ---- u = V-cycle result (the finest level's one-step post-smoothing,
-        // fused), w = A u (+ mean strain), gamma, delta, mean-strain row
+        // ---- u = V-cycle result (FP32: with the finest level's one-step
+        // post-smoothing in the same sweep), w = A u (+ mean strain), gamma, delta, mean-strain row
         Acc<T> acc[2 + NV];
         auto take = [&](const Sums2<T> &sums) {
             acc[0] = sums.ru;
             acc[1] = sums.wu;
             for (int v = 0; v < 3; v++) acc[2 + v].s = T(2) * sums.se[v].s;     // twice half of each cell's stress
         };
-        if (L > 1) {
+        if (PAIR && L > 1) {
             OpFine2<T> &op = *reinterpret_cast<OpFine2<T> *>(s_op);
             static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
             if (lead) {
@@ -896,8 +947,8 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
             __syncthreads();
             take(m2_sweep<T, NT, OFF, OpApply2<T>>(L0.nx, L0.ny, A.zc1[0], bid, nbk));
         }
-        double tt[2 + NV];
-        if (!reduce_barrier<Acc<T>, 2 + NV>(acc, A.partials, A.result, A.bar_count, A.bar_gen, err, tt, bid, nbk)) return -1;
+        double *const tt = S.red;
+        if (!reduce_barrier<Acc<T>, 2 + NV>(acc, A.partials, 0, A.bar_count, A.bar_gen, err, tt, bid, nbk)) return -1;
         if (lead) {
             double s6[6];
             dmat_mul<2>(S.Sl, S.Sm, S.UE, s6);

@@ -811,8 +811,8 @@ __device__ int mg_pass3(const PCGArgs<T, 3> &A, const MGHier<T> &H, PCGState &S,
                 });
         }
         if (!first) {
-            double tr[1];
-            if (!reduce_barrier<Acc<T>, 1>(racc, A.partials, A.result, A.bar_count, A.bar_gen, err, tr, bid, nbk)) return -1;
+            double *const tr = S.red;
+            if (!reduce_barrier<Acc<T>, 1>(racc, A.partials, 1, A.bar_count, A.bar_gen, err, tr, bid, nbk)) return -1;
             if (lead) {
                 double rnew = tr[0];
                 for (int vv = 0; vv < NV; vv++) rnew += S.RE[vv] * S.RE[vv];
@@ -873,8 +873,8 @@ __device__ int mg_pass3(const PCGArgs<T, 3> &A, const MGHier<T> &H, PCGState &S,
 #pragma unroll
                 for (int c = 0; c < 3; c++) prefetch_l1(A.r[cur][c] + n);
             });
-        double tt[2 + NV];
-        if (!reduce_barrier<Acc<T>, 2 + NV>(acc, A.partials, A.result, A.bar_count, A.bar_gen, err, tt, bid, nbk)) return -1;
+        double *const tt = S.red;
+        if (!reduce_barrier<Acc<T>, 2 + NV>(acc, A.partials, 0, A.bar_count, A.bar_gen, err, tt, bid, nbk)) return -1;
         if (lead) {
             double s6[6];
             dmat_mul<3>(S.Sl, S.Sm, S.UE, s6);
