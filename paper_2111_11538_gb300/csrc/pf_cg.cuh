@@ -64,8 +64,8 @@ struct PCGArgs {
     const MGHier<T> *mg;           // multigrid hierarchy (2D, k_pcg<..., MG = true> only)
     double *b64[3];                // MG refinement mode: the FP64 right-hand side, kept from the
                                    // first pass for the later ones
-    int zc1[MG_MAX_LEVELS], zc2[MG_MAX_LEVELS];   // 2D MG: rows per work item of a level's one- and
-                                                  // two-product sweeps (pf_march2.cuh)
+    int zc1[MG_MAX_LEVELS], zc2[MG_MAX_LEVELS];   // MG: rows (3D: planes) per work item of a level's
+                                                  // one- and two-product sweeps (pf_march2.cuh, pf_march3.cuh)
 };
 
 // Grid barrier that also reduces K per-thread values: the warps of a block
@@ -483,6 +483,7 @@ enum { CTL_RUN = 0, CTL_DONE = 1, CTL_ZERO = 2, CTL_STOP = 3 };
 }  // namespace pfdev
 
 #include "pf_march2.cuh"
+#include "pf_march3.cuh"
 #include "pf_mg.cuh"
 #include "pf_mg3.cuh"
 
@@ -501,8 +502,13 @@ template <typename T> struct MGStore<T, false> {};
 template <int D, int S>
 constexpr int tile_threads() { return Tile<D, S>::X * Tile<D, S>::Y * Tile<D, S>::Z; }
 
+// threads of a block: one per tile node; 3D multigrid in FP32: MG3_THREADS
+template <typename T, int D, int S, bool MG>
+constexpr int pcg_threads() { return MG && D == 3 && sizeof(T) == 4 ? MG3_THREADS : tile_threads<D, S>(); }
+
 template <typename T, int D, int SH, bool MG>
-__global__ void __launch_bounds__(tile_threads<D, SH>(), 512 / tile_threads<D, SH>()) k_pcg(const PCGArgs<T, D> *jobs, int njobs)
+__global__ void __launch_bounds__(pcg_threads<T, D, SH, MG>(), MG && D == 3 && sizeof(T) == 4 ? 1 : 512 / tile_threads<D, SH>())
+k_pcg(const PCGArgs<T, D> *jobs, int njobs)
 {
     // this block's job, copied to shared memory
     __shared__ PCGArgs<T, D> sA;
@@ -1075,9 +1081,9 @@ size_t pcg_dyn_smem(int shape, bool mg)
                           : mg_march_offset<T, Tile<2, 0>::X, Tile<2, 0>::Y>() + M2_OP_BYTES;
     }
     if (D == 3 && mg) {
-        // the 3D V-cycle's sweeps (mg_sweep3z in T), or the set-up sweep's
-        // (FP64, three raw streams)
-        const size_t cells = sizeof(T) * (size_t)mg_sweep3z_words<T>();
+        // the FP64 V-cycle's sweeps (mg_sweep3z), or the set-up sweep's (FP64
+        // or double-single, three raw streams)
+        const size_t cells = sizeof(T) == 4 ? 0 : sizeof(T) * (size_t)mg_sweep3z_words<T>();
         const size_t stp = sizeof(double) * (size_t)mg_sweep3z_words<double, true>(3);
         static_assert(sizeof(DS) == sizeof(double) && V3S<DS>::WORDS == V3S<double>::WORDS,
                       "the double-single set-up sweep fits the FP64 one's shared memory");

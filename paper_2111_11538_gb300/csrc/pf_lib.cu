@@ -528,7 +528,8 @@ int setup_cg_launch(pf_handle *h)
     h->pcg_shape = h->cfg.pcg_tile > 0 ? h->cfg.pcg_tile - 1
                                        : (h->mg ? (D == 2 ? mg2_pcg_shape(h->P.N, fp64) : 0)
                                                 : default_pcg_shape(D, h->P.N, fp64));
-    h->cg_block = h->pcg_shape ? tile_threads<D, 1>() : tile_threads<D, 0>();     // one thread per tile node
+    h->cg_block = h->mg ? (h->pcg_shape ? pcg_threads<T, D, 1, true>() : pcg_threads<T, D, 0, true>())
+                        : (h->pcg_shape ? tile_threads<D, 1>() : tile_threads<D, 0>());
     if (h->mg) PF_TRY((build_mg<T, D>(h)));
     int per_sm = 0;
     cudaError_t e = D == 2 ? pcg2_occupancy(fp64, h->pcg_shape, h->mg, h->cg_block, &per_sm)
@@ -711,6 +712,10 @@ int build_plan(pf_handle *h)
             pj[i] = pcg_args<T, D>(I[i]);
             pj[i].block0 = g0;
             pj[i].nblocks = (int)nb;
+            if (D == 3 && I[i]->mg && sizeof(T) == 4)
+                for (int k = 0, nx = I[i]->P.nx, ny = I[i]->P.ny, nz = I[i]->P.nz; k < mg_levels3(I[i]->P.nx, I[i]->P.ny, I[i]->P.nz);
+                     k++, nx /= 2, ny /= 2, nz /= 2)
+                    pj[i].zc1[k] = m3_chunk(nx, ny, nz, (int)nb * (h->cg_block / 32));
             if (D == 2 && I[i]->mg)
                 for (int k = 0, nx = I[i]->P.nx, ny = I[i]->P.ny; k < mg_levels(I[i]->P.nx, I[i]->P.ny); k++, nx /= 2, ny /= 2) {
                     pj[i].zc1[k] = m2_chunk(nx, ny, (int)nb, h->cg_block / 32, 30, 2, sizeof(T) == 8);
@@ -1116,10 +1121,8 @@ int alloc_fields(pf_handle *h)
         }
         if (!h->fp64) {
             h->refine = true;
-            for (int d = 0; d < D; d++) {
-                PF_TRY(h->alloc(&h->corr[d], b));
-                PF_TRY(h->alloc(&h->x64[d], sizeof(double) * (size_t)N));
-            }
+            PF_TRY(h->alloc_comps(h->corr, D, b));
+            for (int d = 0; d < D; d++) PF_TRY(h->alloc(&h->x64[d], sizeof(double) * (size_t)N));
         }
     }
     for (int d = 0; d < D; d++) PF_TRY(h->alloc(&h->u[d], b));

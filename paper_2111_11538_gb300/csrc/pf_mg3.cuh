@@ -56,25 +56,9 @@ __device__ __forceinline__ DS operator*(DS x, DS y)
 }
 __device__ __forceinline__ DS &operator+=(DS &x, DS y) { x = x + y; return x; }
 
-// Shared-memory storage of 3-vectors: FP32 as one float4 per entry (one
-// 128-bit access), FP64 and double-single as three planes of n values.
-// WORDS values of T per entry.
-template <typename T> struct V3S;
-template <> struct V3S<float> {
-    static constexpr int WORDS = 4;
-    __device__ static __forceinline__ void st(float *b, int, int i, const float (&v)[3])
-    {
-        reinterpret_cast<float4 *>(b)[i] = make_float4(v[0], v[1], v[2], 0.f);
-    }
-    __device__ static __forceinline__ void ld(const float *b, int, int i, float (&v)[3])
-    {
-        const float4 a = reinterpret_cast<const float4 *>(b)[i];
-        v[0] = a.x;
-        v[1] = a.y;
-        v[2] = a.z;
-    }
-};
-template <typename T> struct V3Planes {
+// Shared-memory storage of 3-vectors: three planes of n values.  WORDS values
+// of T per entry.
+template <typename T> struct V3S {
     static constexpr int WORDS = 3;
     __device__ static __forceinline__ void st(T *b, int n, int i, const T (&v)[3])
     {
@@ -89,8 +73,6 @@ template <typename T> struct V3Planes {
         v[2] = b[2 * n + i];
     }
 };
-template <> struct V3S<double> : V3Planes<double> {};
-template <> struct V3S<DS> : V3Planes<DS> {};
 
 // Forces of a 3D cell on its eight corner nodes, f[a][comp] with
 // a = ax + 2 ay + 4 az, from its average stress s (mean strain included) and
@@ -118,25 +100,30 @@ __device__ __forceinline__ void corner_forces3(const TC *s, const TC *g, TC (&f)
     }
 }
 
-// Tile of the z-marching 3D sweep: TX x TY nodes per plane, one thread each.
+// Threads of a block of the mixed method's 3D multigrid solve, one block per
+// SM: its sweeps (pf_march3.cuh) take 168 registers a thread without spilling
+// the rows they hold, and are bound by latency, so that more warps beat more
+// rows per warp.  256^3, one V-cycle and CG step: 384 threads 3.29 ms; two
+// blocks of 256 (128 registers) 3.78 ms; 256 (255 registers) with 2 rows per
+// item 4.11 ms, with 4 rows 4.01 ms; 384 with 4 rows 3.61 ms.
+constexpr int MG3_THREADS = 384;
+// Tile of the z-marching 3D sweep of the FP64 V-cycle and of the set-up
+// sweeps: TX x TY nodes per plane, one thread each.
 constexpr int MGZ_TX = 32, MGZ_TY = 8, MGZ_NP = (MGZ_TX + 2) * (MGZ_TY + 2);
 // Streams (arrays read at a staged node) a sweep's operand is formed from,
-// at most; and whether they are copied into shared memory one plane ahead
-// (asynchronous copies, FP32) or read when the plane is staged (FP64, whose
-// sweeps are bound by the FP64 pipe rather than by memory latency).
+// at most (read when the plane is staged: the FP64 V-cycle is bound by the
+// FP64 pipe rather than by memory latency; the set-up sweeps copy theirs one
+// plane ahead, PIPE).
 constexpr int MGZ_NS = 10;
-template <typename T> struct MGZPipe { static constexpr bool on = sizeof(T) == 4; static constexpr int RB = on ? 2 : 1; };
 
 // Shared memory (values of T) of mg_sweep3z with at most ns raw streams: two
-// node planes, the eight corner forces of one cell plane with their halos,
-// the staged nodes' raw streams (two planes when they are copied ahead,
-// PIPE) and, in FP32, the cell moduli of three planes.
-template <typename T, bool PIPE = MGZPipe<T>::on>
+// node planes, the eight corner forces of one cell plane with their halos and
+// the staged nodes' raw streams (two planes when they are copied ahead, PIPE).
+template <typename T, bool PIPE = false>
 __host__ __device__ constexpr int mg_sweep3z_words(int ns = MGZ_NS)
 {
     return V3S<T>::WORDS * (2 * (MGZ_TX + 2) * (MGZ_TY + 2) + 8 * (MGZ_TX + 1) * (MGZ_TY + 1)) +
-           (PIPE ? 2 : 1) * ns * (MGZ_TX + 2) * (MGZ_TY + 2) +
-           (PIPE && sizeof(T) == 4 ? 6 * (MGZ_TX + 1) * (MGZ_TY + 1) : 0);
+           (PIPE ? 2 : 1) * ns * (MGZ_TX + 2) * (MGZ_TY + 2);
 }
 
 // z-chunk of the 3D sweep on an nx x ny x nz level with nbk blocks: the
@@ -164,15 +151,12 @@ __device__ __forceinline__ int mg_zchunk(int nx, int ny, int nz, int nbk)
 // One 3D sweep of the level's Q1 operator, marching along z.  A work item is
 // a TX x TY column of node tiles over zc planes.  Per cell plane zp: the node
 // plane zp + 1 (with its one-node halo in x and y) is formed by
-// make(raw, h, gx, gy, gz, v) from its ns raw streams src[0 .. ns) (FP32:
+// make(raw, h, gx, gy, gz, v) from its ns raw streams src[0 .. ns) (PIPE:
 // copied into shared memory one plane ahead, so that their latency overlaps
 // the previous plane's work; raw[s * NP + h] is stream s at staged node h),
 // every cell of the plane (with the halo cells at x0 - 1, y0 - 1) computes
 // its average stress and hourglass forces once (cell_force3; its moduli, of
-// type TM, are copied with the raw streams two planes ahead in FP32 and read
-// one plane ahead in FP64; PIPE: the raw streams are copied into shared
-// memory one plane ahead, the default in FP32) and its forces on its eight
-// corners
+// type TM, are read one plane ahead) and its forces on its eight corners
 // (corner_forces3), and each own node of plane zp adds its bottom-corner
 // forces to the top-corner forces left by plane zp - 1: q = A v is complete
 // and epi(n, v, q) receives it.  pref(n) runs for each own node of plane zp
@@ -182,7 +166,7 @@ __device__ __forceinline__ int mg_zchunk(int nx, int ny, int nz, int nbk)
 // own cell without it (c[0..5]).  smem: mg_sweep3z_words<T>(ns) values; src:
 // ns pointers (shared memory, set by the caller); two block barriers per
 // plane.
-template <typename T, bool WITH_E, bool PIPE_ = MGZPipe<T>::on, class TM, class Make, class Epi, class CellE,
+template <typename T, bool WITH_E, bool PIPE = false, int NT = MGZ_TX * MGZ_TY, class TM, class Make, class Epi, class CellE,
           class Pref>
 __device__ __forceinline__ void mg_sweep3z(int nx, int ny, int nz, int zc, const TM *lam, const TM *mu, int bid,
                                            int nbk, T *smem, const T *ue, int ns, const T *const *src, Make &&make,
@@ -190,14 +174,11 @@ __device__ __forceinline__ void mg_sweep3z(int nx, int ny, int nz, int zc, const
 {
     constexpr int TX = MGZ_TX, TY = MGZ_TY;
     constexpr int NX = TX + 2, NY = TY + 2, NP = NX * NY;
-    constexpr int CX = TX + 1, CY = TY + 1, NC = CX * CY, NT = TX * TY;
+    constexpr int CX = TX + 1, CY = TY + 1, NC = CX * CY;
     constexpr int W = V3S<T>::WORDS;
-    constexpr bool PIPE = PIPE_, MODC = PIPE && sizeof(T) == 4;   // copied raw streams / moduli
     constexpr int CPT = (NC + NT - 1) / NT;                 // cells per thread
     T *const np0 = smem, *const np1 = smem + W * NP, *const cf = smem + 2 * W * NP;
     T *const rawb = cf + 8 * W * NC;                        // [PIPE ? 2 : 1][ns][NP]
-    T *const modb = rawb + 2 * MGZ_NS * NP;                  // MODC: [3][lam, mu][NC]
-    static_assert(!MODC || std::is_same<TM, T>::value, "copied moduli have the sweep's type");
     const int ntx = (nx + TX - 1) / TX, nty = (ny + TY - 1) / TY, nzc = (nz + zc - 1) / zc;
     const int items = ntx * nty * nzc;
     const bool small = nx < NX || ny < NY;
@@ -207,9 +188,9 @@ __device__ __forceinline__ void mg_sweep3z(int nx, int ny, int nz, int zc, const
         const int x0 = (item % ntx) * TX, y0 = ((item / ntx) % nty) * TY, z0 = (item / (ntx * nty)) * zc;
         const int z1 = min(z0 + zc, nz);
         const int gx = x0 + tx, gy = y0 + ty;
-        const bool own = gx < nx && gy < ny;
+        const bool own = ty < TY && gx < nx && gy < ny;
         auto raw_of = [&](int z) { return rawb + (PIPE ? (z & 1) : 0) * (ns * NP); };
-        // raw streams of node plane z: asynchronous copies (FP32) or loads
+        // raw streams of node plane z: asynchronous copies or loads
         auto issue = [&](int z) {
             const int zw = zwrap(z);
             T *raw = raw_of(z);
@@ -219,21 +200,6 @@ __device__ __forceinline__ void mg_sweep3z(int nx, int ny, int nz, int zc, const
                 for (int q = 0; q < ns; q++) {
                     if constexpr (PIPE) cp_async(raw + q * NP + h, src[q] + g);
                     else raw[q * NP + h] = __ldcg(src[q] + g);
-                }
-            }
-            if constexpr (MODC) {
-                // the moduli of this thread's cells of plane z (read by this
-                // thread only)
-                T *md = modb + ((z + 3) % 3) * 2 * NC;
-#pragma unroll
-                for (int u = 0; u < CPT; u++) {
-                    const int h = threadIdx.x + u * NT;
-                    if (h < NC) {
-                        const int cx = h % CX, cy = h / CX;
-                        const int g = mg_wrap(x0 - 1 + cx, nx, small) + nx * (mg_wrap(y0 - 1 + cy, ny, small) + ny * zw);
-                        cp_async(md + h, reinterpret_cast<const T *>(lam) + g);
-                        cp_async(md + NC + h, reinterpret_cast<const T *>(mu) + g);
-                    }
                 }
             }
         };
@@ -249,7 +215,7 @@ __device__ __forceinline__ void mg_sweep3z(int nx, int ny, int nz, int zc, const
                 V3S<T>::st(buf, NP, h, v);
             }
         };
-        // moduli of this thread's cells of plane z (FP64: into registers)
+        // moduli of this thread's cells of plane z
         auto moduli = [&](int z, T (&l)[CPT], T (&m)[CPT]) {
             const int zw = zwrap(z);
 #pragma unroll
@@ -272,7 +238,7 @@ __device__ __forceinline__ void mg_sweep3z(int nx, int ny, int nz, int zc, const
         }
         form(z0 - 1, ((z0 - 1) & 1) ? np1 : np0);
         T lc[CPT], mc[CPT];
-        if constexpr (!MODC) moduli(z0 - 1, lc, mc);
+        moduli(z0 - 1, lc, mc);
         T qt[3] = {T(0), T(0), T(0)};     // top-corner forces of the previous cell plane on the own node
         for (int zp = z0 - 1; zp < z1; zp++) {
             T *const nlo = (zp & 1) ? np1 : np0;
@@ -288,8 +254,7 @@ __device__ __forceinline__ void mg_sweep3z(int nx, int ny, int nz, int zc, const
             }
             form(zp + 1, nhi);
             T ln[CPT], mn[CPT];
-            if constexpr (!MODC)
-                if (zp + 1 < z1) moduli(zp + 1, ln, mn);
+            if (zp + 1 < z1) moduli(zp + 1, ln, mn);
             __syncthreads();
             const bool inner = zp >= z0;
 #pragma unroll
@@ -297,8 +262,7 @@ __device__ __forceinline__ void mg_sweep3z(int nx, int ny, int nz, int zc, const
                 const int h = threadIdx.x + u * NT;
                 if (h >= NC) continue;
                 const int cx = h % CX, cy = h / CX;
-                const T *md = modb + ((zp + 3) % 3) * 2 * NC;
-                const T l = MODC ? md[h] : lc[u], m = MODC ? md[NC + h] : mc[u];
+                const T l = lc[u], m = mc[u];
                 T uc[8][3];
 #pragma unroll
                 for (int b = 0; b < 8; b++) V3S<T>::ld((b >> 2) ? nhi : nlo, NP, (cx + (b & 1)) + NX * (cy + ((b >> 1) & 1)), uc[b]);
@@ -318,11 +282,9 @@ __device__ __forceinline__ void mg_sweep3z(int nx, int ny, int nz, int zc, const
             }
             T un[3];
             if (own && inner) V3S<T>::ld(nlo, NP, (tx + 1) + NX * (ty + 1), un);
-            if constexpr (!MODC) {
-                if (zp + 1 < z1) {
+            if (zp + 1 < z1) {
 #pragma unroll
-                    for (int u = 0; u < CPT; u++) { lc[u] = ln[u]; mc[u] = mn[u]; }
-                }
+                for (int u = 0; u < CPT; u++) { lc[u] = ln[u]; mc[u] = mn[u]; }
             }
             __syncthreads();
             if (own) {
@@ -489,7 +451,7 @@ __device__ void setup_march3(const PCGArgs<T, 3> &A, bool use_x, bool refine, bo
             for (int c = 0; c < 3; c++) s_xsd[c] = reinterpret_cast<const DS *>(A.x64[c]);
         }
         __syncthreads();
-        mg_sweep3z<DS, true, true>(
+        mg_sweep3z<DS, true, true, MG3_THREADS>(
             P.nx, P.ny, P.nz, mg_zchunk(P.nx, P.ny, P.nz, nbk), A.lam, A.mu, bid, nbk, reinterpret_cast<DS *>(smem),
             s_xd, 3, s_xsd,
             [&](const DS *raw, int h, int, int, int, DS (&v)[3]) {
@@ -575,11 +537,42 @@ __device__ int mg_pass3(const PCGArgs<T, 3> &A, const MGHier<T> &H, PCGState &S,
     };
     auto nopref = [](int) {};
     constexpr int NP = MGZ_NP;
+    // FP32: the warp-marching sweeps (pf_march3.cuh); their operation's record,
+    // filled by the lead thread (every sweep follows a barrier of the whole
+    // block) and read by all
+    constexpr bool F32 = sizeof(T) == 4;
+    __shared__ __align__(16) unsigned char s_op[F32 ? 320 : 16];
+    auto march = [&](auto &op, int k, auto &&fill) {
+        static_assert(sizeof(op) <= 320, "operation record");
+        const MGLevel<T> &V = H.lv[k];
+        if (lead) {
+            fill();
+            op.n = (unsigned)V.nx * V.ny * V.nz;
+            op.lam = V.lam;
+            op.mu = V.mu;
+        }
+        __syncthreads();
+        return m3_sweep(&op, V.nx, V.ny, V.nz, A.zc1[k], bid, nbk);
+    };
 
     // Chebyshev step j on level k (buffer par -> 1 - par); last: also apply
     // step j + 1 and leave the final correction in xpost
     auto cheb = [&](int k, int j, int par, bool post, bool last) {
         const MGLevel<T> &V = H.lv[k];
+        if constexpr (F32) {
+            OpCheb3 &op = *reinterpret_cast<OpCheb3 *>(s_op);
+            march(op, k, [&]() {
+                op.dinv = V.dinv; op.r = V.r[par][0]; op.d = V.d[par][0];
+                // (the iterate after one step from zero is its direction)
+                op.xi = post ? V.xpost[0] : (j == 1 ? V.d[par][0] : V.xpre[0]);
+                op.xo = last || post ? V.xpost[0] : V.xpre[0];
+                op.rn = V.r[1 - par][0]; op.dn = V.d[1 - par][0];
+                op.c1 = H.c1[j]; op.c2 = H.c2[j]; op.n1 = H.c1[j + 1]; op.n2 = H.c2[j + 1];
+                op.last = last;
+                op.dir = j > 0;
+            });
+            return;
+        } else {
         T *const *X = post ? V.xpost : V.xpre;
         const T c1 = H.c1[j], c2 = H.c2[j], n1 = H.c1[j + 1], n2 = H.c2[j + 1];
         sweep(k, j > 0 ? 7 : 4,
@@ -616,6 +609,7 @@ __device__ int mg_pass3(const PCGArgs<T, 3> &A, const MGHier<T> &H, PCGState &S,
                 for (int c = 0; c < 3; c++) { prefetch_l1(X[c] + n); prefetch_l1(V.r[par][c] + n); }
                 if (last) prefetch_l1(V.dinv + n);
             });
+        }
     };
     // restriction (transpose of trilinear prolongation) of level k-1's
     // residual after its pre-smoothing, at node (gx, gy, gz) of level k
@@ -642,6 +636,15 @@ __device__ int mg_pass3(const PCGArgs<T, 3> &A, const MGHier<T> &H, PCGState &S,
     // first pre-smoothing sweep of level k >= 1: f = R r_{k-1}, x = d_0
     auto pre_first = [&](int k) {
         const MGLevel<T> &V = H.lv[k];
+        if constexpr (F32) {
+            OpSmooth3 &op = *reinterpret_cast<OpSmooth3 *>(s_op);
+            march(op, k, [&]() {
+                op.dinv = V.dinv; op.f = V.f[0]; op.r1 = V.r[1][0]; op.d1 = V.d[1][0];
+                op.c2 = H.c2[0];
+                op.dir = (k == L - 1 ? cs - 1 : H.deg[k]) > 1;
+            });
+            return;
+        } else {
         const T c2 = H.c2[0];
         sweep(k, 1, [&](const T **src) { src[0] = V.dinv; },
             [&](const T *raw, int h, int gx, int gy, int gz, T (&v)[3]) {
@@ -673,12 +676,25 @@ __device__ int mg_pass3(const PCGArgs<T, 3> &A, const MGHier<T> &H, PCGState &S,
                 }
             },
             nopref);
+        }
     };
     // first post-smoothing sweep of level k: x = x_pre + P e_{k+1}, r = f - A x;
     // last (one-step smoothing): x + c2[0] D^-1 r is the final correction
     auto post_first = [&](int k, int par, int cur, bool last) {
         const MGLevel<T> &V = H.lv[k];
         const MGLevel<T> &C = H.lv[k + 1];
+        if constexpr (F32) {
+            OpPost3 &op = *reinterpret_cast<OpPost3 *>(s_op);
+            march(op, k, [&]() {
+                op.dinv = V.dinv; op.f = k == 0 ? A.r[cur][0] : V.f[0];
+                op.xpre = V.xpre[0]; op.xc = C.xpost[0];
+                op.xpost = V.xpost[0]; op.rn = V.r[1 - par][0];
+                op.cnx = C.nx; op.cny = C.ny; op.cnz = C.nz; op.cn = (unsigned)C.nx * C.ny * C.nz;
+                op.c2 = H.c2[0];
+                op.last = last;
+            });
+            return;
+        } else
         sweep(k, 3, [&](const T **src) { for (int c = 0; c < 3; c++) src[c] = V.xpre[c]; },
             [&](const T *raw, int h, int gx, int gy, int gz, T (&v)[3]) {
                 const int o[3] = {gx & 1, gy & 1, gz & 1}, ic[3] = {gx >> 1, gy >> 1, gz >> 1};
@@ -730,7 +746,41 @@ __device__ int mg_pass3(const PCGArgs<T, 3> &A, const MGHier<T> &H, PCGState &S,
         }
         return true;
     };
+    // FP32: the restriction in a pass of its own (inside the sweep, every halo
+    // node of every plane restricted again: 500 us on the 128^3 level)
+    auto restrict_pass = [&](int k) {
+        const MGLevel<T> &V = H.lv[k];
+        const MGLevel<T> &F = H.lv[k - 1];
+        const T *fr = F.r[H.deg[k - 1] & 1][0];
+        const unsigned fn = (unsigned)F.nx * F.ny * F.nz, n = (unsigned)V.nx * V.ny * V.nz;
+        for (unsigned i = bid * blockDim.x + threadIdx.x; i < n; i += nbk * blockDim.x) {
+            const int gx = i % V.nx, gy = (i / V.nx) % V.ny, gz = i / ((unsigned)V.nx * V.ny);
+            const int xm = gx == 0 ? F.nx - 1 : 2 * gx - 1;
+            T f[3] = {T(0), T(0), T(0)};
+#pragma unroll
+            for (int cz = -1; cz <= 1; cz++) {
+#pragma unroll
+                for (int cy = -1; cy <= 1; cy++) {
+                    const T *row = fr + (unsigned)(F.nx * (wrap(2 * gy + cy, F.ny) + F.ny * wrap(2 * gz + cz, F.nz)));
+                    const T w = (cz == 0 ? T(1) : T(0.5)) * (cy == 0 ? T(1) : T(0.5));
+#pragma unroll
+                    for (int c = 0; c < 3; c++) {
+                        const T *rc = row + c * fn;
+                        T a[2];
+                        ld_pair(rc + 2 * gx, a);
+                        f[c] += w * (a[0] + T(0.5) * (__ldca(rc + xm) + a[1]));
+                    }
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < 3; c++) V.f[c][i] = f[c];
+        }
+    };
     auto pre = [&](int k) {
+        if constexpr (F32) {
+            restrict_pass(k);
+            if (!sync()) return false;
+        }
         pre_first(k);
         if (!sync()) return false;
         int par = 1;
@@ -761,7 +811,41 @@ __device__ int mg_pass3(const PCGArgs<T, 3> &A, const MGHier<T> &H, PCGState &S,
         // Chebyshev direction is read only by further smoothing steps there
         Acc<T> racc[1];
         const bool d0 = (L == 1 ? cs - 1 : H.deg[0]) > 1;
-        {
+        if constexpr (F32) {
+            // the CG update by itself (p = u + beta p, x += alpha p, s = w + beta
+            // s, r -= alpha s, u: the previous V-cycle's result), so that every
+            // vector is read and written once in whole lines; the smoothing
+            // follows the test of ||r||
+            if (!first) {
+                const unsigned n3 = 3u * (unsigned)L0.nx * L0.ny * L0.nz, n4 = n3 / 4;
+                const float4 *u4 = reinterpret_cast<const float4 *>(L0.xpost[0]), *w4 = reinterpret_cast<const float4 *>(A.w[0][0]);
+                float4 *p4 = reinterpret_cast<float4 *>(A.p[0]), *x4 = reinterpret_cast<float4 *>(A.x[0]);
+                float4 *s4 = reinterpret_cast<float4 *>(A.s[0][0]), *r4 = reinterpret_cast<float4 *>(A.r[0][0]);
+                auto one = [&](float u, float w, float &p, float &x, float &sv, float &r) {
+                    p = u + tb * p;
+                    x = x + ta * p;
+                    sv = w + tb * sv;
+                    r = r - ta * sv;
+                    racc[0].fma_plain(r, r);
+                };
+                for (unsigned i = bid * blockDim.x + threadIdx.x; i < n4; i += nbk * blockDim.x) {
+                    const float4 u = __ldcg(u4 + i), w = __ldcg(w4 + i);
+                    float4 p = __ldcg(p4 + i), x = __ldcg(x4 + i), sv = __ldcg(s4 + i), r = __ldcg(r4 + i);
+                    one(u.x, w.x, p.x, x.x, sv.x, r.x);
+                    one(u.y, w.y, p.y, x.y, sv.y, r.y);
+                    one(u.z, w.z, p.z, x.z, sv.z, r.z);
+                    one(u.w, w.w, p.w, x.w, sv.w, r.w);
+                    p4[i] = p;
+                    x4[i] = x;
+                    s4[i] = sv;
+                    r4[i] = r;
+                }
+                if (bid == 0 && threadIdx.x < (n3 & 3u)) {
+                    const unsigned i = 4 * n4 + threadIdx.x;
+                    one(L0.xpost[0][i], A.w[0][0][i], A.p[0][i], A.x[0][i], A.s[0][0][i], A.r[0][0][i]);
+                }
+            }
+        } else {
             const T c2 = H.c2[0];
             sweep(0, first ? 4 : 10,
                 [&](const T **src) {
@@ -824,11 +908,20 @@ __device__ int mg_pass3(const PCGArgs<T, 3> &A, const MGHier<T> &H, PCGState &S,
                 s_ctl = ctl;
             }
             __syncthreads();
-            cur = nxt;
+            if (!F32) cur = nxt;                 // FP32 updates in place
             const int ctl = s_ctl;
             if (ctl != CTL_RUN) return ctl;
-        } else if (!sync()) {
+        } else if (!F32 && !sync()) {
             return -1;
+        }
+        if constexpr (F32) {
+            OpSmooth3 &op = *reinterpret_cast<OpSmooth3 *>(s_op);
+            march(op, 0, [&]() {
+                op.dinv = L0.dinv; op.f = A.r[0][0]; op.r1 = L0.r[1][0]; op.d1 = L0.d[1][0];
+                op.c2 = H.c2[0];
+                op.dir = d0;
+            });
+            if (!sync()) return -1;
         }
 
         // ---- rest of the V-cycle
@@ -848,6 +941,16 @@ __device__ int mg_pass3(const PCGArgs<T, 3> &A, const MGHier<T> &H, PCGState &S,
 
         // ---- u = V-cycle result, w = A u (+ mean strain), gamma, delta, mean-strain row
         Acc<T> acc[2 + NV];
+        if constexpr (F32) {
+            OpApply3 &op = *reinterpret_cast<OpApply3 *>(s_op);
+            const Sums3 sums = march(op, 0, [&]() {
+                op.u = L0.xpost[0]; op.r = A.r[cur][0]; op.w = A.w[cur][0];
+                for (int v = 0; v < 6; v++) op.ue[v] = s_ue[v];
+            });
+            acc[0] = sums.ru;
+            acc[1] = sums.wu;
+            for (int v = 0; v < 6; v++) acc[2 + v].s = T(4) * sums.se[v].s;     // four times a quarter of each cell's stress
+        } else {
         if (lead)
             for (int c = 0; c < 3; c++) s_src[c] = L0.xpost[c];
         __syncthreads();
@@ -873,6 +976,7 @@ __device__ int mg_pass3(const PCGArgs<T, 3> &A, const MGHier<T> &H, PCGState &S,
 #pragma unroll
                 for (int c = 0; c < 3; c++) prefetch_l1(A.r[cur][c] + n);
             });
+        }
         double *const tt = S.red;
         if (!reduce_barrier<Acc<T>, 2 + NV>(acc, A.partials, 0, A.bar_count, A.bar_gen, err, tt, bid, nbk)) return -1;
         if (lead) {
