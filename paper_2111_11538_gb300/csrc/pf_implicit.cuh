@@ -10,8 +10,9 @@
 // with R the right-hand sides of the explicit update (the same fluxes, the
 // same driving force, the same reaction; the coupling scalars tr eps_e and
 // |dev eps_e|^2 of the mechanics solved at y_n, held over the step).
-// Jacobian-vector products are directional derivatives of F evaluated in
-// forward mode (matrix-free); the linear solves are restarted GMRES
+// Jacobian-vector products are exact (up to rounding): a Newton step's
+// pointwise derivatives are taken once in forward mode and stored, and each
+// product is the linearised stencil with them; the linear solves are restarted GMRES
 // preconditioned by a fixed Chebyshev polynomial of each field's own
 // diffusion block (see k_be_pc_*), in FP64 or FP32 (k_be_pc32_*); FP64
 // everywhere else.
@@ -46,10 +47,10 @@ __device__ __forceinline__ void be_neighbours(const BEArgs &a, long long c, long
     }
 }
 
-// Forward-mode derivative (value, directional derivative): the kernels
-// below evaluate R in it to get J z exactly (up to rounding) rather than by a
-// difference quotient, whose rounding error grows with the stiffness of
-// dt R.
+// Forward-mode derivative (value, directional derivative): the pointwise
+// parts of R are evaluated in it, so that J z is exact (up to rounding)
+// rather than a difference quotient, whose rounding error grows with the
+// stiffness of dt R.
 struct Dual {
     double v, d;
     __device__ __forceinline__ Dual() {}
@@ -68,66 +69,81 @@ __device__ __forceinline__ Dual operator/(Dual a, Dual b)
 __device__ __forceinline__ Dual &operator+=(Dual &a, Dual b) { a = a + b; return a; }
 __device__ __forceinline__ bool be_nonzero(double a) { return a != 0.0; }
 __device__ __forceinline__ bool be_nonzero(Dual a) { return a.v != 0.0; }
-__device__ __forceinline__ double be_val(double a) { return a; }
-__device__ __forceinline__ double be_val(Dual a) { return a.v; }
 
-// mu_O = c sum_a W_a f_a'(x_O) - kappa_O Lap x_O, M_O = D_O / (c sum_a W_a
-// f_a''), D_H, D_H2O (Sec. 2.2, 3.2, Table 1; phase interpolation of the
-// diffusivities) of cell c; ld(b, i) gives field b (theta, x_O, x_H, x_H2O)
-// at cell i.
-template <int D, typename S, class LD>
-__device__ __forceinline__ void be_derive_cell(const BEArgs &a, long long c, LD &&ld, S (&out)[4])
+// The pointwise part of cell c's derived fields: m = c sum_a W_a f_a'(x_O)
+// and M_O = D_O / (c sum_a W_a f_a'') at (theta, x_O) = (th, x).
+template <typename S>
+__device__ __forceinline__ void be_point_cell(const BEArgs &a, long long c, S th, S x, S &m, S &M, S &Wg)
 {
     const CellConst<double> &K = a.K;
-    long long nb[2 * D];
-    be_neighbours<D>(a, c, nb);
-    const S x = ld(1, c);
-    S lap = S(-2.0 * D) * x;
-#pragma unroll
-    for (int q = 0; q < 2 * D; q++) lap += ld(1, nb[q]);
-    S Wf, Ww, Wg;
-    phase_weights<S>(ld(0, c), S(a.phig[c]), Wf, Ww, Wg);
+    S Wf, Ww;
+    phase_weights<S>(th, S(a.phig[c]), Wf, Ww, Wg);
     const S m1 = Wf * f_fe1(x) + Ww * f_wu1(x) + Wg * f_ga1(x);
     const S m2 = Wf * f_fe2(x) + Ww * f_wu2(x) + Wg * f_ga2(x);
-    out[0] = S(K.c) * m1 - S(K.kappa) * lap;
+    m = S(K.c) * m1;
     const S DO = (S(1.0) - Wg) * S(K.DOs) + Wg * S(K.DOg);
     const S den = S(K.c) * m2;
-    out[1] = be_nonzero(den) ? DO / den : S(0.0);
-    out[2] = (S(1.0) - Wg) * S(K.DHs) + Wg * S(K.DHg);
-    out[3] = (S(1.0) - Wg) * S(K.DWs) + Wg * S(K.DWg);
+    M = be_nonzero(den) ? DO / den : S(0.0);
 }
 
-// R(y) of cell c (Sec. 2.4): ld as above, ldd(b, i) the derived field b
-// (mu, M, D_H, D_H2O) at cell i.
-template <int D, typename S, class LD, class LDD>
-__device__ __forceinline__ void be_rates_cell(const BEArgs &a, long long c, LD &&ld, LDD &&ldd, S (&R)[4])
+// The driving force of theta at (th, xo), without the gradient term.
+template <typename S>
+__device__ __forceinline__ S be_force_cell(const BEArgs &a, long long c, S th, S xo)
 {
     const CellConst<double> &K = a.K;
-    long long nb[2 * D];
-    be_neighbours<D>(a, c, nb);
-    const S th = ld(0, c), xo = ld(1, c), xh = ld(2, c), xw = ld(3, c);
-    const S mu0 = ldd(0, c), M0 = ldd(1, c), DH0 = ldd(2, c), DW0 = ldd(3, c);
-    S lapt(0.0), dO(0.0), dH(0.0), dW(0.0);
-#pragma unroll
-    for (int q = 0; q < 2 * D; q++) {
-        const long long n = nb[q];
-        lapt += ld(0, n) - th;
-        dO += S(0.5) * (M0 + ldd(1, n)) * (ldd(0, n) - mu0);
-        dH += S(0.5) * (DH0 + ldd(2, n)) * (ld(2, n) - xh);
-        dW += S(0.5) * (DW0 + ldd(3, n)) * (ld(3, n) - xw);
-    }
-    const double pg = a.phig[c], tE = a.trE[c], s2 = a.devE2[c];
-    const double hg0 = hfun(pg), sol = 1.0 - hg0;
+    const double tE = a.trE[c], s2 = a.devE2[c];
+    const double hg0 = hfun(a.phig[c]), sol = 1.0 - hg0;
     const S hpt = hder(th);
     const S Af = S(K.c) * f_fe(xo) + S(0.5 * K.Ks * tE * tE + K.Gs * s2);
     const S Aw = S(K.c) * f_wu(xo) + S(0.5 * K.Ks * tE * tE + K.Gs * s2);
     const double Kmix = sol * K.Ks + hg0 * K.Kg;
-    const S force = S(sol) * hpt * (Af - Aw) + S(K.w2) * mder(th) - S(K.eig3 * sol * Kmix * tE) * hpt;
-    R[0] = S(K.Lh * a.mob[c]) * (force - S(K.eps2) * lapt);
-    S rr = S(mfun(pg) * K.kf) * xo * xh;
-    if (be_val(xw) >= 1.0) rr = S(0.0);
+    return S(sol) * hpt * (Af - Aw) + S(K.w2) * mder(th) - S(K.eig3 * sol * Kmix * tE) * hpt;
+}
+
+// mu_O = c sum_a W_a f_a'(x_O) - kappa_O Lap x_O, M_O, D_H, D_H2O (Sec. 2.2,
+// 3.2, Table 1; phase interpolation of the diffusivities) of cell c; ld(b, i)
+// gives field b (theta, x_O, x_H, x_H2O) at cell i.
+template <int D, class LD>
+__device__ __forceinline__ void be_derive_cell(const BEArgs &a, long long c, LD &&ld, double (&out)[4])
+{
+    const CellConst<double> &K = a.K;
+    long long nb[2 * D];
+    be_neighbours<D>(a, c, nb);
+    const double x = ld(1, c);
+    double lap = -2.0 * D * x;
+#pragma unroll
+    for (int q = 0; q < 2 * D; q++) lap += ld(1, nb[q]);
+    double m, Wg;
+    be_point_cell<double>(a, c, ld(0, c), x, m, out[1], Wg);
+    out[0] = m - K.kappa * lap;
+    out[2] = (1.0 - Wg) * K.DHs + Wg * K.DHg;
+    out[3] = (1.0 - Wg) * K.DWs + Wg * K.DWg;
+}
+
+// R(y) of cell c (Sec. 2.4): ld as above, ldd(b, i) the derived field b
+// (mu, M, D_H, D_H2O) at cell i.
+template <int D, class LD, class LDD>
+__device__ __forceinline__ void be_rates_cell(const BEArgs &a, long long c, LD &&ld, LDD &&ldd, double (&R)[4])
+{
+    const CellConst<double> &K = a.K;
+    long long nb[2 * D];
+    be_neighbours<D>(a, c, nb);
+    const double th = ld(0, c), xo = ld(1, c), xh = ld(2, c), xw = ld(3, c);
+    const double mu0 = ldd(0, c), M0 = ldd(1, c), DH0 = ldd(2, c), DW0 = ldd(3, c);
+    double lapt = 0.0, dO = 0.0, dH = 0.0, dW = 0.0;
+#pragma unroll
+    for (int q = 0; q < 2 * D; q++) {
+        const long long n = nb[q];
+        lapt += ld(0, n) - th;
+        dO += 0.5 * (M0 + ldd(1, n)) * (ldd(0, n) - mu0);
+        dH += 0.5 * (DH0 + ldd(2, n)) * (ld(2, n) - xh);
+        dW += 0.5 * (DW0 + ldd(3, n)) * (ld(3, n) - xw);
+    }
+    R[0] = K.Lh * a.mob[c] * (be_force_cell<double>(a, c, th, xo) - K.eps2 * lapt);
+    double rr = mfun(a.phig[c]) * K.kf * xo * xh;
+    if (xw >= 1.0) rr = 0.0;
     R[1] = dO - rr;
-    R[2] = dH - S(2.0) * rr;
+    R[2] = dH - 2.0 * rr;
     R[3] = dW + rr;
 }
 
@@ -139,7 +155,7 @@ __global__ void k_be_derive(const BEArgs a, const double *__restrict__ y, double
     auto ld = [&](int b, long long i) { return y[b * N + i]; };
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
         double o[4];
-        be_derive_cell<D, double>(a, c, ld, o);
+        be_derive_cell<D>(a, c, ld, o);
 #pragma unroll
         for (int b = 0; b < 4; b++) der[b * N + c] = o[b];
     }
@@ -164,7 +180,7 @@ __global__ void k_be_rates(const BEArgs a, const double *__restrict__ y, const d
     double mx = 0.0;
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
         double R[4];
-        be_rates_cell<D, double>(a, c, ld, ldd, R);
+        be_rates_cell<D>(a, c, ld, ldd, R);
         if (mode == 1) {
 #pragma unroll
             for (int b = 0; b < 4; b++) out[b * N + c] = R[b];
@@ -187,41 +203,81 @@ __global__ void k_be_rates(const BEArgs a, const double *__restrict__ y, const d
     }
 }
 
-// Jacobian-vector product J z = z - dt R'(y) z (free rows), z (held rows):
-// the derived fields and R in forward mode along z.
-template <int D>
-__global__ void k_be_jderive(const BEArgs a, const double *__restrict__ y, const double *__restrict__ z,
-                             double *__restrict__ dv, double *__restrict__ dd)
+// Pointwise derivatives of a Newton step's state y, for the products with
+// its Jacobian: lin = (dm/dtheta, dm/dx_O, dM/dtheta, dM/dx_O, L mob times
+// dforce/dtheta and dforce/dx_O, d(reaction)/dx_O, d(reaction)/dx_H), 8 N
+// values.  (D_H and D_H2O follow the fixed gas fraction.)
+__global__ void k_be_lin(const BEArgs a, const double *__restrict__ y, double *__restrict__ lin)
 {
     const long long N = a.N;
-    auto ld = [&](int b, long long i) { return Dual(y[b * N + i], z[b * N + i]); };
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
-        Dual o[4];
-        be_derive_cell<D, Dual>(a, c, ld, o);
+        const double th = y[c], xo = y[N + c], xh = y[2 * N + c], xw = y[3 * N + c];
+        const double Lm = a.K.Lh * a.mob[c];
 #pragma unroll
-        for (int b = 0; b < 4; b++) {
-            dv[b * N + c] = o[b].v;
-            dd[b * N + c] = o[b].d;
+        for (int q = 0; q < 2; q++) {
+            const Dual t(th, q == 0 ? 1.0 : 0.0), x(xo, q == 1 ? 1.0 : 0.0);
+            Dual m, M, Wg;
+            be_point_cell<Dual>(a, c, t, x, m, M, Wg);
+            lin[q * N + c] = m.d;
+            lin[(2 + q) * N + c] = M.d;
+            lin[(4 + q) * N + c] = Lm * be_force_cell<Dual>(a, c, t, x).d;
         }
+        const double k = xw >= 1.0 ? 0.0 : mfun(a.phig[c]) * a.K.kf;
+        lin[6 * N + c] = k * xh;
+        lin[7 * N + c] = k * xo;
+    }
+}
+
+// Jacobian-vector product J z = z - dt R'(y) z (free rows), z (held rows), in
+// two passes: the changes of mu and M along z (dv = (dmu, dM)), then the
+// linearised fluxes and sources.  FP64 issue bounds both (GB300 takes 64
+// cycles per warp instruction): ~100 operations per cell against the ~1000 of
+// evaluating R in forward mode for every product.  256^2: 60.5 us -> 17 us.
+template <int D>
+__global__ void k_be_jpoint(const BEArgs a, const double *__restrict__ lin, const double *__restrict__ z,
+                            double *__restrict__ dv)
+{
+    const long long N = a.N;
+    for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
+        long long nb[2 * D];
+        be_neighbours<D>(a, c, nb);
+        const double zt = z[c], zx = z[N + c];
+        double lap = -2.0 * D * zx;
+#pragma unroll
+        for (int q = 0; q < 2 * D; q++) lap += z[N + nb[q]];
+        dv[c] = fma(lin[c], zt, fma(lin[N + c], zx, -a.K.kappa * lap));
+        dv[N + c] = fma(lin[2 * N + c], zt, lin[3 * N + c] * zx);
     }
 }
 
 template <int D>
-__global__ void k_be_jvp(const BEArgs a, const double *__restrict__ y, const double *__restrict__ z,
-                         const double *__restrict__ dv, const double *__restrict__ dd, double *__restrict__ out)
+__global__ void k_be_jvp(const BEArgs a, const double *__restrict__ der, const double *__restrict__ lin,
+                         const double *__restrict__ z, const double *__restrict__ dv, double *__restrict__ out)
 {
     const long long N = a.N;
-    auto ld = [&](int b, long long i) { return Dual(y[b * N + i], z[b * N + i]); };
-    auto ldd = [&](int b, long long i) { return Dual(dv[b * N + i], dd[b * N + i]); };
     for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < N; c += (long long)gridDim.x * blockDim.x) {
-        Dual R[4];
-        be_rates_cell<D, Dual>(a, c, ld, ldd, R);
-        const bool held = a.mask[c] != 0;
+        long long nb[2 * D];
+        be_neighbours<D>(a, c, nb);
+        const double zt = z[c], zx = z[N + c], zh = z[2 * N + c], zw = z[3 * N + c];
+        const double mu0 = der[c], M0 = der[N + c], DH0 = der[2 * N + c], DW0 = der[3 * N + c];
+        const double dmu0 = dv[c], dM0 = dv[N + c];
+        double lapt = -2.0 * D * zt, fo = 0.0, fh = 0.0, fw = 0.0;     // f: twice the flux sums
 #pragma unroll
-        for (int b = 0; b < 4; b++) {
-            const double zz = z[b * N + c];
-            out[b * N + c] = (held && b >= 2) ? zz : zz - a.dt * R[b].d;
+        for (int q = 0; q < 2 * D; q++) {
+            const long long n = nb[q];
+            lapt += z[n];
+            fo = fma(dM0 + dv[N + n], der[n] - mu0, fo);
+            fo = fma(M0 + der[N + n], dv[n] - dmu0, fo);
+            fh = fma(DH0 + der[2 * N + n], z[2 * N + n] - zh, fh);
+            fw = fma(DW0 + der[3 * N + n], z[3 * N + n] - zw, fw);
         }
+        const double r0 = fma(lin[4 * N + c], zt, fma(lin[5 * N + c], zx, -a.K.Lh * a.mob[c] * a.K.eps2 * lapt));
+        const double rr = fma(lin[6 * N + c], zx, lin[7 * N + c] * zh);
+        const bool held = a.mask[c] != 0;
+        out[c] = zt - a.dt * r0;
+        out[N + c] = zx - a.dt * fma(0.5, fo, -rr);
+        out[2 * N + c] = held ? zh : zh - a.dt * fma(0.5, fh, -2.0 * rr);
+        out[3 * N + c] = held ? zw : zw - a.dt * fma(0.5, fw, rr);
     }
 }
 
@@ -364,7 +420,7 @@ struct BEPc32 {
     float *cth;        // N: the theta block's dt L eps mob_c (with its sign)
     float *DO, *DH, *DW;   // N: the diffusivities of the three species blocks
     float *dginv;      // 4N: inverse diagonals
-    float *z, *r, *d0, *d1;   // 4N each: iterate, residual, directions (ping-pong)
+    float *z, *r, *d0, *d1, *r1;   // 4N each: iterate, residual (r1: ping-pong, 2D), directions (ping-pong)
 };
 struct BECheb32 {
     float c1[4], c2[4];
@@ -465,30 +521,245 @@ __global__ void k_be_pc32_final(int N, BEPc32 P, const float *__restrict__ din, 
         }
 }
 
+// The FP32 preconditioner in 2D, several Chebyshev steps per launch.  A step
+// alone moves its 100 bytes per cell through L2 and costs a launch (256^2:
+// 4.9 us + the gap, 31 steps).  Here a block keeps a 32x32 window of all four
+// fields in registers (lane = column, warp = two rows) and takes nsteps <= H
+// steps on it, each spoiling one more ring of cells, so that the
+// (32 - 2H)^2 cells inside are the ones it owns; a step costs it one block
+// barrier, x neighbours by shuffle and y neighbours through shared memory.
+// Redundant cells (32^2 / (32 - 2H)^2) are FP32 work, which is cheap here.
+// Windows wrap around the grid, of any size (a window wider than the grid
+// holds periodic images).
+//   first: r = f v (f: *vf, 1 if null), its owned cells written to vout (the
+//   normalised Krylov vector, not v itself), z = 0, d = c2 D^-1 r;  else r, d
+//   from rin, din and z from P.z.
+//   last: zo = z + d after the steps, else r, d, z are stored for the next.
+constexpr int BE_TILE = 32, BE_TILE_MAXH = 8;
+struct BECheb32Set {
+    BECheb32 k[BE_TILE_MAXH];
+};
+__global__ void __launch_bounds__(512, 1)
+k_be_pc32_tile(int nx, int ny, int N, float dt, const unsigned char *__restrict__ mask, BEPc32 P, int H, int nsteps,
+               BECheb32Set cs, const double *__restrict__ v, const double *__restrict__ vf, double *__restrict__ vout, BECheb32 cinit,
+               const float *__restrict__ rin, const float *__restrict__ din, float *__restrict__ rout,
+               float *__restrict__ dout, double *__restrict__ zo, int first, int last)
+{
+    __shared__ float sd[2][4][BE_TILE][BE_TILE];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int own = BE_TILE - 2 * H, ntx = (nx + own - 1) / own;
+    const int ox = (int)(blockIdx.x % ntx) * own - H, oy = (int)(blockIdx.x / ntx) * own - H;
+    auto modp = [](int a, int n) { a %= n; return a < 0 ? a + n : a; };
+    const int gx = modp(ox + lane, nx);
+    float r[2][4], d[2][4], z[2][4], dg[2][4], cth[2], hf[2], wx[2][3], wl[2][3], wy[3][3];
+    size_t gi[2];
+    bool mine[2];
+    // face weights (D_c + D_n) / 2: right faces, left ones by shuffle, the
+    // three y faces of the two rows
+    {
+        const float *const Ds[3] = {P.DO, P.DH, P.DW};
+        const int gr = modp(gx + 1, nx);
+        float D[4][3];
+#pragma unroll
+        for (int q = 0; q < 4; q++) {
+            const int gy = modp(oy + 2 * wid - 1 + q, ny);
+#pragma unroll
+            for (int f = 0; f < 3; f++) {
+                D[q][f] = Ds[f][gx + (size_t)nx * gy];
+                if (q == 1 || q == 2) wx[q - 1][f] = 0.5f * (D[q][f] + Ds[f][gr + (size_t)nx * gy]);
+            }
+        }
+#pragma unroll
+        for (int f = 0; f < 3; f++) {
+#pragma unroll
+            for (int q = 0; q < 3; q++) wy[q][f] = 0.5f * (D[q][f] + D[q + 1][f]);
+#pragma unroll
+            for (int q = 0; q < 2; q++) wl[q][f] = __shfl_up_sync(0xffffffffu, wx[q][f], 1);
+        }
+    }
+    const double f = first && vf ? *vf : 1.0;
+#pragma unroll
+    for (int q = 0; q < 2; q++) {
+        const int ey = 2 * wid + q, gy = modp(oy + ey, ny);
+        gi[q] = gx + (size_t)nx * gy;
+        mine[q] = lane >= H && lane < BE_TILE - H && ey >= H && ey < BE_TILE - H && ox + lane < nx && oy + ey < ny;
+        cth[q] = P.cth[gi[q]];
+        hf[q] = mask[gi[q]] ? 0.f : dt;
+#pragma unroll
+        for (int b = 0; b < 4; b++) {
+            const size_t i = (size_t)b * N + gi[q];
+            dg[q][b] = P.dginv[i];
+            if (first) {
+                const double vv = v[i] * f;
+                if (mine[q] && vout) vout[i] = vv;
+                r[q][b] = (float)vv;
+                z[q][b] = 0.f;
+                d[q][b] = cinit.c2[b] * r[q][b] * dg[q][b];
+            } else {
+                r[q][b] = rin[i];
+                d[q][b] = din[i];
+                z[q][b] = mine[q] ? P.z[i] : 0.f;
+            }
+        }
+    }
+    for (int k = 0; k < nsteps; k++) {
+        float (*sb)[BE_TILE][BE_TILE] = sd[k & 1];
+#pragma unroll
+        for (int q = 0; q < 2; q++)
+#pragma unroll
+            for (int b = 0; b < 4; b++) sb[b][2 * wid + q][lane] = d[q][b];
+        __syncthreads();
+        const int up = wid == 0 ? 0 : 2 * wid - 1, dn = wid == 15 ? BE_TILE - 1 : 2 * wid + 2;   // the outermost rows are spoilt anyway
+#pragma unroll
+        for (int b = 0; b < 4; b++) {
+            const float dc[2] = {d[0][b], d[1][b]}, du = sb[b][up][lane], dd = sb[b][dn][lane];
+#pragma unroll
+            for (int q = 0; q < 2; q++) {
+                const float l = __shfl_up_sync(0xffffffffu, dc[q], 1), rr_ = __shfl_down_sync(0xffffffffu, dc[q], 1);
+                const float u = q == 0 ? du : dc[0], w = q == 0 ? dc[1] : dd, c = dc[q];
+                float a;
+                if (b == 0) {
+                    a = fmaf(cth[q], (c - l) + (c - rr_) + (c - u) + (c - w), c);
+                } else {
+                    const float f = fmaf(wl[q][b - 1], c - l, fmaf(wx[q][b - 1], c - rr_,
+                                    fmaf(wy[q][b - 1], c - u, wy[q + 1][b - 1] * (c - w))));
+                    a = fmaf(b == 1 ? dt : hf[q], f, c);
+                }
+                z[q][b] += c;
+                r[q][b] -= a;
+                d[q][b] = fmaf(cs.k[k].c1[b], c, cs.k[k].c2[b] * r[q][b] * dg[q][b]);
+            }
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 2; q++)
+        if (mine[q])
+#pragma unroll
+            for (int b = 0; b < 4; b++) {
+                const size_t i = (size_t)b * N + gi[q];
+                if (last) {
+                    zo[i] = (double)(z[q][b] + d[q][b]);
+                } else {
+                    P.z[i] = z[q][b];
+                    rout[i] = r[q][b];
+                    dout[i] = d[q][b];
+                }
+            }
+}
+
 // ---------------------------------------------------------------------------
 // Vector kernels of the Krylov solve (length L = 4N).
 // ---------------------------------------------------------------------------
-// partial dot products of w with nv vectors V + k * L: blockIdx.y = k;
-// part[k * gridDim.x + blockIdx.x]
-__global__ void k_be_dots(long long L, const double *__restrict__ V, int nv, const double *__restrict__ w,
-                          double *__restrict__ part)
+// Classical Gram-Schmidt, one launch per pass: every block owns `per`
+// consecutive elements, which it works on in pieces of BE_CH held in shared
+// memory; the last block to finish adds the blocks' partial sums in block
+// order and leaves them in out.  FP64 issue bounds it: 1 or 2 instructions
+// per element and vector.
+//   GS 0: out[k] = V_k . w;
+//   GS 1: w -= sum_k cin[k] V_k, out[k] = V_k . w (the second pass's
+//         coefficients, on the piece just formed);
+//   GS 2: w -= sum_k cin[k] V_k, out[0] = w . w, out[1] = 1 / |w| (1 if w = 0).
+// 256^2, restarts of 60, per iteration: three dot products of 24 us, two
+// combinations of 15 us, three device-to-host copies with their waits and a
+// scaling before; 16 + 33 + 16 us now.
+constexpr int BE_CH = 1024;
+template <int GS>
+__global__ void __launch_bounds__(256) k_be_gs(long long L, long long per, const double *__restrict__ V, int nv,
+                                               double *w, const double *__restrict__ cin, double *part,
+                                               unsigned int *ticket, double *out)
 {
-    __shared__ double sh[32];
-    const int k = blockIdx.y;
-    if (k >= nv) return;
-    const double *v = V + (size_t)k * L;
-    double s = 0.0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < L; i += (long long)gridDim.x * blockDim.x)
-        s = fma(v[i], w[i], s);
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    __shared__ double sw[BE_CH], sc[64], acc[64];
+    __shared__ bool s_last;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) sh[wid] = s;
-    __syncthreads();
-    if (wid == 0) {
-        s = lane < (int)(blockDim.x >> 5) ? sh[lane] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) part[(size_t)k * gridDim.x + blockIdx.x] = s;
+    if (threadIdx.x < 64) {
+        acc[threadIdx.x] = 0.0;
+        sc[threadIdx.x] = GS > 0 && threadIdx.x < nv ? cin[threadIdx.x] : 0.0;
     }
+    __syncthreads();
+    const long long i0 = blockIdx.x * per, i1 = min(i0 + per, L);
+    double n2 = 0.0;
+    for (long long p0 = i0; p0 < i1; p0 += BE_CH) {
+        const int n = (int)min((long long)BE_CH, i1 - p0);
+        if constexpr (GS > 0) {
+            double s[4] = {0.0, 0.0, 0.0, 0.0};
+            const int t = threadIdx.x;
+#pragma unroll 4
+            for (int k = 0; k < nv; k++) {
+                const double *v = V + (size_t)k * L + p0;
+                const double c = sc[k];
+#pragma unroll
+                for (int q = 0; q < 4; q++)
+                    if (t + 256 * q < n) s[q] = fma(c, v[t + 256 * q], s[q]);
+            }
+#pragma unroll
+            for (int q = 0; q < 4; q++)
+                if (t + 256 * q < n) {
+                    const double x = w[p0 + t + 256 * q] - s[q];
+                    w[p0 + t + 256 * q] = x;
+                    if constexpr (GS == 2) n2 = fma(x, x, n2);
+                    else sw[t + 256 * q] = x;
+                }
+        } else {
+            for (int t = threadIdx.x; t < n; t += 256) sw[t] = w[p0 + t];
+        }
+        if constexpr (GS < 2) {
+            __syncthreads();
+            for (int k = wid; k < nv; k += 8) {
+                const double *v = V + (size_t)k * L + p0;
+                double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
+                int t = lane;
+                for (; t + 96 < n; t += 128) {
+                    s0 = fma(v[t], sw[t], s0);
+                    s1 = fma(v[t + 32], sw[t + 32], s1);
+                    s2 = fma(v[t + 64], sw[t + 64], s2);
+                    s3 = fma(v[t + 96], sw[t + 96], s3);
+                }
+                for (; t < n; t += 32) s0 = fma(v[t], sw[t], s0);
+                double x = (s0 + s1) + (s2 + s3);
+                for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+                if (lane == 0) acc[k] += x;
+            }
+            __syncthreads();
+        }
+    }
+    if constexpr (GS == 2) {
+        for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+        if (lane == 0) sw[wid] = n2;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            double x = 0.0;
+            for (int q = 0; q < 8; q++) x += sw[q];
+            acc[0] = x;
+        }
+        __syncthreads();
+    }
+    const int nk = GS == 2 ? 1 : nv;
+    if (threadIdx.x < nk) part[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = acc[threadIdx.x];
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    for (int k = wid; k < nk; k += 8) {
+        double x = 0.0;
+        for (int b = lane; b < (int)gridDim.x; b += 32) x += __ldcg(part + (size_t)k * gridDim.x + b);
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if (lane == 0) {
+            out[k] = x;
+            if (GS == 2) out[1] = x > 0.0 ? 1.0 / sqrt(x) : 1.0;
+        }
+    }
+    if (threadIdx.x == 0) *ticket = 0u;
+}
+
+// dst = *f v
+__global__ void k_be_scale(long long L, const double *__restrict__ v, const double *__restrict__ f,
+                           double *__restrict__ dst)
+{
+    const double c = *f;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < L; i += (long long)gridDim.x * blockDim.x)
+        dst[i] = c * v[i];
 }
 
 // w += sum_k c[k] V_k (c in device memory, nv <= 64)

@@ -220,6 +220,8 @@ struct pf_handle {
     // first call (be_len values) and the time step of the last step taken
     // that way (0 after explicit steps: the configured dt)
     double *be_ws = nullptr;
+    double *be_host = nullptr;        // pinned: the Krylov sums
+    cudaEvent_t be_ev[2] = {nullptr, nullptr};
     size_t be_len = 0;
     double dt_last = 0.0;
 
@@ -1159,6 +1161,12 @@ void free_all(pf_handle *h)
     h->net_allocs.clear();
     for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
     h->ev_pool.clear();
+    for (cudaEvent_t &e : h->be_ev) {
+        if (e) cudaEventDestroy(e);
+        e = nullptr;
+    }
+    if (h->be_host) cudaFreeHost(h->be_host);
+    h->be_host = nullptr;
     for (void *p : h->allocs) cudaFree(p);
     h->allocs.clear();
     if (h->own) cudaStreamDestroy(h->own);
@@ -1233,43 +1241,57 @@ int create_one(const pf_config *cfg, pf_handle **out, std::string &err)
 // mechanics of the explicit step at y_n, then Newton's method on
 // F(y) = y - y_n - dt R(y) with matrix-free GMRES (pf_implicit.cuh).
 // ---------------------------------------------------------------------------
-constexpr int BE_NDOT = 256;   // blocks of the dot-product kernel
 constexpr int BE_MAX_RESTART = 60;
-// partial sums: the dot products of up to BE_MAX_RESTART + 1 vectors, or the
-// five balance sums of up to 16 blocks per SM on 152 SMs and more
-constexpr size_t BE_NPART = (size_t)BE_NDOT * 65;
+// blocks of the Krylov vector kernels at most, and their partial sums: the
+// dot products of up to BE_MAX_RESTART + 1 vectors, or the five balance sums
+constexpr int BE_NBLK = 512;
+constexpr size_t BE_NPART = (size_t)BE_NBLK * 64;
 
 struct BEWork {
     long long N, L;
     int m;
-    double *y, *y0, *F0, *Ft, *t, *der, *z, *r, *d, *q, *dg, *x, *u, *V;
+    double *y, *y0, *F0, *Ft, *t, *der, *z, *r, *d, *q, *dg, *x, *u, *lin, *V;
     double *part, *hvec;
+    // sums of the Gram-Schmidt passes, two iterations' worth (the host reads
+    // one while the device works on the next): [0, 64) first pass, [64, 128)
+    // second, [128] |w|^2, [129] 1 / |w|; then one such for the other norms
+    double *hs[3];
+    unsigned int *ticket;
     unsigned long long *mx;    // [0] max |F|, [2..3] max |delta|, max |y|, [4..7] Gershgorin s per block
-    BEPc32 pc32;               // the FP32 preconditioner's arrays (24 N floats)
+    BEPc32 pc32;               // the FP32 preconditioner's arrays (28 N floats)
 };
+constexpr int BE_HS = 130;
 
 int be_work(pf_handle *h, int m, BEWork &w)
 {
     const long long N = h->P.N, L = 4 * N;
-    const size_t nvec = 14 + (size_t)(m + 1) + 3;     // the last 3: 24 N floats of the FP32 preconditioner
-    const size_t len = nvec * (size_t)L + BE_NPART + 64 + 8;
+    const size_t nvec = 15 + (size_t)(m + 1) + 4;     // the last 4: 28 N floats of the FP32 preconditioner
+    const size_t len = nvec * (size_t)L + BE_NPART + 64 + 3 * BE_HS + 1 + 8;
     if (h->be_len < len) {
         PF_TRY(h->alloc(&h->be_ws, sizeof(double) * len));
         h->be_len = len;
     }
+    if (!h->be_host) {
+        PF_TRY(h->cuda(cudaMallocHost((void **)&h->be_host, sizeof(double) * 3 * BE_HS), "pinned buffer"));
+        for (cudaEvent_t &e : h->be_ev) PF_TRY(h->cuda(cudaEventCreateWithFlags(&e, cudaEventDisableTiming), "event"));
+    }
     double *p = h->be_ws;
     w.N = N; w.L = L; w.m = m;
+    w.lin = p;                                // 8 N
+    p += 2 * (size_t)L;
     double **vec[14] = {&w.y, &w.y0, &w.F0, &w.Ft, &w.t, &w.der, &w.z, &w.r, &w.d, &w.q, &w.dg, &w.x, &w.u, &w.V};
     for (int k = 0; k < 14; k++) { *vec[k] = p; p += L; }
     p += (size_t)m * L;                       // V holds m + 1 vectors
     float *f = reinterpret_cast<float *>(p);
-    p += 3 * (size_t)L;
-    float **fv[9] = {&w.pc32.cth, &w.pc32.DO, &w.pc32.DH, &w.pc32.DW, &w.pc32.dginv, &w.pc32.z, &w.pc32.r,
-                     &w.pc32.d0, &w.pc32.d1};
-    const long long flen[9] = {N, N, N, N, L, L, L, L, L};
-    for (int k = 0; k < 9; k++) { *fv[k] = f; f += flen[k]; }
+    p += 4 * (size_t)L;
+    float **fv[10] = {&w.pc32.cth, &w.pc32.DO, &w.pc32.DH, &w.pc32.DW, &w.pc32.dginv, &w.pc32.z, &w.pc32.r,
+                     &w.pc32.d0, &w.pc32.d1, &w.pc32.r1};
+    const long long flen[10] = {N, N, N, N, L, L, L, L, L, L};
+    for (int k = 0; k < 10; k++) { *fv[k] = f; f += flen[k]; }
     w.part = p; p += BE_NPART;
     w.hvec = p; p += 64;
+    for (int k = 0; k < 3; k++) { w.hs[k] = p; p += BE_HS; }
+    w.ticket = reinterpret_cast<unsigned int *>(p); p += 1;
     w.mx = reinterpret_cast<unsigned long long *>(p);
     return PF_OK;
 }
@@ -1289,19 +1311,21 @@ int be_steps(pf_handle *h, int nsteps, const pf_implicit_opts &o, pf_implicit_st
     a.K = cell_const<double>(h->P);
     a.phig = (const double *)h->phig; a.mob = (const double *)h->mob;
     a.trE = (const double *)h->trE; a.devE2 = (const double *)h->devE2; a.mask = h->mask;
-    std::vector<double> hp((size_t)BE_NDOT * (m + 1));
     auto check = [&](const char *what) { return h->cuda(cudaGetLastError(), what); };
-    // dot products of w with nv vectors starting at V (fixed summation order)
-    auto dots = [&](const double *Vb, int nv, const double *vw, double *res) -> int {
-        k_be_dots<<<dim3(BE_NDOT, nv), 256, 0, s>>>(L, Vb, nv, vw, w.part);
-        PF_TRY(h->cuda(cudaMemcpyAsync(hp.data(), w.part, sizeof(double) * BE_NDOT * nv, cudaMemcpyDeviceToHost, s),
-                       "dot products"));
-        PF_TRY(h->cuda(cudaStreamSynchronize(s), "dot products"));
-        for (int k = 0; k < nv; k++) {
-            double t = 0.0;
-            for (int b = 0; b < BE_NDOT; b++) t += hp[(size_t)k * BE_NDOT + b];
-            res[k] = t;
-        }
+    // blocks of the Gram-Schmidt passes and their elements (two blocks per SM,
+    // multiples of 64 elements)
+    long long per = (L + 2 * h->sms - 1) / (2 * h->sms);
+    per = (per + 63) / 64 * 64;
+    while ((L + per - 1) / per > BE_NBLK) per += 64;
+    const int gG = (int)((L + per - 1) / per);
+    PF_TRY(h->cuda(cudaMemsetAsync(w.ticket, 0, sizeof(double), s), "ticket"));
+    // |v|^2 and 1 / |v| (in w.hs[2][0, 1])
+    auto norm2 = [&](double *v, double *res) -> int {
+        k_be_gs<2><<<gG, 256, 0, s>>>(L, per, nullptr, 0, v, w.hs[2], w.part, w.ticket, w.hs[2]);
+        double *hp = h->be_host + 2 * BE_HS;
+        PF_TRY(h->cuda(cudaMemcpyAsync(hp, w.hs[2], sizeof(double), cudaMemcpyDeviceToHost, s), "norm"));
+        PF_TRY(h->cuda(cudaStreamSynchronize(s), "norm"));
+        *res = hp[0];
         return PF_OK;
     };
     auto comb = [&](const double *Vb, int nv, const double *c, double *out) -> int {
@@ -1332,7 +1356,43 @@ int be_steps(pf_handle *h, int nsteps, const pf_implicit_opts &o, pf_implicit_st
     std::vector<BECheb32> cheb32;
     BECheb32 cinit32;
     const bool pc32 = o.pc_precision == PF_MIXED;
-    auto precond = [&](const double *v, double *zo) -> int {
+    // steps per launch of the windowed form: launches x (launch, load and store
+    // + steps), each wave of windows counted
+    int tileH = 1;
+    if (D == 2 && pc32 && K > 1) {
+        double best = 1e300;
+        for (int H = 1; H <= BE_TILE_MAXH; H++) {
+            const int own = BE_TILE - 2 * H;
+            const long long nt = (long long)((a.nx + own - 1) / own) * ((a.ny + own - 1) / own);
+            const double waves = (double)((nt + h->sms - 1) / h->sms), nl = (K - 1 + H - 1) / H;
+            const double cost = nl * (2.5 + waves * (3.0 + 0.7 * H));
+            if (cost < best) { best = cost; tileH = H; }
+        }
+    }
+    // zo = M^-1 f v with f = *vf (device; 1 if null); vn: f v itself, a vector
+    // other than v (null: not wanted, f = 1)
+    auto precond = [&](const double *v, const double *vf, double *vn, double *zo) -> int {
+        if (D == 2 && pc32 && K > 0) {
+            const int own = BE_TILE - 2 * tileH;
+            const unsigned nt = (unsigned)(((a.nx + own - 1) / own) * ((a.ny + own - 1) / own));
+            int k0 = 0, par = 0;
+            do {
+                const int ns = std::min(tileH, K - 1 - k0);
+                BECheb32Set set;
+                for (int k = 0; k < BE_TILE_MAXH; k++) set.k[k] = k < ns ? cheb32[k0 + k] : cinit32;
+                k_be_pc32_tile<<<nt, 512, 0, s>>>(a.nx, a.ny, (int)N, (float)a.dt, a.mask, w.pc32, tileH, ns, set, v, vf,
+                                                  vn, cinit32, par ? w.pc32.r1 : w.pc32.r, par ? w.pc32.d1 : w.pc32.d0,
+                                                  par ? w.pc32.r : w.pc32.r1, par ? w.pc32.d0 : w.pc32.d1, zo, k0 == 0,
+                                                  k0 + ns == K - 1);
+                k0 += ns;
+                par ^= 1;
+            } while (k0 < K - 1);
+            return check("preconditioner");
+        }
+        if (vn) {
+            k_be_scale<<<gL, 256, 0, s>>>(L, v, vf, vn);
+            v = vn;
+        }
         if (K == 0) return h->cuda(cudaMemcpyAsync(zo, v, sizeof(double) * L, cudaMemcpyDeviceToDevice, s), "copy");
         if (pc32) {
             const int n32 = (int)N;
@@ -1354,10 +1414,10 @@ int be_steps(pf_handle *h, int nsteps, const pf_implicit_opts &o, pf_implicit_st
         k_be_pc_step<<<gL, 256, 0, s>>>(N, w.q, w.dg, zo, w.r, w.d, cinit, 1);
         return check("preconditioner");
     };
-    // J zz: the directional derivative of F at y, in forward mode
+    // J zz: the directional derivative of F at y (w.der and w.lin of y)
     auto jvp = [&](const double *zz, double *out) -> int {
-        k_be_jderive<D><<<gN, 256, 0, s>>>(a, w.y, zz, w.t, w.Ft);
-        k_be_jvp<D><<<gN, 256, 0, s>>>(a, w.y, zz, w.t, w.Ft, out);
+        k_be_jpoint<D><<<gN, 256, 0, s>>>(a, w.lin, zz, w.t);
+        k_be_jvp<D><<<gN, 256, 0, s>>>(a, w.der, w.lin, zz, w.t, out);
         return check("jvp");
     };
 
@@ -1424,47 +1484,57 @@ int be_steps(pf_handle *h, int nsteps, const pf_implicit_opts &o, pf_implicit_st
             // GMRES(m) on J delta = F0, right preconditioned, from delta = 0
             PF_TRY(h->cuda(cudaMemsetAsync(w.x, 0, sizeof(double) * L, s), "gmres"));
             double beta;
-            PF_TRY(dots(w.F0, 1, w.F0, &beta));
+            PF_TRY(norm2(w.F0, &beta));
             beta = sqrt(beta);
+            k_be_lin<<<gN, 256, 0, s>>>(a, w.y, w.lin);
             const double target = o.gmres_rtol * beta;
             int inner = 0;
             bool first = true;
             while (beta > target && inner < o.gmres_maxit) {
-                if (first) {
-                    k_be_axpby<<<gL, 256, 0, s>>>(L, 1.0 / beta, w.F0, 0.0, w.F0, w.V);
-                } else {
+                // the vector whose direction starts the basis; its 1 / norm is
+                // in w.hs[2][1]
+                const double *v0 = w.F0;
+                if (!first) {
                     // r = F0 - J x
                     PF_TRY(jvp(w.x, w.u));
                     k_be_axpby<<<gL, 256, 0, s>>>(L, 1.0, w.F0, -1.0, w.u, w.u);
                     double b2;
-                    PF_TRY(dots(w.u, 1, w.u, &b2));
+                    PF_TRY(norm2(w.u, &b2));
                     beta = sqrt(b2);
                     if (beta <= target) break;
-                    k_be_axpby<<<gL, 256, 0, s>>>(L, 1.0 / beta, w.u, 0.0, w.u, w.V);
+                    v0 = w.u;
                 }
                 first = false;
                 std::vector<double> H((size_t)(m + 1) * m, 0.0), cs(m), sn(m), g(m + 1, 0.0);
                 g[0] = beta;
                 int j = 0;
                 double res = beta;
-                for (; j < m && inner < o.gmres_maxit;) {
-                    double *vj = w.V + (size_t)j * L, *vn = w.V + (size_t)(j + 1) * L;
-                    PF_TRY(precond(vj, w.z));
-                    PF_TRY(jvp(w.z, vn));
-                    // classical Gram-Schmidt, twice
-                    double hc[64], h2[64], nh[64];
-                    PF_TRY(dots(w.V, j + 1, vn, hc));
-                    for (int k = 0; k <= j; k++) nh[k] = -hc[k];
-                    PF_TRY(comb(w.V, j + 1, nh, vn));
-                    PF_TRY(dots(w.V, j + 1, vn, h2));
-                    for (int k = 0; k <= j; k++) { nh[k] = -h2[k]; hc[k] += h2[k]; }
-                    PF_TRY(comb(w.V, j + 1, nh, vn));
-                    double hn;
-                    PF_TRY(dots(vn, 1, vn, &hn));
-                    hn = sqrt(hn);
-                    for (int k = 0; k <= j; k++) H[(size_t)k * m + j] = hc[k];
+                // iteration q on the stream: V_q = the last vector normalised,
+                // then J M^-1 V_q orthogonalised (classical Gram-Schmidt,
+                // twice) in w.Ft, its coefficients on their way to the host
+                auto enqueue = [&](int q) -> int {
+                    double *hs = w.hs[q & 1];
+                    PF_TRY(precond(q ? w.Ft : v0, q ? w.hs[(q - 1) & 1] + 129 : w.hs[2] + 1, w.V + (size_t)q * L, w.z));
+                    PF_TRY(jvp(w.z, w.Ft));
+                    k_be_gs<0><<<gG, 256, 0, s>>>(L, per, w.V, q + 1, w.Ft, nullptr, w.part, w.ticket, hs);
+                    k_be_gs<1><<<gG, 256, 0, s>>>(L, per, w.V, q + 1, w.Ft, hs, w.part, w.ticket, hs + 64);
+                    k_be_gs<2><<<gG, 256, 0, s>>>(L, per, w.V, q + 1, w.Ft, hs + 64, w.part, w.ticket, hs + 128);
+                    PF_TRY(h->cuda(cudaMemcpyAsync(h->be_host + (q & 1) * BE_HS, hs, sizeof(double) * BE_HS,
+                                                   cudaMemcpyDeviceToHost, s), "Gram-Schmidt"));
+                    return h->cuda(cudaEventRecord(h->be_ev[q & 1], s), "Gram-Schmidt");
+                };
+                PF_TRY(enqueue(0));
+                for (;;) {
+                    // the next iteration is queued before this one's sums are
+                    // waited for (not needed if this one turns out to be the
+                    // last: what it writes is not read then)
+                    const bool more = j + 1 < m && inner + 1 < o.gmres_maxit;
+                    if (more) PF_TRY(enqueue(j + 1));
+                    PF_TRY(h->cuda(cudaEventSynchronize(h->be_ev[j & 1]), "Gram-Schmidt"));
+                    const double *hp = h->be_host + (j & 1) * BE_HS;
+                    const double hn = sqrt(hp[128]);
+                    for (int k = 0; k <= j; k++) H[(size_t)k * m + j] = hp[k] + hp[64 + k];
                     H[(size_t)(j + 1) * m + j] = hn;
-                    if (hn > 0.0) k_be_axpby<<<gL, 256, 0, s>>>(L, 1.0 / hn, vn, 0.0, vn, vn);
                     // Givens rotations of column j
                     for (int k = 0; k < j; k++) {
                         const double a0 = H[(size_t)k * m + j], a1 = H[(size_t)(k + 1) * m + j];
@@ -1482,7 +1552,7 @@ int be_steps(pf_handle *h, int nsteps, const pf_implicit_opts &o, pf_implicit_st
                     res = fabs(g[j + 1]);
                     j++;
                     inner++;
-                    if (res <= target || hn == 0.0) break;
+                    if (res <= target || hn == 0.0 || !more) break;
                 }
                 // x += M^-1 V y, H y = g (upper triangular, j x j)
                 std::vector<double> yv(j, 0.0);
@@ -1493,7 +1563,7 @@ int be_steps(pf_handle *h, int nsteps, const pf_implicit_opts &o, pf_implicit_st
                 }
                 PF_TRY(h->cuda(cudaMemsetAsync(w.u, 0, sizeof(double) * L, s), "gmres"));
                 if (j > 0) PF_TRY(comb(w.V, j, yv.data(), w.u));
-                PF_TRY(precond(w.u, w.z));
+                PF_TRY(precond(w.u, nullptr, nullptr, w.z));
                 k_be_axpby<<<gL, 256, 0, s>>>(L, 1.0, w.x, 1.0, w.z, w.x);
                 beta = res;
             }
