@@ -259,7 +259,7 @@ int pf_step_implicit(pf_handle *h, int nsteps, const pf_implicit_opts *opts, pf_
  * node 0.  Newton's method over opts->nload equal steps of omega, each
  * Newton system solved by conjugate gradients on the energy's Hessian
  * (products evaluated in forward mode, in FP64 or FP32 by opts->precision;
- * the CG scalars stay on the device and the host reads them every 16
+ * the CG scalars stay on the device and the host reads them every 32
  * iterations) with the small-strain diagonal as preconditioner; stops when
  * max |residual| (FP64) <= opts->newton_tol.
  *   theta, phi_g : host arrays of N cells (cell-major, x fastest)
@@ -287,7 +287,8 @@ typedef struct {
     long long cg_iters; /* over all Newton systems                       */
     double residual;    /* max |residual| at the end                     */
     double hvp_ms;      /* device time of the Hessian-vector product
-                           kernel (CUDA events around each launch)       */
+                           kernel (CUDA events around every 32nd launch,
+                           taken for the others as well)                 */
     long long hvp_launches; /* its launches that did work              */
 } pf_fs_stats;
 

@@ -24,8 +24,8 @@
 // preconditioned by the diagonal of the small-strain operator; every
 // product H v is the directional derivative of the residual along v,
 // evaluated in forward mode (value, derivative) through the same cell
-// function as the residual.  FP64 throughout.  Not on the explicit step's
-// hot path: the call allocates and frees its device memory.
+// function as the residual.  Not on the explicit step's hot path: the call
+// allocates and frees its device memory.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -34,6 +34,7 @@
 #include <vector>
 
 #include "pf.h"
+#include "pf_device.cuh"
 
 namespace {
 
@@ -454,14 +455,13 @@ __device__ __forceinline__ void fs_cell(const FSArgs &A, long long c, const FSPa
 // return at once.
 struct FSCG {
     double rz;      // (r, M r)
-    double al;      // step along p
-    double beta;    // direction update
     double tol;     // stop when |r| <= tol
     int stop;       // (p, H p) <= 0: no positive curvature along p
     int done;       // converged or at maxit
     int iters, maxit;
+    int status;     // PF_ETIMEOUT if a barrier gave up
 };
-__device__ __forceinline__ bool fs_cg_over(const FSCG *cg) { return cg && (cg->stop || cg->done); }
+__device__ __forceinline__ bool fs_cg_over(const FSCG *cg) { return cg->stop || cg->done || cg->status; }
 
 // symmetric Fbar (3 x 3) from the m trailing entries of a vector
 template <typename T, typename R>
@@ -521,7 +521,7 @@ __device__ __forceinline__ void fs_block_partials(T (&v)[NV], double *out)
     }
 }
 
-// per cell: corner forces of the state z into cf[c][a][i] (FP64, with the
+// per cell: corner forces of the state z into cf[a * D + i][c] (FP64, with the
 // cell constants pk) and the block partial stress sums into part9
 // (9 x gridDim.x): the residual
 template <int D>
@@ -538,7 +538,7 @@ __global__ void k_fs_res(FSArgs A, const FSPack<double> *pk, const double *z, do
         const FSPack<double> p = pk[c];
         fs_cell<D, double>(A, c, p, [&](long long n, int i) { return z[n * D + i]; }, fb, f, pm);
 #pragma unroll
-        for (int q = 0; q < (1 << D) * D; q++) cf[c * 24 + q] = f[q];
+        for (int q = 0; q < (1 << D) * D; q++) cf[(size_t)q * N + c] = f[q];
 #pragma unroll
         for (int q = 0; q < 9; q++) acc[q] += pm[q];
     }
@@ -570,40 +570,54 @@ k_fs_hvp(FSArgs A, const FSPack<typename RealOf<S>::type> *pk, const typename Re
         const FSPack<R> p = pk[c];
         fs_cell<D, S>(A, c, p, [&](long long n, int i) { return S(z[n * D + i], v[n * D + i]); }, fb, f, pm);
 #pragma unroll
-        for (int q = 0; q < (1 << D) * D; q++) cf[c * 24 + q] = f[q].d;
+        for (int q = 0; q < (1 << D) * D; q++) cf[(size_t)q * N + c] = f[q].d;
 #pragma unroll
         for (int q = 0; q < 9; q++) acc[q] += pm[q].d;
     }
     fs_block_partials<9>(acc, part9);
 }
 
-// nodal forces: each node sums the corner forces of its 2^d cells (in the
-// corner forces' type); node 0 is held (zero).  With p given, also the block
-// partials of (p, out) over the displacement dofs into partdot.
-template <typename R>
-__global__ void k_fs_gather(FSArgs A, const R *cf, double *out, const double *p, double *partdot, const FSCG *cg)
+// nodal force of node n: the sum of the corner forces of its 2^D cells
+// (ld(index in cf))
+template <int D, typename R, class LD>
+__device__ __forceinline__ void fs_node_force(const FSArgs &A, int n, LD &&ld, R (&s)[D])
 {
-    if (fs_cg_over(cg)) return;
-    const int d = A.d, na = 1 << d, nx = A.nx, ny = A.ny;
-    double dot[1] = {0.0};
-    for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < (int)A.N; n += gridDim.x * blockDim.x) {
-        const int i = n % nx, r = n / nx;
-        const int j = r % ny, k = r / ny;
-        const int i0 = i == 0 ? nx - 1 : i - 1, j0 = j == 0 ? ny - 1 : j - 1;
-        const int k0 = d == 3 ? (k == 0 ? A.nz - 1 : k - 1) : 0;
-        R s[3] = {R(0.0), R(0.0), R(0.0)};
-        for (int a = 0; a < na; a++) {
-            const int ci = (a & 1) ? i0 : i, cj = (a & 2) ? j0 : j, ck = (a & 4) ? k0 : k;
-            const size_t c = (size_t)ci + (size_t)nx * (cj + (size_t)ny * ck);
-            for (int q = 0; q < d; q++) s[q] += cf[c * 24 + a * d + q];
-        }
-        for (int q = 0; q < d; q++) {
-            const double o = n == 0 ? 0.0 : (double)s[q];
-            out[n * d + q] = o;
-            if (p) dot[0] = fma(p[n * d + q], o, dot[0]);
-        }
+    const int nx = A.nx, ny = A.ny;
+    const int i = n % nx, r = n / nx;
+    const int j = r % ny, k = r / ny;
+    const int i0 = i == 0 ? nx - 1 : i - 1, j0 = j == 0 ? ny - 1 : j - 1;
+    const int k0 = D == 3 ? (k == 0 ? A.nz - 1 : k - 1) : 0;
+#pragma unroll
+    for (int q = 0; q < D; q++) s[q] = R(0);
+#pragma unroll
+    for (int a = 0; a < (1 << D); a++) {
+        const int ci = (a & 1) ? i0 : i, cj = (a & 2) ? j0 : j, ck = (a & 4) ? k0 : k;
+        const size_t c = (size_t)ci + (size_t)nx * (cj + (size_t)ny * ck);
+#pragma unroll
+        for (int q = 0; q < D; q++) s[q] += ld((size_t)(a * D + q) * A.N + c);
     }
-    if (p) fs_block_partials<1>(dot, partdot);
+}
+
+// nodal forces of the residual; node 0 is held (zero)
+template <int D>
+__global__ void k_fs_gather(FSArgs A, const double *cf, double *out)
+{
+    for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < (int)A.N; n += gridDim.x * blockDim.x) {
+        double s[D];
+        fs_node_force<D, double>(A, n, [&](size_t i) { return cf[i]; }, s);
+#pragma unroll
+        for (int q = 0; q < D; q++) out[(size_t)n * D + q] = n == 0 ? 0.0 : s[q];
+    }
+}
+
+// max |x|
+__global__ void k_fs_maxabs(long long L, const double *x, unsigned long long *out)
+{
+    double m = 0.0;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < L; i += (long long)gridDim.x * blockDim.x)
+        m = fmax(m, fabs(x[i]));
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((threadIdx.x & 31) == 0) atomicMax(out, (unsigned long long)__double_as_longlong(m));
 }
 
 // Jacobi diagonal of the displacement dofs from the small-strain operator
@@ -736,75 +750,181 @@ __global__ void k_fs_rows(int d, int nb, const double *part9, Mat9 pbar, double 
     for (int k = 0; k < (d == 3 ? 6 : 3); k++) outf[k] = rf[k];
 }
 
-// the product's mean-deformation rows into qf, then
-// al = rz / (p, H p) with (p, H p) = the gather's partials + the rows' part
-__global__ void k_fs_cg_alpha(int d, int nb, const double *part9, int ng, const double *partdot, const double *pf,
-                              double *qf, FSCG *cg)
+// ---------------------------------------------------------------------------
+// One CG iteration after its product k_fs_hvp, as one cooperative kernel: the
+// nodes' sums q = H p with (p, q), the update of dz, r and s = M r with |r|^2
+// and (r, s), the new direction; a grid barrier between them.  Every block
+// sums the partials itself, in block order, so all take the same decisions
+// without a broadcast, and in the order of the kernels it replaced (gather,
+// alpha, update, beta, direction: two of them single blocks), so the iterates
+// are theirs bit for bit.
+// 512 threads per block stand for four of those kernels' 128-thread blocks: a
+// quarter of the arrivals at a barrier and of the reads of the partials (608
+// blocks: 55 us).  48^3, FP32 products: 123 us per iteration before (product
+// 60, nodal sums 11, single-block scalar kernels 14, update and direction 12,
+// launches and the host's reads of the state every 16 iterations the rest),
+// 95 us now (product 58, this kernel and its launch 36).  The corner forces
+// lie component by component: 96 bytes per cell one after the other cost the
+// stores and the nodes' loads partial sectors.  (The product inside this
+// kernel: no faster; its derivative in closed form, 2,200 instead of 10,000
+// flops per cell, halves it, but rounds otherwise, and a soft gas region's
+// displacements at the end of a Newton iteration that stops at max |residual|
+// <= 1e-11 follow that rounding by up to 1e-9 of |u|.)
+// ---------------------------------------------------------------------------
+constexpr int FS_CGT = 512, FS_CGV = FS_CGT / 128;
+struct FSCGArgs {
+    FSArgs A;
+    double *p, *q, *dz, *r, *s;
+    float *p32;              // FP32 copy of p, or null
+    const double *dginv;
+    double *part;            // 12 rows of nb partial sums (rows 0..8: the product's stresses)
+    FSCG *cg;
+    unsigned int *bar;       // [0] arrivals, [32] generation
+    int nb;                  // blocks of k_fs_hvp
+};
+
+// grid barrier (bounded: false and PF_ETIMEOUT in *err when it gives up)
+__device__ __forceinline__ bool fs_barrier(unsigned int *bar, int *err)
 {
-    if (fs_cg_over(cg)) return;
-    double ps[9], pd[1];
-    fs_sum_rows<9>(part9, nb, ps);
-    fs_sum_rows<1>(partdot, ng, pd);
-    if (threadIdx.x != 0) return;
-    double rf[6];
-    fs_rows_of(d, ps, rf);
-    double pq = pd[0];
-    for (int k = 0; k < (d == 3 ? 6 : 3); k++) {
-        qf[k] = rf[k];
-        pq = fma(pf[k], rf[k], pq);
+    __shared__ int s_ok;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s_ok = 1;
+        const unsigned int g = pfdev::ld_relaxed_gpu(bar + 32);
+        if (pfdev::atom_add_acq_rel_gpu(bar, 1u) == gridDim.x - 1) {
+            bar[0] = 0u;
+            pfdev::red_add_release_gpu(bar + 32, 1u);
+        } else if (!pfdev::wait_generation(bar + 32, g, err, pfdev::SPIN_LIMIT)) {
+            s_ok = 0;
+        }
     }
-    if (!(pq > 0.0)) {
-        cg->stop = 1;                 // no positive curvature along p
+    __syncthreads();
+    return s_ok != 0;
+}
+// fs_block_partials of each group of 128 threads: group g stands for block
+// blockIdx.x * FS_CGV + g of nb blocks of 128
+template <int NV>
+__device__ __forceinline__ void fs_group_partials(double (&v)[NV], double *out, int nb)
+{
+    __shared__ double sh[FS_CGV][NV][4];
+    const int g = threadIdx.x >> 7, w = (threadIdx.x >> 5) & 3, t = threadIdx.x & 127, vb = (int)blockIdx.x * FS_CGV + g;
+#pragma unroll
+    for (int q = 0; q < NV; q++) {
+        double x = v[q];
+        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+        if ((threadIdx.x & 31) == 0) sh[g][q][w] = x;
+    }
+    __syncthreads();
+    if (t < NV && vb < nb) {
+        double x = 0.0;
+        for (int k = 0; k < 4; k++) x += sh[g][t][k];
+        out[(size_t)t * nb + vb] = x;
+    }
+}
+// rows [0, NV) of nb partials summed into tot, in fs_sum_rows' order (256
+// threads, thread t takes t, t + 256, ...); the two halves of the block take
+// a row each in turn
+template <int NV>
+__device__ __forceinline__ void fs_sum_parts(const double *part, int nb, double *tot)
+{
+    static_assert(FS_CGT == 512, "two groups of fs_sum_rows' threads");
+    __shared__ double sh[NV][8];
+    const int hlf = threadIdx.x >> 8, t = threadIdx.x & 255;
+#pragma unroll
+    for (int q0 = 0; q0 < NV; q0 += 2) {
+        const int q = q0 + hlf;
+        if (q < NV) {
+            double x = 0.0;
+            for (int k = t; k < nb; k += 256) x += __ldcg(part + (size_t)q * nb + k);
+            for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            if ((t & 31) == 0) sh[q][t >> 5] = x;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x < NV) {
+        double x = 0.0;
+        for (int k = 0; k < 8; k++) x += sh[threadIdx.x][k];
+        tot[threadIdx.x] = x;
+    }
+    __syncthreads();
+}
+
+template <int D, typename R>
+__global__ void __launch_bounds__(FS_CGT, 1) k_fs_cg(FSCGArgs a, const R *cf)
+{
+    const FSArgs &A = a.A;
+    if (fs_cg_over(a.cg)) return;
+    constexpr int M = D == 3 ? 6 : 3;
+    __shared__ double tot[12], s_qf[6];
+    __shared__ double s_al;
+    const long long N = A.N, nd = (long long)D * N, L = nd + M;
+    const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x, stp = (long long)a.nb * 128, t1 = t0 < stp ? t0 : 1LL << 62;
+    // (read by every block before the first barrier, written by one after it)
+    const double rz = a.cg->rz, tol = a.cg->tol;
+    const int iters = a.cg->iters, maxit = a.cg->maxit;
+    {
+        double dot[1] = {0.0};
+        for (long long n = t1; n < N; n += stp) {
+            R f[D];
+            fs_node_force<D, R>(A, (int)n, [&](size_t i) { return cf[i]; }, f);
+#pragma unroll
+            for (int q = 0; q < D; q++) {
+                const double o = n == 0 ? 0.0 : (double)f[q];
+                a.q[n * D + q] = o;
+                dot[0] = fma(a.p[n * D + q], o, dot[0]);
+            }
+        }
+        fs_group_partials<1>(dot, a.part + 9 * (size_t)a.nb, a.nb);
+    }
+    if (!fs_barrier(a.bar, &a.cg->status)) return;
+    fs_sum_parts<10>(a.part, a.nb, tot);
+    if (threadIdx.x == 0) {
+        // the product's mean-deformation rows, and al = rz / (p, H p)
+        double ps[9], rf[6], pq = tot[9];
+        for (int q = 0; q < 9; q++) ps[q] = tot[q];
+        fs_rows_of(D, ps, rf);
+        for (int k = 0; k < M; k++) {
+            s_qf[k] = rf[k];
+            pq = fma(a.p[nd + k], rf[k], pq);
+        }
+        s_al = rz / pq;
+        tot[11] = pq;
+    }
+    __syncthreads();
+    const double al = s_al;
+    if (!(tot[11] > 0.0)) {
+        if (t0 == 0) a.cg->stop = 1;            // no positive curvature along p
         return;
     }
-    cg->al = cg->rz / pq;
-}
-
-// dz += al p, r -= al q, s = M r (Jacobi: dginv the inverse diagonal);
-// block partials of (r, r) and (r, s) into part2 (2 x gridDim.x)
-__global__ void k_fs_cg_update(long long L, const double *dginv, const double *p, const double *q, double *dz,
-                               double *r, double *s, const FSCG *cg, double *part2)
-{
-    if (fs_cg_over(cg)) return;
-    const double al = cg->al;
-    double acc[2] = {0.0, 0.0};
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < L; i += (long long)gridDim.x * blockDim.x) {
-        dz[i] = fma(al, p[i], dz[i]);
-        const double ri = fma(-al, q[i], r[i]);
-        r[i] = ri;
-        const double si = ri * dginv[i];
-        s[i] = si;
-        acc[0] = fma(ri, ri, acc[0]);
-        acc[1] = fma(ri, si, acc[1]);
+    {
+        double acc[2] = {0.0, 0.0};
+        for (long long i = t1; i < L; i += stp) {
+            const double qi = i < nd ? __ldcg(a.q + i) : s_qf[i - nd];
+            a.dz[i] = fma(al, a.p[i], a.dz[i]);
+            const double ri = fma(-al, qi, a.r[i]);
+            a.r[i] = ri;
+            const double si = ri * a.dginv[i];
+            a.s[i] = si;
+            acc[0] = fma(ri, ri, acc[0]);
+            acc[1] = fma(ri, si, acc[1]);
+        }
+        fs_group_partials<2>(acc, a.part + 10 * (size_t)a.nb, a.nb);
     }
-    fs_block_partials<2>(acc, part2);
-}
-
-// |r| against the tolerance, then beta = (r, s)_new / (r, s)_old
-__global__ void k_fs_cg_beta(int nb, const double *part2, FSCG *cg)
-{
-    if (fs_cg_over(cg)) return;
-    double t[2];
-    fs_sum_rows<2>(part2, nb, t);
-    if (threadIdx.x != 0) return;
-    cg->iters++;
-    if (sqrt(t[0]) <= cg->tol || cg->iters >= cg->maxit) {
-        cg->done = 1;
-        return;
+    if (!fs_barrier(a.bar, &a.cg->status)) return;
+    fs_sum_parts<2>(a.part + 10 * (size_t)a.nb, a.nb, tot);
+    const bool done = sqrt(tot[0]) <= tol || iters + 1 >= maxit;
+    if (!done) {
+        const double beta = tot[1] / rz;
+        for (long long i = t1; i < L; i += stp) {
+            const double v = fma(beta, a.p[i], a.s[i]);
+            a.p[i] = v;
+            if (a.p32) a.p32[i] = (float)v;
+        }
     }
-    cg->beta = t[1] / cg->rz;
-    cg->rz = t[1];
-}
-
-// p = s + beta p (and its FP32 copy, if kept)
-__global__ void k_fs_cg_dir(long long L, const double *s, double *p, float *p32, const FSCG *cg)
-{
-    if (fs_cg_over(cg)) return;
-    const double b = cg->beta;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < L; i += (long long)gridDim.x * blockDim.x) {
-        const double v = fma(b, p[i], s[i]);
-        p[i] = v;
-        if (p32) p32[i] = (float)v;
+    if (t0 == 0) {
+        a.cg->iters = iters + 1;
+        if (done) a.cg->done = 1;
+        else a.cg->rz = tot[1];
     }
 }
 
@@ -941,7 +1061,7 @@ __global__ void k_fs_force(FSArgs A, const double *z, const double *theta, const
 }
 
 constexpr int FS_NB = 128;     // blocks of the reductions
-constexpr int FS_CHUNK = 16;   // CG iterations launched between two host reads of the CG state
+constexpr int FS_CHUNK = 32;   // CG iterations launched between two host reads of the CG state
 // the mixed method's CG stops at a relative residual of at least this: its
 // FP32 products carry ~1e-7 relative rounding, more along smooth directions
 // (whose nodal sums cancel), and tighter solves only add iterations (inexact
@@ -959,8 +1079,10 @@ struct FSSolver {
     double *dginv = nullptr;             // inverse Jacobi diagonal over [0, L)
     double *cf = nullptr;                // corner forces, N x 24 (FP32 in the mixed product)
     double *part = nullptr;              // FS_NB partials of host-read dot products
-    double *part9 = nullptr, *partdot = nullptr;   // grid x 9 stress and grid (p, Hp) partials
-    double *part2 = nullptr;             // 2 x grid partials of (r, r), (r, s)
+    double *part9 = nullptr;             // 9 x grid partials of the residual's stress sums
+    double *cgpart = nullptr;            // 12 x grid partials of k_fs_cg
+    unsigned long long *mx = nullptr;    // max |residual|
+    unsigned int *bar = nullptr;         // k_fs_cg's barrier words
     double *K = nullptr, *G = nullptr, *Wf = nullptr, *th = nullptr, *pg = nullptr;
     FSPack<double> *pk64 = nullptr;      // cell constants of the load step
     FSPack<float> *pk32 = nullptr;       // their FP32 copy (mixed)
@@ -970,8 +1092,7 @@ struct FSSolver {
     std::vector<double> hp;
     int grid = 0;
     int mixed = 0;                       // FP32 Hessian-vector products
-    cudaEvent_t ev[2 * FS_CHUNK];        // around each product of a chunk
-    bool have_ev = false;
+    cudaEvent_t ev[2] = {nullptr, nullptr};   // around the first product of a chunk
     double hvp_ms = 0.0;
     long long hvp_launches = 0;
 
@@ -985,8 +1106,8 @@ struct FSSolver {
     ~FSSolver()
     {
         for (void *v : mem) cudaFree(v);
-        if (have_ev)
-            for (cudaEvent_t &e : ev) cudaEventDestroy(e);
+        for (cudaEvent_t e : ev)
+            if (e) cudaEventDestroy(e);
     }
     double dot(const double *a, const double *b)
     {
@@ -1007,32 +1128,37 @@ struct FSSolver {
     {
         if (A.d == 3) k_fs_res<3><<<grid, 128>>>(A, pk64, z, cf, part9);
         else k_fs_res<2><<<grid, 128>>>(A, pk64, z, cf, part9);
-        k_fs_gather<double><<<grid, 128>>>(A, cf, r, nullptr, nullptr, nullptr);
+        if (A.d == 3) k_fs_gather<3><<<grid, 128>>>(A, cf, r);
+        else k_fs_gather<2><<<grid, 128>>>(A, cf, r);
         Mat9 pb;
         for (int k = 0; k < 9; k++) pb.v[k] = pbar[k];
         k_fs_rows<<<1, 256>>>(A.d, grid, part9, pb, (double)N, r + nd);
     }
-    // q = H p (events ev0/ev1 around the product kernel), then al
-    void product(cudaEvent_t ev0, cudaEvent_t ev1)
+    // one CG iteration: the product, then the rest of it
+    template <int D, typename S>
+    cudaError_t iteration(const FSPack<typename RealOf<S>::type> *pk, const typename RealOf<S>::type *zr,
+                          const typename RealOf<S>::type *pr, bool timed)
     {
-        const int d = A.d;
-        if (ev0) cudaEventRecord(ev0);
-        if (mixed) {
-            float *cf32 = reinterpret_cast<float *>(cf);
-            if (d == 3) k_fs_hvp<3, FDf><<<grid, 128>>>(A, pk32, z32, p32, cf32, part9, cg);
-            else k_fs_hvp<2, FDf><<<grid, 128>>>(A, pk32, z32, p32, cf32, part9, cg);
-            if (ev1) cudaEventRecord(ev1);
-            k_fs_gather<float><<<grid, 128>>>(A, cf32, q, p, partdot, cg);
-        } else {
-            if (d == 3) k_fs_hvp<3, FD><<<grid, 128>>>(A, pk64, z, p, cf, part9, cg);
-            else k_fs_hvp<2, FD><<<grid, 128>>>(A, pk64, z, p, cf, part9, cg);
-            if (ev1) cudaEventRecord(ev1);
-            k_fs_gather<double><<<grid, 128>>>(A, cf, q, p, partdot, cg);
-        }
-        k_fs_cg_alpha<<<1, 256>>>(d, grid, part9, grid, partdot, p + nd, q + nd, cg);
+        typedef typename RealOf<S>::type R;
+        R *c = reinterpret_cast<R *>(cf);
+        if (timed) cudaEventRecord(ev[0]);
+        k_fs_hvp<D, S><<<grid, 128>>>(A, pk, zr, pr, c, cgpart, cg);
+        if (timed) cudaEventRecord(ev[1]);
+        FSCGArgs a;
+        a.A = A; a.p = p; a.q = q; a.dz = dz; a.r = r; a.s = s; a.p32 = mixed ? p32 : nullptr; a.dginv = dginv;
+        a.part = cgpart; a.cg = cg; a.bar = bar; a.nb = grid;
+        const R *cc = c;
+        void *args[] = {&a, &cc};
+        return cudaLaunchCooperativeKernel((const void *)k_fs_cg<D, R>, dim3((grid + FS_CGV - 1) / FS_CGV), dim3(FS_CGT), args, 0, nullptr);
+    }
+    cudaError_t iteration(bool timed)
+    {
+        if (mixed) return A.d == 3 ? iteration<3, FDf>(pk32, z32, p32, timed) : iteration<2, FDf>(pk32, z32, p32, timed);
+        return A.d == 3 ? iteration<3, FD>(pk64, z, p, timed) : iteration<2, FD>(pk64, z, p, timed);
     }
     // PCG on H dz = -r from dz = 0 (r, p, q, s: residual, direction, H p,
-    // preconditioned residual), then z += dz; returns the iterations taken
+    // preconditioned residual), then z += dz; returns the iterations taken,
+    // -1 after an error (err)
     int cg_solve(double rtol, int maxit)
     {
         cudaMemset(dz, 0, sizeof(double) * L);
@@ -1052,35 +1178,36 @@ struct FSSolver {
         cudaMemcpy(cg, &h, sizeof(h), cudaMemcpyHostToDevice);
         for (;;) {
             const int before = h.iters;
-            for (int k = 0; k < FS_CHUNK; k++) {
-                product(have_ev ? ev[2 * k] : nullptr, have_ev ? ev[2 * k + 1] : nullptr);
-                k_fs_cg_update<<<grid, 128>>>(L, dginv, p, q, dz, r, s, cg, part2);
-                k_fs_cg_beta<<<1, 256>>>(grid, part2, cg);
-                k_fs_cg_dir<<<grid, 128>>>(L, s, p, mixed ? p32 : nullptr, cg);
+            for (int k = 0; k < FS_CHUNK && err == cudaSuccess; k++) err = iteration(k == 0);
+            if (err == cudaSuccess) err = cudaMemcpy(&h, cg, sizeof(h), cudaMemcpyDeviceToHost);
+            if (err != cudaSuccess || h.status) {
+                timeout = h.status != 0;
+                return -1;
             }
-            cudaMemcpy(&h, cg, sizeof(h), cudaMemcpyDeviceToHost);
             // products that did work: one per completed iteration, and the
-            // one that found no positive curvature
+            // one that found no positive curvature; all of a chunk's take
+            // what its first took
             const int ran = h.iters - before + (h.stop ? 1 : 0);
-            if (have_ev)
-                for (int k = 0; k < ran && k < FS_CHUNK; k++) {
-                    float ms = 0.0f;
-                    cudaEventElapsedTime(&ms, ev[2 * k], ev[2 * k + 1]);
-                    hvp_ms += ms;
-                }
+            float ms = 0.0f;
+            cudaEventElapsedTime(&ms, ev[0], ev[1]);
+            hvp_ms += (double)ms * ran;
             hvp_launches += ran;
             if (h.stop || h.done) break;
         }
         k_fs_axpby<<<grid, 128>>>(L, 1.0, dz, 1.0, z);
         return h.iters;
     }
+    cudaError_t err = cudaSuccess;
+    bool timeout = false;
     double maxabs(const double *x)
     {
-        std::vector<double> h((size_t)L);
-        cudaMemcpy(h.data(), x, sizeof(double) * L, cudaMemcpyDeviceToHost);
-        double mx = 0.0;
-        for (double v : h) mx = std::max(mx, std::fabs(v));
-        return mx;
+        unsigned long long v = 0;
+        cudaMemsetAsync(mx, 0, sizeof(v));
+        k_fs_maxabs<<<grid, 128>>>(L, x, mx);
+        cudaMemcpy(&v, mx, sizeof(v), cudaMemcpyDeviceToHost);
+        double m;
+        memcpy(&m, &v, sizeof(m));
+        return m;
     }
 };
 
@@ -1129,26 +1256,21 @@ int fs_run(const pf_config *cfg, const double *theta, const double *phi_g, doubl
     if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
         return fs_fail(PF_ECUDA, "no CUDA device");
     S.grid = (int)std::min<long long>((N + 127) / 128, 4LL * std::max(sms, 1));
-    double **bufs[11] = {&S.z, &S.r, &S.p, &S.q, &S.s, &S.dz, &S.dg, &S.dginv, &S.part, &S.part2, &S.partdot};
-    const size_t lens[11] = {(size_t)L, (size_t)L, (size_t)L, (size_t)L, (size_t)L, (size_t)L, (size_t)S.nd,
-                             (size_t)L, (size_t)FS_NB, (size_t)S.grid * 2, (size_t)S.grid};
-    for (int k = 0; k < 11; k++)
+    double **bufs[10] = {&S.z, &S.r, &S.p, &S.q, &S.s, &S.dz, &S.dg, &S.dginv, &S.part, &S.cgpart};
+    const size_t lens[10] = {(size_t)L, (size_t)L, (size_t)L, (size_t)L, (size_t)L, (size_t)L, (size_t)S.nd,
+                             (size_t)L, (size_t)FS_NB, (size_t)S.grid * 12};
+    for (int k = 0; k < 10; k++)
         if (S.alloc(bufs[k], lens[k]) != cudaSuccess) return fs_fail(PF_ENOMEM, "cudaMalloc failed");
     if (S.alloc(&S.part9, (size_t)S.grid * 9) != cudaSuccess || S.alloc(&S.cg, 1) != cudaSuccess ||
+        S.alloc(&S.mx, 1) != cudaSuccess || S.alloc(&S.bar, 64) != cudaSuccess ||
         S.alloc(&S.pk64, (size_t)N) != cudaSuccess)
         return fs_fail(PF_ENOMEM, "cudaMalloc failed");
     if (S.mixed && (S.alloc(&S.pk32, (size_t)N) != cudaSuccess || S.alloc(&S.z32, (size_t)L) != cudaSuccess ||
                     S.alloc(&S.p32, (size_t)L) != cudaSuccess))
         return fs_fail(PF_ENOMEM, "cudaMalloc failed");
-    {
-        int ok = 0;
-        while (ok < 2 * FS_CHUNK && cudaEventCreate(&S.ev[ok]) == cudaSuccess) ok++;
-        if (ok < 2 * FS_CHUNK) {
-            for (int k = 0; k < ok; k++) cudaEventDestroy(S.ev[k]);
-            return fs_fail(PF_ECUDA, "cudaEventCreate failed");
-        }
-        S.have_ev = true;
-    }
+    cudaMemset(S.bar, 0, sizeof(unsigned int) * 64);
+    for (cudaEvent_t &e : S.ev)
+        if (cudaEventCreate(&e) != cudaSuccess) return fs_fail(PF_ECUDA, "cudaEventCreate failed");
     if (S.alloc(&S.cf, (size_t)N * 24) != cudaSuccess || S.alloc(&S.K, N) != cudaSuccess || S.alloc(&S.G, N) != cudaSuccess || S.alloc(&S.Wf, N) != cudaSuccess ||
         S.alloc(&S.th, N) != cudaSuccess || S.alloc(&S.pg, N) != cudaSuccess)
         return fs_fail(PF_ENOMEM, "cudaMalloc failed");
@@ -1228,7 +1350,13 @@ int fs_run(const pf_config *cfg, const double *theta, const double *phi_g, doubl
                 return fs_fail(PF_ENOTCONV, "finite-strain Newton iteration did not converge");
             }
             st.newton_iters++;
-            st.cg_iters += S.cg_solve(S.mixed ? std::max(opts->cg_rtol, FS_MIXED_RTOL) : opts->cg_rtol, opts->cg_maxit);
+            const int ni = S.cg_solve(S.mixed ? std::max(opts->cg_rtol, FS_MIXED_RTOL) : opts->cg_rtol, opts->cg_maxit);
+            if (ni < 0) {
+                if (stats) *stats = st;
+                return S.timeout ? fs_fail(PF_ETIMEOUT, "a bounded device-side wait gave up")
+                                 : fs_fail(PF_ECUDA, cudaGetErrorString(S.err));
+            }
+            st.cg_iters += ni;
         }
     }
     cudaError_t e = cudaGetLastError();
