@@ -203,7 +203,10 @@ struct pf_handle {
     void *d_cell_jobs[2] = {nullptr, nullptr};
     void *d_fused_jobs[2] = {nullptr, nullptr};
     void *d_pcg_jobs = nullptr;
-    int cell_grid = 0, fused_grid = 0, pcg_grid = 0, njobs = 0;
+    int cell_grid = 0, fused_grid = 0, njobs = 0;
+    // the CG launches of a step: jobs [first, first + n), grid blocks each
+    struct PcgRound { int first, n, grid; };
+    std::vector<PcgRound> pcg_rounds;
     int cg_per_sm = 0;
     int fused_per_sm = 0;               // resident blocks per SM of the marching update
     int pcg_shape = 0;                  // node tile of the PCG sweep (pf_cg.cuh Tile<D, S>)
@@ -690,42 +693,51 @@ int build_plan(pf_handle *h)
         // finish together
         std::vector<long long> tiles(n);
         std::vector<double> work(n);
-        double wtot = 0.0;
         for (int i = 0; i < n; i++) {
             const Params &P = I[i]->P;
             tiles[i] = (long long)((P.nx + TX - 1) / TX) * ((P.ny + TY - 1) / TY) * (D == 3 ? (P.nz + TZ - 1) / TZ : 1);
             const double lin = (double)std::max(P.nx, std::max(P.ny, D == 3 ? P.nz : 1));
             work[i] = (double)tiles[i] * (I[i]->mg ? 1.0 : lin);     // MG: iterations ~ independent of size
-            wtot += work[i];
         }
+        // One launch holds an instance per resident block at most.  3D in
+        // FP32 runs one large block per SM and takes batches of up to two
+        // instances per SM, in two launches then.
         const long long cap = (long long)h->cg_per_sm * h->sms;
-        if (cap < n) return h->fail(PF_EINVAL, "batch of %d instances exceeds the %lld co-resident CG blocks", n, cap);
+        const long long most_n = D == 3 && sizeof(T) == 4 ? std::max(cap, 2LL * h->sms) : cap;
+        if (most_n < n) return h->fail(PF_EINVAL, "batch of %d instances exceeds the %lld co-resident CG blocks", n, most_n);
+        const int rounds = (int)((n + cap - 1) / cap);
         std::vector<PCGArgs<T, D>> pj(n);
-        int g0 = 0;
-        for (int i = 0; i < n; i++) {
-            long long nb = 1 + (long long)((double)(cap - n) * work[i] / wtot);
-            // the marching sweeps of the 2D V-cycle share out single rows:
-            // a block for every 16 nodes in FP64 (its SM's FP64 pipes are what
-            // they wait for, and blocks without rows prepare the dense map of
-            // the block-run levels), for every 256 in FP32
-            const long long most = D == 2 && I[i]->mg ? (I[i]->P.N + (sizeof(T) == 8 ? 15 : 255)) / (sizeof(T) == 8 ? 16 : 256)
-                                                      : tiles[i];
-            if (nb > most) nb = most > 0 ? most : 1;
-            pj[i] = pcg_args<T, D>(I[i]);
-            pj[i].block0 = g0;
-            pj[i].nblocks = (int)nb;
-            if (D == 3 && I[i]->mg && sizeof(T) == 4)
-                for (int k = 0, nx = I[i]->P.nx, ny = I[i]->P.ny, nz = I[i]->P.nz; k < mg_levels3(I[i]->P.nx, I[i]->P.ny, I[i]->P.nz);
-                     k++, nx /= 2, ny /= 2, nz /= 2)
-                    pj[i].zc1[k] = m3_chunk(nx, ny, nz, (int)nb * (h->cg_block / 32));
-            if (D == 2 && I[i]->mg)
-                for (int k = 0, nx = I[i]->P.nx, ny = I[i]->P.ny; k < mg_levels(I[i]->P.nx, I[i]->P.ny); k++, nx /= 2, ny /= 2) {
-                    pj[i].zc1[k] = m2_chunk(nx, ny, (int)nb, h->cg_block / 32, 30, 2, sizeof(T) == 8);
-                    pj[i].zc2[k] = m2_chunk(nx, ny, (int)nb, h->cg_block / 32, 28, 4, sizeof(T) == 8);
-                }
-            g0 += (int)nb;
+        h->pcg_rounds.clear();
+        for (int q = 0; q < rounds; q++) {
+            const int i0 = (int)((long long)n * q / rounds), i1 = (int)((long long)n * (q + 1) / rounds);
+            double wtot = 0.0;
+            for (int i = i0; i < i1; i++) wtot += work[i];
+            int g0 = 0;
+            for (int i = i0; i < i1; i++) {
+                long long nb = 1 + (long long)((double)(cap - (i1 - i0)) * work[i] / wtot);
+                // the marching sweeps of the 2D V-cycle share out single rows:
+                // a block for every 16 nodes in FP64 (its SM's FP64 pipes are what
+                // they wait for, and blocks without rows prepare the dense map of
+                // the block-run levels), for every 256 in FP32
+                const long long most = D == 2 && I[i]->mg ? (I[i]->P.N + (sizeof(T) == 8 ? 15 : 255)) / (sizeof(T) == 8 ? 16 : 256)
+                                                          : tiles[i];
+                if (nb > most) nb = most > 0 ? most : 1;
+                pj[i] = pcg_args<T, D>(I[i]);
+                pj[i].block0 = g0;
+                pj[i].nblocks = (int)nb;
+                if (D == 3 && I[i]->mg && sizeof(T) == 4)
+                    for (int k = 0, nx = I[i]->P.nx, ny = I[i]->P.ny, nz = I[i]->P.nz; k < mg_levels3(I[i]->P.nx, I[i]->P.ny, I[i]->P.nz);
+                         k++, nx /= 2, ny /= 2, nz /= 2)
+                        pj[i].zc1[k] = m3_chunk(nx, ny, nz, (int)nb * (h->cg_block / 32));
+                if (D == 2 && I[i]->mg)
+                    for (int k = 0, nx = I[i]->P.nx, ny = I[i]->P.ny; k < mg_levels(I[i]->P.nx, I[i]->P.ny); k++, nx /= 2, ny /= 2) {
+                        pj[i].zc1[k] = m2_chunk(nx, ny, (int)nb, h->cg_block / 32, 30, 2, sizeof(T) == 8);
+                        pj[i].zc2[k] = m2_chunk(nx, ny, (int)nb, h->cg_block / 32, 28, 4, sizeof(T) == 8);
+                    }
+                g0 += (int)nb;
+            }
+            h->pcg_rounds.push_back({i0, i1 - i0, g0});
         }
-        h->pcg_grid = g0;
         const size_t pbytes = sizeof(PCGArgs<T, D>) * (size_t)n;
         if (!h->d_pcg_jobs) PF_TRY(h->alloc(&h->d_pcg_jobs, pbytes));
         PF_TRY(h->cuda(cudaMemcpy(h->d_pcg_jobs, pj.data(), pbytes, cudaMemcpyHostToDevice), "job table"));
@@ -806,8 +818,13 @@ int launch_mechanics(pf_handle *h, cudaStream_t s, int k)
         }
         h->mark_begin(PF_K_CG, s);
         const bool fp64 = sizeof(T) == 8;
-        cudaError_t e = D == 2 ? pcg2_launch(fp64, h->pcg_shape, h->mg, h->d_pcg_jobs, n, h->pcg_grid, h->cg_block, s)
-                               : pcg3_launch(fp64, h->pcg_shape, h->mg, h->d_pcg_jobs, n, h->pcg_grid, h->cg_block, s);
+        cudaError_t e = cudaSuccess;
+        for (const auto &q : h->pcg_rounds) {
+            const void *jobs = (const PCGArgs<T, D> *)h->d_pcg_jobs + q.first;
+            if (e == cudaSuccess)
+                e = D == 2 ? pcg2_launch(fp64, h->pcg_shape, h->mg, jobs, q.n, q.grid, h->cg_block, s)
+                           : pcg3_launch(fp64, h->pcg_shape, h->mg, jobs, q.n, q.grid, h->cg_block, s);
+        }
         h->mark_end(s);
         if (e != cudaSuccess) return h->cuda(e, "cooperative CG launch");
         h->mark_begin(PF_K_RETURN, s);

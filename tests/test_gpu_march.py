@@ -13,7 +13,7 @@ The stress, linear in u, gets the factor 1e3 (1e-5, 1e-2 of its largest value)."
 import numpy as np
 import pytest
 
-from paper_2111_11538_gb300 import Simulation, inputs, native, workloads
+from paper_2111_11538_gb300 import Batch, Simulation, inputs, native, workloads
 
 pytestmark = pytest.mark.gpu
 
@@ -59,3 +59,30 @@ def test_sweeps_match_jacobi(shape, precision, rtol, tol):
         assert rel(gm[k], gj[k]) < tol, (k, rel(gm[k], gj[k]))
     assert rel(gm["sigma"], gj["sigma"]) < 1e3 * tol, rel(gm["sigma"], gj["sigma"])
     assert rel(gm["Ebar"], gj["Ebar"]) < 1e3 * tol
+
+
+def test_large_3d_batch_in_two_launches():
+    """A batch of more 3D mixed instances than the device has SMs (their CG
+    blocks take an SM each) runs in two launches; every instance ends where a
+    solve of its own does.  The two differ in the blocks that share the work
+    and so in the rounding of FP32 sums: 1e-5, as for the solves above."""
+    shapes = [(8, 8, 8), (16, 8, 10)] * 100
+    prm = workloads.params(plasticity=1, sigma_Y=0.004, H_hard=0.01, cg_rtol=1e-8, precond="mg")
+    fields = {s: inputs.core_shell(s, 2.4, 1.8, delta=1.5) for s in set(shapes)}
+    b = Batch(shapes, prm, precision="mixed")
+    for i, s in enumerate(shapes):
+        b.set_fields(i, fields[s])
+    b.step(2)
+    ref = {}
+    for s in set(shapes):
+        sim = Simulation(s, prm, precision="mixed")
+        sim.set_fields(fields[s])
+        sim.step(2)
+        ref[s] = sim.get_fields()
+        sim.close()
+    for i in (0, 1, 98, 99, 100, 101, 198, 199):
+        got = b.get_fields(i)
+        for k in KEYS:
+            assert rel(got[k], ref[shapes[i]][k]) < 1e-5, (i, k)
+        assert rel(got["sigma"], ref[shapes[i]]["sigma"]) < 1e-2
+    b.close()
