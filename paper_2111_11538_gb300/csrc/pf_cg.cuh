@@ -502,12 +502,43 @@ template <typename T> struct MGStore<T, false> {};
 template <int D, int S>
 constexpr int tile_threads() { return Tile<D, S>::X * Tile<D, S>::Y * Tile<D, S>::Z; }
 
-// threads of a block: one per tile node; 3D multigrid in FP32: MG3_THREADS
+// The Jacobi loops' scalars after a sweep's reduction (tt: gamma, delta,
+// ||r||^2, mean-strain row): counts the iteration, tests ||r|| <= target, takes
+// gamma and delta; returns what to do next to every thread.
+template <int D>
+__device__ __forceinline__ int pcg_step(PCGState &S, const double *tt, bool was_first, double target, int maxit, int &s_ctl)
+{
+    constexpr int NV = Dims<D>::NV;
+    if (threadIdx.x == 0) {
+        double s6[6];
+        dmat_mul<D>(S.Sl, S.Sm, S.UE, s6);
+        for (int vv = 0; vv < NV; vv++) S.WE[vv] = tt[3 + vv] + s6[vv];
+        double gnew = tt[0], dnew = tt[1], rnew = tt[2];
+        for (int vv = 0; vv < NV; vv++) {
+            gnew += S.RE[vv] * S.UE[vv];
+            dnew += S.WE[vv] * S.UE[vv];
+            rnew += S.RE[vv] * S.RE[vv];
+        }
+        int ctl = CTL_RUN;
+        if (!was_first) {
+            S.it++;
+            S.rho_final = rnew;
+            if (rnew <= target * target) ctl = CTL_DONE;      // ||r|| <= target without a square root
+            else if (S.it_total + S.it >= maxit) ctl = CTL_STOP;
+        }
+        cg_take_gamma_delta(S, gnew, dnew, was_first);
+        s_ctl = ctl;
+    }
+    __syncthreads();
+    return s_ctl;
+}
+
+// threads of a block: one per tile node; 3D in FP32 (pf_march3.cuh): MG3_THREADS
 template <typename T, int D, int S, bool MG>
-constexpr int pcg_threads() { return MG && D == 3 && sizeof(T) == 4 ? MG3_THREADS : tile_threads<D, S>(); }
+constexpr int pcg_threads() { return D == 3 && sizeof(T) == 4 ? MG3_THREADS : tile_threads<D, S>(); }
 
 template <typename T, int D, int SH, bool MG>
-__global__ void __launch_bounds__(pcg_threads<T, D, SH, MG>(), MG && D == 3 && sizeof(T) == 4 ? 1 : 512 / tile_threads<D, SH>())
+__global__ void __launch_bounds__(pcg_threads<T, D, SH, MG>(), D == 3 && sizeof(T) == 4 ? 1 : 512 / tile_threads<D, SH>())
 k_pcg(const PCGArgs<T, D> *jobs, int njobs)
 {
     // this block's job, copied to shared memory
@@ -527,17 +558,15 @@ k_pcg(const PCGArgs<T, D> *jobs, int njobs)
     constexpr int CX = TX + 1, CY = TY + 1, CZ = D == 3 ? TZ + 1 : 1;
     constexpr int HN = HX * HY * HZ, HC = CX * CY * CZ;
     constexpr int MAX_OUTER = 24;
+    // 3D FP32: warp-marching sweeps (pf_march3.cuh)
+    constexpr bool MARCH = D == 3 && sizeof(T) == 4;
     // the node and cell tiles of the plain sweep (the multigrid variants
     // keep theirs in the dynamic shared memory)
-    __shared__ T su[MG ? 1 : D * HN];
-    __shared__ T sl[MG ? 1 : HC], sm[MG ? 1 : HC];
-    // per-cell stress and hourglass forces: 2D 5 values per cell; 3D FP32 on
-    // the 16x4x4 tile 20 (five float4); other 3D variants use the
-    // element-matrix path and need none
-    constexpr bool CELL3 = D == 3 && sizeof(T) == 4 && SH == 0;
-    __shared__ __align__(16) T scell2[D == 2 && !MG ? 5 * HC : 1];
-    // pcg_dyn, CELL3: 20 * HC floats; MG: block-run levels, sweeps
-    T *scell = CELL3 ? reinterpret_cast<T *>(pcg_dyn) : scell2;
+    __shared__ T su[MG || MARCH ? 1 : D * HN];
+    __shared__ T sl[MG || MARCH ? 1 : HC], sm[MG || MARCH ? 1 : HC];
+    // 2D: per-cell stress and hourglass forces, 5 values per cell (3D FP64
+    // uses the element-matrix path and needs none)
+    __shared__ __align__(16) T scell[D == 2 && !MG ? 5 * HC : 1];
     __shared__ T s_ta, s_tb, s_ue[6], s_xe[6];
     __shared__ int s_ctl;
 
@@ -554,7 +583,7 @@ k_pcg(const PCGArgs<T, D> *jobs, int njobs)
     const bool small = P.nx < TX + 2 || P.ny < TY + 2 || (D == 3 && P.nz < TZ + 2);
 
     __shared__ PCGState S;
-    double *XE = S.XE, *E64 = S.E64, *DiagE = S.DiagE, *RE = S.RE, *UE = S.UE, *PE = S.PE, *SE = S.SE, *WE = S.WE;
+    double *XE = S.XE, *E64 = S.E64, *DiagE = S.DiagE, *RE = S.RE, *UE = S.UE, *PE = S.PE, *SE = S.SE;
     double &Sl = S.Sl, &Sm = S.Sm, &bnorm = S.bnorm, &rho_final = S.rho_final, &target = S.target;
     double &gamma = S.gamma, &delta = S.delta, &gamma_prev = S.gamma_prev, &alpha_prev = S.alpha_prev;
     double &alpha = S.alpha, &beta = S.beta;
@@ -745,6 +774,61 @@ k_pcg(const PCGArgs<T, D> *jobs, int njobs)
                 rc = mg_pass3<T>(A, sH.h, S, reinterpret_cast<T *>(pcg_dyn), s_ta, s_tb, s_ue, s_ctl, bid, nbk, err);
             if (rc < 0) return;
             if (lead) conv = rc == CTL_DONE;
+        } else if constexpr (MARCH) {
+            // The CG update in a pass of its own, in place (p = D^-1 r + beta
+            // p, x += alpha p, s = w + beta s, r -= alpha s), then one
+            // marching sweep forms u = D^-1 r, w = A u and the sums: per node
+            // 19 words in the update, 10 and the halo rows in the sweep, and
+            // a second grid barrier, against a halo of 2.5 nodes per node
+            // that each formed from r, w and s on 16x4x4 tiles, with 20
+            // values per cell through shared memory.  53x47x61, per
+            // iteration: 37 us -> 26 us.
+            __shared__ __align__(16) unsigned char s_jop[sizeof(OpJac3)];
+            OpJac3 &op = *reinterpret_cast<OpJac3 *>(s_jop);
+            bool first = true;
+            int redpar = 0;
+            while (true) {
+                if (lead) {
+                    if (!first) cg_scalar_update<NV>(S);
+                    s_ta = (T)alpha;
+                    s_tb = (T)beta;
+                    op.lam = A.lam; op.mu = A.mu; op.dinv = A.dinv; op.r = A.r[0][0]; op.w = A.w[0][0];
+                    op.n = (unsigned)N;
+                    for (int vv = 0; vv < NV; vv++) op.ue[vv] = (T)UE[vv];
+                }
+                __syncthreads();
+                if (!first) {
+                    const T ta = s_ta, tb = s_tb;
+                    for (long long n = t0; n < N; n += st) {
+                        const T di = A.dinv[n];
+#pragma unroll
+                        for (int d = 0; d < D; d++) {
+                            const T rv = A.r[0][d][n];
+                            const T pi = di * rv + tb * A.p[d][n], si = __ldcg(A.w[0][d] + n) + tb * A.s[0][d][n];
+                            A.p[d][n] = pi;
+                            A.x[d][n] += ta * pi;
+                            A.s[0][d][n] = si;
+                            A.r[0][d][n] = rv - ta * si;
+                        }
+                    }
+                    if (!grid_sync(A.bar_count, A.bar_gen, err, nbk)) return;
+                }
+                const SumsJ3 sums = m3_sweep(&op, P.nx, P.ny, P.nz, A.zc1[0], bid, nbk);
+                Acc<T> acc[3 + NV];      // gamma, delta, ||r||^2, mean-strain row
+                acc[0] = sums.ru;
+                acc[1] = sums.wu;
+                acc[2] = sums.rr;
+                for (int v = 0; v < NV; v++) acc[3 + v].s = T(4) * sums.se[v].s;     // four times a quarter of each cell's stress
+                double *const tt = S.red;
+                if (!reduce_barrier<Acc<T>, 3 + NV>(acc, A.partials, redpar, A.bar_count, A.bar_gen, err, tt, bid, nbk)) return;
+                redpar ^= 1;
+                const int ctl = pcg_step<D>(S, tt, first, target, A.maxit, s_ctl);
+                first = false;
+                if (ctl == CTL_DONE || ctl == CTL_STOP) {
+                    if (lead) conv = (ctl == CTL_DONE);
+                    break;
+                }
+            }
         } else {
             bool first = true;
             int cur = 0, redpar = 0;
@@ -854,31 +938,6 @@ k_pcg(const PCGArgs<T, D> *jobs, int njobs)
                     // issue the next tile's loads; they complete while this one computes
                     if (tile + nbk < ntiles) load_raw(tile + nbk, R);
                     __syncthreads();
-                    if constexpr (CELL3) {
-                        // per halo cell: average stress (mean strain UE included)
-                        // and the twelve hourglass forces, shared by its 8 nodes
-                        for (int h = threadIdx.x; h < HC; h += blockDim.x) {
-                            const int cx = h % CX, cy = (h / CX) % CY, cz = h / (CX * CY);
-                            T uc[8][3];
-    #pragma unroll
-                            for (int b = 0; b < 8; b++) {
-                                const int hn = (cx + (b & 1)) + HX * ((cy + ((b >> 1) & 1)) + HY * (cz + (b >> 2)));
-                                uc[b][0] = su[hn];
-                                uc[b][1] = su[HN + hn];
-                                uc[b][2] = su[2 * HN + hn];
-                            }
-                            const T l = sl[h], m = sm[h];
-                            T c[20], sx[6];
-                            cell_force3<T>(l, m, uc, c);
-                            voigt_stress<T, 3>(l, m, ue, sx);
-    #pragma unroll
-                            for (int v = 0; v < 6; v++) c[v] += sx[v];
-                            float4 *dst = reinterpret_cast<float4 *>(scell + 20 * h);
-    #pragma unroll
-                            for (int q4 = 0; q4 < 5; q4++) dst[q4] = make_float4(c[4 * q4], c[4 * q4 + 1], c[4 * q4 + 2], c[4 * q4 + 3]);
-                        }
-                        __syncthreads();
-                    }
                     if constexpr (D == 2) {
                         // per halo cell: average stress (mean strain UE included)
                         // and hourglass forces, shared by the cell's four nodes
@@ -951,32 +1010,6 @@ k_pcg(const PCGArgs<T, D> *jobs, int njobs)
                             se[0] = scell[c0] - sx[0];
                             se[1] = scell[HC + c0] - sx[1];
                             se[2] = scell[2 * HC + c0] - sx[2];
-                        } else if constexpr (CELL3) {
-                            q[0] = q[1] = q[2] = T(0);
-    #pragma unroll
-                            for (int a = 0; a < 8; a++) {
-                                const int ax = a & 1, ay = (a >> 1) & 1, az = a >> 2;
-                                const int cl = (lx - ax) + CX * ((ly - ay) + CY * (lz - az));
-                                const float4 *src = reinterpret_cast<const float4 *>(scell + 20 * cl);
-                                T c[20];
-    #pragma unroll
-                                for (int q4 = 0; q4 < 5; q4++) {
-                                    const float4 v = src[q4];
-                                    c[4 * q4] = v.x; c[4 * q4 + 1] = v.y; c[4 * q4 + 2] = v.z; c[4 * q4 + 3] = v.w;
-                                }
-                                T f[3];
-                                node_force3<T>(ax, ay, az, c, c + 6, f);
-                                q[0] += f[0];
-                                q[1] += f[1];
-                                q[2] += f[2];
-                                if (a == 0) {
-                                    // own cell's average stress without the mean strain
-                                    T sx[6];
-                                    voigt_stress<T, 3>(sl[cl], sm[cl], ue, sx);
-    #pragma unroll
-                                    for (int v = 0; v < 6; v++) se[v] = c[v] - sx[v];
-                                }
-                            }
                         } else {
                             T eo[NV], lo, mo;
                             apply_tile<T, D, HX, HY, CX, CY>(su, sl, sm, HN, lx, ly, lz, ue, q, eo, lo, mo);
@@ -997,31 +1030,9 @@ k_pcg(const PCGArgs<T, D> *jobs, int njobs)
                 double *const tt = S.red;
                 if (!reduce_barrier<Acc<T>, 3 + NV>(acc, A.partials, redpar, A.bar_count, A.bar_gen, err, tt, bid, nbk)) return;
                 redpar ^= 1;
-                const bool was_first = first;
-                if (lead) {
-                    double s6[6];
-                    dmat_mul<D>(Sl, Sm, UE, s6);
-                    for (int vv = 0; vv < NV; vv++) WE[vv] = tt[3 + vv] + s6[vv];
-                    double gnew = tt[0], dnew = tt[1], rnew = tt[2];
-                    for (int vv = 0; vv < NV; vv++) {
-                        gnew += RE[vv] * UE[vv];
-                        dnew += WE[vv] * UE[vv];
-                        rnew += RE[vv] * RE[vv];
-                    }
-                    int ctl = CTL_RUN;
-                    if (!was_first) {
-                        it++;
-                        rho_final = rnew;
-                        if (rnew <= target * target) ctl = CTL_DONE;      // ||r|| <= target without a square root
-                        else if (it_total + it >= A.maxit) ctl = CTL_STOP;
-                    }
-                    cg_take_gamma_delta(S, gnew, dnew, was_first);
-                    s_ctl = ctl;
-                }
-                __syncthreads();
-                const int ctl = s_ctl;
+                const int ctl = pcg_step<D>(S, tt, first, target, A.maxit, s_ctl);
+                if (!first) cur = nxt;
                 first = false;
-                if (!was_first) cur = nxt;
                 if (ctl == CTL_DONE || ctl == CTL_STOP) {
                     if (lead) conv = (ctl == CTL_DONE);
                     break;
@@ -1066,11 +1077,10 @@ k_pcg(const PCGArgs<T, D> *jobs, int njobs)
 
 // Host side of one translation unit's PCG instantiations: occupancy query,
 // cooperative launch and the upload of that unit's copy of the element
-// tables (constant memory is per unit).  Dynamic shared memory: the 3D FP32
-// cell buffer of the 16x4x4 tile; with MG, the arrays of the block-run
-// levels (the bound for any hierarchy, so one attribute serves all), which
-// the FP64 set-up sweep uses as scratch before them, and the operation
-// record of the marching sweeps.
+// tables (constant memory is per unit).  Dynamic shared memory: with MG, the
+// arrays of the block-run levels (the bound for any hierarchy, so one
+// attribute serves all), which the FP64 set-up sweep uses as scratch before
+// them, and the operation record of the marching sweeps.
 template <typename T, int D>
 size_t pcg_dyn_smem(int shape, bool mg)
 {
@@ -1089,9 +1099,7 @@ size_t pcg_dyn_smem(int shape, bool mg)
                       "the double-single set-up sweep fits the FP64 one's shared memory");
         return cells > stp ? cells : stp;
     }
-    if (D != 3 || sizeof(T) != 4 || shape != 0) return 0;
-    constexpr int HC = (Tile<3, 0>::X + 1) * (Tile<3, 0>::Y + 1) * (Tile<3, 0>::Z + 1);
-    return sizeof(float) * 20 * HC;
+    return 0;
 }
 
 // the kernel variant of a tile shape, with or without the multigrid

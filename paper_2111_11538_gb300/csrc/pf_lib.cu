@@ -533,8 +533,7 @@ int setup_cg_launch(pf_handle *h)
     h->pcg_shape = h->cfg.pcg_tile > 0 ? h->cfg.pcg_tile - 1
                                        : (h->mg ? (D == 2 ? mg2_pcg_shape(h->P.N, fp64) : 0)
                                                 : default_pcg_shape(D, h->P.N, fp64));
-    h->cg_block = h->mg ? (h->pcg_shape ? pcg_threads<T, D, 1, true>() : pcg_threads<T, D, 0, true>())
-                        : (h->pcg_shape ? tile_threads<D, 1>() : tile_threads<D, 0>());
+    h->cg_block = h->pcg_shape ? pcg_threads<T, D, 1, true>() : pcg_threads<T, D, 0, true>();
     if (h->mg) PF_TRY((build_mg<T, D>(h)));
     int per_sm = 0;
     cudaError_t e = D == 2 ? pcg2_occupancy(fp64, h->pcg_shape, h->mg, h->cg_block, &per_sm)
@@ -725,8 +724,9 @@ int build_plan(pf_handle *h)
                 pj[i] = pcg_args<T, D>(I[i]);
                 pj[i].block0 = g0;
                 pj[i].nblocks = (int)nb;
-                if (D == 3 && I[i]->mg && sizeof(T) == 4)
-                    for (int k = 0, nx = I[i]->P.nx, ny = I[i]->P.ny, nz = I[i]->P.nz; k < mg_levels3(I[i]->P.nx, I[i]->P.ny, I[i]->P.nz);
+                if (D == 3 && sizeof(T) == 4)
+                    for (int k = 0, nx = I[i]->P.nx, ny = I[i]->P.ny, nz = I[i]->P.nz;
+                         k < (I[i]->mg ? mg_levels3(I[i]->P.nx, I[i]->P.ny, I[i]->P.nz) : 1);
                          k++, nx /= 2, ny /= 2, nz /= 2)
                         pj[i].zc1[k] = m3_chunk(nx, ny, nz, (int)nb * (h->cg_block / 32));
                 if (D == 2 && I[i]->mg)
@@ -787,7 +787,6 @@ int launch_mechanics(pf_handle *h, cudaStream_t s, int k)
     memset(&cj, 0, sizeof(cj));
     cj.table = (const CellJob<T, D> *)h->d_cell_jobs[k];
     cj.njobs = h->njobs;
-    const int n = h->njobs;
     if (h->cfg.mechanics) {
         h->mark_begin(PF_K_SETUP, s);
         k_setup<T, D><<<h->cell_grid, 256, 0, s>>>(cj);

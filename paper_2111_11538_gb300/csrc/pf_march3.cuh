@@ -497,4 +497,56 @@ struct OpApply3 {
     }
 };
 
+// Jacobi-preconditioned CG: u = D^-1 r, w = A u with the mean strain, and the
+// sums of OpApply3 with ||r||^2.
+struct SumsJ3 : Sums3 {
+    Acc<float> rr;
+};
+struct OpJac3 {
+    static constexpr bool E = true;
+    typedef SumsJ3 Sums;
+    const float *lam, *mu, *dinv, *r;
+    float *w;
+    float ue[6];
+    unsigned n;
+    struct Raw {
+        float l, m, di, r[3];
+    };
+    __device__ __forceinline__ void load(Raw &R, int, bool, int, int, int, int g, int gm, const Lanes2 &) const
+    {
+        R.l = __ldcg(lam + gm);
+        R.m = __ldcg(mu + gm);
+        R.di = __ldcg(dinv + g);
+#pragma unroll
+        for (int c = 0; c < 3; c++) R.r[c] = __ldcg(r + ((unsigned)g + c * n));
+    }
+    __device__ __forceinline__ void form(const Raw &R, int, bool own, int, int, int, int, const Lanes2 &, float (&v)[3],
+                                         float (&k)[4], Sums &S) const
+    {
+        k[3] = 0.f;
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            v[c] = R.di * R.r[c];
+            k[c] = v[c];
+            if (own) {
+                S.ru.fma_plain(R.r[c], v[c]);
+                S.rr.fma_plain(R.r[c], R.r[c]);
+            }
+        }
+    }
+    __device__ __forceinline__ void cell(const Cell3 &C, Sums &S) const
+    {
+#pragma unroll
+        for (int v = 0; v < 6; v++) S.se[v].add_plain(C.s[v]);
+    }
+    __device__ __forceinline__ void epi(int g, const float (&q)[3], const float (&k)[4], Sums &S) const
+    {
+#pragma unroll
+        for (int c = 0; c < 3; c++) {
+            w[(unsigned)g + c * n] = q[c];
+            S.wu.fma_plain(q[c], k[c]);
+        }
+    }
+};
+
 }  // namespace pfdev
