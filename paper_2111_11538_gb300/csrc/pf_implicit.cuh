@@ -659,63 +659,79 @@ k_be_pc32_tile(int nx, int ny, int N, float dt, const unsigned char *__restrict_
 //   GS 1: w -= sum_k cin[k] V_k, out[k] = V_k . w (the second pass's
 //         coefficients, on the piece just formed);
 //   GS 2: w -= sum_k cin[k] V_k, out[0] = w . w, out[1] = 1 / |w| (1 if w = 0).
+// The vectors stream from L2 and beyond (60 of 2.1 MB), so that what counts
+// is the loads in flight: 16 bytes per lane, eight vectors (the update) or
+// seven pieces (the products) at a time, 32 warps per SM.
 // 256^2, restarts of 60, per iteration: three dot products of 24 us, two
 // combinations of 15 us, three device-to-host copies with their waits and a
-// scaling before; 16 + 33 + 16 us now.
-constexpr int BE_CH = 1024;
+// scaling before; 26 + 41 + 22 us now at 40 vectors (8-byte loads and
+// 16 warps per SM: 38 + 47 + 24).
+constexpr int BE_CH = 1024, BE_GST = 512;
 template <int GS>
-__global__ void __launch_bounds__(256) k_be_gs(long long L, long long per, const double *__restrict__ V, int nv,
-                                               double *w, const double *__restrict__ cin, double *part,
-                                               unsigned int *ticket, double *out)
+__global__ void __launch_bounds__(BE_GST, 2) k_be_gs(long long L, long long per, const double *__restrict__ V, int nv,
+                                                     double *w, const double *__restrict__ cin, double *part,
+                                                     unsigned int *ticket, double *out)
 {
-    __shared__ double sw[BE_CH], sc[64], acc[64];
+    __shared__ __align__(16) double sw[BE_CH];
+    __shared__ double sc[64], acc[64];
     __shared__ bool s_last;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (threadIdx.x < 64) {
-        acc[threadIdx.x] = 0.0;
-        sc[threadIdx.x] = GS > 0 && threadIdx.x < nv ? cin[threadIdx.x] : 0.0;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, t = threadIdx.x;
+    constexpr int NW = BE_GST / 32;
+    if (t < 64) {
+        acc[t] = 0.0;
+        sc[t] = GS > 0 && t < nv ? cin[t] : 0.0;
     }
     __syncthreads();
+    // (L and per are multiples of 4: pieces have even lengths and 16-byte
+    // boundaries)
     const long long i0 = blockIdx.x * per, i1 = min(i0 + per, L);
     double n2 = 0.0;
+    double2 *const sw2 = reinterpret_cast<double2 *>(sw);
     for (long long p0 = i0; p0 < i1; p0 += BE_CH) {
-        const int n = (int)min((long long)BE_CH, i1 - p0);
-        if constexpr (GS > 0) {
-            double s[4] = {0.0, 0.0, 0.0, 0.0};
-            const int t = threadIdx.x;
-#pragma unroll 4
-            for (int k = 0; k < nv; k++) {
-                const double *v = V + (size_t)k * L + p0;
-                const double c = sc[k];
-#pragma unroll
-                for (int q = 0; q < 4; q++)
-                    if (t + 256 * q < n) s[q] = fma(c, v[t + 256 * q], s[q]);
-            }
-#pragma unroll
-            for (int q = 0; q < 4; q++)
-                if (t + 256 * q < n) {
-                    const double x = w[p0 + t + 256 * q] - s[q];
-                    w[p0 + t + 256 * q] = x;
-                    if constexpr (GS == 2) n2 = fma(x, x, n2);
-                    else sw[t + 256 * q] = x;
+        const int n = (int)min((long long)BE_CH, i1 - p0) / 2;      // pairs
+        double2 *const w2 = reinterpret_cast<double2 *>(w + p0);
+        if (t < n) {
+            double2 x = w2[t];
+            if constexpr (GS > 0) {
+                const double2 *v = reinterpret_cast<const double2 *>(V + p0) + t;
+                double2 s = make_double2(0.0, 0.0);
+#pragma unroll 8
+                for (int k = 0; k < nv; k++) {
+                    const double2 a = v[(size_t)k * (L / 2)];
+                    s.x = fma(sc[k], a.x, s.x);
+                    s.y = fma(sc[k], a.y, s.y);
                 }
-        } else {
-            for (int t = threadIdx.x; t < n; t += 256) sw[t] = w[p0 + t];
+                x.x -= s.x;
+                x.y -= s.y;
+                w2[t] = x;
+            }
+            if constexpr (GS == 2) n2 = fma(x.x, x.x, fma(x.y, x.y, n2));
+            else sw2[t] = x;
         }
         if constexpr (GS < 2) {
             __syncthreads();
-            for (int k = wid; k < nv; k += 8) {
-                const double *v = V + (size_t)k * L + p0;
-                double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
-                int t = lane;
-                for (; t + 96 < n; t += 128) {
-                    s0 = fma(v[t], sw[t], s0);
-                    s1 = fma(v[t + 32], sw[t + 32], s1);
-                    s2 = fma(v[t + 64], sw[t + 64], s2);
-                    s3 = fma(v[t + 96], sw[t + 96], s3);
+            for (int k = wid; k < nv; k += NW) {
+                const double2 *v = reinterpret_cast<const double2 *>(V + (size_t)k * L + p0);
+                double2 s = make_double2(0.0, 0.0), r = s;
+                int q = lane;
+                for (; q + 32 * 6 < n; q += 32 * 7) {
+                    double2 a[7];
+#pragma unroll
+                    for (int u = 0; u < 7; u++) a[u] = v[q + 32 * u];
+#pragma unroll
+                    for (int u = 0; u < 7; u++) {
+                        const double2 b = sw2[q + 32 * u];
+                        double2 &z = (u & 1) ? r : s;
+                        z.x = fma(a[u].x, b.x, z.x);
+                        z.y = fma(a[u].y, b.y, z.y);
+                    }
                 }
-                for (; t < n; t += 32) s0 = fma(v[t], sw[t], s0);
-                double x = (s0 + s1) + (s2 + s3);
+                for (; q < n; q += 32) {
+                    const double2 a = v[q], b = sw2[q];
+                    s.x = fma(a.x, b.x, s.x);
+                    s.y = fma(a.y, b.y, s.y);
+                }
+                double x = (s.x + s.y) + (r.x + r.y);
                 for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
                 if (lane == 0) acc[k] += x;
             }
@@ -726,22 +742,22 @@ __global__ void __launch_bounds__(256) k_be_gs(long long L, long long per, const
         for (int o = 16; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
         if (lane == 0) sw[wid] = n2;
         __syncthreads();
-        if (threadIdx.x == 0) {
+        if (t == 0) {
             double x = 0.0;
-            for (int q = 0; q < 8; q++) x += sw[q];
+            for (int q = 0; q < NW; q++) x += sw[q];
             acc[0] = x;
         }
         __syncthreads();
     }
     const int nk = GS == 2 ? 1 : nv;
-    if (threadIdx.x < nk) part[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = acc[threadIdx.x];
+    if (t < nk) part[(size_t)t * gridDim.x + blockIdx.x] = acc[t];
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+    if (t == 0) s_last = atomicAdd(ticket, 1u) == gridDim.x - 1;
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    for (int k = wid; k < nk; k += 8) {
+    for (int k = wid; k < nk; k += NW) {
         double x = 0.0;
         for (int b = lane; b < (int)gridDim.x; b += 32) x += __ldcg(part + (size_t)k * gridDim.x + b);
         for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
@@ -750,7 +766,7 @@ __global__ void __launch_bounds__(256) k_be_gs(long long L, long long per, const
             if (GS == 2) out[1] = x > 0.0 ? 1.0 / sqrt(x) : 1.0;
         }
     }
-    if (threadIdx.x == 0) *ticket = 0u;
+    if (t == 0) *ticket = 0u;
 }
 
 // dst = *f v

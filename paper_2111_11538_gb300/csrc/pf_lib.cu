@@ -1337,7 +1337,7 @@ int be_steps(pf_handle *h, int nsteps, const pf_implicit_opts &o, pf_implicit_st
     PF_TRY(h->cuda(cudaMemsetAsync(w.ticket, 0, sizeof(double), s), "ticket"));
     // |v|^2 and 1 / |v| (in w.hs[2][0, 1])
     auto norm2 = [&](double *v, double *res) -> int {
-        k_be_gs<2><<<gG, 256, 0, s>>>(L, per, nullptr, 0, v, w.hs[2], w.part, w.ticket, w.hs[2]);
+        k_be_gs<2><<<gG, BE_GST, 0, s>>>(L, per, nullptr, 0, v, w.hs[2], w.part, w.ticket, w.hs[2]);
         double *hp = h->be_host + 2 * BE_HS;
         PF_TRY(h->cuda(cudaMemcpyAsync(hp, w.hs[2], sizeof(double), cudaMemcpyDeviceToHost, s), "norm"));
         PF_TRY(h->cuda(cudaStreamSynchronize(s), "norm"));
@@ -1532,9 +1532,9 @@ int be_steps(pf_handle *h, int nsteps, const pf_implicit_opts &o, pf_implicit_st
                     double *hs = w.hs[q & 1];
                     PF_TRY(precond(q ? w.Ft : v0, q ? w.hs[(q - 1) & 1] + 129 : w.hs[2] + 1, w.V + (size_t)q * L, w.z));
                     PF_TRY(jvp(w.z, w.Ft));
-                    k_be_gs<0><<<gG, 256, 0, s>>>(L, per, w.V, q + 1, w.Ft, nullptr, w.part, w.ticket, hs);
-                    k_be_gs<1><<<gG, 256, 0, s>>>(L, per, w.V, q + 1, w.Ft, hs, w.part, w.ticket, hs + 64);
-                    k_be_gs<2><<<gG, 256, 0, s>>>(L, per, w.V, q + 1, w.Ft, hs + 64, w.part, w.ticket, hs + 128);
+                    k_be_gs<0><<<gG, BE_GST, 0, s>>>(L, per, w.V, q + 1, w.Ft, nullptr, w.part, w.ticket, hs);
+                    k_be_gs<1><<<gG, BE_GST, 0, s>>>(L, per, w.V, q + 1, w.Ft, hs, w.part, w.ticket, hs + 64);
+                    k_be_gs<2><<<gG, BE_GST, 0, s>>>(L, per, w.V, q + 1, w.Ft, hs + 64, w.part, w.ticket, hs + 128);
                     PF_TRY(h->cuda(cudaMemcpyAsync(h->be_host + (q & 1) * BE_HS, hs, sizeof(double) * BE_HS,
                                                    cudaMemcpyDeviceToHost, s), "Gram-Schmidt"));
                     return h->cuda(cudaEventRecord(h->be_ev[q & 1], s), "Gram-Schmidt");
