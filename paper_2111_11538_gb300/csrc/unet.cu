@@ -440,10 +440,10 @@ struct pf_unet {
 
 namespace {
 
-template <int D, int C>
+template <int D, int C, bool AHEAD = false>
 void set_smem_attrs()
 {
-    cudaFuncSetAttribute(k_conv3<D, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv3_smem<D, C>());
+    cudaFuncSetAttribute(k_conv3<D, C, AHEAD>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)conv3_smem<D, C>());
 }
 
 template <int D, int C>
@@ -455,21 +455,28 @@ void set_wgrad_attrs()
 template <int D>
 bool prepare_kernels()
 {
+    set_smem_attrs<D, 16, true>();
     set_smem_attrs<D, 16>(); set_smem_attrs<D, 32>(); set_smem_attrs<D, 48>(); set_smem_attrs<D, 64>();
     set_smem_attrs<D, 80>(); set_smem_attrs<D, 96>(); set_smem_attrs<D, 112>(); set_smem_attrs<D, 128>();
     set_wgrad_attrs<D, 16>(); set_wgrad_attrs<D, 32>(); set_wgrad_attrs<D, 48>(); set_wgrad_attrs<D, 64>();
     return cudaGetLastError() == cudaSuccess;
 }
 
-template <int D, int C>
+template <int D, int C, bool AHEAD = false>
 void launch_conv_t(const ConvArgs &a, long long tiles, cudaStream_t s)
 {
-    k_conv3<D, C><<<(unsigned)tiles, 256, conv3_smem<D, C>(), s>>>(a);
+    k_conv3<D, C, AHEAD><<<dim3((unsigned)tiles, (unsigned)(a.cout / C)), 256, conv3_smem<D, C>(), s>>>(a);
 }
 
 template <int D>
-int launch_conv(int cout, const ConvArgs &a, long long tiles, cudaStream_t s)
+int launch_conv(int cout, ConvArgs a, long long tiles, cudaStream_t s)
 {
+    a.cout = cout;
+    // fewer tiles than SMs: 16 output channels per block (see k_conv3)
+    if (tiles < 152) {
+        launch_conv_t<D, 16, true>(a, tiles, s);
+        return PF_OK;
+    }
     switch (cout) {
     case 16: launch_conv_t<D, 16>(a, tiles, s); break;
     case 32: launch_conv_t<D, 32>(a, tiles, s); break;

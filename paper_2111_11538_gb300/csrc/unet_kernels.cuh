@@ -64,7 +64,8 @@ struct ConvArgs {
     int C0, C1;
     const __nv_bfloat16 *wt;    // [taps][COUT][C0 + C1]
     const float *bias;          // [COUT] or null
-    __nv_bfloat16 *out;         // [cells][COUT]
+    __nv_bfloat16 *out;         // [cells][cout]
+    int cout;
     int relu;
     int mirror;                 // 1: tap t reads the cell at -offset(t) (input-gradient pass)
     Dims dim;
@@ -73,9 +74,16 @@ struct ConvArgs {
 // ---------------------------------------------------------------------------
 // Periodic 3^D convolution as an implicit GEMM: out[p, co] = bias[co] +
 // sum_{tap, ci} in[p + off(tap), ci] * W[tap, co, ci].  One block computes a
-// tile of 128 cells x COUT channels; 8 warps, warp w owns the tile's row w
-// (16 cells = one m16 fragment).  The K loop runs over 16-channel chunks of
-// the input (staged with a one-cell halo) and over the taps.
+// tile of 128 cells x COUT of the cout output channels (blockIdx.y); 8 warps,
+// warp w owns the tile's row w (16 cells = one m16 fragment).  The K loop runs
+// over 16-channel chunks of the input (staged with a one-cell halo) and over
+// the taps.  The deep levels have few tiles (16 for 152 SMs at 8 samples of 16
+// x 16 cells) and a block waits for its chunks one after the other; there a
+// block takes 16 channels only and loads the next chunk's words into registers
+// while this one is contracted (AHEAD).  Every sum keeps its order.  64 to 64
+// channels, 16 tiles: 14.0 us -> 6.8 us; 64 tiles: 14.4 -> 8.8.  With tiles for
+// every SM neither helps: 256 tiles of 32 channels 7.6 us, split in two and
+// ahead 8.8; 1024 tiles of 16 channels 8.9, ahead 9.3.
 // ---------------------------------------------------------------------------
 template <int D, int COUT>
 __host__ __device__ constexpr size_t conv3_smem()
@@ -84,7 +92,7 @@ __host__ __device__ constexpr size_t conv3_smem()
     return sizeof(__nv_bfloat16) * 24 * (HP + (D == 3 ? 27 : 9) * COUT);
 }
 
-template <int D, int COUT>
+template <int D, int COUT, bool AHEAD>
 __global__ void __launch_bounds__(256) k_conv3(const ConvArgs a)
 {
     constexpr int TX = CTile<D>::X, TY = CTile<D>::Y, TZ = CTile<D>::Z;
@@ -122,29 +130,54 @@ __global__ void __launch_bounds__(256) k_conv3(const ConvArgs a)
     // this warp's row in the tile
     const int wy = warp % TY, wz = warp / TY;
 
+    const int co0 = (int)blockIdx.y * COUT;
+    constexpr int NI = (HP * 2 + 255) / 256, NW = (TAPS * COUT * 2 + 255) / 256;
+    // a chunk: HP cells x 16 channels = 2 x 16 B per cell, and the weights
+    // [tap][co][16]
+    auto ld_in = [&](int q, int ci0) {
+        const int cell = q >> 1, half = q & 1;
+        const int hxi = cell % HX, r = cell / HX, hyi = r % HY, hzi = r / HY;
+        const int gx = wrapc(x0 + hxi - 1, nx), gy = wrapc(y0 + hyi - 1, ny);
+        const int gz = D == 3 ? wrapc(z0 + hzi - 1, nz) : 0;
+        if (ci0 < a.C0) {
+            const long long p = gx + (long long)nx * (gy + (long long)ny * gz);
+            return *(const uint4 *)(in0 + p * a.C0 + ci0 + half * 8);
+        }
+        const long long p = (gx >> 1) + (long long)hx * ((gy >> 1) + (long long)hy * (gz >> 1));
+        return *(const uint4 *)(in1 + p * a.C1 + (ci0 - a.C0) + half * 8);
+    };
+    auto ld_w = [&](int q, int ci0) {
+        const int row = q >> 1, half = q & 1, tap = row / COUT, co = row % COUT;
+        return *(const uint4 *)(a.wt + (size_t)(tap * a.cout + co0 + co) * Cin + ci0 + half * 8);
+    };
+    uint4 vi[AHEAD ? NI : 1], vw[AHEAD ? NW : 1];
+    auto fetch = [&](int ci0) {
+#pragma unroll
+        for (int k = 0; k < NI; k++)
+            if ((int)threadIdx.x + 256 * k < HP * 2) vi[AHEAD ? k : 0] = ld_in(threadIdx.x + 256 * k, ci0);
+#pragma unroll
+        for (int k = 0; k < NW; k++)
+            if ((int)threadIdx.x + 256 * k < TAPS * COUT * 2) vw[AHEAD ? k : 0] = ld_w(threadIdx.x + 256 * k, ci0);
+    };
+    if constexpr (AHEAD) fetch(0);
     for (int ci0 = 0; ci0 < Cin; ci0 += 16) {
         __syncthreads();
-        // stage the input chunk: HP cells x 16 channels = 2 x 16 B per cell
-        for (int q = threadIdx.x; q < HP * 2; q += blockDim.x) {
-            const int cell = q >> 1, half = q & 1;
-            const int hxi = cell % HX, r = cell / HX, hyi = r % HY, hzi = r / HY;
-            const int gx = wrapc(x0 + hxi - 1, nx), gy = wrapc(y0 + hyi - 1, ny);
-            const int gz = D == 3 ? wrapc(z0 + hzi - 1, nz) : 0;
-            uint4 v;
-            if (ci0 < a.C0) {
-                const long long p = gx + (long long)nx * (gy + (long long)ny * gz);
-                v = *(const uint4 *)(in0 + p * a.C0 + ci0 + half * 8);
-            } else {
-                const long long p = (gx >> 1) + (long long)hx * ((gy >> 1) + (long long)hy * (gz >> 1));
-                v = *(const uint4 *)(in1 + p * a.C1 + (ci0 - a.C0) + half * 8);
+        if constexpr (AHEAD) {
+#pragma unroll
+            for (int k = 0; k < NI; k++) {
+                const int q = threadIdx.x + 256 * k;
+                if (q < HP * 2) *(uint4 *)(s_in + (q >> 1) * PS + (q & 1) * 8) = vi[k];
             }
-            *(uint4 *)(s_in + cell * PS + half * 8) = v;
-        }
-        // stage the weights of this chunk: [tap][co][16]
-        for (int q = threadIdx.x; q < TAPS * COUT * 2; q += blockDim.x) {
-            const int row = q >> 1, half = q & 1;
-            const uint4 v = *(const uint4 *)(a.wt + (size_t)row * Cin + ci0 + half * 8);
-            *(uint4 *)(s_w + row * PS + half * 8) = v;
+#pragma unroll
+            for (int k = 0; k < NW; k++) {
+                const int q = threadIdx.x + 256 * k;
+                if (q < TAPS * COUT * 2) *(uint4 *)(s_w + (q >> 1) * PS + (q & 1) * 8) = vw[k];
+            }
+            if (ci0 + 16 < Cin) fetch(ci0 + 16);
+        } else {
+            for (int q = threadIdx.x; q < HP * 2; q += 256) *(uint4 *)(s_in + (q >> 1) * PS + (q & 1) * 8) = ld_in(q, ci0);
+            for (int q = threadIdx.x; q < TAPS * COUT * 2; q += 256)
+                *(uint4 *)(s_w + (q >> 1) * PS + (q & 1) * 8) = ld_w(q, ci0);
         }
         __syncthreads();
 #pragma unroll 1
@@ -179,13 +212,13 @@ __global__ void __launch_bounds__(256) k_conv3(const ConvArgs a)
     const long long rowbase = (long long)b * cells + (long long)nx * (yy + (long long)ny * zz) + x0;
 #pragma unroll
     for (int j = 0; j < NT; j++) {
-        const int co = j * 8 + qd * 2;
+        const int co = co0 + j * 8 + qd * 2;
         float bb0 = a.bias ? a.bias[co] : 0.f, bb1 = a.bias ? a.bias[co + 1] : 0.f;
         float v0 = acc[j][0] + bb0, v1 = acc[j][1] + bb1, v2 = acc[j][2] + bb0, v3 = acc[j][3] + bb1;
         if (a.relu) { v0 = fmaxf(v0, 0.f); v1 = fmaxf(v1, 0.f); v2 = fmaxf(v2, 0.f); v3 = fmaxf(v3, 0.f); }
         __nv_bfloat162 lo = __floats2bfloat162_rn(v0, v1), hi = __floats2bfloat162_rn(v2, v3);
-        *(__nv_bfloat162 *)(a.out + (rowbase + g) * COUT + co) = lo;
-        *(__nv_bfloat162 *)(a.out + (rowbase + g + 8) * COUT + co) = hi;
+        *(__nv_bfloat162 *)(a.out + (rowbase + g) * a.cout + co) = lo;
+        *(__nv_bfloat162 *)(a.out + (rowbase + g + 8) * a.cout + co) = hi;
     }
 }
 
