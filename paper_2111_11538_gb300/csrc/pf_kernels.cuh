@@ -378,29 +378,6 @@ __global__ void __launch_bounds__(256) k_update(const __grid_constant__ JobSet<C
     }
 }
 
-// ---------------------------------------------------------------------------
-// K1: the fused explicit step -- oxygen chemical potential and mobility
-// (K1a) and the explicit Euler update (K1b) in one pass over the grid.
-//
-// Each block walks tiles of TX x TY (x TZ) cells.  Per tile it stages in
-// shared memory x_O with a halo of two cells and theta, phi_g, x_H, x_H2O
-// with a halo of one, evaluates mu_O and M_O on the tile plus one halo
-// cell, then updates the tile's cells from shared memory.  HBM sees each
-// field once per step (the halo re-reads hit L2); mu_O and M_O never leave
-// the SM.  Arithmetic and operand order per cell are those of k_mu and
-// k_update.
-// ---------------------------------------------------------------------------
-template <int D, int TX, int TY, int TZ>
-struct FusedTile {
-    static constexpr int EX = TX + 2, EY = TY + 2, EZ = D == 3 ? TZ + 2 : 1;   // halo 1
-    static constexpr int GX = TX + 4, GY = TY + 4, GZ = D == 3 ? TZ + 4 : 1;   // halo 2
-    static constexpr int E = EX * EY * EZ, G = GX * GY * GZ, C = TX * TY * (D == 3 ? TZ : 1);
-    // shared words: x_O (G); theta, phi_g, x_H, x_H2O, mu_O, M_O, D_H, D_H2O (E each)
-    static constexpr int WORDS = G + 8 * E;
-    static constexpr int NT = 256;                       // threads per block
-    static constexpr int CPT = (C + NT - 1) / NT;        // tile cells per thread
-};
-
 // Quotient for the mobility M_O = D_O / psi'': the FP32 method takes the
 // hardware approximate divide (2 ulp; its fields are held to 1e-4), FP64 the
 // IEEE divide.
@@ -416,476 +393,10 @@ __device__ __forceinline__ int pwrap(int a, int n)
     return a;
 }
 
-template <typename T, int D, int TX, int TY, int TZ>
-__global__ void __launch_bounds__(256, (sizeof(T) == 4 && D == 2) ? 3 : 2) k_fused(const __grid_constant__ JobSet<CellJob<T, D>> js)
-{
-    using FT = FusedTile<D, TX, TY, TZ>;
-    static_assert(TX == 32, "the staging maps one warp lane to one tile column");
-    constexpr int EX = FT::EX, EY = FT::EY, GX = FT::GX, GY = FT::GY, NT = FT::NT, CPT = FT::CPT;
-    constexpr int TZe = D == 3 ? TZ : 1;
-    extern __shared__ __align__(16) unsigned char fsm_raw[];
-    T *sXO = (T *)fsm_raw;
-    T *sTh = sXO + FT::G, *sPg = sTh + FT::E, *sXH = sPg + FT::E, *sXW = sXH + FT::E;
-    T *sMu = sXW + FT::E, *sM = sMu + FT::E, *sDH = sM + FT::E, *sDW = sDH + FT::E;
-
-    // the job lives in shared memory: its parameters are read where they
-    // are used instead of occupying registers for the whole kernel
-    __shared__ __align__(16) CellJob<T, D> sJ;
-    {
-        const CellJob<T, D> *J_ = my_job(js);
-        const int *src = (const int *)J_;
-        int *dst = (int *)&sJ;
-        for (int w = threadIdx.x; w < (int)(sizeof(CellJob<T, D>) / sizeof(int)); w += NT) dst[w] = src[w];
-    }
-    __syncthreads();
-    const Params &P = sJ.P;
-    const FieldPtrs<T, D> &F = sJ.F;
-    const long long bid = (long long)blockIdx.x - sJ.block0;
-    const long long nbk = sJ.nblocks;
-    const int nx = P.nx, ny = P.ny, nz = D == 3 ? P.nz : 1;
-    const int tiles_x = (nx + TX - 1) / TX, tiles_y = (ny + TY - 1) / TY, tiles_z = (nz + TZe - 1) / TZe;
-    const long long ntiles = (long long)tiles_x * tiles_y * tiles_z;
-    const unsigned sxy = (unsigned)nx * (unsigned)ny;   // grids hold < 2^31 cells
-
-    Acc<T> acc[5];           // sum x_O, x_H, x_H2O, removed water, supplied H
-    bool bad = false;
-
-    for (long long t = bid; t < ntiles; t += nbk) {
-        const int tx = (int)(t % tiles_x);
-        const long long tr = t / tiles_x;
-        const int ty = (int)(tr % tiles_y), tz = (int)(tr / tiles_y);
-        const int x0 = tx * TX, y0 = ty * TY, z0 = tz * TZe;
-
-        // per-cell inputs of this thread's cells, requested first so that
-        // they arrive while the tile is staged
-        int gc[CPT];
-        T pre_tE[CPT], pre_s2[CPT], pre_mob[CPT];
-        unsigned char pre_mask[CPT];
-#pragma unroll
-        for (int u = 0; u < CPT; u++) {
-            const int l = threadIdx.x + u * NT;
-            const int a = l % TX, r = l / TX, b = r % TY, c = r / TY;
-            const int i = x0 + a, j = y0 + b, k = z0 + c;
-            const bool in = l < FT::C && i < nx && j < ny && (D == 2 || k < nz);
-            gc[u] = in ? (int)((unsigned)i + (unsigned)nx * (unsigned)j + sxy * (unsigned)k) : -1;
-            if (in) {
-                pre_tE[u] = F.trE[gc[u]];
-                pre_s2[u] = F.devE2[gc[u]];
-                pre_mob[u] = F.mob[gc[u]];
-                pre_mask[u] = F.mask[gc[u]];
-            }
-        }
-        // Stage x_O (halo 2) and theta, phi_g, x_H, x_H2O (halo 1).  Warps take
-        // whole rows: lane L loads column L, lanes 0..(extra-1) the columns
-        // past 32; the periodic wrap is computed once per row and column, and
-        // every load of a thread is issued before its shared-memory stores.
-        {
-            const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-            constexpr int NW = NT / 32;
-            constexpr int RG = FT::GY * FT::GZ, RE = EY * FT::EZ;
-            constexpr int NRG = (RG + NW - 1) / NW, NRE = (RE + NW - 1) / NW;
-            const int ci2 = pwrap(x0 + lane - 2, nx), ci2x = pwrap(x0 + 32 + lane - 2, nx);
-            const int ci1 = pwrap(x0 + lane - 1, nx), ci1x = pwrap(x0 + 32 + lane - 1, nx);
-            const bool xg = lane < GX - 32, xe = lane < EX - 32;
-            T v[NRG], vx[NRG];
-#pragma unroll
-            for (int u = 0; u < NRG; u++) {
-                const int row = warp + u * NW;
-                if (row < RG) {
-                    const int b = row % GY, c = row / GY;
-                    const int gj = pwrap(y0 + b - 2, ny), gk = D == 3 ? pwrap(z0 + c - 2, nz) : 0;
-                    const T *src = F.xO + ((unsigned)nx * (unsigned)gj + sxy * (unsigned)gk);
-                    v[u] = src[ci2];
-                    if (xg) vx[u] = src[ci2x];
-                }
-            }
-            T e0[NRE], e1[NRE], e2[NRE], e3[NRE], x0v[NRE], x1v[NRE], x2v[NRE], x3v[NRE];
-#pragma unroll
-            for (int u = 0; u < NRE; u++) {
-                const int row = warp + u * NW;
-                if (row < RE) {
-                    const int b = row % EY, c = row / EY;
-                    const int gj = pwrap(y0 + b - 1, ny), gk = D == 3 ? pwrap(z0 + c - 1, nz) : 0;
-                    const unsigned rb = (unsigned)nx * (unsigned)gj + sxy * (unsigned)gk;
-                    e0[u] = F.theta[rb + ci1]; e1[u] = F.phig[rb + ci1]; e2[u] = F.xH[rb + ci1]; e3[u] = F.xW[rb + ci1];
-                    if (xe) {
-                        x0v[u] = F.theta[rb + ci1x]; x1v[u] = F.phig[rb + ci1x];
-                        x2v[u] = F.xH[rb + ci1x]; x3v[u] = F.xW[rb + ci1x];
-                    }
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < NRG; u++) {
-                const int row = warp + u * NW;
-                if (row < RG) {
-                    sXO[row * GX + lane] = v[u];
-                    if (xg) sXO[row * GX + 32 + lane] = vx[u];
-                }
-            }
-#pragma unroll
-            for (int u = 0; u < NRE; u++) {
-                const int row = warp + u * NW;
-                if (row < RE) {
-                    const int q = row * EX + lane;
-                    sTh[q] = e0[u]; sPg[q] = e1[u]; sXH[q] = e2[u]; sXW[q] = e3[u];
-                    if (xe) { sTh[q + 32] = x0v[u]; sPg[q + 32] = x1v[u]; sXH[q + 32] = x2v[u]; sXW[q + 32] = x3v[u]; }
-                }
-            }
-        }
-        __syncthreads();
-        // mu_O, M_O (Sec. 2.2, 3.2) and the species diffusivities (R4) on the
-        // tile plus one halo cell
-        {
-            const CellConst<T> &K = sJ.K;
-            const T cc = K.c, kap = K.kappa;
-            const T DOs = K.DOs, DOg = K.DOg, DHs = K.DHs, DHg = K.DHg, DWs = K.DWs, DWg = K.DWg;
-            constexpr int NI = (FT::E + NT - 1) / NT;
-#pragma unroll
-            for (int u = 0; u < NI; u++) {
-                const int l = threadIdx.x + u * NT;
-                if (l < FT::E) {
-                    const int a = l % EX, r = l / EX, b = r % EY, c = r / EY;
-                    const int q = (a + 1) + GX * ((b + 1) + GY * (D == 3 ? c + 1 : 0));
-                    const T x = sXO[q];
-                    T lap = sXO[q - 1] + sXO[q + 1] + sXO[q - GX] + sXO[q + GX] - T(2 * D) * x;
-                    if constexpr (D == 3) lap += sXO[q - GX * GY] + sXO[q + GX * GY];
-                    T Wf, Ww, Wg;
-                    phase_weights(sTh[l], sPg[l], Wf, Ww, Wg);
-                    const T m1 = Wf * f_fe1(x) + Ww * f_wu1(x) + Wg * f_ga1(x);
-                    const T m2 = Wf * f_fe2(x) + Ww * f_wu2(x) + Wg * f_ga2(x);
-                    sMu[l] = cc * m1 - kap * lap;
-                    const T DO = (T(1) - Wg) * DOs + Wg * DOg;
-                    const T den = cc * m2;
-                    sM[l] = den != T(0) ? fast_div(DO, den) : T(0);
-                    sDH[l] = (T(1) - Wg) * DHs + Wg * DHg;
-                    sDW[l] = (T(1) - Wg) * DWs + Wg * DWg;
-                }
-            }
-        }
-        __syncthreads();
-        // explicit Euler update of the tile's cells (Sec. 2.4, R2)
-        {
-            const CellConst<T> &K = sJ.K;
-            const T cc = K.c, eps2 = K.eps2, dt = K.dt;
-            const T Ks = K.Ks, Gs = K.Gs, Kg = K.Kg, w2 = K.w2, eig3 = K.eig3;
-            const T Lh = K.Lh, kf = K.kf, xHbc = K.xHbc;
-#pragma unroll
-            for (int u = 0; u < CPT; u++) {
-                if (gc[u] < 0) continue;
-                const int l = threadIdx.x + u * NT;
-                const int a = l % TX, r = l / TX, b = r % TY, c = r / TY;
-                const int e = (a + 1) + EX * ((b + 1) + EY * (D == 3 ? c + 1 : 0));
-                int nb[2 * D];
-                nb[0] = e - 1; nb[1] = e + 1; nb[2] = e - EX; nb[3] = e + EX;
-                if constexpr (D == 3) { nb[4] = e - EX * EY; nb[5] = e + EX * EY; }
-                const T th = sTh[e], pg = sPg[e];
-                const T xo = sXO[(a + 2) + GX * ((b + 2) + GY * (D == 3 ? c + 2 : 0))];
-                const T xh = sXH[e], xw = sXW[e];
-                const T mu0 = sMu[e], M0 = sM[e], DH0 = sDH[e], DW0 = sDW[e];
-                T lapt = T(0), dO = T(0), dH = T(0), dW = T(0);
-#pragma unroll
-                for (int q = 0; q < 2 * D; q++) {
-                    const int m = nb[q];
-                    lapt += sTh[m] - th;
-                    dO += T(0.5) * (M0 + sM[m]) * (sMu[m] - mu0);
-                    dH += T(0.5) * (DH0 + sDH[m]) * (sXH[m] - xh);
-                    dW += T(0.5) * (DW0 + sDW[m]) * (sXW[m] - xw);
-                }
-                const T tE = pre_tE[u], s2 = pre_s2[u];
-                const T hg0 = hfun(pg);
-                const T hpt = hder(th);
-                const T sol = T(1) - hg0;
-                const T Af = cc * f_fe(xo) + T(0.5) * Ks * tE * tE + Gs * s2;
-                const T Aw = cc * f_wu(xo) + T(0.5) * Ks * tE * tE + Gs * s2;
-                const T Kmix = sol * Ks + hg0 * Kg;
-                const T force = sol * hpt * (Af - Aw) + w2 * mder(th) - eig3 * sol * hpt * Kmix * tE;
-                const T rate = Lh * pre_mob[u] * (force - eps2 * lapt);
-                T rr = mfun(pg) * kf * xo * xh;
-                if (xw >= T(1)) rr = T(0);
-                const T nth = th + dt * rate;
-                const T nxo = xo + dt * (dO - rr);
-                T nxh = xh + dt * (dH - T(2) * rr);
-                T nxw = xw + dt * (dW + rr);
-                if (pre_mask[u]) {
-                    acc[3].add(nxw);
-                    acc[4].add(xHbc - nxh);
-                    nxh = xHbc;
-                    nxw = T(0);
-                }
-                const unsigned g = (unsigned)gc[u];
-                F.theta_o[g] = nth;
-                F.xO_o[g] = nxo;
-                F.xH_o[g] = nxh;
-                F.xW_o[g] = nxw;
-                acc[0].add(nxo); acc[1].add(nxh); acc[2].add(nxw);
-                // a non-finite value anywhere makes the sum non-finite
-                bad |= !isfinite(nth + nxo + nxh + nxw);
-            }
-        }
-        __syncthreads();
-    }
-    Acc<T> acc6[6];
-#pragma unroll
-    for (int q = 0; q < 5; q++) acc6[q] = acc[q];
-    acc6[5].add(T(bad ? 1 : 0));
-    double *partials = sJ.partials;
-    unsigned int *counter = sJ.counter;
-    block_reduce_store<6>(acc6, partials + (size_t)bid * PSTRIDE);
-    __shared__ bool last;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        unsigned int tk = atomicAdd(counter, 1u);
-        last = (tk == (unsigned int)nbk - 1);
-    }
-    __syncthreads();
-    if (last) {
-        __threadfence();
-        __shared__ double tot[6];
-        last_block_sums<6>(partials, (int)nbk, tot);
-        if (threadIdx.x == 0) {
-            Diag *dg = sJ.dg;
-            dg->sumO_prev = dg->sumO;
-            dg->sumO = tot[0]; dg->sumH = tot[1]; dg->sumW = tot[2];
-            dg->removedW += tot[3];
-            dg->suppliedH += tot[4];
-            if (tot[5] > 0.0 && dg->status == 0) dg->status = 5;
-            *counter = 0u;
-        }
-    }
-}
-
 // ---------------------------------------------------------------------------
-// K1 in 2D by column strips (k_fused_cm): the same arithmetic as k_fused,
-// without shared memory.  Each warp walks one strip of 32 lanes over a
-// block's range of rows; lane L holds column x0 - 1 + L (x0 = 30 * strip column),
-// so lanes 1..30 are the strip's output columns and lanes 0 and 31 its halo.
-// Every lane evaluates mu_O, M_O and the diffusivities of its own column in
-// a three-row register window (x_O at the lane's left/right from shuffles,
-// from an extra load at lanes 0 and 31); the update of row j takes its
-// vertical neighbours from the window and its horizontal ones by shuffle.
-// Raw fields are loaded two rows ahead of their use.
-// ---------------------------------------------------------------------------
-template <typename T>
-struct CmRaw {
-    T th, pg, xo, xh, xw;
-};
-
-template <typename T>
-__device__ __forceinline__ void cm_load(const FieldPtrs<T, 2> &F, unsigned g, CmRaw<T> &R)
-{
-    R.th = F.theta[g];
-    R.pg = F.phig[g];
-    R.xo = F.xO[g];
-    R.xh = F.xH[g];
-    R.xw = F.xW[g];
-}
-
-template <typename T>
-struct CmDer {
-    T mu, M, DH, DW;
-};
-
-// mu_O, M_O, D_H, D_H2O of a cell from its theta, phi_g, x_O and the
-// Laplacian of x_O (Sec. 2.2, 3.2; R4)
-template <typename T>
-__device__ __forceinline__ void cm_derive(const CellConst<T> &K, T th, T pg, T x, T lap, CmDer<T> &Dv)
-{
-    T Wf, Ww, Wg;
-    phase_weights(th, pg, Wf, Ww, Wg);
-    const T m1 = Wf * f_fe1(x) + Ww * f_wu1(x) + Wg * f_ga1(x);
-    const T m2 = Wf * f_fe2(x) + Ww * f_wu2(x) + Wg * f_ga2(x);
-    Dv.mu = K.c * m1 - K.kappa * lap;
-    const T DO = (T(1) - Wg) * K.DOs + Wg * K.DOg;
-    const T den = K.c * m2;
-    Dv.M = den != T(0) ? fast_div(DO, den) : T(0);
-    Dv.DH = (T(1) - Wg) * K.DHs + Wg * K.DHg;
-    Dv.DW = (T(1) - Wg) * K.DWs + Wg * K.DWg;
-}
-
-template <typename T>
-__device__ __forceinline__ T up1(T v) { return __shfl_up_sync(0xffffffffu, v, 1); }
-template <typename T>
-__device__ __forceinline__ T dn1(T v) { return __shfl_down_sync(0xffffffffu, v, 1); }
-
-template <typename T>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 3 : 1) k_fused_cm(const __grid_constant__ JobSet<CellJob<T, 2>> js)
-{
-    __shared__ __align__(16) CellJob<T, 2> sJ;
-    {
-        const CellJob<T, 2> *J_ = my_job(js);
-        const int *src = (const int *)J_;
-        int *dst = (int *)&sJ;
-        for (int w = threadIdx.x; w < (int)(sizeof(CellJob<T, 2>) / sizeof(int)); w += blockDim.x) dst[w] = src[w];
-    }
-    __syncthreads();
-    const FieldPtrs<T, 2> &F = sJ.F;       // pointers and constants are read from the
-    const CellConst<T> &K = sJ.K;          // job's shared-memory copy where used
-    const int nx = sJ.P.nx, ny = sJ.P.ny;
-    const int bid = (int)blockIdx.x - sJ.block0, nbk = sJ.nblocks;
-    const int lane = threadIdx.x & 31;
-    const int WB = blockDim.x >> 5, wib = threadIdx.x >> 5;
-    // strips are grouped WB at a time (one per warp of a block: adjacent
-    // strips share the 128-byte lines of their boundary columns, and the
-    // warps of one block read them together); the (group, row) space is
-    // cut into equal contiguous chunks, one per block, and a chunk that
-    // crosses a group is two segments
-    const int nsx = (nx + 29) / 30;
-    const int ngx = (nsx + WB - 1) / WB;
-    const long long total = (long long)ngx * ny;
-    const long long per = (total + nbk - 1) / nbk;
-    long long u = (long long)bid * per;
-    const long long uend = u + per < total ? u + per : total;
-    Acc<T> acc[5];
-    bool bad = false;
-    while (u < uend) {
-        const int gxi = (int)(u / ny), j0 = (int)(u % ny);
-        const int j1 = (int)((ny - j0) < (uend - u) ? ny : j0 + (uend - u));
-        u += j1 - j0;
-        const int sxi = gxi * WB + wib;
-        if (sxi >= nsx) continue;                                // warp-uniform
-        const int x0 = sxi * 30;
-        const int craw = x0 - 1 + lane;
-        const int c = craw < 0 ? craw + nx : (craw >= nx ? craw - nx : craw);
-        const int cw = c % nx;                                   // grids narrower than a strip wrap again
-        const bool out = lane >= 1 && lane <= 30 && craw < nx;   // this lane writes its column
-        int cext = lane == 0 ? cw - 1 : cw + 1;                  // x_O beyond the halo lanes
-        cext = cext < 0 ? cext + nx : (cext >= nx ? cext - nx : cext);
-        auto row = [&](int j) {
-            int r = j < 0 ? j + ny : (j >= ny ? j - ny : j);
-            if ((unsigned)r >= (unsigned)ny) r = ((j % ny) + ny) % ny;   // grids of a few rows
-            return r;
-        };
-        auto at = [&](int col, int j) { return (unsigned)col + (unsigned)nx * (unsigned)row(j); };
-        // window: raw rows j-1 .. j+2, derived rows j-1, j
-        CmRaw<T> rm, r0, r1, r2;
-        T xe0, xe1, xe2;          // x_O beyond the halo lane, rows j, j+1, j+2 (lanes 0 and 31)
-        CmDer<T> dm, d0;
-        {
-            const T xo_m2 = F.xO[at(cw, j0 - 2)];
-            T xe_m1 = T(0);
-            cm_load(F, at(cw, j0 - 1), rm);
-            cm_load(F, at(cw, j0), r0);
-            cm_load(F, at(cw, j0 + 1), r1);
-            cm_load(F, at(cw, j0 + 2), r2);
-            if (lane == 0 || lane == 31) {
-                xe_m1 = F.xO[at(cext, j0 - 1)];
-                xe0 = F.xO[at(cext, j0)];
-                xe1 = F.xO[at(cext, j0 + 1)];
-                xe2 = F.xO[at(cext, j0 + 2)];
-            } else {
-                xe0 = xe1 = xe2 = T(0);
-            }
-            // derived of rows j0-1 and j0: Laplacians of x_O
-            T l, r;
-            l = up1(rm.xo); r = dn1(rm.xo);
-            if (lane == 0) l = xe_m1;
-            if (lane == 31) r = xe_m1;
-            cm_derive(K, rm.th, rm.pg, rm.xo, l + r + xo_m2 + r0.xo - T(4) * rm.xo, dm);
-            l = up1(r0.xo); r = dn1(r0.xo);
-            if (lane == 0) l = xe0;
-            if (lane == 31) r = xe0;
-            cm_derive(K, r0.th, r0.pg, r0.xo, l + r + rm.xo + r1.xo - T(4) * r0.xo, d0);
-        }
-        for (int j = j0; j < j1; j++) {
-            // raw values two rows ahead, and this row's per-cell inputs
-            CmRaw<T> r3;
-            T xe3 = T(0);
-            cm_load(F, at(cw, j + 3), r3);
-            if (lane == 0 || lane == 31) xe3 = F.xO[at(cext, j + 3)];
-            const unsigned g = at(cw, j);
-            T tE = T(0), s2 = T(0), mob = T(0);
-            unsigned char msk = 0;
-            if (out) { tE = F.trE[g]; s2 = F.devE2[g]; mob = F.mob[g]; msk = F.mask[g]; }
-            // derived of row j+1
-            CmDer<T> d1;
-            {
-                T l = up1(r1.xo), r = dn1(r1.xo);
-                if (lane == 0) l = xe1;
-                if (lane == 31) r = xe1;
-                cm_derive(K, r1.th, r1.pg, r1.xo, l + r + r0.xo + r2.xo - T(4) * r1.xo, d1);
-            }
-            // horizontal neighbours of row j
-            const T thl = up1(r0.th), thr = dn1(r0.th);
-            const T mul = up1(d0.mu), mur = dn1(d0.mu), Ml = up1(d0.M), Mr = dn1(d0.M);
-            const T DHl = up1(d0.DH), DHr = dn1(d0.DH), DWl = up1(d0.DW), DWr = dn1(d0.DW);
-            const T xhl = up1(r0.xh), xhr = dn1(r0.xh), xwl = up1(r0.xw), xwr = dn1(r0.xw);
-            if (out) {
-                const T th = r0.th, pg = r0.pg, xo = r0.xo, xh = r0.xh, xw = r0.xw;
-                const T mu0 = d0.mu, M0 = d0.M, DH0 = d0.DH, DW0 = d0.DW;
-                const T half = T(0.5);
-                const T lapt = (thl - th) + (thr - th) + (rm.th - th) + (r1.th - th);
-                const T dO = half * (M0 + Ml) * (mul - mu0) + half * (M0 + Mr) * (mur - mu0)
-                           + half * (M0 + dm.M) * (dm.mu - mu0) + half * (M0 + d1.M) * (d1.mu - mu0);
-                const T dH = half * (DH0 + DHl) * (xhl - xh) + half * (DH0 + DHr) * (xhr - xh)
-                           + half * (DH0 + dm.DH) * (rm.xh - xh) + half * (DH0 + d1.DH) * (r1.xh - xh);
-                const T dW = half * (DW0 + DWl) * (xwl - xw) + half * (DW0 + DWr) * (xwr - xw)
-                           + half * (DW0 + dm.DW) * (rm.xw - xw) + half * (DW0 + d1.DW) * (r1.xw - xw);
-                const T hg0 = hfun(pg);
-                const T hpt = hder(th);
-                const T sol = T(1) - hg0;
-                const T Af = K.c * f_fe(xo) + half * K.Ks * tE * tE + K.Gs * s2;
-                const T Aw = K.c * f_wu(xo) + half * K.Ks * tE * tE + K.Gs * s2;
-                const T Kmix = sol * K.Ks + hg0 * K.Kg;
-                const T force = sol * hpt * (Af - Aw) + K.w2 * mder(th) - K.eig3 * sol * hpt * Kmix * tE;
-                const T rate = K.Lh * mob * (force - K.eps2 * lapt);
-                T rr = mfun(pg) * K.kf * xo * xh;
-                if (xw >= T(1)) rr = T(0);
-                const T nth = th + K.dt * rate;
-                const T nxo = xo + K.dt * (dO - rr);
-                T nxh = xh + K.dt * (dH - T(2) * rr);
-                T nxw = xw + K.dt * (dW + rr);
-                if (msk) {
-                    acc[3].add(nxw);
-                    acc[4].add(K.xHbc - nxh);
-                    nxh = K.xHbc;
-                    nxw = T(0);
-                }
-                F.theta_o[g] = nth;
-                F.xO_o[g] = nxo;
-                F.xH_o[g] = nxh;
-                F.xW_o[g] = nxw;
-                acc[0].add(nxo); acc[1].add(nxh); acc[2].add(nxw);
-                bad |= !isfinite(nth + nxo + nxh + nxw);
-            }
-            // shift the window one row up
-            rm = r0; r0 = r1; r1 = r2; r2 = r3;
-            xe0 = xe1; xe1 = xe2; xe2 = xe3;
-            dm = d0; d0 = d1;
-        }
-    }
-    Acc<T> acc6[6];
-#pragma unroll
-    for (int q = 0; q < 5; q++) acc6[q] = acc[q];
-    acc6[5].add(T(bad ? 1 : 0));
-    double *partials = sJ.partials;
-    unsigned int *counter = sJ.counter;
-    block_reduce_store<6>(acc6, partials + (size_t)bid * PSTRIDE);
-    __shared__ bool last;
-    if (threadIdx.x == 0) {
-        __threadfence();
-        unsigned int tk = atomicAdd(counter, 1u);
-        last = (tk == (unsigned int)nbk - 1);
-    }
-    __syncthreads();
-    if (last) {
-        __threadfence();
-        __shared__ double tot[6];
-        last_block_sums<6>(partials, nbk, tot);
-        if (threadIdx.x == 0) {
-            Diag *dg = sJ.dg;
-            dg->sumO_prev = dg->sumO;
-            dg->sumO = tot[0]; dg->sumH = tot[1]; dg->sumW = tot[2];
-            dg->removedW += tot[3];
-            dg->suppliedH += tot[4];
-            if (tot[5] > 0.0 && dg->status == 0) dg->status = 5;
-            *counter = 0u;
-        }
-    }
-}
-
-// ---------------------------------------------------------------------------
-// K1 marching along the slowest axis (k_fusedz): the same arithmetic as
-// k_fused, with the grid cut into planes (3D: 32 x 8 cells of an x-y plane,
+// K1 marching along the slowest axis (k_fusedz): mu_O and M_O are evaluated on
+// the fly and never leave the SM, the arithmetic and operand order per cell are
+// those of k_mu and k_update.  The grid is cut into planes (3D: 32 x 8 cells of an x-y plane,
 // marching along z; 2D: 256-cell row segments, marching along y).  A block
 // walks a chunk of planes of one tile column: x_O with a halo of two cells
 // in the plane and theta, phi_g, x_H, x_H2O with a halo of one are copied
