@@ -317,27 +317,40 @@ __global__ void k_up_bwd(Dims d, int C0, int C1, const __nv_bfloat16 *gin, float
     }
 }
 
+// The 3^D convolution layers, a table in device memory: one launch (layer =
+// blockIdx.y) handles all of them.  8 x 128 x 128 training step: 13 + 13 + 13
+// launches of 2-3 us and their gaps, and 20 memsets, before; 3 and 2 now.
+struct WLay {
+    const float *W;                 // master [co][ci][taps]
+    __nv_bfloat16 *fwd, *bwd;
+    const float *gk;                // weight gradient in the kernels' layout
+    float *gW;                      // in the master layout
+    int co, ci, cip, taps;
+};
+
 // weights in the kernels' layouts from the FP32 master W[co][ci][taps]:
 // fwd[tap][co][cip] and, for the input-gradient pass, bwd[tap][cip][co]
-__global__ void k_weights(int co_n, int ci_n, int cip, int taps, const float *W, __nv_bfloat16 *fwd, __nv_bfloat16 *bwd)
+__global__ void k_weights(const WLay *lay)
 {
-    const int n = taps * co_n * cip;
+    const WLay l = lay[blockIdx.y];
+    const int n = l.taps * l.co * l.cip;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int ci = i % cip, r = i / cip, co = r % co_n, tap = r / co_n;
-        const float w = ci < ci_n ? W[((size_t)co * ci_n + ci) * taps + tap] : 0.f;
+        const int ci = i % l.cip, r = i / l.cip, co = r % l.co, tap = r / l.co;
+        const float w = ci < l.ci ? l.W[((size_t)co * l.ci + ci) * l.taps + tap] : 0.f;
         const __nv_bfloat16 v = __float2bfloat16(w);
-        fwd[i] = v;
-        if (bwd) bwd[((size_t)tap * cip + ci) * co_n + co] = v;
+        l.fwd[i] = v;
+        l.bwd[((size_t)tap * l.cip + ci) * l.co + co] = v;
     }
 }
 
 // gW master layout [co][ci][taps] += kernel layout [tap][co][cip]
-__global__ void k_wgrad_to_master(int co_n, int ci_n, int cip, int taps, const float *gk, float *gW)
+__global__ void k_wgrad_to_master(const WLay *lay)
 {
-    const int n = co_n * ci_n * taps;
+    const WLay l = lay[blockIdx.y];
+    const int n = l.co * l.ci * l.taps;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const int tap = i % taps, r = i / taps, ci = r % ci_n, co = r / ci_n;
-        gW[i] += gk[((size_t)tap * co_n + co) * cip + ci];
+        const int tap = i % l.taps, r = i / l.taps, ci = r % l.ci, co = r / l.ci;
+        l.gW[i] += l.gk[((size_t)tap * l.co + co) * l.cip + ci];
     }
 }
 
@@ -353,6 +366,8 @@ __global__ void k_adam(long long n, float *w, const float *g, float *m, float *v
         w[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
     }
 }
+
+constexpr int LAY_BLOCKS = 48;     // blocks per layer of the all-layer kernels
 
 int blocks_for(long long n, int per = 256)
 {
@@ -371,7 +386,7 @@ struct ConvLayer {
     int ci, cip, co, taps;          // input channels (padded cip), output channels, taps
     long long woff, boff;           // offsets in the flat parameter vector
     __nv_bfloat16 *wf = nullptr, *wb = nullptr;   // kernel layouts
-    float *gk = nullptr;            // weight gradient in the kernel layout
+    float *gk = nullptr;            // weight gradient in the kernel layout (a piece of pf_unet::gk)
 };
 
 // Activations (and, for training, gradients) of one (nb, nx, ny, nz).  The
@@ -385,6 +400,8 @@ struct UWork {
     __nv_bfloat16 *x0 = nullptr;
     std::vector<__nv_bfloat16 *> enc1, enc2, pool, dec1, dec2;     // per level
     std::vector<float *> g_a, g_d, g_p;                            // FP32 gradients per level
+    float *g_zero = nullptr;                                       // g_a and g_p, one block
+    size_t n_zero = 0;
     __nv_bfloat16 *gz = nullptr, *gin = nullptr;                   // scratch (largest level)
     float *y = nullptr, *gy = nullptr, *gd0 = nullptr;
     void release()
@@ -403,6 +420,10 @@ struct pf_unet {
     float *params = nullptr, *grad = nullptr, *m = nullptr, *v = nullptr;
     long long adam_t = 0;
     double *part = nullptr;         // loss partials
+    float *gk = nullptr;            // the layers' weight gradients in the kernel layout
+    size_t ngk = 0;
+    WLay *lay = nullptr;            // table of the 3^D convolutions (nlay of them)
+    int nlay = 0;
     std::vector<void *> allocs;
     UWork train;                    // workspace of pf_unet_forward / pf_unet_loss_grad
     int loss_kind = 0;              // PF_UNET_LOSS_MSE / PF_UNET_LOSS_GRAD
@@ -575,9 +596,7 @@ int ensure_work(pf_unet *n, UWork *w, int nb, int nx, int ny, int nz, bool grads
             UN_TRY(n->alloc(&w->dec2[l], sizeof(__nv_bfloat16) * c * C, w->work));
         }
         if (grads) {
-            UN_TRY(n->alloc(&w->g_a[l], sizeof(float) * c * C, w->work));
             UN_TRY(n->alloc(&w->g_d[l], sizeof(float) * c * C, w->work));
-            if (l > 0) UN_TRY(n->alloc(&w->g_p[l], sizeof(float) * c * n->cfg.channels[l - 1], w->work));
         }
         // widest per-cell tensor of this level: a decoder input, a pooled
         // input or the padded network input
@@ -589,6 +608,22 @@ int ensure_work(pf_unet *n, UWork *w, int nb, int nx, int ny, int nz, bool grads
     }
     UN_TRY(n->alloc(&w->y, sizeof(float) * c0 * D, w->work));
     if (grads) {
+        // the gradients that are added to: one block, zeroed by one memset
+        // (every piece a multiple of 16 floats)
+        w->n_zero = 0;
+        for (int l = 0; l < L; l++)
+            w->n_zero += (size_t)level_cells(n, w, l) * nb * (n->cfg.channels[l] + (l > 0 ? n->cfg.channels[l - 1] : 0));
+        UN_TRY(n->alloc(&w->g_zero, sizeof(float) * w->n_zero, w->work));
+        float *q = w->g_zero;
+        for (int l = 0; l < L; l++) {
+            const size_t c = (size_t)level_cells(n, w, l) * nb;
+            w->g_a[l] = q;
+            q += c * n->cfg.channels[l];
+            if (l > 0) {
+                w->g_p[l] = q;
+                q += c * n->cfg.channels[l - 1];
+            }
+        }
         UN_TRY(n->alloc(&w->gz, sizeof(__nv_bfloat16) * big, w->work));
         UN_TRY(n->alloc(&w->gin, sizeof(__nv_bfloat16) * big, w->work));
         UN_TRY(n->alloc(&w->gy, sizeof(float) * c0 * D, w->work));
@@ -599,10 +634,7 @@ int ensure_work(pf_unet *n, UWork *w, int nb, int nx, int ny, int nz, bool grads
 
 int upload_weights(pf_unet *n, cudaStream_t s)
 {
-    for (ConvLayer &c : n->layers) {
-        if (c.taps == 1) continue;
-        k_weights<<<blocks_for((long long)c.taps * c.co * c.cip), 256, 0, s>>>(c.co, c.ci, c.cip, c.taps, n->params + c.woff, c.wf, c.wb);
-    }
+    k_weights<<<dim3(LAY_BLOCKS, n->nlay), 256, 0, s>>>(n->lay);
     return n->cuda(cudaGetLastError(), "weight layout");
 }
 
@@ -687,13 +719,8 @@ int backward_t(pf_unet *n, UWork *w, const float *in, const float *target, doubl
     const int nparts = n->loss_kind == PF_UNET_LOSS_GRAD ? blocks_for(c0) : nblk;
     // zero gradients
     UN_TRY(n->cuda(cudaMemsetAsync(n->grad, 0, sizeof(float) * n->nparam, s), "zero"));
-    for (ConvLayer &c : n->layers)
-        if (c.gk) UN_TRY(n->cuda(cudaMemsetAsync(c.gk, 0, sizeof(float) * c.taps * c.co * c.cip, s), "zero"));
-    for (int l = 0; l < L; l++) {
-        UN_TRY(n->cuda(cudaMemsetAsync(w->g_a[l], 0, sizeof(float) * level_cells(n, w, l) * w->wnb * n->cfg.channels[l], s), "zero"));
-        if (l > 0)
-            UN_TRY(n->cuda(cudaMemsetAsync(w->g_p[l], 0, sizeof(float) * level_cells(n, w, l) * w->wnb * n->cfg.channels[l - 1], s), "zero"));
-    }
+    UN_TRY(n->cuda(cudaMemsetAsync(n->gk, 0, sizeof(float) * n->ngk, s), "zero"));
+    UN_TRY(n->cuda(cudaMemsetAsync(w->g_zero, 0, sizeof(float) * w->n_zero, s), "zero"));
     // output layer
     int k = (int)n->layers.size() - 1;
     const ConvLayer &O = n->layers[k];
@@ -748,10 +775,7 @@ int backward_t(pf_unet *n, UWork *w, const float *in, const float *target, doubl
         }
     }
     // kernel-layout weight gradients into the master layout
-    for (ConvLayer &c : n->layers) {
-        if (c.taps == 1) continue;
-        k_wgrad_to_master<<<blocks_for((long long)c.co * c.ci * c.taps), 256, 0, s>>>(c.co, c.ci, c.cip, c.taps, c.gk, n->grad + c.woff);
-    }
+    k_wgrad_to_master<<<dim3(LAY_BLOCKS, n->nlay), 256, 0, s>>>(n->lay);
     std::vector<double> part(nparts);
     UN_TRY(n->cuda(cudaMemcpyAsync(part.data(), n->part, sizeof(double) * nparts, cudaMemcpyDeviceToHost, s), "loss"));
     UN_TRY(n->cuda(cudaStreamSynchronize(s), "backward"));
@@ -857,8 +881,20 @@ int pf_unet_create(const pf_unet_config *cfg, pf_unet **out)
         if (lay.taps == 1) continue;
         A(&lay.wf, sizeof(__nv_bfloat16) * lay.taps * lay.co * lay.cip);
         A(&lay.wb, sizeof(__nv_bfloat16) * lay.taps * lay.co * lay.cip);
-        A(&lay.gk, sizeof(float) * lay.taps * lay.co * lay.cip);
+        n->ngk += (size_t)lay.taps * lay.co * lay.cip;
     }
+    A(&n->gk, sizeof(float) * n->ngk);
+    std::vector<WLay> tab;
+    size_t o = 0;
+    for (ConvLayer &lay : n->layers) {
+        if (lay.taps == 1) continue;
+        lay.gk = n->gk + o;
+        o += (size_t)lay.taps * lay.co * lay.cip;
+        tab.push_back({n->params + lay.woff, lay.wf, lay.wb, lay.gk, n->grad + lay.woff, lay.co, lay.ci, lay.cip, lay.taps});
+    }
+    n->nlay = (int)tab.size();
+    A(&n->lay, sizeof(WLay) * tab.size());
+    if (rc == PF_OK) rc = n->cuda(cudaMemcpy(n->lay, tab.data(), sizeof(WLay) * tab.size(), cudaMemcpyHostToDevice), "layer table");
     if (rc == PF_OK && !(c.ndim == 2 ? prepare_kernels<2>() : prepare_kernels<3>())) rc = n->fail(PF_ECUDA, "kernel attributes");
     if (rc == PF_OK) rc = n->cuda(cudaMemset(n->params, 0, sizeof(float) * n->nparam), "init");
     if (rc == PF_OK) rc = n->cuda(cudaMemset(n->m, 0, sizeof(float) * n->nparam), "init");
