@@ -642,9 +642,9 @@ k_pcg(const PCGArgs<T, D> *jobs, int njobs)
                 // only form the residual
                 setup_tiled<T, TX, TY>(A, use_x, refine, refine && outer > 0, xe64,
                                        reinterpret_cast<double *>(pcg_dyn), acc, bid, nbk);
-            } else if constexpr (MG) {
-                // 3D multigrid variant: the z-marching sweep in FP64
-                setup_march3<T>(A, use_x, refine, refine && outer > 0, xe64, reinterpret_cast<double *>(pcg_dyn), acc,
+            } else if constexpr (MG || MARCH) {
+                // 3D multigrid variant and the mixed method: the z-marching sweep
+                setup_march3<T, MG>(A, use_x, refine, MG && refine && outer > 0, xe64, reinterpret_cast<double *>(pcg_dyn), acc,
                                 bid, nbk);
             } else
             for (long long n = t0; n < N; n += st) {
@@ -1090,7 +1090,7 @@ size_t pcg_dyn_smem(int shape, bool mg)
         return shape == 1 ? mg_march_offset<T, Tile<2, 1>::X, Tile<2, 1>::Y>() + M2_OP_BYTES
                           : mg_march_offset<T, Tile<2, 0>::X, Tile<2, 0>::Y>() + M2_OP_BYTES;
     }
-    if (D == 3 && mg) {
+    if (D == 3 && (mg || sizeof(T) == 4)) {
         // the FP64 V-cycle's sweeps (mg_sweep3z), or the set-up sweep's (FP64
         // or double-single, three raw streams)
         const size_t cells = sizeof(T) == 4 ? 0 : sizeof(T) * (size_t)mg_sweep3z_words<T>();

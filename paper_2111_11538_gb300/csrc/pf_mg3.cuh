@@ -395,7 +395,10 @@ __device__ __forceinline__ void node_rhs_ds3(const Params &P, long long n, const
 // like the FP32 sweeps' (8-byte asynchronous copies).  The mixed method runs
 // the operator in double-single arithmetic (DS) on the FP32 pipes, the FP64
 // method in FP64.  smem: mg_sweep3z_words<double, true>(3) doubles.
-template <typename T>
+// MG = false (the Jacobi solve of the mixed method): FP64 like the node-wise
+// form it replaced, and b formed in every pass (577 us per set-up at 53x47x61,
+// where every node took its eight cells' element matrices; 290 us now).
+template <typename T, bool MG>
 __device__ void setup_march3(const PCGArgs<T, 3> &A, bool use_x, bool refine, bool resid, const double *xe,
                              double *smem, Acc<double> (&acc)[16], int bid, int nbk)
 {
@@ -407,14 +410,14 @@ __device__ void setup_march3(const PCGArgs<T, 3> &A, bool use_x, bool refine, bo
             for (int c = 0; c < 3; c++) b[c] = __ldcg(A.b64[c] + n);
         } else {
             double so[6], dgn, lo, mo;
-            if constexpr (sizeof(T) == 4) {
+            if constexpr (sizeof(T) == 4 && MG) {
                 node_rhs_ds3(P, n, A.lam, A.mu, A.sig, b, dgn, so, lo, mo);
             } else {
                 double unused[3], unused6[6];
                 node_setup<T, double, double, 3>(P, n, A.lam, A.mu, A.sig, A.x64, xe, false, b, unused, dgn, so,
                                                  unused6, lo, mo);
             }
-            if (refine)
+            if (MG && refine)
 #pragma unroll
                 for (int c = 0; c < 3; c++) A.b64[c][n] = b[c];
             A.dinv[n] = (T)(1.0 / dgn);
@@ -441,7 +444,8 @@ __device__ void setup_march3(const PCGArgs<T, 3> &A, bool use_x, bool refine, bo
         for (long long n = t0; n < P.N; n += st) node((int)n, zero);
         return;
     }
-    if constexpr (sizeof(T) == 4) {
+    constexpr int NT = sizeof(T) == 4 ? MG3_THREADS : MGZ_TX * MGZ_TY;
+    if constexpr (sizeof(T) == 4 && MG) {
         // mixed method: the sweep in double-single arithmetic; x64 is copied
         // as 8-byte words and split into hi + lo when its node plane is formed
         __shared__ DS s_xd[6];
@@ -451,7 +455,7 @@ __device__ void setup_march3(const PCGArgs<T, 3> &A, bool use_x, bool refine, bo
             for (int c = 0; c < 3; c++) s_xsd[c] = reinterpret_cast<const DS *>(A.x64[c]);
         }
         __syncthreads();
-        mg_sweep3z<DS, true, true, MG3_THREADS>(
+        mg_sweep3z<DS, true, true, NT>(
             P.nx, P.ny, P.nz, mg_zchunk(P.nx, P.ny, P.nz, nbk), A.lam, A.mu, bid, nbk, reinterpret_cast<DS *>(smem),
             s_xd, 3, s_xsd,
             [&](const DS *raw, int h, int, int, int, DS (&v)[3]) {
@@ -472,12 +476,12 @@ __device__ void setup_march3(const PCGArgs<T, 3> &A, bool use_x, bool refine, bo
             },
             [](int) {});
     } else {
-        // x: the solution itself (FP64 method)
+        // x: the solution itself (FP64 method), or x64
         __shared__ const double *s_xs[3];
         if (threadIdx.x == 0)
             for (int c = 0; c < 3; c++) s_xs[c] = refine ? A.x64[c] : reinterpret_cast<const double *>(A.x[c]);
         __syncthreads();
-        mg_sweep3z<double, true, true>(
+        mg_sweep3z<double, true, true, NT>(
             P.nx, P.ny, P.nz, mg_zchunk(P.nx, P.ny, P.nz, nbk), A.lam, A.mu, bid, nbk, smem, xe, 3, s_xs,
             [&](const double *raw, int h, int, int, int, double (&v)[3]) {
 #pragma unroll
