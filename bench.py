@@ -549,8 +549,8 @@ def finite_strain_line(n=64, omega=0.2, nload=2, only="both"):
     stretch, Newton-CG to max |residual| <= 1e-10, then the multiplicative J2
     update per cell) on the n^3 core-shell with gas, with FP32 and with FP64
     Hessian-vector products: wall time, Newton and CG counts, and the
-    product kernel's device time (CUDA events around each launch on its
-    stream, pf_fs_stats.hvp_ms).  The call allocates its own memory, so the
+    product kernel's device time (CUDA events around every 32nd launch on
+    its stream, pf_fs_stats.hvp_ms).  The call allocates its own memory, so the
     wall time includes that; the first call (untimed) loads the kernels."""
     import time
     import torch
