@@ -1041,6 +1041,9 @@ k_pcg(const PCGArgs<T, D> *jobs, int njobs)
         }
         if (lead) it_total += it;
         if (!refine) break;
+        // every warp has read s_ctl of the pass's last iteration before the
+        // lead thread writes it again
+        __syncthreads();
         // refinement: x64 += correction, then a grid-wide sync before the
         // next pass reads x64 around every node
         for (long long n = t0; n < N; n += st)
