@@ -439,7 +439,10 @@ struct PCGState {
     double tot0[10];   // first pass's set-up sums [0, 10) (fixed during a solve; MG refinement reuses them)
     double red[16];    // totals of the last reduction
     int it, it_total, conv;
-    int met;           // refinement: the FP64 residual has met the tolerance
+    // refinement: the FP64 residual has met the tolerance, its square there, and
+    // the mean-strain part of the correction added since
+    int met;
+    double rho_met, cE[6];
 };
 
 // Scalar part of one CG update, thread 0 only: beta and alpha from gamma and
@@ -478,7 +481,7 @@ __device__ __forceinline__ void cg_take_gamma_delta(PCGState &S, double gnew, do
 }
 
 // Control words broadcast by thread 0.
-enum { CTL_RUN = 0, CTL_DONE = 1, CTL_ZERO = 2, CTL_STOP = 3 };
+enum { CTL_RUN = 0, CTL_DONE = 1, CTL_ZERO = 2, CTL_STOP = 3, CTL_UNDO = 4 };
 
 }  // namespace pfdev
 
@@ -720,15 +723,23 @@ k_pcg(const PCGArgs<T, D> *jobs, int njobs)
                 int ctl = CTL_RUN;
                 // refinement goes on to half the tolerance: its passes end
                 // anywhere below their targets, and a residual just under the
-                // tolerance would leave an error several times the usual one
+                // tolerance would leave an error several times the usual one.
+                // A solution that meets the tolerance but not its half (met)
+                // gets one more pass, and comes back if that pass's correction
+                // takes the residual above the tolerance again
                 const double res = sqrt(rho), tol = A.rtol * bnorm;
-                if (refine && res <= tol) S.met = 1;
                 if (bnorm == 0.0) ctl = CTL_ZERO;
                 else if (res <= (refine ? 0.5 * tol : tol)) ctl = CTL_DONE;
+                else if (refine && S.met && !(res <= tol)) ctl = CTL_UNDO;
                 // refinement that no longer halves the FP64 residual has
                 // reached what the FP32 passes can resolve: stop (not
                 // converged unless the tolerance is met)
-                else if (refine && outer > 0 && res > 0.5 * S.prev_res) ctl = S.met ? CTL_DONE : CTL_STOP;
+                else if (refine && outer > 0 && res > 0.5 * S.prev_res) ctl = res <= tol ? CTL_DONE : CTL_STOP;
+                else if (refine && res <= tol) {
+                    S.met = 1;
+                    S.rho_met = rho;
+                }
+                if (ctl == CTL_UNDO) rho_final = S.rho_met;
                 S.prev_res = res;
                 // target of this pass: the requested tolerance, or in refinement
                 // mode what an FP32 iteration can deliver on this correction
@@ -764,6 +775,16 @@ k_pcg(const PCGArgs<T, D> *jobs, int njobs)
         }
         if (ctl0 == CTL_DONE) { conv = true; break; }
         if (ctl0 == CTL_STOP) { conv = false; break; }
+        if (ctl0 == CTL_UNDO) {
+            // (A.u holds the last correction; x64 comes back to its rounding)
+            for (long long n = t0; n < N; n += st)
+#pragma unroll
+                for (int d = 0; d < D; d++) A.x64[d][n] -= (double)A.u[d][n];
+            if (lead)
+                for (int vv = 0; vv < NV; vv++) E64[vv] -= S.cE[vv];
+            conv = true;
+            break;
+        }
 
         // ---------------- sweeps: the first builds w_0, then iterations -----
         if constexpr (MG) {
@@ -1044,21 +1065,37 @@ k_pcg(const PCGArgs<T, D> *jobs, int njobs)
         // every warp has read s_ctl of the pass's last iteration before the
         // lead thread writes it again
         __syncthreads();
-        // refinement: x64 += correction, then a grid-wide sync before the
-        // next pass reads x64 around every node
-        for (long long n = t0; n < N; n += st)
-#pragma unroll
-            for (int d = 0; d < D; d++) A.x64[d][n] += (double)A.x[d][n];
         if (lead) {
-            for (int vv = 0; vv < NV; vv++) E64[vv] += XE[vv];
-            s_ctl = (it_total >= A.maxit) ? CTL_STOP : CTL_RUN;
-            if (bid == 0)
-                for (int vv = 0; vv < NV; vv++) A.result[24 + vv] = E64[vv];
+            // A pass that spent cg_maxit, and the last one, are followed by no
+            // residual: what has met the tolerance stays as it was before
+            // them, as it does before a pass that missed its target
+            const bool last = it_total >= A.maxit || outer + 1 == MAX_OUTER;
+            s_ctl = S.met && (last || !(rho_final <= target * target)) ? CTL_DONE : (last ? CTL_STOP : CTL_RUN);
+            if (s_ctl == CTL_DONE) rho_final = S.rho_met;
         }
         __syncthreads();
         const int stop = s_ctl;
+        if (stop == CTL_DONE) { conv = true; break; }
+        // x64 += correction, then a grid-wide sync before the next pass reads
+        // x64 around every node
+        const bool keep = S.met != 0;
+        for (long long n = t0; n < N; n += st)
+#pragma unroll
+            for (int d = 0; d < D; d++) {
+                const T c = A.x[d][n];
+                A.x64[d][n] += (double)c;
+                if (keep) A.u[d][n] = c;
+            }
+        if (lead) {
+            for (int vv = 0; vv < NV; vv++) {
+                S.cE[vv] = XE[vv];
+                E64[vv] += XE[vv];
+            }
+            if (bid == 0)
+                for (int vv = 0; vv < NV; vv++) A.result[24 + vv] = E64[vv];
+        }
         if (!grid_sync(A.bar_count, A.bar_gen, err, nbk)) return;
-        if (stop == CTL_STOP) { if (lead) conv = S.met != 0; break; }
+        if (stop == CTL_STOP) { conv = false; break; }
     }
     if (refine) {
         for (long long n = t0; n < N; n += st)
