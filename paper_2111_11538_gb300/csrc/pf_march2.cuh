@@ -37,10 +37,10 @@ struct Lanes2 {
     }
 };
 
-// the row's displacement with its right neighbour: sum and difference
+// the row's displacement and its difference to the right neighbour
 template <typename T>
 struct Row2 {
-    T e[2], d[2];
+    T v[2], d[2];
 };
 
 template <typename T>
@@ -48,34 +48,39 @@ __device__ __forceinline__ void row2(const T (&v)[2], const Lanes2 &Ln, Row2<T> 
 {
 #pragma unroll
     for (int c = 0; c < 2; c++) {
-        const T r = __shfl_sync(0xffffffffu, v[c], Ln.nxt);
-        R.e[c] = v[c] + r;
-        R.d[c] = r - v[c];
+        R.v[c] = v[c];
+        R.d[c] = __shfl_sync(0xffffffffu, v[c], Ln.nxt) - v[c];
     }
 }
 
 // Corner-force coefficients of the cell between rows lo and hi (l4, m4: a
 // quarter of its moduli): the force on its corner (sx, sy), s = -1 or +1, is
 // sx ax + sy ay + sx sy axy per component.  This is cell_force2 /
-// node_force2 with the sums along x and y taken apart.
+// node_force2 with the sums along x and y taken apart.  Differences of
+// neighbours come first, as there: they are nearly exact where the field is
+// smooth (the y gradient, the sum of both columns' differences, is 2 (hi.v -
+// lo.v) + (hi.d - lo.d)).  The difference of the rows' sums, as many
+// operations, costs digits: relative error of A u in FP64 at 256^2, a smooth
+// u, 2.6e-14 against 1.3e-15.
 template <typename T>
 struct Cell2 {
     T ax0, sh, ay1, xy[2];          // ax = (ax0, sh), ay = (sh, ay1)
 };
 
 template <typename T>
-__device__ __forceinline__ Cell2<T> cell2(T l4, T m4, const Row2<T> &lo, const Row2<T> &hi)
+__host__ __device__ __forceinline__ Cell2<T> cell2(T l4, T m4, const Row2<T> &lo, const Row2<T> &hi)
 {
     const T gxu = lo.d[0] + hi.d[0], gxv = lo.d[1] + hi.d[1];
-    const T gyu = hi.e[0] - lo.e[0], gyv = hi.e[1] - lo.e[1];
+    const T xyu = hi.d[0] - lo.d[0], xyv = hi.d[1] - lo.d[1];
+    const T gyu = T(2) * (hi.v[0] - lo.v[0]) + xyu, gyv = T(2) * (hi.v[1] - lo.v[1]) + xyv;
     const T lt = l4 * (gxu + gyv), m2 = m4 + m4;
     const T ch = (l4 + T(3) * m4) * T(1.0 / 3.0);
     Cell2<T> C;
     C.ax0 = lt + m2 * gxu;
     C.ay1 = lt + m2 * gyv;
     C.sh = m4 * (gyu + gxv);
-    C.xy[0] = ch * (hi.d[0] - lo.d[0]);
-    C.xy[1] = ch * (hi.d[1] - lo.d[1]);
+    C.xy[0] = ch * xyu;
+    C.xy[1] = ch * xyv;
     return C;
 }
 
