@@ -268,7 +268,8 @@ int pf_step_implicit(pf_handle *h, int nsteps, const pf_implicit_opts *opts, pf_
  *   Fbar         : out, host, ndim * ndim row-major
  * Uses the current device; allocates and frees its own device memory;
  * blocking.  Returns PF_EINVAL (arguments), PF_ENOMEM, PF_ECUDA, PF_ENOTCONV
- * (Newton over newton_maxit in a load step; stats still filled);
+ * (Newton over newton_maxit in a load step, or a residual that is not
+ * finite; stats still filled);
  * pf_fs_last_error() gives the text.  Not part of the explicit step. */
 typedef struct {
     int nload;          /* load steps of omega (>= 1)                    */

@@ -610,12 +610,13 @@ __global__ void k_fs_gather(FSArgs A, const double *cf, double *out)
     }
 }
 
-// max |x|
+// max |x|; infinite if an entry is not finite (fmax alone drops NaN, and the
+// maximum is what Newton's method stops at)
 __global__ void k_fs_maxabs(long long L, const double *x, unsigned long long *out)
 {
     double m = 0.0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < L; i += (long long)gridDim.x * blockDim.x)
-        m = fmax(m, fabs(x[i]));
+        m = fmax(m, isfinite(x[i]) ? fabs(x[i]) : (double)INFINITY);
     for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
     if ((threadIdx.x & 31) == 0) atomicMax(out, (unsigned long long)__double_as_longlong(m));
 }
@@ -1342,12 +1343,13 @@ int fs_run(const pf_config *cfg, const double *theta, const double *phi_g, doubl
             S.residual();
             res = S.maxabs(S.r);
             if (res <= opts->newton_tol) break;
-            if (it == opts->newton_maxit) {
+            if (it == opts->newton_maxit || !std::isfinite(res)) {
                 st.residual = res;
                 st.hvp_ms = S.hvp_ms;
                 st.hvp_launches = S.hvp_launches;
                 if (stats) *stats = st;
-                return fs_fail(PF_ENOTCONV, "finite-strain Newton iteration did not converge");
+                return fs_fail(PF_ENOTCONV, std::isfinite(res) ? "finite-strain Newton iteration did not converge"
+                                                               : "finite-strain residual is not finite");
             }
             st.newton_iters++;
             const int ni = S.cg_solve(S.mixed ? std::max(opts->cg_rtol, FS_MIXED_RTOL) : opts->cg_rtol, opts->cg_maxit);
