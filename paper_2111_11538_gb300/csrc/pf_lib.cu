@@ -1217,6 +1217,12 @@ int create_one(const pf_config *cfg, pf_handle **out, std::string &err)
     if (!(c.p.nu > -1.0 && c.p.nu < 0.5) || !(c.p.E_s > 0.0) || !(c.p.E_g_ratio > 0.0)) { err = "elastic constants out of range"; return PF_EINVAL; }
     const long long N = (long long)c.nx * c.ny * (c.ndim == 3 ? c.nz : 1);
     if (N > (1LL << 31)) { err = "grid too large (more than 2^31 cells)"; return PF_EINVAL; }
+    // the 3D sweeps in FP32 address a vector's 3 N values with 32 bits (at that
+    // size the arrays, 276 bytes per cell, would not fit the device)
+    if (c.mechanics && c.ndim == 3 && c.precision == PF_MIXED && 3 * N >= (1LL << 32)) {
+        err = "grid too large (3D mixed mechanics: fewer than 2^32 / 3 cells)";
+        return PF_EINVAL;
+    }
 
     pf_handle *h = new (std::nothrow) pf_handle();
     if (!h) { err = "host allocation failed"; return PF_ENOMEM; }

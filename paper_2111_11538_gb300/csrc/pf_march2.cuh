@@ -355,7 +355,7 @@ struct Restrict2 {
     };
     __device__ __forceinline__ void load(int gx, int gy, const Lanes2 &Ln, Raw &R) const
     {
-        const int n = fnx * fny;
+        const unsigned n = (unsigned)fnx * fny;
 #pragma unroll
         for (int b = 0; b < 3; b++) {
             const T *row = r + fnx * wrap(2 * gy + b - 1, fny);
@@ -384,7 +384,7 @@ struct Restrict2 {
 // ---------------------------------------------------------------------------
 // The sweeps of the V-cycle.  An operation is a plain record, filled in shared
 // memory by one thread; component 1 of a vector lies n values after
-// component 0.  What a thread sums goes into Sums.
+// component 0 (unsigned: g + n reaches 2^32 on a grid of 2^31 nodes).  What a thread sums goes into Sums.
 // ---------------------------------------------------------------------------
 // gamma = r.u, delta = w.u and half the own cells' stresses (of u, without
 // the mean strain)
@@ -403,7 +403,7 @@ struct OpFirst2 {
     const T *lam, *mu, *dinv, *r, *w, *s, *u;
     T *p, *x[2], *sn, *rn, *xpre, *r1, *d1;
     T ta, tb, c2;
-    int n;
+    unsigned n;
     bool upd, dir;              // dir: keep the direction for further smoothing steps
     typedef Acc<T> Sums;        // ||r||^2
     struct Raw {
@@ -471,7 +471,7 @@ struct OpCheb2 {
     const T *lam, *mu, *dinv, *r, *d, *xi;
     T *xo, *rn, *dn;
     T c1, c2, n1, n2;
-    int n;
+    unsigned n;
     bool last, dir;            // dir: the step has a previous direction d
     typedef Acc<T> Sums;
     struct Raw {
@@ -527,7 +527,7 @@ struct OpPre2 {
     Restrict2<T> Rs;
     T *f, *xpre, *r1, *d1;
     T c2;
-    int n;
+    unsigned n;
     typedef Acc<T> Sums;
     struct Raw {
         T l, m, di;
@@ -569,7 +569,7 @@ struct OpApply2 {
     const T *lam, *mu, *u, *r;
     T *w;
     T ue[3];
-    int n;
+    unsigned n;
     typedef Sums2<T> Sums;
     struct Raw {
         T l, m, u[2], r[2];
@@ -620,7 +620,7 @@ struct OpPrePair2 {
     Restrict2<T> Rs;
     T *f, *xpre, *r2;
     T c20, c11, c21;
-    int n;
+    unsigned n;
     typedef Acc<T> Sums;
     struct Raw {
         T l, m, di;
@@ -692,7 +692,7 @@ struct OpPost2 {
     Prolong2<T> P;
     T *xpost, *r;
     T c2;
-    int n;
+    unsigned n;
     bool last;
     typedef Acc<T> Sums;
     typedef PostRaw2<T> Raw;
@@ -728,7 +728,7 @@ struct OpPostPair2 {
     Prolong2<T> P;
     T *xpost;
     T c20, c11, c21;
-    int n;
+    unsigned n;
     typedef Acc<T> Sums;
     typedef PostRaw2<T> Raw;
     __device__ __forceinline__ void load(int g, int gx, int gy, const Lanes2 &Ln, Raw &R) const { post_load2(*this, f, g, gx, gy, Ln, R); }
@@ -768,7 +768,7 @@ struct OpFine2 {
     T *u, *w;
     T c20;
     T ue[3];
-    int n;
+    unsigned n;
     typedef Sums2<T> Sums;
     typedef PostRaw2<T> Raw;
     __device__ __forceinline__ void load(int g, int gx, int gy, const Lanes2 &Ln, Raw &R) const { post_load2(*this, r, g, gx, gy, Ln, R); }

@@ -561,7 +561,7 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
         OpCheb2<T> &op = *reinterpret_cast<OpCheb2<T> *>(s_op);
         static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
         if (lead) {
-            op.lam = V.lam; op.mu = V.mu; op.dinv = V.dinv; op.n = V.nx * V.ny;
+            op.lam = V.lam; op.mu = V.mu; op.dinv = V.dinv; op.n = (unsigned)V.nx * V.ny;
             op.r = V.r[par][0]; op.d = V.d[par][0]; op.xi = post ? V.xpost[0] : V.xpre[0];
             op.xo = last || post ? V.xpost[0] : V.xpre[0];
             op.rn = V.r[1 - par][0]; op.dn = V.d[1 - par][0];
@@ -619,7 +619,7 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
             OpPostPair2<T> &op = *reinterpret_cast<OpPostPair2<T> *>(s_op);
             static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
             if (lead) {
-                op.lam = V.lam; op.mu = V.mu; op.dinv = V.dinv; op.n = V.nx * V.ny;
+                op.lam = V.lam; op.mu = V.mu; op.dinv = V.dinv; op.n = (unsigned)V.nx * V.ny;
                 op.f = V.f[0]; op.xpre = V.xpre[0]; op.xpost = V.xpost[0];
                 op.P = prolong_of(k);
                 op.c20 = H.c2[0]; op.c11 = H.c1[1]; op.c21 = H.c2[1];
@@ -631,7 +631,7 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
             OpPost2<T> &op = *reinterpret_cast<OpPost2<T> *>(s_op);
             static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
             if (lead) {
-                op.lam = V.lam; op.mu = V.mu; op.dinv = V.dinv; op.n = V.nx * V.ny;
+                op.lam = V.lam; op.mu = V.mu; op.dinv = V.dinv; op.n = (unsigned)V.nx * V.ny;
                 op.f = k == 0 ? A.r[cur][0] : V.f[0];
                 op.xpre = V.xpre[0]; op.xpost = V.xpost[0]; op.r = V.r[0][0];
                 op.P = prolong_of(k);
@@ -654,7 +654,7 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
             OpPrePair2<T> &op = *reinterpret_cast<OpPrePair2<T> *>(s_op);
             static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
             if (lead) {
-                op.lam = V.lam; op.mu = V.mu; op.dinv = V.dinv; op.n = V.nx * V.ny;
+                op.lam = V.lam; op.mu = V.mu; op.dinv = V.dinv; op.n = (unsigned)V.nx * V.ny;
                 op.f = V.f[0]; op.xpre = V.xpre[0]; op.r2 = V.r[0][0];
                 op.Rs = restrict_of(k);
                 op.c20 = H.c2[0]; op.c11 = H.c1[1]; op.c21 = H.c2[1];
@@ -666,7 +666,7 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
         OpPre2<T> &op = *reinterpret_cast<OpPre2<T> *>(s_op);
         static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
         if (lead) {
-            op.lam = V.lam; op.mu = V.mu; op.dinv = V.dinv; op.n = V.nx * V.ny;
+            op.lam = V.lam; op.mu = V.mu; op.dinv = V.dinv; op.n = (unsigned)V.nx * V.ny;
             op.f = V.f[0]; op.xpre = V.xpre[0]; op.r1 = V.r[1][0]; op.d1 = V.d[1][0];
             op.Rs = restrict_of(k);
             op.c2 = H.c2[0];
@@ -862,7 +862,7 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
             OpFirst2<T> &op = *reinterpret_cast<OpFirst2<T> *>(s_op);
             static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
             if (lead) {
-                op.lam = L0.lam; op.mu = L0.mu; op.dinv = L0.dinv; op.n = L0.nx * L0.ny;
+                op.lam = L0.lam; op.mu = L0.mu; op.dinv = L0.dinv; op.n = (unsigned)L0.nx * L0.ny;
                 op.r = A.r[cur][0]; op.w = A.w[cur][0]; op.s = A.s[cur][0]; op.u = L0.xpost[0];
                 op.p = A.p[0]; op.x[0] = A.x[0]; op.x[1] = A.x[1]; op.sn = A.s[nxt][0]; op.rn = A.r[nxt][0];
                 op.xpre = L0.xpre[0]; op.r1 = L0.r[1][0]; op.d1 = L0.d[1][0];
@@ -928,7 +928,7 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
             OpFine2<T> &op = *reinterpret_cast<OpFine2<T> *>(s_op);
             static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
             if (lead) {
-                op.lam = L0.lam; op.mu = L0.mu; op.dinv = L0.dinv; op.n = L0.nx * L0.ny;
+                op.lam = L0.lam; op.mu = L0.mu; op.dinv = L0.dinv; op.n = (unsigned)L0.nx * L0.ny;
                 op.r = A.r[cur][0]; op.xpre = L0.xpre[0]; op.u = L0.xpost[0]; op.w = A.w[cur][0];
                 for (int v = 0; v < 3; v++) op.ue[v] = s_ue[v];
                 op.P = prolong_of(0);
@@ -940,7 +940,7 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
             OpApply2<T> &op = *reinterpret_cast<OpApply2<T> *>(s_op);
             static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
             if (lead) {
-                op.lam = L0.lam; op.mu = L0.mu; op.n = L0.nx * L0.ny;
+                op.lam = L0.lam; op.mu = L0.mu; op.n = (unsigned)L0.nx * L0.ny;
                 op.u = L0.xpost[0]; op.r = A.r[cur][0]; op.w = A.w[cur][0];
                 for (int v = 0; v < 3; v++) op.ue[v] = s_ue[v];
             }
