@@ -99,7 +99,10 @@ typedef struct {
     pf_params p;
     int pcg_tile;       /* node tile of the PCG sweep: 0 = the library's choice for the
                            grid size (measured per size class), 1 = 32x8 (2D) / 16x4x4
-                           (3D), 2 = 32x16 / 32x4x2.  Results agree to rounding.        */
+                           (3D), 2 = 32x16 / 32x4x2.  In the 2D multigrid solve it sets
+                           the block size (256 / 512 threads) and the set-up's tile, in
+                           3D mixed nothing (their sweeps march warps).  Results agree
+                           to rounding.                                                 */
     int precond;        /* CG preconditioner: PF_PC_AUTO (the library's choice: PF_PC_MG
                            for grids whose sizes are all divisible by 4 and >= 32, else
                            Jacobi; one choice for a whole batch), PF_PC_JACOBI

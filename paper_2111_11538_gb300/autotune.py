@@ -8,10 +8,11 @@ or are identical for the marching update):
 
   * PCG node tile (pf_config.pcg_tile = 1, 2) of the Jacobi-preconditioned
     solve, per size class (2D up to 2^18 nodes, 2D above, 3D) and storage
-    type: a core-shell grid of the class is stepped with each tile and the
+    type (not 3D FP32, whose sweeps use no tile): a core-shell grid of the class is stepped with each tile and the
     solve time per CG iteration (the library's CUDA-event profile) decides;
-  * the same tiles for the 2D multigrid-preconditioned solve (its V-cycle
-    sweeps use the tile), per 2D size class and storage type, decided by
+  * the same choice for the 2D multigrid-preconditioned solve, where it sets
+    the block size (256 or 512 threads; its V-cycle's sweeps use no tile)
+    and the set-up's tile, per 2D size class and storage type, decided by
     the solve time per step on a porous grid of the class;
   * the start-up weight w of the marching field update's chunk choice (the
     cost model (items per block) x (planes per item + w)), per dimension:
@@ -127,6 +128,8 @@ def main(argv=None):
     table, rows = {}, []
     for dim, cls, shape in PCG_CLASSES:
         for prec, tag in (("mixed", "F32"), ("fp64", "F64")):
+            if dim == "3D" and prec == "mixed":
+                continue
             times = [measure_pcg(shape, prec, t) for t in (1, 2)]
             best = min(range(2), key=lambda k: times[k])
             key = "PCG_TABLE_%s_%s%s" % (dim, tag, "_" + cls if cls else "")

@@ -25,11 +25,13 @@
 
 namespace pfdev {
 
-// Node tiles of the PCG sweep (one node per thread: the block has X*Y*Z
-// threads); the shape is a launch option (pf_config.pcg_tile), picked per
-// size class from measurements when left to the library.  The 32x16 tile
-// runs one 512-thread block per SM: fewer blocks in each grid reduction and
-// a smaller idle tail in the halo passes than two 256-thread blocks.
+// Node tiles of the Jacobi PCG's sweep and of the 2D multigrid's set-up (one
+// node per thread: the block has X*Y*Z threads); the shape is a launch option
+// (pf_config.pcg_tile), picked per size class from measurements when left to
+// the library.  The 32x16 tile runs one 512-thread block per SM: fewer blocks
+// in each grid reduction and a smaller idle tail in the halo passes than two
+// 256-thread blocks.  The marching sweeps (2D multigrid, 3D FP32) use no tile;
+// in 2D the shape still sets their block size, in 3D FP32 nothing.
 template <int D, int S> struct Tile;
 template <> struct Tile<2, 0> { static constexpr int X = 32, Y = 8, Z = 1; };
 template <> struct Tile<2, 1> { static constexpr int X = 32, Y = 16, Z = 1; };
@@ -53,7 +55,7 @@ struct PCGArgs {
     int refine;                    // 1: FP64 outer residual around the FP32 iteration
     double eta;                    // refinement mode: relative target of one FP32 pass
     double *partials;
-    double *result;                // 32 doubles: [0,16) reductions, [24,30) FP64 mean strain
+    double *emean;                 // refinement mode: FP64 mean strain between two passes, 6 doubles
     unsigned int *bar_count, *bar_gen;
     Scalars *sc;
     Diag *dg;
@@ -635,7 +637,7 @@ k_pcg(const PCGArgs<T, D> *jobs, int njobs)
             double xe64[6];
             T xeT[6];
             for (int v = 0; v < NV; v++) {
-                xe64[v] = outer == 0 ? (A.warm ? A.sc->E[v] : 0.0) : __ldcg(A.result + 24 + v);
+                xe64[v] = outer == 0 ? (A.warm ? A.sc->E[v] : 0.0) : __ldcg(A.emean + v);
                 xeT[v] = s_xe[v];
             }
             Acc<double> acc[16];
@@ -1092,7 +1094,7 @@ k_pcg(const PCGArgs<T, D> *jobs, int njobs)
                 E64[vv] += XE[vv];
             }
             if (bid == 0)
-                for (int vv = 0; vv < NV; vv++) A.result[24 + vv] = E64[vv];
+                for (int vv = 0; vv < NV; vv++) A.emean[vv] = E64[vv];
         }
         if (!grid_sync(A.bar_count, A.bar_gen, err, nbk)) return;
         if (stop == CTL_STOP) { conv = false; break; }
@@ -1143,12 +1145,16 @@ size_t pcg_dyn_smem(int shape, bool mg)
 }
 
 // the kernel variant of a tile shape, with or without the multigrid
-// preconditioner (2D only)
+// preconditioner (3D FP32 marches warps and has one)
 template <typename T, int D>
 const void *pcg_kernel(int shape, bool mg)
 {
-    if (mg) return shape == 1 ? (const void *)k_pcg<T, D, 1, true> : (const void *)k_pcg<T, D, 0, true>;
-    return shape == 1 ? (const void *)k_pcg<T, D, 1, false> : (const void *)k_pcg<T, D, 0, false>;
+    if constexpr (D == 3 && sizeof(T) == 4)
+        return mg ? (const void *)k_pcg<T, D, 0, true> : (const void *)k_pcg<T, D, 0, false>;
+    else if (mg)
+        return shape == 1 ? (const void *)k_pcg<T, D, 1, true> : (const void *)k_pcg<T, D, 0, true>;
+    else
+        return shape == 1 ? (const void *)k_pcg<T, D, 1, false> : (const void *)k_pcg<T, D, 0, false>;
 }
 
 template <typename T, int D>

@@ -86,8 +86,6 @@ struct Diag {
 // ---------------------------------------------------------------------------
 // Small helpers
 // ---------------------------------------------------------------------------
-template <typename T> __device__ __forceinline__ T ldg_(const T *p) { return __ldg(p); }
-template <typename T> __device__ __forceinline__ T ldcg_(const T *p) { return __ldcg(p); }
 
 __device__ __forceinline__ double warp_sum(double v)
 {

@@ -426,20 +426,17 @@ struct BECheb32 {
     float c1[4], c2[4];
 };
 
-template <int D>
-__device__ __forceinline__ void be_neighbours32(int nx, int ny, int nz, int c, int (&nb)[2 * D])
+__device__ __forceinline__ void be_neighbours32(int nx, int ny, int nz, int c, int (&nb)[6])
 {
     const int i = c % nx, r = c / nx;
-    const int j = r % ny, k = D == 3 ? r / ny : 0;
+    const int j = r % ny, k = r / ny;
     const int base = c - i, pl = nx * ny;
     nb[0] = base + (i == 0 ? nx - 1 : i - 1);
     nb[1] = base + (i == nx - 1 ? 0 : i + 1);
     nb[2] = c + nx * ((j == 0 ? ny - 1 : j - 1) - j);
     nb[3] = c + nx * ((j == ny - 1 ? 0 : j + 1) - j);
-    if constexpr (D == 3) {
-        nb[4] = c + pl * ((k == 0 ? nz - 1 : k - 1) - k);
-        nb[5] = c + pl * ((k == nz - 1 ? 0 : k + 1) - k);
-    }
+    nb[4] = c + pl * ((k == 0 ? nz - 1 : k - 1) - k);
+    nb[5] = c + pl * ((k == nz - 1 ? 0 : k + 1) - k);
 }
 
 // the FP32 coefficients of the four blocks (after k_be_pc_diag)
@@ -473,20 +470,19 @@ __global__ void k_be_pc32_init(int N, const double *__restrict__ v, BEPc32 P, BE
         }
 }
 
-// one Chebyshev step: q = A din at cell c, then z += din, r -= q,
-// dout = c1 din + c2 D^-1 r
-template <int D>
+// one Chebyshev step in 3D: q = A din at cell c, then z += din, r -= q,
+// dout = c1 din + c2 D^-1 r (2D: k_be_pc32_tile)
 __global__ void k_be_pc32_step(int nx, int ny, int nz, int N, float dt, const unsigned char *__restrict__ mask,
                                BEPc32 P, const float *__restrict__ din, float *__restrict__ dout, BECheb32 cf)
 {
     for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < N; c += gridDim.x * blockDim.x) {
-        int nb[2 * D];
-        be_neighbours32<D>(nx, ny, nz, c, nb);
+        int nb[6];
+        be_neighbours32(nx, ny, nz, c, nb);
         const float d0c = din[c], d1c = din[N + c], d2c = din[2 * N + c], d3c = din[3 * N + c];
         const float DOc = P.DO[c], DHc = P.DH[c], DWc = P.DW[c];
         float lt = 0.0f, fo = 0.0f, fh = 0.0f, fw = 0.0f;
 #pragma unroll
-        for (int k = 0; k < 2 * D; k++) {
+        for (int k = 0; k < 6; k++) {
             const int n = nb[k];
             lt += d0c - din[n];
             fo += 0.5f * (DOc + P.DO[n]) * (d1c - din[N + n]);

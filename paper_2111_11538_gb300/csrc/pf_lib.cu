@@ -183,7 +183,7 @@ struct pf_handle {
     void *corr[3] = {};                // mixed mode: FP32 correction of one refinement pass
     double *x64[3] = {};               // mixed mode: FP64 displacement
     bool refine = false;
-    double *result = nullptr;
+    double *emean = nullptr;
     unsigned char *mask = nullptr;
     double *partials = nullptr;
     int npart = 0;
@@ -353,20 +353,20 @@ std::vector<pf_handle *> instances(pf_handle *h)
     return h->is_batch ? h->members : std::vector<pf_handle *>{h};
 }
 
-// Node tile of the PCG sweep for a grid of N nodes: pf_config.pcg_tile if
-// set (1 or 2 select shape 0 or 1), else the per-size-class choice measured
-// on GB300 (paper_2111_11538_gb300/autotune.py prints the table).
+// Node tile of the Jacobi PCG's sweep for a grid of N nodes (pf_config.pcg_tile
+// 1 or 2 select shape 0 or 1): the per-size-class choice measured on GB300
+// (paper_2111_11538_gb300/autotune.py prints the table).
 int default_pcg_shape(int ndim, long long N, bool fp64)
 {
     if (ndim == 2) {
         if (fp64) return N <= (1LL << 18) ? PCG_TABLE_2D_F64_SMALL : PCG_TABLE_2D_F64_LARGE;
         return N <= (1LL << 18) ? PCG_TABLE_2D_F32_SMALL : PCG_TABLE_2D_F32_LARGE;
     }
-    return fp64 ? PCG_TABLE_3D_F64 : PCG_TABLE_3D_F32;
+    return PCG_TABLE_3D_F64;
 }
 
-// Node tile of the 2D multigrid-preconditioned solve (its V-cycle sweeps use
-// the same tile), per size class.
+// Block size (256 or 512 threads) and set-up tile of the 2D multigrid solve,
+// per size class.
 int mg2_pcg_shape(long long N, bool fp64)
 {
     if (fp64) return N <= (1LL << 18) ? PCG_TABLE_MG2D_F64_SMALL : PCG_TABLE_MG2D_F64_LARGE;
@@ -527,12 +527,11 @@ int setup_cg_launch(pf_handle *h)
 {
     const bool fp64 = sizeof(T) == 8;
     h->mg = h->cfg.precond == PF_PC_MG || (h->cfg.precond == PF_PC_AUTO && auto_mg(h->cfg));
-    // 2D: the V-cycle's coarse grid levels have few tiles, and the 32x16
-    // tile (one 512-thread block per SM) halves the blocks in each of their
-    // barriers; 3D: the 16x4x4 tile of the cell path
-    h->pcg_shape = h->cfg.pcg_tile > 0 ? h->cfg.pcg_tile - 1
-                                       : (h->mg ? (D == 2 ? mg2_pcg_shape(h->P.N, fp64) : 0)
-                                                : default_pcg_shape(D, h->P.N, fp64));
+    // (3D FP32 has one shape: its sweeps march warps)
+    h->pcg_shape = D == 3 && !fp64       ? 0
+                   : h->cfg.pcg_tile > 0 ? h->cfg.pcg_tile - 1
+                   : h->mg               ? (D == 2 ? mg2_pcg_shape(h->P.N, fp64) : 0)
+                                         : default_pcg_shape(D, h->P.N, fp64);
     h->cg_block = h->pcg_shape ? pcg_threads<T, D, 1, true>() : pcg_threads<T, D, 0, true>();
     if (h->mg) PF_TRY((build_mg<T, D>(h)));
     int per_sm = 0;
@@ -562,7 +561,7 @@ PCGArgs<T, D> pcg_args(pf_handle *m)
     A.eta = 1e-3;
     A.dinv = (T *)m->diag;
     A.partials = m->partials;
-    A.result = m->result;
+    A.emean = m->emean;
     A.bar_count = m->sync; A.bar_gen = m->sync + SYNC_GEN;
     A.sc = m->sc; A.dg = m->dg;
     A.rtol = m->cfg.cg_rtol; A.maxit = m->cfg.cg_maxit;
@@ -1130,7 +1129,7 @@ int alloc_fields(pf_handle *h)
             PF_TRY(h->alloc_comps(h->w[k], D, b));
             PF_TRY(h->alloc_comps(h->s[k], D, b));
         }
-        PF_TRY(h->alloc(&h->result, sizeof(double) * 32));
+        PF_TRY(h->alloc(&h->emean, sizeof(double) * 6));
         PF_TRY(h->alloc(&h->diag, b));
         if (h->cfg.warm_start == PF_WS_EXTRAP || h->cfg.warm_start == PF_WS_EXTRAP2) {
             const int nh = h->cfg.warm_start == PF_WS_EXTRAP2 ? 2 : 1;
@@ -1398,7 +1397,7 @@ int be_steps(pf_handle *h, int nsteps, const pf_implicit_opts &o, pf_implicit_st
     // zo = M^-1 f v with f = *vf (device; 1 if null); vn: f v itself, a vector
     // other than v (null: not wanted, f = 1)
     auto precond = [&](const double *v, const double *vf, double *vn, double *zo) -> int {
-        if (D == 2 && pc32 && K > 0) {
+        if constexpr (D == 2) if (pc32 && K > 0) {
             const int own = BE_TILE - 2 * tileH;
             const unsigned nt = (unsigned)(((a.nx + own - 1) / own) * ((a.ny + own - 1) / own));
             int k0 = 0, par = 0;
@@ -1420,13 +1419,12 @@ int be_steps(pf_handle *h, int nsteps, const pf_implicit_opts &o, pf_implicit_st
             v = vn;
         }
         if (K == 0) return h->cuda(cudaMemcpyAsync(zo, v, sizeof(double) * L, cudaMemcpyDeviceToDevice, s), "copy");
-        if (pc32) {
+        if constexpr (D == 3) if (pc32) {
             const int n32 = (int)N;
             k_be_pc32_init<<<gN, 256, 0, s>>>(n32, v, w.pc32, cinit32);
             float *din = w.pc32.d0, *dout = w.pc32.d1;
             for (int k = 0; k + 1 < K; k++) {
-                k_be_pc32_step<D><<<gN, 256, 0, s>>>(a.nx, a.ny, a.nz, n32, (float)a.dt, a.mask, w.pc32, din, dout,
-                                                     cheb32[k]);
+                k_be_pc32_step<<<gN, 256, 0, s>>>(a.nx, a.ny, a.nz, n32, (float)a.dt, a.mask, w.pc32, din, dout, cheb32[k]);
                 std::swap(din, dout);
             }
             k_be_pc32_final<<<gN, 256, 0, s>>>(n32, w.pc32, din, zo);

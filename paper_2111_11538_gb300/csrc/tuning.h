@@ -8,7 +8,6 @@
 #define PCG_TABLE_2D_F32_SMALL 0
 #define PCG_TABLE_2D_F64_LARGE 0
 #define PCG_TABLE_2D_F64_SMALL 1
-#define PCG_TABLE_3D_F32 0
 #define PCG_TABLE_3D_F64 0
 #define PCG_TABLE_MG2D_F32_LARGE 1
 #define PCG_TABLE_MG2D_F32_SMALL 1
