@@ -728,16 +728,12 @@ int build_plan(pf_handle *h)
                          k < (I[i]->mg ? mg_levels3(I[i]->P.nx, I[i]->P.ny, I[i]->P.nz) : 1);
                          k++, nx /= 2, ny /= 2, nz /= 2)
                         pj[i].zc1[k] = m3_chunk(nx, ny, nz, (int)nb * (h->cg_block / 32));
+                if (D == 2 && I[i]->mg)
+                    for (int k = 0, nx = I[i]->P.nx, ny = I[i]->P.ny; k < mg_levels(I[i]->P.nx, I[i]->P.ny); k++, nx /= 2, ny /= 2) {
+                        pj[i].zc1[k] = m2_chunk(nx, ny, (int)nb, h->cg_block / 32, 30, 2, sizeof(T) == 8);
+                        pj[i].zc2[k] = m2_chunk(nx, ny, (int)nb, h->cg_block / 32, 28, 4, sizeof(T) == 8);
+                    }
                 g0 += (int)nb;
-            }
-            for (int i = i0; i < i1; i++) {
-                if (D != 2 || !I[i]->mg) continue;
-                const bool fp64 = sizeof(T) == 8;
-                const long long units = fp64 ? m2_pipes(pj[i].nblocks, g0, h->sms) : (long long)pj[i].nblocks * (h->cg_block / 32);
-                for (int k = 0, nx = I[i]->P.nx, ny = I[i]->P.ny; k < mg_levels(I[i]->P.nx, I[i]->P.ny); k++, nx /= 2, ny /= 2) {
-                    pj[i].zc1[k] = m2_chunk(nx, ny, units, 30, 2, fp64);
-                    pj[i].zc2[k] = m2_chunk(nx, ny, units, 28, 4, fp64);
-                }
             }
             h->pcg_rounds.push_back({i0, i1 - i0, g0});
         }

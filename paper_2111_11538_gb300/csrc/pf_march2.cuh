@@ -120,35 +120,27 @@ struct Node2 {
 constexpr int M2_OP_BYTES = 320;
 extern __shared__ __align__(16) unsigned char pcg_dyn[];
 
-// Rows per work item of an nx x ny level, with strips of OW columns and
-// `extra` rows of start-up, for `units` workers: the candidate with the least
-// time by a simple count, items per worker (rounded up) times rows.  FP32
-// sweeps are bound by a warp's latency (the units are warps; a first row's
-// copies cost about four rows' work); FP64 ones by the FP64 pipes, four to an
-// SM however many blocks share it (a row of a lone warp takes as long as its
-// FP64 instructions, 64 cycles each).
-inline int m2_chunk(int nx, int ny, long long units, int OW, int extra, bool fp64)
+// Rows per work item of an nx x ny level for nbk blocks of nwb warps, with
+// strips of OW columns and `extra` rows of start-up: the candidate with the
+// least time by a simple count.  FP32 sweeps are bound by a warp's latency
+// (items per warp, rounded up, times rows; a first row's copies cost about
+// four rows' work); FP64 ones by the FP64 pipes, one per quarter of an SM (a
+// row of a lone warp takes as long as its FP64 instructions, 64 cycles each).
+inline int m2_chunk(int nx, int ny, int nbk, int nwb, int OW, int extra, bool fp64)
 {
     const long long ns = nx <= 32 ? 1 : (nx + OW - 1) / OW;
     int best = ny;
     long long bcost = -1;
     for (int zc = 1; zc <= ny; zc++) {
         const long long items = ns * ((ny + zc - 1) / zc);
-        const long long cost = ((items + units - 1) / units) * (zc + extra + (fp64 ? 0 : 4));
+        const long long cost = fp64 ? ((items + 4LL * nbk - 1) / (4LL * nbk)) * (zc + extra)
+                                    : ((items + (long long)nbk * nwb - 1) / ((long long)nbk * nwb)) * (zc + extra + 4);
         if (bcost < 0 || cost < bcost) {
             bcost = cost;
             best = zc;
         }
     }
     return best;
-}
-
-// FP64 pipes that a job of nbk blocks has in a launch of `grid` blocks on
-// `sms` SMs.
-inline long long m2_pipes(int nbk, int grid, int sms)
-{
-    const long long per_sm = (grid + sms - 1) / sms, n = 4LL * nbk / (per_sm > 1 ? per_sm : 1);
-    return n > 0 ? n : 1;
 }
 
 // One product: op.load(g, gx, gy, own, lanes, R) loads the words of node g
