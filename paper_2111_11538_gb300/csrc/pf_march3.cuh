@@ -5,8 +5,8 @@
 // and 31 are halo) by M3_ROWS rows over a chunk of planes; one warp marches it
 // along z with everything in registers.  Per plane it walks its node rows
 // (and a halo row on each side): a row's operand is formed from its own
-// lane's words, loaded while the row before is worked on, and kept as its
-// difference to the right neighbour beside it (one shuffle per component); a cell
+// lane's words, loaded while the row before is worked on, and kept as its sum
+// and difference with the right neighbour (one shuffle per component); a cell
 // row takes four such rows, two of this plane and two of the plane before,
 // which stay in registers; what a cell row leaves on the plane above is
 // carried to the next plane as left/right sums, and a finished node row takes
@@ -29,17 +29,17 @@
 
 namespace pfdev {
 
-// a row's displacement and its difference to the right neighbour
 struct Row3 {
-    float v[3], d[3];
+    float e[3], d[3];
 };
 
 __device__ __forceinline__ void row3(const float (&v)[3], const Lanes2 &Ln, Row3 &R)
 {
 #pragma unroll
     for (int c = 0; c < 3; c++) {
-        R.v[c] = v[c];
-        R.d[c] = __shfl_sync(0xffffffffu, v[c], Ln.nxt) - v[c];
+        const float r = __shfl_sync(0xffffffffu, v[c], Ln.nxt);
+        R.e[c] = v[c] + r;
+        R.d[c] = r - v[c];
     }
 }
 
@@ -48,29 +48,26 @@ __device__ __forceinline__ void row3(const float (&v)[3], const Lanes2 &Ln, Row3
 // (sx, sy, sz), s = -1 or +1, is sx ax + sy ay + sz az + sx sy xy + sy sz yz +
 // sz sx zx + sx sy sz xyz per component; ax, ay, az are the rows of the
 // symmetric s.  This is cell_force3 / corner_forces3 with the sums along each
-// axis taken apart, and with the differences of neighbours first, which are
-// nearly exact where the field is smooth (see cell2): the sum of both columns'
-// differences between two rows is 2 (v' - v) + (d' - d).
+// axis taken apart.
 struct Cell3 {
     float s[6];                     // xx yy zz yz xz xy, a quarter of the average stress
     float xy[3], yz[3], zx[3], xyz[3];
 };
 
-__host__ __device__ __forceinline__ void cell3(float l, float m, const Row3 &a, const Row3 &b, const Row3 &a1, const Row3 &b1,
+__device__ __forceinline__ void cell3(float l, float m, const Row3 &a, const Row3 &b, const Row3 &a1, const Row3 &b1,
                                       Cell3 &C)
 {
     float gx[3], gy[3], gz[3], hxy[3], hyz[3], hzx[3];
 #pragma unroll
     for (int k = 0; k < 3; k++) {
-        const float sd0 = a.d[k] + b.d[k], dd0 = b.d[k] - a.d[k], de0 = 2.0f * (b.v[k] - a.v[k]) + dd0;
-        const float sd1 = a1.d[k] + b1.d[k], dd1 = b1.d[k] - a1.d[k], de1 = 2.0f * (b1.v[k] - a1.v[k]) + dd1;
-        const float va = a1.v[k] - a.v[k], vb = b1.v[k] - b.v[k];
+        const float sd0 = a.d[k] + b.d[k], dd0 = b.d[k] - a.d[k], se0 = a.e[k] + b.e[k], de0 = b.e[k] - a.e[k];
+        const float sd1 = a1.d[k] + b1.d[k], dd1 = b1.d[k] - a1.d[k], se1 = a1.e[k] + b1.e[k], de1 = b1.e[k] - a1.e[k];
         gx[k] = sd0 + sd1;
         gy[k] = de0 + de1;
+        gz[k] = se1 - se0;
         hxy[k] = dd0 + dd1;
         hyz[k] = de1 - de0;
         hzx[k] = sd1 - sd0;
-        gz[k] = 2.0f * (va + vb) + hzx[k];
         C.xyz[k] = dd1 - dd0;
     }
     const float lt = l * (gx[0] + gy[1] + gz[2]), m2 = m + m;
