@@ -39,14 +39,17 @@ CG_ITER_WORDS = {2: 16, 3: 24}
 CG_INIT_WORDS = {2: 10, 3: 15}
 # The compulsory traffic of one multigrid-preconditioned iteration (a V-cycle)
 # per finest-level node, in FP32 words (model, reported beside the figure
-# above).  2D: finest level 29 (CG update fused into the first smoothing
-# sweep) + 9.5 (post-smoothing) + 8 (w = A u); coarse grid levels ~18;
-# shared-memory levels none.  3D (three components per vector): first sweep
-# 46 (r, w, s, p, x, xpost and dinv, lam, mu read; p, x, s, r, xpre, r1, d1
-# written), post-smoothing sweep 19 (xpre, r, xpost-correction, dinv, lam,
-# mu read; xpost written), w = A u 17 (xpost, r, lam, mu read; w written),
-# every coarse level 1/8 of the nodes with four sweeps of ~20 words: ~11.
-MG_ITER_WORDS = {2: 64, 3: 93}
+# above).  2D: first sweep with the CG update 27 (r, w, s, u, p, x, dinv, lam,
+# mu read; p, x, s, r, xpre, r1 written), post-smoothing with w = A u 11.5
+# (r, xpre, dinv, lam, mu and the coarse correction read; u, w written), every
+# coarse grid level ~22 on 1/4 of the nodes, with the restriction's 2 words per
+# fine node: ~9.5; shared-memory levels none.  3D: CG update 30 (u, w, p, x, s,
+# r read; p, x, s, r written), first smoothing 9 (r, dinv, lam, mu read; r1
+# written), post-smoothing 9.4 (r, dinv, lam, mu and the coarse correction
+# read; xpost written), w = A u 11 (xpost, r, lam, mu read; w written), every
+# coarse level ~62 on 1/8 of the nodes, with the restriction's 3 words per
+# fine and 3 per coarse node: ~12.6.
+MG_ITER_WORDS = {2: 48, 3: 72}
 MG_INIT_WORDS = {2: 28, 3: 40}
 # DRAM bytes per k_pcg launch (dram__bytes_read.sum + dram__bytes_write.sum)
 # from one ncu capture of the current kernel on the named workload, per

@@ -1,5 +1,5 @@
-// Persistent Jacobi-PCG for the mechanics (K3/K4), one grid barrier per
-// iteration.
+// Persistent PCG for the mechanics (K3/K4); here the Jacobi-preconditioned
+// loops and what they share with the multigrid ones (pf_mg.cuh, pf_mg3.cuh).
 //
 // The iteration is the Chronopoulos-Gear form of preconditioned CG: with
 // u = M^-1 r, w = A u, gamma = r.u, delta = w.u,
@@ -8,11 +8,14 @@
 //     p_i = u_i + beta_i p_{i-1},  s_i = w_i + beta_i s_{i-1}
 //     x_{i+1} = x_i + alpha_i p_i,  r_{i+1} = r_i - alpha_i s_i
 // which produces the iterates of standard PCG but needs all its inner
-// products at one point per iteration.  One sweep over node tiles does the
-// vector updates, rebuilds u_{i+1} on the tile and its halo in shared memory
-// from r_i, w_i, s_{i-1} (double-buffered in global memory), applies the Q1
-// operator to it and accumulates gamma, delta and ||r||^2; the grid barrier
-// then reduces those in a fixed order (the last block to arrive reduces).
+// products at one point per iteration.  In 2D and in 3D FP64 one sweep over
+// node tiles does the vector updates, rebuilds u_{i+1} on the tile and its halo
+// in shared memory from r_i, w_i, s_{i-1} (double-buffered in global memory),
+// applies the Q1 operator to it and accumulates gamma, delta and ||r||^2: one
+// grid barrier per iteration, after which every block sums the blocks'
+// partials in the same fixed order.  In 3D FP32 the update is a pass of its
+// own, in place, and a marching sweep (pf_march3.cuh) does the rest: two
+// barriers.
 //
 // The few FP64 scalars of the iteration (alpha, beta, the mean-strain dofs)
 // are computed by thread 0 of every block (identically, from the same

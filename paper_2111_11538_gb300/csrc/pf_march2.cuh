@@ -124,16 +124,25 @@ extern __shared__ __align__(16) unsigned char pcg_dyn[];
 // strips of OW columns and `extra` rows of start-up: the candidate with the
 // least time by a simple count.  FP32 sweeps are bound by a warp's latency
 // (items per warp, rounded up, times rows; a first row's copies cost about
-// four rows' work); FP64 ones by the FP64 pipes, one per quarter of an SM (a
-// row of a lone warp takes as long as its FP64 instructions, 64 cycles each).
+// four rows' work); FP64 ones by the FP64 pipes, one per quarter of an SM, and
+// by the loads between (a row of a lone warp takes as long as its FP64
+// instructions, 64 cycles each): two items to a pipe, so that one's loads
+// overlap another's arithmetic, but one in a job of one or two blocks, whose
+// short chunks cost more rows of start-up than that gains.  One / two / four
+// items per pipe, ms per step: 512^2 7.18 / 6.68 / 7.22, batches of 32 x 128^2
+// 12.05 / 10.63 / 10.35, of 16 x 256^2 17.9 / 14.9 / 14.5, of 64 x 64^2 (two
+// blocks each) 6.56 / 6.74 / 7.00; one in all, the batch of 32 was slower than
+// the tiled sweeps (11.57).  Where two blocks share an SM (more than 2^18
+// nodes) the count is still per block: 1024^2 73.6, counted per SM 90.4.
 inline int m2_chunk(int nx, int ny, int nbk, int nwb, int OW, int extra, bool fp64)
 {
     const long long ns = nx <= 32 ? 1 : (nx + OW - 1) / OW;
+    const long long units = (nbk > 2 ? 8LL : 4LL) * nbk;
     int best = ny;
     long long bcost = -1;
     for (int zc = 1; zc <= ny; zc++) {
         const long long items = ns * ((ny + zc - 1) / zc);
-        const long long cost = fp64 ? ((items + 4LL * nbk - 1) / (4LL * nbk)) * (zc + extra)
+        const long long cost = fp64 ? ((items + units - 1) / units) * (zc + extra)
                                     : ((items + (long long)nbk * nwb - 1) / ((long long)nbk * nwb)) * (zc + extra + 4);
         if (bcost < 0 || cost < bcost) {
             bcost = cost;

@@ -218,8 +218,9 @@ __device__ void mg_coarsen_blk(const T *fl, const T *fm, int fnx, bool global, c
     __syncthreads();
 }
 
-// Hierarchy set-up at the start of a solve (the cell moduli change every
-// step): the grid levels below Lg, with a barrier after each.  Returns false
+// Hierarchy set-up at the start of a solve (the cell moduli are written anew
+// every step; they follow phi_g, which is held fixed, to rounding): the grid
+// levels below Lg, with a barrier after each.  Returns false
 // if a barrier timed out.
 template <typename T>
 __device__ bool mg_setup(const MGHier<T> &H, unsigned int *bc, unsigned int *bg, int *err, int bid, int nbk)
@@ -534,7 +535,8 @@ __device__ void setup_tiled(const PCGArgs<T, 2> &A, bool use_x, bool refine, boo
 //   V-cycle on r_i, its first sweep also doing the update of iteration i-1
 //   (p, s, x, r) and reducing ||r_i||^2 for the stopping test;
 //   u_i = the V-cycle's result, w_i = A u_i, gamma_i = r_i.u_i, delta_i =
-//   w_i.u_i and the mean-strain row in one sweep and one reduction.
+//   w_i.u_i and the mean-strain row in one sweep (FP32: with the finest
+//   level's post-smoothing) and one reduction.
 // Returns CTL_DONE or CTL_STOP, or -1 when a barrier timed out.
 template <typename T, int TX, int TY>
 __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, T *sblk, T &s_ta, T &s_tb, T *s_ue,

@@ -6,15 +6,18 @@
 // operator matches the fine one under trilinear prolongation); restriction
 // is the transpose of trilinear prolongation (27 fine nodes per coarse
 // node).  The Chebyshev bound is the largest eigenvalue of diag(K_e)^-1 K_e
-// of the 3D element.  All levels run on the whole grid, one tiled sweep of
-// the operator (the exact cell decomposition of cell_force3 / node_force3)
-// and one grid barrier per Chebyshev step; the CG update and the last step
-// of each smoothing are folded into neighbouring sweeps as in 2D.  Data
-// written by other blocks is read only after the grid barrier that follows
-// the write (an acquire at GPU scope), so such loads may be cached in L1:
-// the epilogues' operands are prefetched into L1 when a plane's work begins,
-// and the restriction and prolongation gathers, which read each value from
-// several neighbouring nodes, go through L1.
+// of the 3D element.  All levels run on the whole grid, one sweep of the
+// operator and one grid barrier per Chebyshev step; the last step of each
+// smoothing is applied in the epilogue of the step before it.  FP32: warps
+// march (pf_march3.cuh), the CG update and the restriction are passes of their
+// own.  FP64: tiled sweeps (mg_sweep3z, the exact cell decomposition of
+// cell_force3 / node_force3) with the CG update folded into the finest level's
+// first one and the restriction into a coarse level's, as in 2D.  Data written
+// by other blocks is read only after the grid barrier that follows the write
+// (an acquire at GPU scope), so such loads may be cached in L1: the FP64
+// epilogues' operands are prefetched into L1 when a plane's work begins, and
+// the restriction and prolongation gathers, which read each value from several
+// neighbouring nodes, go through L1.
 #pragma once
 
 namespace pfdev {

@@ -368,11 +368,13 @@ __global__ void k_adam(long long n, float *w, const float *g, float *m, float *v
 }
 
 constexpr int LAY_BLOCKS = 48;     // blocks per layer of the all-layer kernels
+constexpr int UN_SMS = 152;        // SMs of the GPU this is written for: sizes grids, nothing depends on it
+constexpr int UN_MAX_BLOCKS = 32 * UN_SMS;
 
 int blocks_for(long long n, int per = 256)
 {
     long long b = (n + per - 1) / per;
-    if (b > 152 * 32) b = 152 * 32;
+    if (b > UN_MAX_BLOCKS) b = UN_MAX_BLOCKS;
     if (b < 1) b = 1;
     return (int)b;
 }
@@ -494,7 +496,7 @@ int launch_conv(int cout, ConvArgs a, long long tiles, cudaStream_t s)
 {
     a.cout = cout;
     // fewer tiles than SMs: 16 output channels per block (see k_conv3)
-    if (tiles < 152) {
+    if (tiles < UN_SMS) {
         launch_conv_t<D, 16, true>(a, tiles, s);
         return PF_OK;
     }
@@ -515,7 +517,7 @@ int launch_conv(int cout, ConvArgs a, long long tiles, cudaStream_t s)
 template <int D, int C>
 void launch_wgrad_t(const WGradArgs &a, int cin, cudaStream_t s)
 {
-    long long gx = a.ntiles < 152 * 2 ? a.ntiles : 152 * 2;
+    long long gx = a.ntiles < 2 * UN_SMS ? a.ntiles : 2 * UN_SMS;
     dim3 grid((unsigned)gx, (unsigned)(cin / 16), (unsigned)wgrad_zsplit<D, C>());
     k_conv3_wgrad<D, C><<<grid, 256, wgrad_smem<D, C>(), s>>>(a);
 }
@@ -727,7 +729,7 @@ int backward_t(pf_unet *n, UWork *w, const float *in, const float *target, doubl
     const __nv_bfloat16 *d0 = L > 1 ? w->dec2[0] : w->enc2[0];
     {
         float *gd = L > 1 ? w->g_d[0] : w->g_a[0], *gW = n->grad + O.woff, *gb = n->grad + O.boff;
-        const int nb = std::min(blocks_for(c0 * (O.ci / 8)), 608);
+        const int nb = std::min(blocks_for(c0 * (O.ci / 8)), 4 * UN_SMS);
         const float *W = n->params + O.woff;
         switch (O.co) {
         case 2: k_out_bwd<2><<<nb, chan_threads(O.ci), 0, s>>>(c0, O.ci, d0, W, w->gy, gd, gW, gb); break;
@@ -876,7 +878,7 @@ int pf_unet_create(const pf_unet_config *cfg, pf_unet **out)
     A(&n->grad, sizeof(float) * n->nparam);
     A(&n->m, sizeof(float) * n->nparam);
     A(&n->v, sizeof(float) * n->nparam);
-    A(&n->part, sizeof(double) * 152 * 32);
+    A(&n->part, sizeof(double) * UN_MAX_BLOCKS);
     for (ConvLayer &lay : n->layers) {
         if (lay.taps == 1) continue;
         A(&lay.wf, sizeof(__nv_bfloat16) * lay.taps * lay.co * lay.cip);
