@@ -84,15 +84,16 @@ struct PCGArgs {
 // `region` picks one of PCG_REGIONS sets of partials: a set may be written
 // again only after another barrier has passed since it was read.  Waits are
 // bounded (SPIN_LIMIT polls, then PF_ETIMEOUT in *err and false is returned).
-constexpr int PCG_REGIONS = 3;
+// The scratch is sized for the largest block, 512 threads.
+constexpr int PCG_REGIONS = 3, PCG_MAX_WARPS = 16;
 
 template <typename AccT, int K>
 __device__ __forceinline__ bool reduce_barrier(AccT (&acc)[K], double *partials, int region, unsigned int *count,
                                             unsigned int *gen, int *err, double *out, int bid, int nbk)
 {
     constexpr bool pairs = std::is_same<AccT, Acc<float>>::value;
-    __shared__ float sh[pairs ? K : 1][32], sl[pairs ? K : 1][32];
-    __shared__ double sd[pairs ? 1 : K][32];
+    __shared__ float sh[pairs ? K : 1][PCG_MAX_WARPS], sl[pairs ? K : 1][PCG_MAX_WARPS];
+    __shared__ double sd[pairs ? 1 : K][PCG_MAX_WARPS];
     __shared__ int s_ok;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
     double *const part = partials + (size_t)region * nbk * PSTRIDE;
@@ -509,6 +510,8 @@ template <typename T> struct MGStore<T, false> {};
 
 template <int D, int S>
 constexpr int tile_threads() { return Tile<D, S>::X * Tile<D, S>::Y * Tile<D, S>::Z; }
+static_assert(tile_threads<2, 1>() <= 32 * PCG_MAX_WARPS && tile_threads<3, 0>() <= 32 * PCG_MAX_WARPS &&
+              MG3_THREADS <= 32 * PCG_MAX_WARPS, "warps of a block");
 
 // The Jacobi loops' scalars after a sweep's reduction (tt: gamma, delta,
 // ||r||^2, mean-strain row): counts the iteration, tests ||r|| <= target, takes
@@ -539,6 +542,41 @@ __device__ __forceinline__ int pcg_step(PCGState &S, const double *tt, bool was_
     }
     __syncthreads();
     return s_ctl;
+}
+
+// Refinement, own nodes: the pass's correction (A.x, S.XE) added to the
+// solution.  If the solution had met the tolerance, A.u (written at the end of
+// the solve) and S.cE keep the correction for refine_undo.
+template <typename T, int D>
+__device__ __noinline__ void refine_add(const PCGArgs<T, D> &A, PCGState &S, int bid, int nbk)
+{
+    const long long N = A.P.N, t0 = bid * (long long)blockDim.x + threadIdx.x, st = (long long)nbk * blockDim.x;
+    const bool keep = S.met != 0;
+    for (int d = 0; d < D; d++) {
+        const T *__restrict__ x = A.x[d];
+        double *__restrict__ y = A.x64[d];
+#pragma unroll 4
+        for (long long n = t0; n < N; n += st) y[n] += (double)x[n];
+        T *__restrict__ u = A.u[d];
+        if (keep)
+            for (long long n = t0; n < N; n += st) u[n] = x[n];
+    }
+    if (threadIdx.x == 0)
+        for (int v = 0; v < Dims<D>::NV; v++) {
+            S.cE[v] = S.XE[v];
+            S.E64[v] += S.XE[v];
+            if (bid == 0) A.emean[v] = S.E64[v];
+        }
+}
+// ... and taken back (x64 to its rounding)
+template <typename T, int D>
+__device__ __noinline__ void refine_undo(const PCGArgs<T, D> &A, PCGState &S, int bid, int nbk)
+{
+    for (long long n = bid * (long long)blockDim.x + threadIdx.x; n < A.P.N; n += (long long)nbk * blockDim.x)
+#pragma unroll
+        for (int d = 0; d < D; d++) A.x64[d][n] -= (double)A.u[d][n];
+    if (threadIdx.x == 0)
+        for (int v = 0; v < Dims<D>::NV; v++) S.E64[v] -= S.cE[v];
 }
 
 // threads of a block: one per tile node; 3D in FP32 (pf_march3.cuh): MG3_THREADS
@@ -781,12 +819,7 @@ k_pcg(const PCGArgs<T, D> *jobs, int njobs)
         if (ctl0 == CTL_DONE) { conv = true; break; }
         if (ctl0 == CTL_STOP) { conv = false; break; }
         if (ctl0 == CTL_UNDO) {
-            // (A.u holds the last correction; x64 comes back to its rounding)
-            for (long long n = t0; n < N; n += st)
-#pragma unroll
-                for (int d = 0; d < D; d++) A.x64[d][n] -= (double)A.u[d][n];
-            if (lead)
-                for (int vv = 0; vv < NV; vv++) E64[vv] -= S.cE[vv];
+            refine_undo<T, D>(A, S, bid, nbk);
             conv = true;
             break;
         }
@@ -1083,22 +1116,7 @@ k_pcg(const PCGArgs<T, D> *jobs, int njobs)
         if (stop == CTL_DONE) { conv = true; break; }
         // x64 += correction, then a grid-wide sync before the next pass reads
         // x64 around every node
-        const bool keep = S.met != 0;
-        for (long long n = t0; n < N; n += st)
-#pragma unroll
-            for (int d = 0; d < D; d++) {
-                const T c = A.x[d][n];
-                A.x64[d][n] += (double)c;
-                if (keep) A.u[d][n] = c;
-            }
-        if (lead) {
-            for (int vv = 0; vv < NV; vv++) {
-                S.cE[vv] = XE[vv];
-                E64[vv] += XE[vv];
-            }
-            if (bid == 0)
-                for (int vv = 0; vv < NV; vv++) A.emean[vv] = E64[vv];
-        }
+        refine_add<T, D>(A, S, bid, nbk);
         if (!grid_sync(A.bar_count, A.bar_gen, err, nbk)) return;
         if (stop == CTL_STOP) { conv = false; break; }
     }
