@@ -7,9 +7,11 @@ Tuned choices (every one changes speed only: the results agree to rounding,
 or are identical for the marching update):
 
   * PCG node tile (pf_config.pcg_tile = 1, 2) of the Jacobi-preconditioned
-    solve, per size class (2D up to 2^18 nodes, 2D above, 3D) and storage
-    type (not 3D FP32, whose sweeps use no tile): a core-shell grid of the class is stepped with each tile and the
-    solve time per CG iteration (the library's CUDA-event profile) decides;
+    solve, per size class (2D up to 2^18 nodes, 2D above, 3D; a 2D grid with
+    no more 32x8 tiles than SMs takes those) and storage type (not 3D FP32,
+    whose sweeps use no tile): a core-shell grid of the class is stepped with
+    each tile and the solve time per CG iteration (the library's CUDA-event
+    profile) decides;
   * the same choice for the 2D multigrid-preconditioned solve, where it sets
     the block size (256 or 512 threads; its V-cycle's sweeps use no tile)
     and the set-up's tile, per 2D size class and storage type, decided by
@@ -33,7 +35,7 @@ JSON_PATH = os.path.join(HERE, "data", "autotune_gb300.json")
 HEADER_PATH = os.path.join(HERE, "csrc", "tuning.h")
 
 PCG_CLASSES = [
-    ("2D", "SMALL", (512, 512)),        # <= 2^18 nodes
+    ("2D", "SMALL", (320, 320)),        # <= 2^18 nodes, more 32x8 tiles than SMs
     ("2D", "LARGE", (1024, 1024)),
     ("3D", None, (96, 96, 96)),
 ]

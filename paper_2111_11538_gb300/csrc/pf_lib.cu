@@ -356,9 +356,15 @@ std::vector<pf_handle *> instances(pf_handle *h)
 // Node tile of the Jacobi PCG's sweep for a grid of N nodes (pf_config.pcg_tile
 // 1 or 2 select shape 0 or 1): the per-size-class choice measured on GB300
 // (paper_2111_11538_gb300/autotune.py prints the table).
-int default_pcg_shape(int ndim, long long N, bool fp64)
+// A 2D grid whose 32x8 tiles do not outnumber the SMs takes them: each block
+// then has an SM to itself with half the threads of the other shape's (37 x 29,
+// us per iteration, 32x8 / 32x16: FP64 19.0 / 28.8, mixed 9.3 / 11.2; 101 x 99
+// FP64 19.0 / 28.4; 255 x 257, 264 tiles, FP64 32.1 / 29.6).
+int default_pcg_shape(int ndim, int nx, int ny, int sms, bool fp64)
 {
+    const long long N = (long long)nx * ny;
     if (ndim == 2) {
+        if ((long long)((nx + Tile<2, 0>::X - 1) / Tile<2, 0>::X) * ((ny + Tile<2, 0>::Y - 1) / Tile<2, 0>::Y) <= sms) return 0;
         if (fp64) return N <= (1LL << 18) ? PCG_TABLE_2D_F64_SMALL : PCG_TABLE_2D_F64_LARGE;
         return N <= (1LL << 18) ? PCG_TABLE_2D_F32_SMALL : PCG_TABLE_2D_F32_LARGE;
     }
@@ -531,7 +537,7 @@ int setup_cg_launch(pf_handle *h)
     h->pcg_shape = D == 3 && !fp64       ? 0
                    : h->cfg.pcg_tile > 0 ? h->cfg.pcg_tile - 1
                    : h->mg               ? (D == 2 ? mg2_pcg_shape(h->P.N, fp64) : 0)
-                                         : default_pcg_shape(D, h->P.N, fp64);
+                                         : default_pcg_shape(D, h->P.nx, h->P.ny, h->sms, fp64);
     h->cg_block = h->pcg_shape ? pcg_threads<T, D, 1, true>() : pcg_threads<T, D, 0, true>();
     if (h->mg) PF_TRY((build_mg<T, D>(h)));
     int per_sm = 0;

@@ -4,8 +4,8 @@
 #pragma once
 #define FUSED_STARTUP_2D 1
 #define FUSED_STARTUP_3D 1
-#define PCG_TABLE_2D_F32_LARGE 0
-#define PCG_TABLE_2D_F32_SMALL 0
+#define PCG_TABLE_2D_F32_LARGE 1
+#define PCG_TABLE_2D_F32_SMALL 1
 #define PCG_TABLE_2D_F64_LARGE 0
 #define PCG_TABLE_2D_F64_SMALL 1
 #define PCG_TABLE_3D_F64 0
