@@ -546,7 +546,6 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
     const bool lead = threadIdx.x == 0;
     const int L = H.L, Lgw = H.Lg < H.L ? H.Lg : H.L, cs = H.csteps;
     const MGLevel<T> &L0 = H.lv[0];
-    unsigned int *bc = A.bar_count, *bg = A.bar_gen;
     // the sweeps' place in the dynamic shared memory; the operation's record
     // there is filled by the lead thread (every sweep follows a barrier of the
     // whole block) and read by all
@@ -628,7 +627,7 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
             }
             __syncthreads();
             m2_sweep2<T, NT, OFF, OpPostPair2<T>>(V.nx, V.ny, A.zc2[k], bid, nbk);
-            return grid_sync(bc, bg, err, nbk);
+            return grid_sync(A.bar_count, A.bar_gen, err, nbk);
         } else {
             OpPost2<T> &op = *reinterpret_cast<OpPost2<T> *>(s_op);
             static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
@@ -642,10 +641,10 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
             }
             __syncthreads();
             m2_sweep<T, NT, OFF, OpPost2<T>>(V.nx, V.ny, A.zc1[k], bid, nbk);
-            if (!grid_sync(bc, bg, err, nbk)) return false;
+            if (!grid_sync(A.bar_count, A.bar_gen, err, nbk)) return false;
             if (k == 0) return true;
             cheb(k, 0, 0, true, true);
-            return grid_sync(bc, bg, err, nbk);
+            return grid_sync(A.bar_count, A.bar_gen, err, nbk);
         }
     };
     // pre-smoothing of grid level k >= 1 (two steps), or the coarsest solve
@@ -663,7 +662,7 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
             }
             __syncthreads();
             m2_sweep2<T, NT, OFF, OpPrePair2<T>>(V.nx, V.ny, A.zc2[k], bid, nbk);
-            return grid_sync(bc, bg, err, nbk);
+            return grid_sync(A.bar_count, A.bar_gen, err, nbk);
         }
         OpPre2<T> &op = *reinterpret_cast<OpPre2<T> *>(s_op);
         static_assert(sizeof(op) <= M2_OP_BYTES, "operation record");
@@ -675,13 +674,13 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
         }
         __syncthreads();
         m2_sweep<T, NT, OFF, OpPre2<T>>(V.nx, V.ny, A.zc1[k], bid, nbk);
-        if (!grid_sync(bc, bg, err, nbk)) return false;
+        if (!grid_sync(A.bar_count, A.bar_gen, err, nbk)) return false;
         int par = 1;
         const bool co = k == L - 1;
         const int nk = co ? cs - 1 : H.deg[k];
         for (int j = 1; j < nk; j++) {
             cheb(k, j, par, co && j + 1 == nk, false);
-            if (!grid_sync(bc, bg, err, nbk)) return false;
+            if (!grid_sync(A.bar_count, A.bar_gen, err, nbk)) return false;
             par ^= 1;
         }
         return true;
@@ -892,7 +891,7 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
             cur = nxt;
             const int ctl = s_ctl;
             if (ctl != CTL_RUN) return ctl;
-        } else if (!grid_sync(bc, bg, err, nbk)) {
+        } else if (!grid_sync(A.bar_count, A.bar_gen, err, nbk)) {
             return -1;
         }
 
@@ -901,7 +900,7 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
             int par = 1;
             for (int j = 1; j < cs - 1; j++) {
                 cheb(0, j, par, j + 2 == cs, false);
-                if (!grid_sync(bc, bg, err, nbk)) return -1;
+                if (!grid_sync(A.bar_count, A.bar_gen, err, nbk)) return -1;
                 par ^= 1;
             }
         }
@@ -913,7 +912,7 @@ __device__ int mg_pass(const PCGArgs<T, 2> &A, const MGHier<T> &H, PCGState &S, 
             } else {
                 block64();
             }
-            if (!grid_sync(bc, bg, err, nbk)) return -1;
+            if (!grid_sync(A.bar_count, A.bar_gen, err, nbk)) return -1;
         }
         for (int k = (Lgw < L - 1 ? Lgw : L - 1) - 1; k >= (PAIR ? 1 : 0); k--)
             if (!post(k, cur)) return -1;
