@@ -55,10 +55,10 @@ MG_INIT_WORDS = {2: 28, 3: 40}
 # from one ncu capture of the current kernel on the named workload, per
 # finest node and V-cycle (so that it scales with the launch's iterations);
 # None where the current kernel has not been captured.  porous256cube: the
-# first timed solve of `bench.py --only mixed --steps 1 --warmup 4` (44
-# V-cycles), 139.35 GB read + 85.84 GB written = 305.1 B per node and V-cycle
+# timed solve of `bench.py --only mixed --steps 1 --warmup 4` (51 V-cycles),
+# 162.31 GB read + 92.74 GB written = 298.1 B per node and V-cycle
 # (profiles/launches_porous256_mixed.md).
-PCG_TRAFFIC_PER_NODE_ITER = {"porous256cube": 305.05}
+PCG_TRAFFIC_PER_NODE_ITER = {"porous256cube": 298.08}
 # Algorithmic bytes per cell of the fused explicit update (k_fusedz): theta,
 # phi_g, x_O, x_H, x_H2O, tr eps_e, |dev eps_e|^2, mobility read, the 1-byte
 # supply mask read, theta, x_O, x_H, x_H2O written.
