@@ -37,7 +37,8 @@ struct Lanes2 {
     }
 };
 
-// the row's displacement and its difference to the right neighbour
+// the row's displacement (FP32: its sum with the right neighbour's) and its
+// difference to the right neighbour
 template <typename T>
 struct Row2 {
     T v[2], d[2];
@@ -48,20 +49,25 @@ __device__ __forceinline__ void row2(const T (&v)[2], const Lanes2 &Ln, Row2<T> 
 {
 #pragma unroll
     for (int c = 0; c < 2; c++) {
-        R.v[c] = v[c];
-        R.d[c] = __shfl_sync(0xffffffffu, v[c], Ln.nxt) - v[c];
+        const T r = __shfl_sync(0xffffffffu, v[c], Ln.nxt);
+        R.v[c] = sizeof(T) == 8 ? v[c] : v[c] + r;
+        R.d[c] = r - v[c];
     }
 }
 
 // Corner-force coefficients of the cell between rows lo and hi (l4, m4: a
 // quarter of its moduli): the force on its corner (sx, sy), s = -1 or +1, is
 // sx ax + sy ay + sx sy axy per component.  This is cell_force2 /
-// node_force2 with the sums along x and y taken apart.  Differences of
-// neighbours come first, as there: they are nearly exact where the field is
-// smooth (the y gradient, the sum of both columns' differences, is 2 (hi.v -
-// lo.v) + (hi.d - lo.d)).  The difference of the rows' sums, as many
-// operations, costs digits: relative error of A u in FP64 at 256^2, a smooth
-// u, 2.6e-14 against 1.3e-15.
+// node_force2 with the sums along x and y taken apart.
+// FP64 takes differences of neighbours first, as there: they are nearly exact
+// where the field is smooth (the y gradient, the sum of both columns'
+// differences, is 2 (hi.v - lo.v) + (hi.d - lo.d)).  The difference of the rows'
+// sums, as many operations, costs digits: relative error of A u at 256^2, a
+// smooth u, 5.1e-14 against 2.6e-15, at 2048^2 3.3e-12 against 2.1e-14.
+// FP32, whose passes only precondition the FP64 residual, takes the rows' sums:
+// the FP64 residual after a pass is the pass's own to 2 % up to 8192^2, the
+// V-cycles are as many either way, and differences first take 2 to 3 % longer
+// (a chain longer by one operation; 2048^2 0.471 and 0.481 ms per V-cycle).
 template <typename T>
 struct Cell2 {
     T ax0, sh, ay1, xy[2];          // ax = (ax0, sh), ay = (sh, ay1)
@@ -72,7 +78,8 @@ __host__ __device__ __forceinline__ Cell2<T> cell2(T l4, T m4, const Row2<T> &lo
 {
     const T gxu = lo.d[0] + hi.d[0], gxv = lo.d[1] + hi.d[1];
     const T xyu = hi.d[0] - lo.d[0], xyv = hi.d[1] - lo.d[1];
-    const T gyu = T(2) * (hi.v[0] - lo.v[0]) + xyu, gyv = T(2) * (hi.v[1] - lo.v[1]) + xyv;
+    const T dyu = hi.v[0] - lo.v[0], dyv = hi.v[1] - lo.v[1];
+    const T gyu = sizeof(T) == 8 ? T(2) * dyu + xyu : dyu, gyv = sizeof(T) == 8 ? T(2) * dyv + xyv : dyv;
     const T lt = l4 * (gxu + gyv), m2 = m4 + m4;
     const T ch = (l4 + T(3) * m4) * T(1.0 / 3.0);
     Cell2<T> C;
