@@ -788,16 +788,17 @@ k_pcg(const PCGArgs<T, D> *jobs, int njobs)
                 // mode what an FP32 iteration can deliver on this correction
                 // (eta); when the final tolerance is not far below that, the pass
                 // aims for it directly, which saves a pass that would otherwise
-                // start just above the tolerance: within a factor 100 with the
-                // V-cycle, 10 without.  (Jacobi-preconditioned FP32 passes on 2D
-                // grids of 10^4 nodes and more do not always get down to 3e-5 of
-                // where they start, and ran on to cg_maxit: of 30 core-shells of
-                // 224 x 138, rtol 1e-10, 15 failed with 100 here, none with 10;
-                // 0.5 tol and 100, before the solves went on to half the
-                // tolerance, 6.  The iterations are as many.)
+                // start just above the tolerance: within a factor 100, but 10
+                // with the Jacobi preconditioner on axes of more than 64 nodes.
+                // (FP32 passes there do not always get down to 3e-5 of where they
+                // start, and ran on to cg_maxit: of 30 core-shells of 224 x 138,
+                // rtol 1e-10, 15 failed with 100 here, none with 10; 0.5 tol and
+                // 100, before the solves went on to half the tolerance, 6.  The
+                // iterations are as many; on small grids 10 costs a few per cent.)
                 if (refine) {
+                    const bool deep = MG || max(P.nx, max(P.ny, D == 3 ? P.nz : 1)) <= 64;
                     const double fin = 0.25 * tol, pass = A.eta * res;
-                    target = fin >= (MG ? 0.01 : 0.1) * pass ? fin : pass;
+                    target = fin >= (deep ? 0.01 : 0.1) * pass ? fin : pass;
                 } else {
                     target = A.rtol * bnorm;
                 }
