@@ -542,7 +542,7 @@ def backward_euler_line(n=256, steps=3, dt=0.05, explicit_steps=20):
 # FP32 lanes x 2 flops x 2.07 GHz (the counters' FFMA peak of 128 per cycle
 # and SM; the maximum SM clock).
 FS_HVP_FLOPS_PER_CELL = 10036.4
-FS_HVP_DRAM_PER_CELL = 114.4
+FS_HVP_DRAM_PER_CELL = 115.2
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 
 
