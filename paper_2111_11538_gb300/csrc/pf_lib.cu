@@ -371,6 +371,14 @@ int default_pcg_shape(int ndim, int nx, int ny, int sms, bool fp64)
     return PCG_TABLE_3D_F64;
 }
 
+// The same for a 2D batch, by its first grid.  A launch holds an instance per
+// resident block at most: FP32 takes 32x8 tiles, two blocks to an SM, whatever
+// the size (304 instances; the 512-thread blocks of the other shape 152).
+int batch_pcg_shape(long long N, bool fp64)
+{
+    return !fp64 ? 0 : N <= (1LL << 18) ? PCG_TABLE_2D_F64_SMALL : PCG_TABLE_2D_F64_LARGE;
+}
+
 // Block size (256 or 512 threads) and set-up tile of the 2D multigrid solve,
 // per size class.
 int mg2_pcg_shape(long long N, bool fp64)
@@ -1671,6 +1679,8 @@ int pf_batch_create(const pf_config *cfgs, int n, pf_handle **out)
         std::string err;
         pf_config ci = cfgs[i];
         if (ci.precond == PF_PC_AUTO) ci.precond = all_mg ? PF_PC_MG : PF_PC_JACOBI;
+        if (n > 1 && ci.ndim == 2 && ci.precond == PF_PC_JACOBI && ci.pcg_tile == 0)
+            ci.pcg_tile = 1 + batch_pcg_shape((long long)cfgs[0].nx * cfgs[0].ny, ci.precision == PF_FP64);
         int rc = create_one(&ci, &m, err);
         if (rc != PF_OK) {
             char buf[64];
